@@ -11,7 +11,10 @@
 // and the same for each component of A with (U, sigma2, J^{n+1/2}).
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "pic_internal.h"
+#include "orbit_cell.cuh"
 
 namespace pic {
 namespace {
@@ -355,6 +358,38 @@ __global__ void k_backsub_table(MeshParams p, const double* __restrict__ F0, con
     }
 }
 
+// Cell table (orbit_cell.cuh) from the gather table: one thread per cell and column takes the
+// column's 8 node values to their mixed differences.  Writes 576 B a cell, 18 doubles apart per
+// thread with a cell's columns on neighbouring threads.
+__global__ void k_cell_table(MeshDims m, const double* __restrict__ table, double2* __restrict__ ctab) {
+    const int64_t total = m.ncell * CELL_COLS;
+    GRID_LOOP(idx, total) {
+        const int64_t cell = idx / CELL_COLS;
+        const int col = (int)(idx - cell * CELL_COLS);
+        int c[3];
+        c[0] = (int)(cell % m.n[0]);
+        const int64_t t = cell / m.n[0];
+        c[1] = (int)(t % m.n[1]);
+        c[2] = (int)(t / m.n[1]);
+        int64_t g[8];
+        cell_nodes8(c, m, g);
+        double f[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const double* q = table + 12 * g[k];
+            f[k] = col < 3 ? q[3 + col] : (col < 6 ? q[col] - q[col - 3] : -q[col]);
+        }
+#pragma unroll
+        for (int bit = 1; bit < 8; bit <<= 1)
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (k & bit) f[k] -= f[k ^ bit];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            ctab[cell * (CELL_VALUES / 2) + q * CELL_COLS + col] = make_double2(f[2 * q], f[2 * q + 1]);
+    }
+}
+
 // Field energy W = sum_g (|E|^2 / (2 sigma1) + |B|^2 / (2 sigma2)) dV, E = -grad phi - U, B = curl A.
 __device__ __forceinline__ double node_energy(const MeshParams& p, const double* F, const double* W, const Nb& b) {
     const int64_t N = p.m.ncell;
@@ -584,6 +619,13 @@ int cheb_coop_capacity(const Ctx& c) {
 
 void launch_backsub_table(Ctx& c, bool) {
     k_backsub_table<<<mesh_blocks(c), THREADS, 0, c.stream>>>(mesh_params(c), c.F0, c.W0, c.F1, c.W1, c.table);
+    ++c.launches;
+}
+
+void launch_cell_table(Ctx& c) {
+    const int64_t b = (c.m.ncell * CELL_COLS + THREADS - 1) / THREADS;
+    const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)c.sms * 16));
+    k_cell_table<<<nb, THREADS, 0, c.stream>>>(c.m, c.table, reinterpret_cast<double2*>(c.ctab));
     ++c.launches;
 }
 

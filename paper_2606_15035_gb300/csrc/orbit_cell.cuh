@@ -1,0 +1,297 @@
+// Orbit integrals in centred form, and the cell table they contract with.
+//
+// The orbit of one particle over a step is cut at the knots it crosses (§4.7, Eq.
+// (breakpoint-set)).  Inside one piece [s0, s0 + h] the orbit stays in one cell, where every
+// mesh field of linear splines is the trilinear polynomial
+//     f(w) = sum_k f_k prod_{a in k} w_a,   k = subsets of {x, y, z} (bit a = axis a),
+// w_a in [0, 1] the coordinate in the cell and f_k the mixed differences of the cell's 8 node
+// values.  With u = s - s_mid running over [-h/2, h/2] the orbit is w_a = m_a + beta_a u, m_a its
+// midpoint, and odd powers of u integrate to zero, so the closed forms of Appendices A and B
+// become, per unit of h and with e_a = beta_a h^2 / 12,
+//     <w_a>         = m_a                         <u w_a>     = e_a
+//     <w_p w_q>     = P_pq = m_p m_q + e_p beta_q  <u w_p w_q> = m_p e_q + m_q e_p
+//     <w_x w_y w_z> = m_x P_yz + m_y e_x beta_z + m_z e_x beta_y          <u> = 0.
+// That is 20 operations where the integrals from the piece's start took 74, and the 8 node
+// weights with their 8-node differences (16 + 84) disappear into the table.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "pic_device.cuh"
+
+namespace pic {
+
+// Cell table: per cell and k the 9 columns A^{n+1} (3), A^{n+1} - A^n (3), -grad phi^{n+1/2} (3),
+// k in pairs (2 p, 2 p + 1) that one 16-byte load brings: entry [p][column][k & 1].
+constexpr int CELL_COLS = 9;
+constexpr int CELL_VALUES = 8 * CELL_COLS;
+
+// Order and range tests of the walk.  On doubles they run on the integer pipe (for values >= 0
+// the bit patterns order like the values; the sign and exponent decide t < 0 and t >= 1): the
+// FP64 pipe, which has 1/64 of the issue rate, is what bounds the particle kernels.
+__device__ __forceinline__ bool less_pos(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
+__device__ __forceinline__ bool same_bits(double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); }
+__device__ __forceinline__ bool at_least_one(double t) { return __double2hiint(t) >= 0x3ff00000; }
+__device__ __forceinline__ bool below_zero(double t) { return __double2hiint(t) < 0; }
+__device__ __forceinline__ bool is_zero(double t) { return (__double_as_longlong(t) << 1) == 0; }
+
+// A particle's start: cell and coordinate in it.
+template <typename T>
+struct CellStart {
+    T f[3];
+    int c[3];
+};
+
+// c + 1 and c - 1 on a periodic axis of n cells, c in [0, n)
+__device__ __forceinline__ int next_cell(int c, int n) { return c + 1 >= n ? 0 : c + 1; }
+__device__ __forceinline__ int prev_cell(int c, int n) { return c > 0 ? c - 1 : n - 1; }
+
+// Visit the knot-free pieces of the orbit st.f + s beta: visit(h, s_mid, mid, cell), h > 0.  On
+// return st.c is the end point's cell and st.f the end point's coordinate in it (in [0, 1]; an
+// end exactly on a knot keeps the cell it came from, where the fields have the same value).
+// Returns the number of breakpoint intervals, or -1 if MAX_SEGMENTS was exceeded.  Cells stay in
+// [0, n) whatever the input.
+template <typename T, typename F>
+__device__ __forceinline__ int for_each_piece(CellStart<T>& st, const T beta[3], const MeshDims& m, F&& visit) {
+    T fd[3], te[3], sn[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        fd[a] = st.f[a];                       // start coordinate relative to the current cell
+        te[a] = fd[a] + beta[a];               // end coordinate relative to the current cell
+        if (below_zero(te[a]) && is_zero(fd[a])) {   // on a knot, moving down: the cell below
+            st.c[a] = prev_cell(st.c[a], m.n[a]);
+            fd[a] = T(1);
+            te[a] = T(1) + beta[a];
+        }
+        sn[a] = T(2);                          // next crossing of this axis (2: none)
+        if (at_least_one(te[a])) sn[a] = (T(1) - fd[a]) / beta[a];
+        else if (below_zero(te[a])) sn[a] = fd[a] / -beta[a];
+        if (!less_pos(sn[a], T(1))) sn[a] = T(2);
+    }
+    T s0 = T(0);
+    int count = -1;
+    for (int it = 0; it < MAX_SEGMENTS; ++it) {
+        T s1 = T(1);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) s1 = less_pos(sn[a], s1) ? sn[a] : s1;
+        if (less_pos(s0, s1)) {
+            const T h = s1 - s0, sm = T(0.5) * (s0 + s1);
+            T mid[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) mid[a] = fd[a] + sm * beta[a];
+            visit(h, sm, mid, st.c);
+        }
+        if (same_bits(s1, T(1))) {
+            count = it + 1;
+            break;
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if (!same_bits(sn[a], s1)) continue;
+            sn[a] = T(2);
+            if (!below_zero(te[a])) {
+                st.c[a] = next_cell(st.c[a], m.n[a]);
+                fd[a] = fd[a] - T(1);
+                te[a] = te[a] - T(1);
+                if (at_least_one(te[a])) sn[a] = (T(1) - fd[a]) / beta[a];
+            } else {
+                st.c[a] = prev_cell(st.c[a], m.n[a]);
+                fd[a] = fd[a] + T(1);
+                te[a] = te[a] + T(1);
+                if (below_zero(te[a])) sn[a] = fd[a] / -beta[a];
+            }
+            if (!less_pos(sn[a], T(1))) sn[a] = T(2);
+        }
+        s0 = s1;
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) st.f[a] = te[a];
+    return count;
+}
+
+// The moments of one piece per unit of h (see the file comment).
+template <typename T>
+struct PieceMoments {
+    T m[3];              // <w_a>
+    T Pxy, Pxz, Pyz, S;  // <w_p w_q>, <w_x w_y w_z>
+    T e[3];              // <u w_a>
+};
+
+template <typename T>
+__device__ __forceinline__ PieceMoments<T> piece_moments(T h, const T mid[3], const T beta[3]) {
+    PieceMoments<T> q;
+    const T k = h * h * T(1.0 / 12.0);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        q.m[a] = mid[a];
+        q.e[a] = k * beta[a];
+    }
+    const T kxy = q.e[0] * beta[1], kxz = q.e[0] * beta[2], kyz = q.e[1] * beta[2];
+    q.Pxy = mid[0] * mid[1] + kxy;
+    q.Pxz = mid[0] * mid[2] + kxz;
+    q.Pyz = mid[1] * mid[2] + kyz;
+    q.S = mid[0] * q.Pyz + (mid[1] * kxz + mid[2] * kxy);
+    return q;
+}
+
+// The 8 node weights of Appendix A per unit of h, node nu = nx + 2 ny + 4 nz.
+template <typename T>
+__device__ __forceinline__ void node_weights(const PieceMoments<T>& q, T W[8]) {
+    W[7] = q.S;
+    W[3] = q.Pxy - q.S;
+    W[5] = q.Pxz - q.S;
+    W[6] = q.Pyz - q.S;
+    W[1] = q.m[0] - q.Pxy - W[5];
+    W[2] = q.m[1] - q.Pyz - W[3];
+    W[4] = q.m[2] - q.Pxz - W[6];
+    W[0] = T(1) - q.m[0] - W[2] - W[4] - W[6];
+}
+
+// One piece's impulse, acc_j += int ((D_j A)^T v - d_j phi) over the piece (Eqs.
+// (gphibar-definition) and (DA-def)), vs = scale v and ihs_j = 1 / (scale H_j).  `ld(p, col, a, b)`
+// loads entries k = 2 p and 2 p + 1 of a column of the cell.  A at the time s is
+// A^{n+1} - (1 - s) (A^{n+1} - A^n), contracted with v first.
+template <typename T, typename L>
+__device__ __forceinline__ void piece_impulse(T h, T sm, const T mid[3], const T beta[3], const T vs[3],
+                                              const T ihs[3], L&& ld, T acc[3]) {
+    const PieceMoments<T> q = piece_moments(h, mid, beta);
+    const T oms = T(1) - sm;
+    T F[3], g[3];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        T a[2], cc[2];
+        {
+            T x0, x1, y0, y1, z0, z1;
+            ld(p, 3, x0, x1);
+            ld(p, 4, y0, y1);
+            ld(p, 5, z0, z1);
+            if (p > 0) cc[0] = x0 * vs[0] + y0 * vs[1] + z0 * vs[2];
+            cc[1] = x1 * vs[0] + y1 * vs[1] + z1 * vs[2];
+            ld(p, 0, x0, x1);
+            ld(p, 1, y0, y1);
+            ld(p, 2, z0, z1);
+            if (p > 0) a[0] = x0 * vs[0] + y0 * vs[1] + z0 * vs[2] - oms * cc[0];
+            a[1] = x1 * vs[0] + y1 * vs[1] + z1 * vs[2] - oms * cc[1];
+        }
+        if (p == 0) {            // k = 1: x
+            F[0] = a[1];
+        } else if (p == 1) {     // k = 2: y, k = 3: xy
+            F[0] = F[0] + a[1] * mid[1] + cc[1] * q.e[1];
+            F[1] = a[0] + a[1] * mid[0] + cc[1] * q.e[0];
+        } else if (p == 2) {     // k = 4: z, k = 5: xz
+            F[0] = F[0] + a[1] * mid[2] + cc[1] * q.e[2];
+            F[2] = a[0] + a[1] * mid[0] + cc[1] * q.e[0];
+        } else {                 // k = 6: yz, k = 7: xyz
+            F[1] = F[1] + a[0] * mid[2] + cc[0] * q.e[2];
+            F[2] = F[2] + a[0] * mid[1] + cc[0] * q.e[1];
+            F[0] = F[0] + a[1] * q.Pyz + cc[1] * (mid[1] * q.e[2] + mid[2] * q.e[1]);
+            F[1] = F[1] + a[1] * q.Pxz + cc[1] * (mid[0] * q.e[2] + mid[2] * q.e[0]);
+            F[2] = F[2] + a[1] * q.Pxy + cc[1] * (mid[0] * q.e[1] + mid[1] * q.e[0]);
+        }
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            T g0, g1;
+            ld(p, 6 + j, g0, g1);
+            if (p == 0) g[j] = g0 + g1 * mid[0];
+            else if (p == 1) g[j] = g[j] + g0 * mid[1] + g1 * q.Pxy;
+            else if (p == 2) g[j] = g[j] + g0 * mid[2] + g1 * q.Pxz;
+            else g[j] = g[j] + g0 * q.Pyz + g1 * q.S;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) acc[j] = acc[j] + h * (g[j] + ihs[j] * F[j]);
+}
+
+// A^{n+1} at coordinate r of the cell (Eq. (Ah-mesh)).
+template <typename T, typename L>
+__device__ __forceinline__ void cell_A1(const T r[3], L&& ld, T out[3]) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        T k0, k1, k2, k3, k4, k5, k6, k7;
+        ld(0, c, k0, k1);
+        ld(1, c, k2, k3);
+        ld(2, c, k4, k5);
+        ld(3, c, k6, k7);
+        const T lo = (k0 + k1 * r[0]) + r[1] * (k2 + k3 * r[0]);
+        const T hi = (k4 + k5 * r[0]) + r[1] * (k6 + k7 * r[0]);
+        out[c] = lo + r[2] * hi;
+    }
+}
+
+// Row index of a cell's lowest node, and the 8 node rows of the cell.
+__device__ __forceinline__ int64_t cell_row(const int c[3], const MeshDims& m) {
+    return (int64_t)c[0] + (int64_t)m.n[0] * ((int64_t)c[1] + (int64_t)m.n[1] * c[2]);
+}
+
+__device__ __forceinline__ void cell_nodes8(const int c[3], const MeshDims& m, int64_t g[8]) {
+    const int64_t dx = next_cell(c[0], m.n[0]) - c[0];
+    const int64_t dy = (int64_t)m.n[0] * (next_cell(c[1], m.n[1]) - c[1]);
+    const int64_t dz = (int64_t)m.n[0] * m.n[1] * (next_cell(c[2], m.n[2]) - c[2]);
+    g[0] = cell_row(c, m);
+    g[1] = g[0] + dx;
+    g[2] = g[0] + dy;
+    g[3] = g[2] + dx;
+    g[4] = g[0] + dz;
+    g[5] = g[4] + dx;
+    g[6] = g[4] + dy;
+    g[7] = g[6] + dx;
+}
+
+// Loader of a cell's entries for piece_impulse and cell_A1: from the FP64 cell table, or (CELLS
+// = false, contexts without that table) from the gather table, taking the differences of the
+// cell's nodes each time.
+template <bool CELLS>
+struct FieldLoad {
+    const double2* t;
+    __device__ __forceinline__ FieldLoad(const double* table, const int c[3], const MeshDims& m)
+        : t(reinterpret_cast<const double2*>(table + CELL_VALUES * cell_row(c, m))) {}
+    __device__ __forceinline__ void operator()(int p, int col, double& a, double& b) const {
+        const double2 q = __ldg(t + p * CELL_COLS + col);
+        a = q.x;
+        b = q.y;
+    }
+};
+
+template <>
+struct FieldLoad<false> {
+    const double* t;
+    int64_t g[8];
+    __device__ __forceinline__ FieldLoad(const double* table, const int c[3], const MeshDims& m) : t(table) {
+        cell_nodes8(c, m, g);
+    }
+    __device__ __forceinline__ double node(int k, int col) const {
+        const double* q = t + 12 * g[k];
+        return col < 3 ? __ldg(q + 3 + col) : (col < 6 ? __ldg(q + col) - __ldg(q + col - 3) : -__ldg(q + col));
+    }
+    __device__ __forceinline__ void operator()(int p, int col, double& a, double& b) const {
+        a = node(0, col);
+        b = node(1, col) - a;
+        if (p == 0) return;
+        if (p == 3) {
+            double lo = node(2, col), hi = node(3, col) - lo;
+            a = lo - a;
+            b = hi - b;
+            lo = node(4, col);
+            hi = node(5, col) - lo;
+            const double l6 = node(6, col);
+            a = (l6 - lo) - a;
+            b = ((node(7, col) - l6) - hi) - b;
+        } else {
+            const double lo = node(2 * p, col);
+            a = lo - a;
+            b = (node(2 * p + 1, col) - lo) - b;
+        }
+    }
+};
+
+// The cell and coordinate of an FP64 position in [0, n) (cell units).
+__device__ __forceinline__ void cell_start(const double x0[3], const MeshDims& m, CellStart<double>& st) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double fl = floor(x0[a]);
+        st.f[a] = x0[a] - fl;
+        st.c[a] = min(max((int)fl, 0), m.n[a] - 1);
+    }
+}
+
+}  // namespace pic

@@ -9,6 +9,7 @@
 
 #include "pic_internal.h"
 #include "particle_common.cuh"
+#include "orbit_cell.cuh"
 
 namespace pic {
 
@@ -48,25 +49,27 @@ namespace {
 
 // ---- orbit current scatter (Eq. (orbit-current)) -------------------------------------
 
-// J_c[g] += w_c * Sbar contribution of every piece (closed form, Appendix A).
-__device__ __forceinline__ int scatter_closed(const StepParams& p, const double x0[3], const double beta[3],
+// J_c[g] += w_c * Sbar contribution of every piece (closed form, Appendix A), from the centred
+// moments of orbit_cell.cuh.
+__device__ __forceinline__ int scatter_closed(const StepParams& p, CellStart<double> st, const double beta[3],
                                               const double w[3], double* __restrict__ J) {
     const int64_t N = p.m.ncell;
-    return for_each_segment(x0, beta, true, [&](const Segment<double>& sg) {
-        double I[8];
+    return for_each_piece(st, beta, p.m, [&](double h, double, const double mid[3], const int c[3]) {
+        double W[8];
         int64_t g[8];
-        weights_from_ints(piece_integrals(sg, beta, false), I);
-        segment_nodes8(sg, p.m, g);
+        node_weights(piece_moments(h, mid, beta), W);
+        cell_nodes8(c, p.m, g);
+        const double wh[3] = {h * w[0], h * w[1], h * w[2]};
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             if (p.det) {
-                exact_add(p.acc, g[k], w[0] * I[k]);
-                exact_add(p.acc, N + g[k], w[1] * I[k]);
-                exact_add(p.acc, 2 * N + g[k], w[2] * I[k]);
+                exact_add(p.acc, g[k], wh[0] * W[k]);
+                exact_add(p.acc, N + g[k], wh[1] * W[k]);
+                exact_add(p.acc, 2 * N + g[k], wh[2] * W[k]);
             } else {
-                atomicAdd(J + g[k], w[0] * I[k]);
-                atomicAdd(J + N + g[k], w[1] * I[k]);
-                atomicAdd(J + 2 * N + g[k], w[2] * I[k]);
+                atomicAdd(J + g[k], wh[0] * W[k]);
+                atomicAdd(J + N + g[k], wh[1] * W[k]);
+                atomicAdd(J + 2 * N + g[k], wh[2] * W[k]);
             }
         }
     });
@@ -199,8 +202,11 @@ __device__ __forceinline__ int scatter_gauss_r(const StepParams& p, const double
 template <int QUAD>
 __device__ __forceinline__ int scatter_orbit(const StepParams& p, const double x0[3], const double beta[3],
                                              const double w[3], double* J) {
-    if constexpr (QUAD == 0) return scatter_closed(p, x0, beta, w, J);
-    else {
+    if constexpr (QUAD == 0) {
+        CellStart<double> st;
+        cell_start(x0, p.m, st);
+        return scatter_closed(p, st, beta, w, J);
+    } else {
         if (p.order == 2) return scatter_gauss_r<2>(p, x0, beta, w, J);
         if (p.order == 3) return scatter_gauss_r<3>(p, x0, beta, w, J);
         return scatter_gauss(p, x0, beta, w, J);
@@ -287,48 +293,6 @@ __device__ __forceinline__ void push_piece_closed(const StepParams& p, const Seg
                 acc.DAv[l] += Am * G0 + (t[3 + l] - t[l]) * G1;
             }
         }
-    }
-}
-
-// The same piece contribution from the base integrals (no diagnostics).  For derivative
-// direction j with transverse axes (p, q), sum over the four transverse offsets (a, b) of
-// T0(a, b) D_ab with T0 = int w_{p,a} w_{q,b} and D_ab the difference across j of the nodes'
-// A^{(m)}.vbar, is D00 h + (D10 - D00) Sp + (D01 - D00) Sq + (D11 - D10 - D01 + D00) Spq;
-// the T1 (eta-weighted, C^{(m)}.vbar) sum has the same form with h^2/2, Ep, Eq, Epq.
-__device__ __forceinline__ void push_piece_fast(const StepParams& p, const Segment<double>& sg, const double beta[3],
-                                                const double vb[3], const double* __restrict__ table, PushAcc& acc) {
-    const PieceInts<double> I = piece_integrals(sg, beta, true);
-    double W[8];
-    weights_from_ints(I, W);
-    int64_t g[8];
-    segment_nodes8(sg, p.m, g);
-    const double s = sg.s0, oms = 1.0 - s, h = sg.h, hh2 = 0.5 * h * h;
-    double am[8], cc[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const double* t = table + 12 * g[k];
-        const double an = t[0] * vb[0] + t[1] * vb[1] + t[2] * vb[2];   // A^n_g . vbar
-        const double a1 = t[3] * vb[0] + t[4] * vb[1] + t[5] * vb[2];   // A^{n+1}_g . vbar
-        am[k] = oms * an + s * a1;                                       // A^{(m)}_nu . vbar
-        cc[k] = a1 - an;                                                 // C^{(m)}_nu . vbar
-        acc.gphi[0] += W[k] * t[6];
-        acc.gphi[1] += W[k] * t[7];
-        acc.gphi[2] += W[k] * t[8];
-    }
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        const int pa = j == 0 ? 1 : 0, qa = j == 2 ? 1 : 2;              // transverse axes
-        const int sp = j == 0 ? 2 : 1, sq = j == 2 ? 2 : 4;              // their index strides
-        const int sj = j == 0 ? 1 : (j == 1 ? 2 : 4);                    // stride of axis j
-        const double D00 = am[sj] - am[0], D10 = am[sp + sj] - am[sp];
-        const double D01 = am[sq + sj] - am[sq], D11 = am[sp + sq + sj] - am[sp + sq];
-        const double C00 = cc[sj] - cc[0], C10 = cc[sp + sj] - cc[sp];
-        const double C01 = cc[sq + sj] - cc[sq], C11 = cc[sp + sq + sj] - cc[sp + sq];
-        const double t0 = D00 * h + (D10 - D00) * I.S1[pa] + (D01 - D00) * I.S1[qa] +
-                          (D11 - D10 - D01 + D00) * I.S2[j];
-        const double t1 = C00 * hh2 + (C10 - C00) * I.E1[pa] + (C01 - C00) * I.E1[qa] +
-                          (C11 - C10 - C01 + C00) * I.E2[j];
-        acc.F[j] += p.invH[j] * (t0 + t1);
     }
 }
 
@@ -584,8 +548,7 @@ __device__ __forceinline__ void push_eval(const StepParams& p, const double x0[3
     acc = PushAcc{};
     if constexpr (QUAD == 0) {
         o.nseg = for_each_segment(x0, beta, true, [&](const Segment<double>& sg) {
-            if constexpr (DIAG) push_piece_closed<true>(p, sg, beta, vb, table, acc);
-            else push_piece_fast(p, sg, beta, vb, table, acc);
+            push_piece_closed<DIAG>(p, sg, beta, vb, table, acc);
         });
     } else {
         // pieces between the knots of the shape's degree (shifted by 1/2 for even degrees)
@@ -604,6 +567,263 @@ __device__ __forceinline__ void push_eval(const StepParams& p, const double x0[3
     point_gather3(p, o.xe, table, 3, o.Ae);
 #pragma unroll
     for (int a = 0; a < 3; ++a) o.vw[a] = (o.Pw[a] - p.q * o.Ae[a]) * p.inv_mass;
+}
+
+// G(u) from the cell table (closed forms, no diagnostics): the push of push_eval in the centred
+// form of orbit_cell.cuh, from the start (cell, coordinate) and vs = u + v^n = 2 vbar.
+struct CellOut {
+    double Pw[3], Ae[3], vw[3];
+    int nseg;
+};
+
+template <bool CELLS>
+__device__ __forceinline__ void push_eval_cell(const StepParams& p, CellStart<double> st, const double vs[3],
+                                               const double Pn[3], const double* __restrict__ ctab, CellOut& o) {
+    double beta[3], acc[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) beta[a] = p.cb[a] * vs[a];
+    o.nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
+        piece_impulse(h, sm, mid, beta, vs, p.ihs, FieldLoad<CELLS>(ctab, c, p.m), acc);
+    });
+    cell_A1(st.f, FieldLoad<CELLS>(ctab, st.c, p.m), o.Ae);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        o.Pw[a] = Pn[a] + p.dtq * acc[a];
+        o.vw[a] = (o.Pw[a] - p.q * o.Ae[a]) * p.inv_mass;
+    }
+}
+
+// Shared-memory hand-over of a chunk's particles to the threads in order of orbit-piece count:
+// what the ranking computed (cell, coordinate, v^{p} + v^n) travels with the particle.
+struct ChunkOrder {
+    int order[THREADS];
+    int wcount[THREADS / 32][PIECE_CLASSES];
+    double f[3][THREADS], vs[3][THREADS];
+    int c[3][THREADS];
+};
+
+// Knots crossed by an axis whose orbit ends at te (relative to its start cell).
+__device__ __forceinline__ unsigned crossings(double te) {
+    return (at_least_one(te) || below_zero(te)) ? min((unsigned)abs(__double2int_rd(te)), 3u) : 0u;
+}
+
+// Rank the chunk's particles by piece count and hand them over; ends with a barrier.  Returns the
+// index of this thread's particle (>= np: none).
+__device__ __forceinline__ int64_t chunk_exchange(const StepParams& p, ChunkOrder& co, int64_t base, bool valid,
+                                                  const double x0[3], const double v2[3], CellStart<double>& st,
+                                                  double vs[3]) {
+    int cls = PIECE_CLASSES - 1;
+    if (valid) {
+        cell_start(x0, p.m, st);
+        unsigned pieces = 1;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) pieces += crossings(st.f[a] + p.cb[a] * v2[a]);
+        cls = (int)min(pieces, (unsigned)(PIECE_CLASSES - 1)) - 1;
+    }
+    const int r = stable_class_rank(cls, co.wcount);
+    co.order[r] = threadIdx.x;
+    if (valid) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            co.f[a][r] = st.f[a];
+            co.vs[a][r] = v2[a];
+            co.c[a][r] = st.c[a];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        st.f[a] = co.f[a][threadIdx.x];
+        vs[a] = co.vs[a][threadIdx.x];
+        st.c[a] = co.c[a][threadIdx.x];
+    }
+    return base + co.order[threadIdx.x];
+}
+
+// k_first_scatter for the closed forms.
+__global__ void __launch_bounds__(THREADS, 2) k_first_scatter_cell(
+    StepParams p, const double* __restrict__ xi, const double* __restrict__ v, const double* __restrict__ vprev,
+    const double* __restrict__ vgiven, double* __restrict__ vit, double* __restrict__ J, double* __restrict__ partials,
+    int* __restrict__ status) {
+    __shared__ double sm[32];
+    __shared__ ChunkOrder co;
+    const int64_t np = p.np, nchunks = (np + THREADS - 1) / THREADS;
+    double jsc = 0.0;
+    for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
+        const int64_t base = ch * THREADS, j = base + threadIdx.x;
+        double x0[3], v2[3], vs[3];
+        CellStart<double> st;
+        if (j < np) {
+            double vn[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                x0[a] = xi[a * np + j];
+                vn[a] = v[a * np + j];
+                const double vi = vgiven ? vgiven[a * np + j] : 2.0 * vn[a] - vprev[a * np + j];
+                vit[a * np + j] = vi;
+                v2[a] = vi + vn[a];
+            }
+            jsc += sqrt(vn[0] * vn[0] + vn[1] * vn[1] + vn[2] * vn[2]);
+        }
+        const int64_t i = chunk_exchange(p, co, base, j < np, x0, v2, st, vs);
+        if (i < np) {
+            double beta[3], w[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                beta[a] = p.cb[a] * vs[a];
+                w[a] = p.q_dV_half * vs[a];
+            }
+            if (scatter_closed(p, st, beta, w, J) < 0) atomicOr(status, DEV_ERR_SEGMENTS);
+        }
+        __syncthreads();   // the hand-over buffers are rewritten by the next chunk
+    }
+    write_partial<double>(partials, S_JSCALE, jsc, sm, false);
+}
+
+// is_creeping from the start's cell coordinate: on an axis with |beta| < BETA_CREEP, does twice
+// the orbit reach a knot, or does it start within D_KNOT of one?  Integer comparisons throughout.
+__device__ __forceinline__ bool is_creeping_cell(const double f[3], const double beta[3]) {
+    bool r = false;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double u = f[a] + 2.0 * beta[a];
+        const bool reach = at_least_one(u) || below_zero(u);
+        const bool near = less_pos(f[a], D_KNOT) || less_pos(1.0 - D_KNOT, f[a]);
+        r |= less_pos(fabs(beta[a]), BETA_CREEP) && (reach || near);
+    }
+    return r;
+}
+
+__device__ __forceinline__ double max_pos(double a, double b) { return less_pos(a, b) ? b : a; }
+
+// The Algorithm 1 push for the closed forms without diagnostics: as k_push (below), from the
+// cell table (CELLS) or the gather table.
+//
+// Bound by the FP64 pipe (one warp instruction in 16 clocks per SM), so what counts is the number of
+// FP64 instructions: the centred moments and the cell's mixed differences take 120 a piece where
+// node weights took 270 (57 against 88 for the scatter), and the walk, the creeping test and the
+// piece count compare on the integer pipe.  Measured at 32^3 with 2,097,152 particles (1.31 pieces
+// each): iterate 3.52 -> 1.59 ms, final sweep 2.40 -> 1.11 ms; 25.6M FP64 warp instructions where
+// there were 58.2M, the pipe 83% busy (88% in the final sweep).  Two blocks per SM (128 registers).
+template <bool COMMIT, bool CELLS>
+__global__ void __launch_bounds__(THREADS, 2) k_push_cell(StepParams p, const double* __restrict__ xi,
+                                                          const double* __restrict__ v, const double* __restrict__ P,
+                                                          const double* __restrict__ vit,
+                                                          const double* __restrict__ ctab, double* __restrict__ vnew,
+                                                          double* __restrict__ Jnext, double* __restrict__ xi_out,
+                                                          double* __restrict__ P_out,
+                                                          int32_t* __restrict__ creep_list,
+                                                          int* __restrict__ creep_count,
+                                                          uint8_t* __restrict__ creep_flag,
+                                                          const uint8_t* __restrict__ slide,
+                                                          double* __restrict__ partials, int* __restrict__ status) {
+    __shared__ double sm[32];
+    __shared__ ChunkOrder co;
+    const int64_t np = p.np, nchunks = (np + THREADS - 1) / THREADS;
+    double ev_num = 0.0, ev_den = 0.0;
+    long long pieces_push = 0, pieces_scatter = 0;
+    for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
+        const int64_t base = ch * THREADS, j = base + threadIdx.x;
+        double x0[3], vs[3];
+        CellStart<double> st;
+        {
+            double v2[3];
+            if (j < np) {
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    x0[a] = xi[a * np + j];
+                    v2[a] = vit[a * np + j] + v[a * np + j];
+                }
+            }
+            const int64_t i = chunk_exchange(p, co, base, j < np, x0, v2, st, vs);
+            if (i < np) {
+                double vi[3], vn[3], Pn[3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) Pn[a] = P[a * np + i];
+                CellOut o;
+                push_eval_cell<CELLS>(p, st, vs, Pn, ctab, o);
+                if (o.nseg < 0) atomicOr(status, DEV_ERR_SEGMENTS);
+                pieces_push += o.nseg;
+                if (!(isfinite(o.vw[0]) && isfinite(o.vw[1]) && isfinite(o.vw[2]))) atomicOr(status, DEV_ERR_NONFINITE);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    vi[a] = vit[a * np + i];
+                    vn[a] = v[a * np + i];
+                }
+                if constexpr (!COMMIT) {
+                    // a particle solved locally earlier in this step keeps the local solve, so that
+                    // none alternates between it and the plain update.  So does one whose change did
+                    // not shrink below SLOW_RATIO of the previous one: its own feedback is too strong
+                    // for the outer iteration (orbits crossing a knot just past the creeping range,
+                    // once the force jumps at knots grow).  A contracting outer loop shrinks
+                    // field-driven changes far faster, so it flags almost none.
+                    double d[3], beta[3];
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        d[a] = o.vw[a] - vi[a];   // change of the iterate, v^{p+1} - v^p
+                        beta[a] = p.cb[a] * vs[a];
+                    }
+                    bool slow = false;
+                    if (p.hist) {
+                        double dold = 0.0;
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) dold = max_pos(dold, fabs(vi[a] - vnew[a * np + i]));
+                        const double dn = max_pos(max_pos(fabs(d[0]), fabs(d[1])), fabs(d[2]));
+                        if (less_pos(SLOW_RATIO * dold, dn))
+                            slow = dn > p.slow_floor * sqrt(vi[0] * vi[0] + vi[1] * vi[1] + vi[2] * vi[2]);
+                    }
+                    const bool creep = p.accel && (is_creeping_cell(st.f, beta) || (slide[i] & SLIDE_CREPT) || slow);
+                    if (creep_flag) creep_flag[i] = creep ? 1 : 0;   // deterministic mode: k_local walks the flags
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) vnew[a * np + i] = o.vw[a];   // G(v^p)
+                    if (creep) {
+                        if (!creep_flag) {
+                            const int k = atomicAdd(creep_count, 1);   // k_local solves it and adds its e_v terms
+                            creep_list[k] = (int32_t)i;
+                        }
+                    } else {
+                        double w[3];
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) {
+                            ev_num += d[a] * d[a];
+                            ev_den += o.vw[a] * o.vw[a];
+                            const double v2n = o.vw[a] + vn[a];
+                            beta[a] = p.cb[a] * v2n;
+                            w[a] = p.q_dV_half * v2n;
+                        }
+                        const int ns = scatter_closed(p, st, beta, w, Jnext);
+                        if (ns < 0) atomicOr(status, DEV_ERR_SEGMENTS);
+                        pieces_scatter += ns;
+                    }
+                } else {
+                    // components sliding onto a knot (set by k_local): the orbit lands on the knot,
+                    // v^{n+1}_a is the iterate itself and P_a follows from v = (P - q A_h(x)) / m
+                    const uint8_t sb = slide ? slide[i] : 0;
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        if (sb & (1u << a)) {
+                            o.vw[a] = vi[a];
+                            o.Pw[a] = p.mass * o.vw[a] + p.q * o.Ae[a];
+                        }
+                        vnew[a * np + i] = o.vw[a];
+                        xi_out[a * np + i] = wrap_pos(xi[a * np + i] + p.cb[a] * vs[a], (double)p.m.n[a]);
+                        P_out[a * np + i] = o.Pw[a];
+                        // the residual of the accepted iterate itself, ||G(v*) - v*||
+                        const double d = o.vw[a] - vi[a];
+                        ev_num += d * d;
+                        ev_den += o.vw[a] * o.vw[a];
+                    }
+                }
+            }
+        }
+        __syncthreads();   // the hand-over buffers are rewritten by the next chunk
+    }
+    write_partial<double>(partials, S_EV_NUM, ev_num, sm, false);
+    write_partial<double>(partials, S_EV_DEN, ev_den, sm, false);
+    if constexpr (!COMMIT) {
+        write_partial<double>(partials, S_PIECES_PUSH, (double)pieces_push, sm, false);
+        write_partial<double>(partials, S_PIECES_SCATTER, (double)pieces_scatter, sm, false);
+    }
 }
 
 // The Algorithm 1 push for iterate vit, then either
@@ -791,7 +1011,7 @@ __global__ void __launch_bounds__(THREADS, DIAG ? 1 : 2) k_push(StepParams p, co
 // and the commit push sets v^{n+1}_a to it with P_a from the canonical relation.  The energy
 // identities hold to the size of vbar_a = d H / dt < D_KNOT H / dt.  The plain image G(v^p)
 // is saved in gsave (diagnostics), then the orbit current of the result is scattered.
-template <int QUAD>
+template <int QUAD, bool CELLS>
 __global__ void __launch_bounds__(THREADS) k_local(StepParams p, const double* __restrict__ xi,
                                                    const double* __restrict__ v, const double* __restrict__ P,
                                                    const double* __restrict__ vit, const double* __restrict__ table,
@@ -949,10 +1169,23 @@ __global__ void __launch_bounds__(THREADS) k_local(StepParams p, const double* _
                 }
             }
         }
-        PushAcc acc;
         PushOut o;
         if (active) {
-            push_eval<QUAD, false>(p, x0, vn, Pn, ue, table, acc, o);
+            if constexpr (QUAD == 0) {
+                CellStart<double> st;
+                CellOut co;
+                double vs[3];
+                cell_start(x0, p.m, st);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) vs[a] = ue[a] + vn[a];
+                push_eval_cell<CELLS>(p, st, vs, Pn, table, co);
+                o.nseg = co.nseg;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) o.vw[a] = co.vw[a];
+            } else {
+                PushAcc acc;
+                push_eval<QUAD, false>(p, x0, vn, Pn, ue, table, acc, o);
+            }
             if (phase >= 2 && o.nseg < 0) atomicOr(status, DEV_ERR_SEGMENTS);
             neval += 1.0;
         }
@@ -1334,6 +1567,12 @@ StepParams make_params(const Ctx& c) {
     p.mass = c.mass;
     p.inv_mass = 1.0 / c.mass;
     p.q_dV = c.q / c.dV;
+    for (int a = 0; a < 3; ++a) {
+        p.cb[a] = 0.5 * c.cfg.dt / c.H[a];
+        p.ihs[a] = 0.5 * c.invH[a];
+    }
+    p.dtq = c.cfg.dt * c.q;
+    p.q_dV_half = 0.5 * p.q_dV;
     p.np = c.np;
     p.split = c.cfg.split_orbit_at_knots;
     p.nq = c.cfg.nq;
@@ -1380,8 +1619,8 @@ void launch_first_scatter(Ctx& c, double* J, const double* v_iter_or_null) {
     StepParams p = make_params(c);
     int nb = particle_blocks(c);
     if (c.cfg.quadrature == PIC_QUAD_CLOSED)
-        k_first_scatter<0><<<nb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.vprev, v_iter_or_null, c.vit, J, c.partials,
-                                                         c.dev_status);
+        k_first_scatter_cell<<<nb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.vprev, v_iter_or_null, c.vit, J, c.partials,
+                                                           c.dev_status);
     else
         k_first_scatter<1><<<nb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.vprev, v_iter_or_null, c.vit, J, c.partials,
                                                          c.dev_status);
@@ -1401,17 +1640,28 @@ void launch_push(Ctx& c, const double* vit, double* vnew, double* Jnext, bool co
                                                   c.creep_list, c.creep_count, det ? c.creep_flag : nullptr,  \
                                                   c.slide,                                                    \
                                                   c.partials, c.dev_status)
-    if (!commit) {
-        if (closed) PIC_PUSH(0, false, false);
-        else PIC_PUSH(1, false, false);
+#define PIC_PUSH_CELL(C, T)                                                                                       \
+    k_push_cell<C, T><<<nb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.P, vit, T ? c.ctab : c.table, vnew, Jnext,     \
+                                                    c.xi_new, c.P_new, c.creep_list, c.creep_count,                \
+                                                    det ? c.creep_flag : nullptr, c.slide, c.partials, c.dev_status)
+    if (closed && !diag) {
+        if (commit) {
+            if (c.ctab) PIC_PUSH_CELL(true, true);
+            else PIC_PUSH_CELL(true, false);
+        } else {
+            if (c.ctab) PIC_PUSH_CELL(false, true);
+            else PIC_PUSH_CELL(false, false);
+        }
+    } else if (!commit) {
+        PIC_PUSH(1, false, false);
     } else if (!diag) {
-        if (closed) PIC_PUSH(0, true, false);
-        else PIC_PUSH(1, true, false);
+        PIC_PUSH(1, true, false);
     } else {
         if (closed) PIC_PUSH(0, true, true);
         else PIC_PUSH(1, true, true);
     }
 #undef PIC_PUSH
+#undef PIC_PUSH_CELL
     ++c.launches;
     // in deterministic mode the exact current is rounded once all of its deposits are in
     if (det && Jnext && !c.cfg.picard_accel) launch_exact_finish(c, Jnext, 3 * c.m.ncell, c.inv_u_J);
@@ -1421,14 +1671,14 @@ void launch_local(Ctx& c, const double* vit, double* vnew, double* Jnext) {
     StepParams p = make_params(c);
     const bool det = c.cfg.deterministic != 0;
     const int lb = local_blocks(c);
-    if (c.cfg.quadrature == PIC_QUAD_CLOSED)
-        k_local<0><<<lb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.P, vit, c.table, vnew, c.gsave, Jnext, c.creep_list,
-                                                 c.creep_count, det ? c.creep_flag : nullptr, c.slide,
-                                                 c.creep_count + 1, c.partials, c.dev_status);
-    else
-        k_local<1><<<lb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.P, vit, c.table, vnew, c.gsave, Jnext, c.creep_list,
-                                                 c.creep_count, det ? c.creep_flag : nullptr, c.slide,
-                                                 c.creep_count + 1, c.partials, c.dev_status);
+#define PIC_LOCAL(Q, T, TAB)                                                                                      \
+    k_local<Q, T><<<lb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.P, vit, TAB, vnew, c.gsave, Jnext, c.creep_list,   \
+                                                c.creep_count, det ? c.creep_flag : nullptr, c.slide,              \
+                                                c.creep_count + 1, c.partials, c.dev_status)
+    if (c.cfg.quadrature != PIC_QUAD_CLOSED) PIC_LOCAL(1, false, c.table);
+    else if (c.ctab) PIC_LOCAL(0, true, c.ctab);
+    else PIC_LOCAL(0, false, c.table);
+#undef PIC_LOCAL
     ++c.launches;
     if (det && Jnext) launch_exact_finish(c, Jnext, 3 * c.m.ncell, c.inv_u_J);
 }

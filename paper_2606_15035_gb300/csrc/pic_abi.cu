@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "pic_internal.h"
+#include "orbit_cell.cuh"
 
 using namespace pic;
 
@@ -32,8 +33,7 @@ pic_status fail(pic_ctx* ctx, pic_status s, const std::string& why) {
     return s;
 }
 
-void* dev_alloc(pic_ctx* ctx, size_t bytes) {
-    if (bytes == 0) bytes = 16;
+void* dev_alloc_once(pic_ctx* ctx, size_t bytes) {
     void* p = nullptr;
     if (ctx->c.has_alloc) {
         p = ctx->c.alloc.alloc(bytes, (void*)ctx->c.stream, ctx->c.alloc.user);
@@ -42,6 +42,29 @@ void* dev_alloc(pic_ctx* ctx, size_t bytes) {
         p = nullptr;
     }
     if (p) ctx->allocs.emplace_back(p, bytes);
+    return p;
+}
+
+// Give the optional cell table back (between calls: the kernels then read the gather table).
+bool drop_cell_table(pic_ctx* ctx) {
+    Ctx& c = ctx->c;
+    if (!c.ctab) return false;
+    cudaStreamSynchronize(c.stream);
+    for (size_t k = 0; k < ctx->allocs.size(); ++k) {
+        if (ctx->allocs[k].first != c.ctab) continue;
+        if (c.has_alloc) c.alloc.free(c.ctab, ctx->allocs[k].second, (void*)c.stream, c.alloc.user);
+        else cudaFree(c.ctab);
+        ctx->allocs.erase(ctx->allocs.begin() + (long)k);
+        break;
+    }
+    c.ctab = nullptr;
+    return true;
+}
+
+void* dev_alloc(pic_ctx* ctx, size_t bytes) {
+    if (bytes == 0) bytes = 16;
+    void* p = dev_alloc_once(ctx, bytes);
+    if (!p && drop_cell_table(ctx)) p = dev_alloc_once(ctx, bytes);
     return p;
 }
 
@@ -256,6 +279,13 @@ void setup_geometry(Ctx& c) {
     c.cheb_rate = (c.cheb_iters > 1 && rho > 0.0) ? 1.0 / std::log(1.0 / rho) : 0.0;
 }
 
+// Rule of the cell table (576 B per cell, orbit_cell.cuh): from one particle per cell on.  Three
+// FP64 steps measured with the table | without it: 64^3 at 1 per cell 11.18 | 11.19 ms a step, at 4
+// 15.0 | 17.9, at 16 32.6 | 45.7; 128^3 at 1 68.7 | 72.8, at 16 314 | 454; 32^3 at 1 4.34 | 4.53.
+// The byte limit keeps the table a small part of the device's memory (it is reached at 310^3).
+constexpr int64_t CELL_TABLE_MIN_PPC = 1;
+constexpr size_t CELL_TABLE_MAX_BYTES = (size_t)16 << 30;
+
 #define ALLOC(ptr, type, count)                                                          \
     do {                                                                                 \
         (ptr) = (type*)dev_alloc(ctx, sizeof(type) * (size_t)(count));                   \
@@ -391,6 +421,13 @@ pic_status allocate(pic_ctx* ctx) {
         cudaGetLastError();
         return fail(ctx, PIC_ERR_OOM, "pinned host allocation failed");
     }
+    // last, because it is optional: the closed forms' cell table, where there are particles enough to
+    // repay building it and it stays a small part of the device's memory
+    const size_t cells = sizeof(double) * CELL_VALUES * (size_t)N;
+    if (c.cfg.quadrature == PIC_QUAD_CLOSED && c.np >= CELL_TABLE_MIN_PPC * N && cells <= CELL_TABLE_MAX_BYTES) {
+        c.ctab = (double*)dev_alloc_once(ctx, cells);
+        if (c.ctab && reinterpret_cast<uintptr_t>(c.ctab) % 16 != 0) drop_cell_table(ctx);
+    }
     cudaMemsetAsync(c.partials, 0, sizeof(double) * (size_t)NSLOT * MAX_BLOCKS, c.stream);
     cudaMemsetAsync(c.results, 0, sizeof(double) * NSLOT, c.stream);
     cudaMemsetAsync(c.dev_status, 0, sizeof(int), c.stream);
@@ -479,19 +516,21 @@ void mesh_begin(Ctx& c) {
 // The mesh half of one Algorithm 1 iteration: continuity, CN solve (warm-started from F1),
 // back-substitution and the gather table.
 // tol: the Chebyshev solve's relative accuracy (helmholtz_tol when not positive).
-void mesh_phase(Ctx& c, const double* Jcur, const double* Jprev, double tol = 0.0) {
+// cells: also the cell table, for the FP64 closed-form kernels that follow.
+void mesh_phase(Ctx& c, const double* Jcur, const double* Jprev, double tol = 0.0, bool cells = true) {
     ProfScope ps(c, PH_MESH);
     if (c.cfg.ops == PIC_OPS_SPECTRAL) {
         launch_spec_mesh_phase(c, Jcur, Jprev);
-        return;
-    }
-    launch_source(c, Jcur, Jprev);
-    if (c.helm_fft) {
-        launch_helmholtz_fft_refined(c, c.F1);   // to roundoff: the tolerance does not apply
     } else {
-        launch_helmholtz_cn(c, &c.F1, &c.F1b, tol > 0.0 ? std::max(tol, c.cfg.helmholtz_tol) : c.cfg.helmholtz_tol);
+        launch_source(c, Jcur, Jprev);
+        if (c.helm_fft) {
+            launch_helmholtz_fft_refined(c, c.F1);   // to roundoff: the tolerance does not apply
+        } else {
+            launch_helmholtz_cn(c, &c.F1, &c.F1b, tol > 0.0 ? std::max(tol, c.cfg.helmholtz_tol) : c.cfg.helmholtz_tol);
+        }
+        launch_backsub_table(c, false);
     }
-    launch_backsub_table(c, false);
+    if (cells && c.ctab) launch_cell_table(c);
 }
 
 // PIC_MIXED: the fields of an FP32 iteration need no more accuracy than its iterate has
@@ -569,7 +608,7 @@ void iter_issue(Ctx& c) {
     const int64_t N = c.m.ncell;
     const double mesh_tol = r.fp32 ? MESH_TOL32
                             : (r.began32 && c.cfg.mixed_tol64 > 0.0 ? 1e-3 * c.cfg.mixed_tol64 : 0.0);
-    mesh_phase(c, c.J[r.cur], r.p > 0 ? c.J[r.prev] : nullptr, mesh_tol);
+    mesh_phase(c, c.J[r.cur], r.p > 0 ? c.J[r.prev] : nullptr, mesh_tol, !r.fp32);
     if (r.fp32) {
         launch_table32(c);
         cudaMemsetAsync(c.J[r.next], 0, sizeof(double) * 3 * N, c.stream);

@@ -66,6 +66,7 @@ struct StepParams {
     MeshDims m;
     double H[3], invH[3];
     double dt, q, mass, inv_mass, q_dV;  // q_dV = q / dV
+    double cb[3], ihs[3], dtq, q_dV_half;   // dt / (2 H), 1 / (2 H), dt q, q / (2 dV): factors of v^{p} + v^n
     int64_t np;
     int split;                 // split orbits at knots
     int nq;                    // Gauss points (Gauss quadrature only)
@@ -149,6 +150,7 @@ struct Ctx {
     double *cheb_d = nullptr, *rhs0 = nullptr, *rhs = nullptr;
     double *J[3] = {nullptr, nullptr, nullptr};
     double* table = nullptr;             // 12 * ncell gather table
+    double* ctab = nullptr;              // closed forms: CELL_VALUES * ncell cell table (orbit_cell.cuh)
 
     // FP32 working set of the mixed path (allocated only for PIC_MIXED)
     std::vector<double> hist_ev, hist_eJ;   // residuals of the last step's iterations
@@ -295,6 +297,8 @@ void launch_jdiff(Ctx& c, const double* Jnew, const double* Jold);
 void launch_helmholtz(Ctx& c, const double* b, double c_id, double c_lap, int nfields, int iters,
                       const double* alpha, const double* beta, double** x_io, double** x_spare);
 void launch_backsub_table(Ctx& c, bool diag);
+// The cell table of the FP64 closed-form particle kernels from the gather table.
+void launch_cell_table(Ctx& c);
 void launch_helmholtz_cn(Ctx& c, double** x_io, double** x_spare, double tol);
 void launch_helmholtz_fft_refined(Ctx& c, double* x);
 int cheb_coop_capacity(const Ctx& c);

@@ -1,0 +1,88 @@
+"""The centred closed-form particle kernels (orbit_cell.cuh) at the edges of their walk: starts
+exactly on knots moving either way or not at all, ends exactly on knots, orbits of several cells,
+axes of 2 nodes, with the cell table and, where the allocator refuses it, with the gather table.
+
+One Picard body against the oracle, with the tolerances of the general parity test (an orbit's
+integrals are sums of a few dozen products of order one, so 1e-13 leaves two digits of margin)."""
+
+import numpy as np
+import pytest
+
+from oracle import pic as opic
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sim(cuda_ok):
+    from paper_2606_15035_gb300 import build
+    build.build()
+    from paper_2606_15035_gb300 import sim as s
+    return s
+
+
+def _edge_particles(n, npart, seed):
+    """Cell-unit starts and displacements; H = 1 and dt = 1, so that knots are hit exactly."""
+    rng = np.random.default_rng(seed)
+    x = rng.uniform(0, 1, size=(npart, 3)) * n
+    b = rng.normal(scale=0.8, size=(npart, 3))
+    k = npart // 8
+    x[:k] = np.floor(x[:k])                                   # on a knot in every axis
+    b[k // 2:k, 1] = 0.0                                      # ... resting on it in one
+    b[k:2 * k] = np.round(b[k:2 * k])                         # whole cells: ends keep the offset
+    x[2 * k:3 * k] = np.floor(x[2 * k:3 * k]) + 0.5
+    b[2 * k:3 * k] = rng.integers(-3, 4, size=(k, 3)) + 0.5   # end exactly on a knot
+    b[3 * k:4 * k] = 0.0
+    b[4 * k:5 * k] = 2.6 * np.sign(b[4 * k:5 * k])            # two or three knots an axis
+    b[5 * k:6 * k] *= 1e-9
+    return x, np.clip(b, 0.5 - n, n - 0.5)                    # less than one box length
+
+
+@pytest.mark.parametrize("n", [(8, 8, 8), (2, 5, 3), (9, 2, 4)])
+@pytest.mark.parametrize("table", ["cells", "nodes"])
+def test_one_body_matches_oracle_at_the_edges(sim, monkeypatch, n, table):
+    refused = []
+    if table == "nodes":
+        want = 576 * n[0] * n[1] * n[2]
+        base = sim._TorchAllocator
+
+        class Refusing(base):
+            def __init__(self, device):
+                super().__init__(device)
+                inner = self._alloc_cb
+
+                def alloc(nbytes, stream, user):
+                    if nbytes == want:
+                        refused.append(nbytes)
+                        return None
+                    return inner(nbytes, stream, user)
+
+                self._outer_cb = sim._lib.ALLOC_FN(alloc)
+                self.struct = sim.PicAllocator(self._outer_cb, self._free_cb, None)
+
+        monkeypatch.setattr(sim, "_TorchAllocator", Refusing)
+    L = tuple(float(k) for k in n)
+    x, b = _edge_particles(np.asarray(n), 1601, 40 + n[0])
+    v = 0.3 * b[::-1].copy()
+    v_it = 2.0 * b - v                                        # vbar = b exactly up to rounding
+    q = -1e-3
+    cfg = sim.pic_config_default(n=n, L=L, dt=1.0, picard_tol=1e-13)
+    s = sim.PicSim(cfg, x, v, q, 1e-3)
+    assert bool(refused) == (table == "nodes")
+    ocfg = opic.Config(n=n, L=L, dt=1.0, picard_tol=1e-13)
+    o = opic.init(x, v, q, 1e-3, ocfg)
+    g = s.iterate(v_it)
+    it = opic.picard_iteration(o, v_it, ocfg, ocfg.grid())
+    s.close()
+
+    def rel(a, r):
+        return np.linalg.norm(a - r) / max(np.linalg.norm(r), 1e-300)
+
+    assert rel(g["J"], it["J"]) <= 1e-13
+    for name in ("phi", "psi", "A", "U"):
+        assert rel(g[name], it[name]) <= 1e-12, (name, rel(g[name], it[name]))
+    assert rel(g["P"], it["P"]) <= 1e-13
+    assert rel(g["v"], it["v_new"]) <= 1e-13
+    d = g["x"] - it["xi"] * np.asarray(ocfg.grid().H)
+    Lv = np.asarray(L)
+    assert np.abs((d + 0.5 * Lv) % Lv - 0.5 * Lv).max() <= 1e-14 * Lv.max()
