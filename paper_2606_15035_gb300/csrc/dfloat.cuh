@@ -81,6 +81,14 @@ __device__ __forceinline__ DF operator/(DF a, DF b) {
     return fast_two_sum(q1, q2);
 }
 
+// a b + c with one renormalisation (15 operations for the 18 of the two operators)
+__device__ __forceinline__ DF mad(DF a, DF b, DF c) {
+    const DF p = two_prod(a.hi, b.hi);
+    const DF s = two_sum(p.hi, c.hi);
+    const float e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, p.lo));
+    return fast_two_sum(s.hi, s.lo + (e + c.lo));
+}
+
 __device__ __forceinline__ DF& operator+=(DF& a, DF b) { return a = a + b; }
 __device__ __forceinline__ DF& operator-=(DF& a, DF b) { return a = a - b; }
 __device__ __forceinline__ DF& operator*=(DF& a, DF b) { return a = a * b; }
@@ -104,9 +112,32 @@ __device__ __forceinline__ DF ceil(DF a) {
     return fast_two_sum(ch, ceilf(a.lo));
 }
 
+// order and range tests of the orbit walk (orbit_cell.cuh)
+__device__ __forceinline__ bool less_pos(DF a, DF b) { return a < b; }
+__device__ __forceinline__ bool same_bits(DF a, DF b) { return a == b; }
+__device__ __forceinline__ bool at_least_one(DF t) { return t.hi > 1.f || (t.hi == 1.f && t.lo >= 0.f); }
+__device__ __forceinline__ bool below_zero(DF t) { return t.hi < 0.f || (t.hi == 0.f && t.lo < 0.f); }
+__device__ __forceinline__ bool is_zero(DF t) { return t.hi == 0.f && t.lo == 0.f; }
+
 __device__ __forceinline__ DF fmin(DF a, DF b) { return b < a ? b : a; }
 __device__ __forceinline__ DF fmax(DF a, DF b) { return a < b ? b : a; }
 __device__ __forceinline__ DF fabs(DF a) { return a.hi < 0.f ? -a : a; }
+
+// double -> pair from the bit pattern (integer and FP32 pipes only): the upper 24 bits of the
+// significand, then the lower 29 as an integer.  Small or huge values convert in FP64.
+__device__ __forceinline__ DF df_bits(double d) {
+    const int hw = __double2hiint(d);
+    const unsigned lw = (unsigned)__double2loint(d);
+    const int fe = ((hw >> 20) & 0x7ff) - 896;            // the float's biased exponent
+    if (fe < 60 || fe > 250) {
+        const float h = (float)d;
+        return DF(h, (float)(d - (double)h));
+    }
+    const int sign = hw & 0x80000000;
+    const float hi = __int_as_float(sign | (fe << 23) | ((hw & 0xfffff) << 3) | (int)(lw >> 29));
+    const float unit = __int_as_float(sign | ((fe - 52) << 23));
+    return fast_two_sum(hi, (float)(int)(lw & 0x1fffffffu) * unit);
+}
 
 // double -> pair and pair -> double (two FP64 operations each way; used at the kernel's edges)
 __device__ __forceinline__ DF df_of(double d) {

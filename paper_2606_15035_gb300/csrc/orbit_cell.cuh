@@ -26,6 +26,12 @@ namespace pic {
 constexpr int CELL_COLS = 9;
 constexpr int CELL_VALUES = 8 * CELL_COLS;
 
+// a b + c (FP32 pairs have an overload that rounds once).
+template <typename T>
+__device__ __forceinline__ T mad(T a, T b, T c) {
+    return a * b + c;
+}
+
 // Order and range tests of the walk.  On doubles they run on the integer pipe (for values >= 0
 // the bit patterns order like the values; the sign and exponent decide t < 0 and t >= 1): the
 // FP64 pipe, which has 1/64 of the issue rate, is what bounds the particle kernels.
@@ -46,56 +52,58 @@ struct CellStart {
 __device__ __forceinline__ int next_cell(int c, int n) { return c + 1 >= n ? 0 : c + 1; }
 __device__ __forceinline__ int prev_cell(int c, int n) { return c > 0 ? c - 1 : n - 1; }
 
-// Visit the knot-free pieces of the orbit st.f + s beta: visit(h, s_mid, mid, cell), h > 0.  On
-// return st.c is the end point's cell and st.f the end point's coordinate in it (in [0, 1]; an
-// end exactly on a knot keeps the cell it came from, where the fields have the same value).
-// Returns the number of breakpoint intervals, or -1 if MAX_SEGMENTS was exceeded.  Cells stay in
-// [0, n) whatever the input.
-template <typename T, typename F>
-__device__ __forceinline__ int for_each_piece(CellStart<T>& st, const T beta[3], const MeshDims& m, F&& visit) {
-    T fd[3], te[3], sn[3];
+// The knot-free pieces of the orbit f + s beta of a start, one per next().  c stays in [0, n)
+// whatever the input.  After the last piece c is the end point's cell and te its coordinate in it
+// (in [0, 1]; an end exactly on a knot keeps the cell it came from, where the fields have the same
+// value), and count the number of breakpoint intervals, or -1 if MAX_SEGMENTS was exceeded.
+template <typename T>
+struct PieceWalk {
+    T fd[3], te[3], sn[3], s0;   // start and end coordinate relative to cell c, next crossing per axis
+    int c[3];
+    int it, count;
+
+    __device__ __forceinline__ PieceWalk(const CellStart<T>& st, const T beta[3], const MeshDims& m) {
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        fd[a] = st.f[a];                       // start coordinate relative to the current cell
-        te[a] = fd[a] + beta[a];               // end coordinate relative to the current cell
-        if (below_zero(te[a]) && is_zero(fd[a])) {   // on a knot, moving down: the cell below
-            st.c[a] = prev_cell(st.c[a], m.n[a]);
-            fd[a] = T(1);
-            te[a] = T(1) + beta[a];
+        for (int a = 0; a < 3; ++a) {
+            c[a] = st.c[a];
+            fd[a] = st.f[a];
+            te[a] = fd[a] + beta[a];
+            if (below_zero(te[a]) && is_zero(fd[a])) {   // on a knot, moving down: the cell below
+                c[a] = prev_cell(c[a], m.n[a]);
+                fd[a] = T(1);
+                te[a] = T(1) + beta[a];
+            }
+            sn[a] = T(2);                          // 2: no crossing ahead
+            if (at_least_one(te[a])) sn[a] = (T(1) - fd[a]) / beta[a];
+            else if (below_zero(te[a])) sn[a] = fd[a] / -beta[a];
+            if (!less_pos(sn[a], T(1))) sn[a] = T(2);
         }
-        sn[a] = T(2);                          // next crossing of this axis (2: none)
-        if (at_least_one(te[a])) sn[a] = (T(1) - fd[a]) / beta[a];
-        else if (below_zero(te[a])) sn[a] = fd[a] / -beta[a];
-        if (!less_pos(sn[a], T(1))) sn[a] = T(2);
+        s0 = T(0);
+        it = 0;
+        count = 0;
     }
-    T s0 = T(0);
-    int count = -1;
-    for (int it = 0; it < MAX_SEGMENTS; ++it) {
+
+    // The next breakpoint (1: the end of the orbit).
+    __device__ __forceinline__ T upcoming() const {
         T s1 = T(1);
 #pragma unroll
         for (int a = 0; a < 3; ++a) s1 = less_pos(sn[a], s1) ? sn[a] : s1;
-        if (less_pos(s0, s1)) {
-            const T h = s1 - s0, sm = T(0.5) * (s0 + s1);
-            T mid[3];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) mid[a] = fd[a] + sm * beta[a];
-            visit(h, sm, mid, st.c);
-        }
-        if (same_bits(s1, T(1))) {
-            count = it + 1;
-            break;
-        }
+        return s1;
+    }
+
+    // Cross the knots met at s1.
+    __device__ __forceinline__ void cross(T s1, const T beta[3], const MeshDims& m) {
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             if (!same_bits(sn[a], s1)) continue;
             sn[a] = T(2);
             if (!below_zero(te[a])) {
-                st.c[a] = next_cell(st.c[a], m.n[a]);
+                c[a] = next_cell(c[a], m.n[a]);
                 fd[a] = fd[a] - T(1);
                 te[a] = te[a] - T(1);
                 if (at_least_one(te[a])) sn[a] = (T(1) - fd[a]) / beta[a];
             } else {
-                st.c[a] = prev_cell(st.c[a], m.n[a]);
+                c[a] = prev_cell(c[a], m.n[a]);
                 fd[a] = fd[a] + T(1);
                 te[a] = te[a] + T(1);
                 if (below_zero(te[a])) sn[a] = fd[a] / -beta[a];
@@ -104,8 +112,62 @@ __device__ __forceinline__ int for_each_piece(CellStart<T>& st, const T beta[3],
         }
         s0 = s1;
     }
+
+    // The next piece [s_mid - h/2, s_mid + h/2], h > 0, in cell pc with the midpoint mid; false when
+    // there is none.  `last` is set with the orbit's last interval.
+    __device__ __forceinline__ bool next(const T beta[3], const MeshDims& m, T& h, T& sm, T mid[3], int pc[3], bool& last) {
+        last = false;
+        while (true) {
+            const T s1 = upcoming();
+            ++it;
+            const bool piece = less_pos(s0, s1);
+            if (piece) {
+                h = s1 - s0;
+                sm = T(0.5) * (s0 + s1);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) st.f[a] = te[a];
+                for (int a = 0; a < 3; ++a) {
+                    mid[a] = fd[a] + sm * beta[a];
+                    pc[a] = c[a];
+                }
+            }
+            if (same_bits(s1, T(1)) || it == MAX_SEGMENTS) {
+                last = true;
+                count = same_bits(s1, T(1)) ? it : -1;
+                return piece;
+            }
+            cross(s1, beta, m);
+            if (piece) return true;
+        }
+    }
+};
+
+// Visit the pieces of the orbit: visit(h, s_mid, mid, cell).  On return st is the end point's cell
+// and coordinate.  Returns PieceWalk's count.  (The kernels that visit inside this loop measured 10%
+// faster than through next(), which keeps the walk's state across calls.)
+template <typename T, typename F>
+__device__ __forceinline__ int for_each_piece(CellStart<T>& st, const T beta[3], const MeshDims& m, F&& visit) {
+    PieceWalk<T> wk(st, beta, m);
+    int count = -1;
+    for (int it = 0; it < MAX_SEGMENTS; ++it) {
+        const T s1 = wk.upcoming();
+        if (less_pos(wk.s0, s1)) {
+            const T h = s1 - wk.s0, sm = T(0.5) * (wk.s0 + s1);
+            T mid[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) mid[a] = wk.fd[a] + sm * beta[a];
+            visit(h, sm, mid, wk.c);
+        }
+        if (same_bits(s1, T(1))) {
+            count = it + 1;
+            break;
+        }
+        wk.cross(s1, beta, m);
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        st.c[a] = wk.c[a];
+        st.f[a] = wk.te[a];
+    }
     return count;
 }
 
@@ -127,10 +189,10 @@ __device__ __forceinline__ PieceMoments<T> piece_moments(T h, const T mid[3], co
         q.e[a] = k * beta[a];
     }
     const T kxy = q.e[0] * beta[1], kxz = q.e[0] * beta[2], kyz = q.e[1] * beta[2];
-    q.Pxy = mid[0] * mid[1] + kxy;
-    q.Pxz = mid[0] * mid[2] + kxz;
-    q.Pyz = mid[1] * mid[2] + kyz;
-    q.S = mid[0] * q.Pyz + (mid[1] * kxz + mid[2] * kxy);
+    q.Pxy = mad(mid[0], mid[1], kxy);
+    q.Pxz = mad(mid[0], mid[2], kxz);
+    q.Pyz = mad(mid[1], mid[2], kyz);
+    q.S = mad(mid[0], q.Pyz, mad(mid[1], kxz, mid[2] * kxy));
     return q;
 }
 
@@ -155,7 +217,7 @@ template <typename T, typename L>
 __device__ __forceinline__ void piece_impulse(T h, T sm, const T mid[3], const T beta[3], const T vs[3],
                                               const T ihs[3], L&& ld, T acc[3]) {
     const PieceMoments<T> q = piece_moments(h, mid, beta);
-    const T oms = T(1) - sm;
+    const T nms = sm - T(1);
     T F[3], g[3];
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
@@ -165,41 +227,41 @@ __device__ __forceinline__ void piece_impulse(T h, T sm, const T mid[3], const T
             ld(p, 3, x0, x1);
             ld(p, 4, y0, y1);
             ld(p, 5, z0, z1);
-            if (p > 0) cc[0] = x0 * vs[0] + y0 * vs[1] + z0 * vs[2];
-            cc[1] = x1 * vs[0] + y1 * vs[1] + z1 * vs[2];
+            if (p > 0) cc[0] = mad(z0, vs[2], mad(y0, vs[1], x0 * vs[0]));
+            cc[1] = mad(z1, vs[2], mad(y1, vs[1], x1 * vs[0]));
             ld(p, 0, x0, x1);
             ld(p, 1, y0, y1);
             ld(p, 2, z0, z1);
-            if (p > 0) a[0] = x0 * vs[0] + y0 * vs[1] + z0 * vs[2] - oms * cc[0];
-            a[1] = x1 * vs[0] + y1 * vs[1] + z1 * vs[2] - oms * cc[1];
+            if (p > 0) a[0] = mad(nms, cc[0], mad(z0, vs[2], mad(y0, vs[1], x0 * vs[0])));
+            a[1] = mad(nms, cc[1], mad(z1, vs[2], mad(y1, vs[1], x1 * vs[0])));
         }
         if (p == 0) {            // k = 1: x
             F[0] = a[1];
         } else if (p == 1) {     // k = 2: y, k = 3: xy
-            F[0] = F[0] + a[1] * mid[1] + cc[1] * q.e[1];
-            F[1] = a[0] + a[1] * mid[0] + cc[1] * q.e[0];
+            F[0] = mad(cc[1], q.e[1], mad(a[1], mid[1], F[0]));
+            F[1] = mad(cc[1], q.e[0], mad(a[1], mid[0], a[0]));
         } else if (p == 2) {     // k = 4: z, k = 5: xz
-            F[0] = F[0] + a[1] * mid[2] + cc[1] * q.e[2];
-            F[2] = a[0] + a[1] * mid[0] + cc[1] * q.e[0];
+            F[0] = mad(cc[1], q.e[2], mad(a[1], mid[2], F[0]));
+            F[2] = mad(cc[1], q.e[0], mad(a[1], mid[0], a[0]));
         } else {                 // k = 6: yz, k = 7: xyz
-            F[1] = F[1] + a[0] * mid[2] + cc[0] * q.e[2];
-            F[2] = F[2] + a[0] * mid[1] + cc[0] * q.e[1];
-            F[0] = F[0] + a[1] * q.Pyz + cc[1] * (mid[1] * q.e[2] + mid[2] * q.e[1]);
-            F[1] = F[1] + a[1] * q.Pxz + cc[1] * (mid[0] * q.e[2] + mid[2] * q.e[0]);
-            F[2] = F[2] + a[1] * q.Pxy + cc[1] * (mid[0] * q.e[1] + mid[1] * q.e[0]);
+            F[1] = mad(cc[0], q.e[2], mad(a[0], mid[2], F[1]));
+            F[2] = mad(cc[0], q.e[1], mad(a[0], mid[1], F[2]));
+            F[0] = mad(cc[1], mad(mid[1], q.e[2], mid[2] * q.e[1]), mad(a[1], q.Pyz, F[0]));
+            F[1] = mad(cc[1], mad(mid[0], q.e[2], mid[2] * q.e[0]), mad(a[1], q.Pxz, F[1]));
+            F[2] = mad(cc[1], mad(mid[0], q.e[1], mid[1] * q.e[0]), mad(a[1], q.Pxy, F[2]));
         }
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
             T g0, g1;
             ld(p, 6 + j, g0, g1);
-            if (p == 0) g[j] = g0 + g1 * mid[0];
-            else if (p == 1) g[j] = g[j] + g0 * mid[1] + g1 * q.Pxy;
-            else if (p == 2) g[j] = g[j] + g0 * mid[2] + g1 * q.Pxz;
-            else g[j] = g[j] + g0 * q.Pyz + g1 * q.S;
+            if (p == 0) g[j] = mad(g1, mid[0], g0);
+            else if (p == 1) g[j] = mad(g1, q.Pxy, mad(g0, mid[1], g[j]));
+            else if (p == 2) g[j] = mad(g1, q.Pxz, mad(g0, mid[2], g[j]));
+            else g[j] = mad(g1, q.S, mad(g0, q.Pyz, g[j]));
         }
     }
 #pragma unroll
-    for (int j = 0; j < 3; ++j) acc[j] = acc[j] + h * (g[j] + ihs[j] * F[j]);
+    for (int j = 0; j < 3; ++j) acc[j] = mad(h, mad(ihs[j], F[j], g[j]), acc[j]);
 }
 
 // A^{n+1} at coordinate r of the cell (Eq. (Ah-mesh)).
@@ -212,9 +274,9 @@ __device__ __forceinline__ void cell_A1(const T r[3], L&& ld, T out[3]) {
         ld(1, c, k2, k3);
         ld(2, c, k4, k5);
         ld(3, c, k6, k7);
-        const T lo = (k0 + k1 * r[0]) + r[1] * (k2 + k3 * r[0]);
-        const T hi = (k4 + k5 * r[0]) + r[1] * (k6 + k7 * r[0]);
-        out[c] = lo + r[2] * hi;
+        const T lo = mad(r[1], mad(k3, r[0], k2), mad(k1, r[0], k0));
+        const T hi = mad(r[1], mad(k7, r[0], k6), mad(k5, r[0], k4));
+        out[c] = mad(r[2], hi, lo);
     }
 }
 

@@ -10,6 +10,7 @@
 #include "pic_internal.h"
 #include "particle_common.cuh"
 #include "orbit_cell.cuh"
+#include "chunk.cuh"
 
 namespace pic {
 
@@ -593,60 +594,19 @@ __device__ __forceinline__ void push_eval_cell(const StepParams& p, CellStart<do
     }
 }
 
-// Shared-memory hand-over of a chunk's particles to the threads in order of orbit-piece count:
-// what the ranking computed (cell, coordinate, v^{p} + v^n) travels with the particle.
-struct ChunkOrder {
-    int order[THREADS];
-    int wcount[THREADS / 32][PIECE_CLASSES];
-    double f[3][THREADS], vs[3][THREADS];
-    int c[3][THREADS];
-};
-
-// Knots crossed by an axis whose orbit ends at te (relative to its start cell).
-__device__ __forceinline__ unsigned crossings(double te) {
-    return (at_least_one(te) || below_zero(te)) ? min((unsigned)abs(__double2int_rd(te)), 3u) : 0u;
-}
-
-// Rank the chunk's particles by piece count and hand them over; ends with a barrier.  Returns the
-// index of this thread's particle (>= np: none).
-__device__ __forceinline__ int64_t chunk_exchange(const StepParams& p, ChunkOrder& co, int64_t base, bool valid,
-                                                  const double x0[3], const double v2[3], CellStart<double>& st,
-                                                  double vs[3]) {
-    int cls = PIECE_CLASSES - 1;
-    if (valid) {
-        cell_start(x0, p.m, st);
-        unsigned pieces = 1;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) pieces += crossings(st.f[a] + p.cb[a] * v2[a]);
-        cls = (int)min(pieces, (unsigned)(PIECE_CLASSES - 1)) - 1;
-    }
-    const int r = stable_class_rank(cls, co.wcount);
-    co.order[r] = threadIdx.x;
-    if (valid) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            co.f[a][r] = st.f[a];
-            co.vs[a][r] = v2[a];
-            co.c[a][r] = st.c[a];
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        st.f[a] = co.f[a][threadIdx.x];
-        vs[a] = co.vs[a][threadIdx.x];
-        st.c[a] = co.c[a][threadIdx.x];
-    }
-    return base + co.order[threadIdx.x];
-}
+// Blocks per SM of the scatter: 3 (80 registers, a few spills) measured 43.6 ms at 128^3 with 134M
+// particles, 2 (128 registers) 46.0, 4 (64) 48.5.
+constexpr int SCATTER_MINB = 3;
 
 // k_first_scatter for the closed forms.
-__global__ void __launch_bounds__(THREADS, 2) k_first_scatter_cell(
+__global__ void __launch_bounds__(THREADS, SCATTER_MINB) k_first_scatter_cell(
     StepParams p, const double* __restrict__ xi, const double* __restrict__ v, const double* __restrict__ vprev,
     const double* __restrict__ vgiven, double* __restrict__ vit, double* __restrict__ J, double* __restrict__ partials,
     int* __restrict__ status) {
     __shared__ double sm[32];
-    __shared__ ChunkOrder co;
+    extern __shared__ __align__(16) unsigned char dyn[];
+    ChunkOrder& co = *reinterpret_cast<ChunkOrder*>(dyn);
+    long long* tile = reinterpret_cast<long long*>(dyn + sizeof(ChunkOrder)) + (threadIdx.x >> 5) * DEPOSIT_TILE;
     const int64_t np = p.np, nchunks = (np + THREADS - 1) / THREADS;
     double jsc = 0.0;
     for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
@@ -666,35 +626,17 @@ __global__ void __launch_bounds__(THREADS, 2) k_first_scatter_cell(
             jsc += sqrt(vn[0] * vn[0] + vn[1] * vn[1] + vn[2] * vn[2]);
         }
         const int64_t i = chunk_exchange(p, co, base, j < np, x0, v2, st, vs);
-        if (i < np) {
-            double beta[3], w[3];
+        double beta[3], w[3];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                beta[a] = p.cb[a] * vs[a];
-                w[a] = p.q_dV_half * vs[a];
-            }
-            if (scatter_closed(p, st, beta, w, J) < 0) atomicOr(status, DEV_ERR_SEGMENTS);
+        for (int a = 0; a < 3; ++a) {
+            beta[a] = p.cb[a] * vs[a];
+            w[a] = p.q_dV_half * vs[a];
         }
+        if (scatter_warp(p.m, i < np, st, beta, w, tile, p.det, p.acc, J) < 0) atomicOr(status, DEV_ERR_SEGMENTS);
         __syncthreads();   // the hand-over buffers are rewritten by the next chunk
     }
     write_partial<double>(partials, S_JSCALE, jsc, sm, false);
 }
-
-// is_creeping from the start's cell coordinate: on an axis with |beta| < BETA_CREEP, does twice
-// the orbit reach a knot, or does it start within D_KNOT of one?  Integer comparisons throughout.
-__device__ __forceinline__ bool is_creeping_cell(const double f[3], const double beta[3]) {
-    bool r = false;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const double u = f[a] + 2.0 * beta[a];
-        const bool reach = at_least_one(u) || below_zero(u);
-        const bool near = less_pos(f[a], D_KNOT) || less_pos(1.0 - D_KNOT, f[a]);
-        r |= less_pos(fabs(beta[a]), BETA_CREEP) && (reach || near);
-    }
-    return r;
-}
-
-__device__ __forceinline__ double max_pos(double a, double b) { return less_pos(a, b) ? b : a; }
 
 // The Algorithm 1 push for the closed forms without diagnostics: as k_push (below), from the
 // cell table (CELLS) or the gather table.
@@ -703,8 +645,9 @@ __device__ __forceinline__ double max_pos(double a, double b) { return less_pos(
 // FP64 instructions: the centred moments and the cell's mixed differences take 120 a piece where
 // node weights took 270 (57 against 88 for the scatter), and the walk, the creeping test and the
 // piece count compare on the integer pipe.  Measured at 32^3 with 2,097,152 particles (1.31 pieces
-// each): iterate 3.52 -> 1.59 ms, final sweep 2.40 -> 1.11 ms; 25.6M FP64 warp instructions where
-// there were 58.2M, the pipe 83% busy (88% in the final sweep).  Two blocks per SM (128 registers).
+// each): iterate 3.52 -> 1.59 ms (1.43 with the fixed-point deposit), final sweep 2.40 -> 1.11 ms;
+// 25.6M FP64 warp instructions (22.7M) where there were 58.2M, the pipe 83% busy (88% in the final
+// sweep).  Two blocks per SM (128 registers).
 template <bool COMMIT, bool CELLS>
 __global__ void __launch_bounds__(THREADS, 2) k_push_cell(StepParams p, const double* __restrict__ xi,
                                                           const double* __restrict__ v, const double* __restrict__ P,
@@ -718,7 +661,9 @@ __global__ void __launch_bounds__(THREADS, 2) k_push_cell(StepParams p, const do
                                                           const uint8_t* __restrict__ slide,
                                                           double* __restrict__ partials, int* __restrict__ status) {
     __shared__ double sm[32];
-    __shared__ ChunkOrder co;
+    extern __shared__ __align__(16) unsigned char dyn[];
+    ChunkOrder& co = *reinterpret_cast<ChunkOrder*>(dyn);
+    long long* tile = reinterpret_cast<long long*>(dyn + sizeof(ChunkOrder)) + (threadIdx.x >> 5) * DEPOSIT_TILE;
     const int64_t np = p.np, nchunks = (np + THREADS - 1) / THREADS;
     double ev_num = 0.0, ev_den = 0.0;
     long long pieces_push = 0, pieces_scatter = 0;
@@ -736,6 +681,8 @@ __global__ void __launch_bounds__(THREADS, 2) k_push_cell(StepParams p, const do
                 }
             }
             const int64_t i = chunk_exchange(p, co, base, j < np, x0, v2, st, vs);
+            bool scat = false;               // this lane's next orbit is scattered here
+            double bn[3] = {0.0, 0.0, 0.0}, w[3] = {0.0, 0.0, 0.0};
             if (i < np) {
                 double vi[3], vn[3], Pn[3];
 #pragma unroll
@@ -782,18 +729,15 @@ __global__ void __launch_bounds__(THREADS, 2) k_push_cell(StepParams p, const do
                             creep_list[k] = (int32_t)i;
                         }
                     } else {
-                        double w[3];
+                        scat = true;
 #pragma unroll
                         for (int a = 0; a < 3; ++a) {
                             ev_num += d[a] * d[a];
                             ev_den += o.vw[a] * o.vw[a];
                             const double v2n = o.vw[a] + vn[a];
-                            beta[a] = p.cb[a] * v2n;
+                            bn[a] = p.cb[a] * v2n;
                             w[a] = p.q_dV_half * v2n;
                         }
-                        const int ns = scatter_closed(p, st, beta, w, Jnext);
-                        if (ns < 0) atomicOr(status, DEV_ERR_SEGMENTS);
-                        pieces_scatter += ns;
                     }
                 } else {
                     // components sliding onto a knot (set by k_local): the orbit lands on the knot,
@@ -814,6 +758,11 @@ __global__ void __launch_bounds__(THREADS, 2) k_push_cell(StepParams p, const do
                         ev_den += o.vw[a] * o.vw[a];
                     }
                 }
+            }
+            if constexpr (!COMMIT) {
+                const int ns = scatter_warp(p.m, scat, st, bn, w, tile, p.det, p.acc, Jnext);
+                if (ns < 0) atomicOr(status, DEV_ERR_SEGMENTS);
+                pieces_scatter += ns;
             }
         }
         __syncthreads();   // the hand-over buffers are rewritten by the next chunk
@@ -1586,6 +1535,16 @@ StepParams make_params(const Ctx& c) {
     return p;
 }
 
+// Opt the depositing kernels in to their dynamic shared memory (above the 48 KB default; once per
+// context, on its device).
+bool setup_particle_kernels() {
+    const int bytes = (int)CHUNK_SMEM;
+    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    return cudaFuncSetAttribute(k_first_scatter_cell, at, bytes) == cudaSuccess &&
+           cudaFuncSetAttribute(k_push_cell<false, true>, at, bytes) == cudaSuccess &&
+           cudaFuncSetAttribute(k_push_cell<false, false>, at, bytes) == cudaSuccess;
+}
+
 int local_blocks(const Ctx& c) { return std::max(1, std::min(particle_blocks(c), c.sms * 2)); }
 
 int particle_blocks(const Ctx& c) {
@@ -1619,7 +1578,7 @@ void launch_first_scatter(Ctx& c, double* J, const double* v_iter_or_null) {
     StepParams p = make_params(c);
     int nb = particle_blocks(c);
     if (c.cfg.quadrature == PIC_QUAD_CLOSED)
-        k_first_scatter_cell<<<nb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.vprev, v_iter_or_null, c.vit, J, c.partials,
+        k_first_scatter_cell<<<nb, THREADS, CHUNK_SMEM, c.stream>>>(p, c.xi, c.v, c.vprev, v_iter_or_null, c.vit, J, c.partials,
                                                            c.dev_status);
     else
         k_first_scatter<1><<<nb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.vprev, v_iter_or_null, c.vit, J, c.partials,
@@ -1641,7 +1600,7 @@ void launch_push(Ctx& c, const double* vit, double* vnew, double* Jnext, bool co
                                                   c.slide,                                                    \
                                                   c.partials, c.dev_status)
 #define PIC_PUSH_CELL(C, T)                                                                                       \
-    k_push_cell<C, T><<<nb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.P, vit, T ? c.ctab : c.table, vnew, Jnext,     \
+    k_push_cell<C, T><<<nb, THREADS, C ? sizeof(ChunkOrder) : CHUNK_SMEM, c.stream>>>(p, c.xi, c.v, c.P, vit, T ? c.ctab : c.table, vnew, Jnext,     \
                                                     c.xi_new, c.P_new, c.creep_list, c.creep_count,                \
                                                     det ? c.creep_flag : nullptr, c.slide, c.partials, c.dev_status)
     if (closed && !diag) {

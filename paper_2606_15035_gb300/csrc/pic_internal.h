@@ -319,6 +319,7 @@ int cheb_schedule(double lmin, double lmax, double eps, double* alpha, double* b
 // Kernel parameters of the FP64 particle kernels for this context (particles.cu).
 StepParams make_params(const Ctx& c);
 
+bool setup_particle_kernels();
 int particle_blocks(const Ctx& c);
 int local_blocks(const Ctx& c);
 int mesh_blocks(const Ctx& c);

@@ -1,0 +1,170 @@
+// The orbit current of a warp's particles, summed per cell on the integer pipe (sm_103a).
+//
+// Depositing a piece in FP64 takes 46 FP64 instructions and 24 L2 reductions per particle, on a
+// pipe with 1/64 of the issue rate and with one L2 request per lane and reduction (equal addresses
+// of a warp are not merged): both bound the scatters.  Every factor of a deposit is bounded (the
+// moments of orbit_cell.cuh lie in [0, 1], the weights below the warp's largest), so the products
+// and sums run in 64-bit fixed point instead: moments to 2^-62, weights to 2^-57 of the warp's
+// largest, at least as fine as the FP64 products they replace (2^-53 of each, and one more rounding
+// per addition to J), and exact sums.  The warp's particles hold few distinct cells (the store is
+// cell-sorted), so each cell's 24 sums (8 moments, 3 components) are taken by 24 lanes from a
+// transposed shared tile, turned into node weights by three exchanges, and added to J once.
+#pragma once
+
+#include "orbit_cell.cuh"
+
+namespace pic {
+
+constexpr int DEPOSIT_ROWS = 24;
+constexpr int DEPOSIT_STRIDE = 33;   // 33 x 8 B: a row's lanes and a column's rows miss each other's banks
+constexpr int DEPOSIT_TILE = DEPOSIT_ROWS * DEPOSIT_STRIDE;   // 64-bit words per warp
+
+// x times 2^s truncated to an integer, |x| 2^s < 2^63: `drop` is how far the exponent of x is below
+// the one whose mantissa is shifted left by `up`.
+__device__ __forceinline__ long long fixed_of(double x, int top, int up) {
+    const int hi = __double2hiint(x);
+    const int drop = min(max(top - ((hi >> 20) & 0x7ff), 0), 63);
+    const unsigned long long mant =
+        ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x);
+    const long long r = (long long)((mant << up) >> drop);
+    return hi < 0 ? -r : r;
+}
+
+// A factor: its signed high word and the upper 31 bits of its low word.
+struct Fx {
+    int h, l;
+};
+
+__device__ __forceinline__ Fx fx_split(long long v) { return Fx{(int)(v >> 32), (int)((unsigned)v >> 1)}; }
+
+// a b 2^-62 from three 32 x 32 products; the constant stands for the mean of the dropped low product
+// and rounds (errors within about 2 units, mean below a quarter).
+__device__ __forceinline__ long long fx_mul(Fx a, Fx b) {
+    const long long u = (long long)a.h * b.l + ((long long)a.l * b.h + 912680550LL);   // 1.7 x 2^29
+    return (((long long)a.h * b.h) << 2) + (u >> 29);
+}
+
+// Measured at 32^3 with 2,097,152 particles (1.31 pieces each): the first scatter 0.82 -> 0.49 ms with
+// 4.5M L2 reduction requests where there were 67M; at 128^3 with 134M (2.2 pieces) 96 -> 44 ms.
+// In the push it takes 46 FP64 instructions a piece off the pipe that bounds it (1.59 -> 1.43 ms).
+//
+// Add the orbit currents q v_bar S_bar / dV (weights w, orbits st.f + s beta) of the lanes with `act`
+// to J.  Every lane of the warp calls it; `tile` is the warp's DEPOSIT_TILE words.  bs = beta /
+// sqrt(12).  Returns the lane's number of breakpoint intervals (-1: too many; 0: not active).
+__device__ __forceinline__ int scatter_warp(const MeshDims& m, bool act, const CellStart<double>& st,
+                                            const double beta[3], const double w[3], long long* tile, int det,
+                                            const ExactAcc& acc, double* __restrict__ J) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int64_t N = m.ncell;
+    int top[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int e = act ? (__double2hiint(w[a]) >> 20) & 0x7ff : 0;
+        // 64: the unit 2^(top - 1079) stays a normal number
+        top[a] = max((int)__reduce_max_sync(full, (unsigned)e), 64);
+    }
+    if (max(max(top[0], top[1]), top[2]) == 0x7ff) {
+        // a weight that is not finite: the plain deposit, which hands it on to J
+        if (!act) return 0;
+        CellStart<double> s = st;
+        return for_each_piece(s, beta, m, [&](double h, double, const double mid[3], const int c[3]) {
+            double W[8];
+            int64_t g[8];
+            node_weights(piece_moments(h, mid, beta), W);
+            cell_nodes8(c, m, g);
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    if (det) exact_add(acc, a * N + g[k], h * w[a] * W[k]);
+                    else atomicAdd(J + a * N + g[k], h * w[a] * W[k]);
+                }
+        });
+    }
+    if (lane < DEPOSIT_ROWS) tile[lane * DEPOSIT_STRIDE + 32] = 0;
+    // this lane's unit: component lane / 8 (lanes 24..31 sum nothing)
+    const int comp = min(lane >> 3, 2);
+    const double unit = __hiloint2double(((comp == 0 ? top[0] : (comp == 1 ? top[1] : top[2])) - 56) << 20, 0);
+    const double rs12 = 0.28867513459481288225;   // 1 / sqrt(12)
+    double bs[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) bs[a] = rs12 * beta[a];
+    PieceWalk<double> wk(st, beta, m);
+    bool last = !act;
+    while (__any_sync(full, !last)) {
+        bool has = false;
+        int row = -1, pc[3] = {0, 0, 0};
+        if (!last) {
+            double h, sm, mid[3];
+            has = wk.next(beta, m, h, sm, mid, pc, last);
+            if (has) {
+                row = (int)cell_row(pc, m);
+                long long M[8];
+                Fx q[3], d[3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    M[1 << a] = fixed_of(mid[a], 1023, 10);
+                    q[a] = fx_split(M[1 << a]);
+                    d[a] = fx_split(fixed_of(h * bs[a], 1023, 10));
+                }
+                const long long kxy = fx_mul(d[0], d[1]), kxz = fx_mul(d[0], d[2]), kyz = fx_mul(d[1], d[2]);
+                M[3] = fx_mul(q[0], q[1]) + kxy;
+                M[5] = fx_mul(q[0], q[2]) + kxz;
+                M[6] = fx_mul(q[1], q[2]) + kyz;
+                M[7] = fx_mul(q[0], fx_split(M[6])) + fx_mul(q[1], fx_split(kxz)) + fx_mul(q[2], fx_split(kxy));
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const long long wf = fixed_of(h * w[a], top[a], 4);
+                    const Fx ws = fx_split(wf);
+                    tile[(8 * a) * DEPOSIT_STRIDE + lane] = wf;
+#pragma unroll
+                    for (int k = 1; k < 8; ++k) tile[(8 * a + k) * DEPOSIT_STRIDE + lane] = fx_mul(ws, fx_split(M[k]));
+                }
+            }
+        }
+        __syncwarp();
+        unsigned rest = __ballot_sync(full, has);
+        while (rest) {
+            const int lead = __ffs(rest) - 1;
+            const int r = __shfl_sync(full, row, lead);
+            const unsigned group = __ballot_sync(full, row == r);
+            rest &= ~group;
+            int c[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) c[a] = __shfl_sync(full, pc[a], lead);
+            long long s = 0;
+            if (lane < DEPOSIT_ROWS) {
+                const long long* rowp = tile + lane * DEPOSIT_STRIDE;
+                for (unsigned g = group; g;) {   // four loads in flight; the zero column pads the last ones
+                    long long v[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        v[k] = rowp[min((unsigned)(__ffs(g) - 1), 32u)];
+                        g &= g - 1;
+                    }
+                    s += (v[0] + v[1]) + (v[2] + v[3]);
+                }
+            }
+            // moments of the subsets -> weights of the nodes (inclusion--exclusion, axis by axis)
+#pragma unroll
+            for (int bit = 1; bit < 8; bit <<= 1) {
+                const long long o = __shfl_xor_sync(full, s, bit);
+                if (!(lane & bit)) s -= o;
+            }
+            if (lane < DEPOSIT_ROWS && s != 0) {
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+                    if ((lane >> a) & 1) c[a] = next_cell(c[a], m.n[a]);
+                const int64_t at = comp * N + cell_row(c, m);
+                const double v = (double)s * unit;
+                if (det) exact_add(acc, at, v);
+                else atomicAdd(J + at, v);
+            }
+        }
+        __syncwarp();   // the tile is rewritten by the next pieces
+    }
+    return act ? wk.count : 0;
+}
+
+}  // namespace pic
