@@ -11,35 +11,29 @@
 // size), so its fixed point is the FP64 fixed point to that level.  What checks the iterate
 // is FP64: the FP64 final sweep, which measures ||G(v*) - v*|| of the pair iterate itself
 // before committing it (the mixed path's default with mixed_tol64 > 0), or the FP64
-// iterations that follow.  Compiled for four resident blocks per SM (64 registers, with
-// spills): the pair arithmetic's dependent chains need the warps more than the registers.
+// iterations that follow.
 //
-// Per chunk of THREADS cell-sorted particles the next-orbit current goes into a shared-memory
-// tile of 64-bit fixed-point sums (exact, order independent, 2^-52 of the chunk's largest
-// weight per unit), added to the FP64 J once per node; a chunk whose orbits' node box does not
-// fit the tile adds its contributions to J directly.
+// The orbit integrals are those of the FP64 kernels (orbit_cell.cuh) on pairs, from a cell table of
+// pairs; the hand-over by piece count, the gates and the next orbit's current (fixed point,
+// scatter_warp.cuh) are theirs too.
 #include <algorithm>
 #include <climits>
 #include <cmath>
 
 #include "pic_internal.h"
-#include "particle_common.cuh"
 #include "dfloat.cuh"
+#include "chunk.cuh"
 
 namespace pic {
 namespace {
 
-constexpr int DF_TILE_CAP = 320;   // nodes of a chunk's current tile
-constexpr int DF_NODE4 = 5;        // float4 per node of the pair table: A^n, A^{n+1}, grad phi (9 pairs)
+// Blocks per SM: 2 (128 registers) measured 88.5 ms at 128^3 with 134M particles, 3 (85) 100.4.
+constexpr int DF_MINB = 2;
 
 struct ParamsDF {
     StepParams p;       // the FP64 parameters (creeping tests, residual sums, iterate I/O)
-    DF dth[3];          // dt / (2 H_a): beta_a = dth_a (u_a + v^n_a)
-    DF dt_invH[3];      // dt / H_a
-    DF invH[3];         // 1 / H_a
-    DF dt_q;            // dt q
-    DF q;
-    DF q_dV;            // q / dV
+    DF cb[3], ihs[3];   // dt / (2 H), 1 / (2 H): factors of v^p + v^n
+    DF dtq, q;          // dt q, q
 };
 
 DF pair_of(double d) {
@@ -47,365 +41,187 @@ DF pair_of(double d) {
     return DF(h, (float)(d - (double)h));
 }
 
-// The 9 pairs of node g: A^n (3), A^{n+1} (3), grad_h phi^{n+1/2} (3).
-struct NodeDF {
-    DF An[3], A1[3], g[3];
+// Loader of a cell's pair entries, as FieldLoad: from the pair cell table, or from the pairs of the
+// gather table (5 float4 per node: A^n, A^{n+1}, grad phi), taking the nodes' differences.
+template <bool CELLS>
+struct PairLoad {
+    const float4* t;
+    __device__ __forceinline__ PairLoad(const float4* table, const int c[3], const MeshDims& m)
+        : t(table + (CELL_VALUES / 2) * cell_row(c, m)) {}
+    __device__ __forceinline__ void operator()(int p, int col, DF& a, DF& b) const {
+        const float4 q = __ldg(t + p * CELL_COLS + col);
+        a = DF(q.x, q.y);
+        b = DF(q.z, q.w);
+    }
 };
 
-__device__ __forceinline__ NodeDF load_node(const float4* __restrict__ t, int64_t g) {
-    const float4* q = t + DF_NODE4 * g;
-    const float4 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + 2), d = __ldg(q + 3), e = __ldg(q + 4);
-    NodeDF n;
-    n.An[0] = DF(a.x, a.y);
-    n.An[1] = DF(a.z, a.w);
-    n.An[2] = DF(b.x, b.y);
-    n.A1[0] = DF(b.z, b.w);
-    n.A1[1] = DF(c.x, c.y);
-    n.A1[2] = DF(c.z, c.w);
-    n.g[0] = DF(d.x, d.y);
-    n.g[1] = DF(d.z, d.w);
-    n.g[2] = DF(e.x, e.y);
-    return n;
-}
+constexpr int DF_NODE = 10;   // pairs per node of the pair gather table (9 and a pad)
 
-__device__ __forceinline__ void cell_nodes(const int c[3], const MeshDims& m, int64_t g[8]) {
-    Segment<float> s;
-    s.cell[0] = c[0];
-    s.cell[1] = c[1];
-    s.cell[2] = c[2];
-    segment_nodes8(s, m, g);
-}
-
-// One knot-free piece of the push (Appendices A and B), as push_piece_fast in FP64: the
-// orbit gather of grad phi and (D_i A)^T vbar, contracted with vbar first.  Piece cells are
-// relative to the particle's start cell c0.
-__device__ __forceinline__ void push_piece_df(const ParamsDF& pd, const Segment<DF>& sg, const int c0[3],
-                                              const DF beta[3], const DF vb[3], const float4* __restrict__ table,
-                                              DF gphi[3], DF F[3]) {
-    const PieceInts<DF> I = piece_integrals(sg, beta, true);
-    DF W[8];
-    weights_from_ints(I, W);
-    const int c[3] = {c0[0] + sg.cell[0], c0[1] + sg.cell[1], c0[2] + sg.cell[2]};
+template <>
+struct PairLoad<false> {
+    const float2* t;
     int64_t g[8];
-    cell_nodes(c, pd.p.m, g);
-    const DF s = sg.s0, oms = DF(1) - sg.s0, h = sg.h, hh2 = DF(0.5f) * (sg.h * sg.h);
-    DF am[8], cc[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const NodeDF n = load_node(table, g[k]);
-        const DF an = n.An[0] * vb[0] + n.An[1] * vb[1] + n.An[2] * vb[2];   // A^n_g . vbar
-        const DF a1 = n.A1[0] * vb[0] + n.A1[1] * vb[1] + n.A1[2] * vb[2];   // A^{n+1}_g . vbar
-        am[k] = oms * an + s * a1;                                           // A^{(m)}_nu . vbar
-        cc[k] = a1 - an;                                                     // C^{(m)}_nu . vbar
-        gphi[0] += W[k] * n.g[0];
-        gphi[1] += W[k] * n.g[1];
-        gphi[2] += W[k] * n.g[2];
+    __device__ __forceinline__ PairLoad(const float4* table, const int c[3], const MeshDims& m)
+        : t(reinterpret_cast<const float2*>(table)) {
+        cell_nodes8(c, m, g);
     }
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        const int pa = j == 0 ? 1 : 0, qa = j == 2 ? 1 : 2;
-        const int sp = j == 0 ? 2 : 1, sq = j == 2 ? 2 : 4;
-        const int sj = j == 0 ? 1 : (j == 1 ? 2 : 4);
-        const DF D00 = am[sj] - am[0], D10 = am[sp + sj] - am[sp];
-        const DF D01 = am[sq + sj] - am[sq], D11 = am[sp + sq + sj] - am[sp + sq];
-        const DF C00 = cc[sj] - cc[0], C10 = cc[sp + sj] - cc[sp];
-        const DF C01 = cc[sq + sj] - cc[sq], C11 = cc[sp + sq + sj] - cc[sp + sq];
-        const DF t0 = D00 * h + (D10 - D00) * I.S1[pa] + (D01 - D00) * I.S1[qa] + (D11 - D10 - D01 + D00) * I.S2[j];
-        const DF t1 = C00 * hh2 + (C10 - C00) * I.E1[pa] + (C01 - C00) * I.E1[qa] + (C11 - C10 - C01 + C00) * I.E2[j];
-        F[j] += pd.invH[j] * (t0 + t1);
+    __device__ __forceinline__ DF get(int k, int col) const {
+        const float2 q = __ldg(t + DF_NODE * g[k] + col);
+        return DF(q.x, q.y);
     }
-}
-
-// Minimal-image offset of cell c from cell ref on a periodic axis of n cells.
-__device__ __forceinline__ int rel_cell_df(int c, int ref, int n) {
-    int d = c - ref;
-    if (2 * d > n) d -= n;
-    else if (2 * d < -n) d += n;
-    return d;
-}
-
-// Block-wide box of node ranges [lo, hi] and maxima of amax (non-negative floats, reduced
-// through their bit patterns); sm holds 9 * 32 + 9 ints.  Every thread gets the result.
-__device__ __forceinline__ void block_box_df(int lo[3], int hi[3], float amax[3], int* sm) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int v[9];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        v[a] = __reduce_min_sync(0xffffffffu, lo[a]);
-        v[3 + a] = __reduce_max_sync(0xffffffffu, hi[a]);
-        v[6 + a] = __reduce_max_sync(0xffffffffu, __float_as_int(amax[a]));
+    __device__ __forceinline__ DF node(int k, int col) const {
+        return col < 3 ? get(k, 3 + col) : (col < 6 ? get(k, col) - get(k, col - 3) : -get(k, col));
     }
-    if (lane == 0) {
-#pragma unroll
-        for (int t = 0; t < 9; ++t) sm[t * 32 + wid] = v[t];
+    __device__ __forceinline__ void operator()(int p, int col, DF& a, DF& b) const {
+        a = node(0, col);
+        b = node(1, col) - a;
+        if (p == 0) return;
+        if (p == 3) {
+            DF lo = node(2, col), hi = node(3, col) - lo;
+            a = lo - a;
+            b = hi - b;
+            lo = node(4, col);
+            hi = node(5, col) - lo;
+            const DF l6 = node(6, col);
+            a = (l6 - lo) - a;
+            b = ((node(7, col) - l6) - hi) - b;
+        } else {
+            const DF lo = node(2 * p, col);
+            a = lo - a;
+            b = (node(2 * p + 1, col) - lo) - b;
+        }
     }
-    __syncthreads();
-    if (threadIdx.x < 9) {
-        const int t = threadIdx.x;
-        int r = sm[t * 32];
-        for (int w = 1; w < nw; ++w) r = t < 3 ? min(r, sm[t * 32 + w]) : max(r, sm[t * 32 + w]);
-        sm[288 + t] = r;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        lo[a] = sm[288 + a];
-        hi[a] = sm[291 + a];
-        amax[a] = __int_as_float(sm[294 + a]);
-    }
-    __syncthreads();   // sm is reused by the next reduction
-}
-
-// The chunk's current tile: node (lx, ly, lz) of the box at lx + ex (ly + ey lz), one 64-bit
-// fixed-point sum per component in units of 1 / scale[a].
-struct TileDF {
-    long long* jt;
-    int lo[3], ext[3];
-    int vol;
-    float scale[3];
 };
 
-__device__ __forceinline__ long long fixed64(DF c, float scale) {
-    return __float2ll_rn(c.hi * scale) + __float2ll_rn(c.lo * scale);   // exact scaling by a power of 2
-}
-
-// Next-orbit current of one particle (closed-form weights, Appendix A): into the tile when
-// `tiled`, else straight into the FP64 J.
-__device__ __forceinline__ int scatter_df(const ParamsDF& pd, const TileDF& tl, bool tiled, const int c0[3],
-                                          const int co[3], const DF x0[3], const DF beta[3], const DF w[3],
-                                          double* __restrict__ J) {
-    const int64_t N = pd.p.m.ncell;
-    return for_each_segment(x0, beta, true, [&](const Segment<DF>& sg) {
-        DF I[8];
-        weights_from_ints(piece_integrals(sg, beta, false), I);
-        if (tiled) {
-            const int lx = co[0] + sg.cell[0] - tl.lo[0], ly = co[1] + sg.cell[1] - tl.lo[1];
-            const int lz = co[2] + sg.cell[2] - tl.lo[2];
-            const int ex = tl.ext[0], exy = tl.ext[0] * tl.ext[1];
-            const int base = lx + ex * ly + exy * lz;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int l = base + (k & 1) + ((k >> 1) & 1) * ex + (k >> 2) * exy;
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-                    atomicAdd(reinterpret_cast<unsigned long long*>(tl.jt + a * DF_TILE_CAP + l),
-                              (unsigned long long)fixed64(w[a] * I[k], tl.scale[a]));
-            }
-        } else {
-            const int c[3] = {c0[0] + sg.cell[0], c0[1] + sg.cell[1], c0[2] + sg.cell[2]};
-            int64_t g[8];
-            cell_nodes(c, pd.p.m, g);
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-#pragma unroll
-                for (int a = 0; a < 3; ++a) atomicAdd(J + a * N + g[k], dbl_of(w[a] * I[k]));
-        }
-    });
-}
-
-// The FP32-pair iteration: G(v^p) for every particle, creeping ones listed for k_local (as in
-// k_push), the e_v partial sums, and the orbit current of v^{p+1} = G(v^p) into Jnext.
-__global__ void __launch_bounds__(THREADS, 4) k_push_df(ParamsDF pd, const double* __restrict__ xi,
-                                                         const double* __restrict__ v, const double* __restrict__ P,
-                                                         const double* __restrict__ vit,
-                                                         const float4* __restrict__ table, double* __restrict__ vnew,
-                                                         double* __restrict__ Jnext, int32_t* __restrict__ creep_list,
-                                                         int* __restrict__ creep_count,
-                                                         uint8_t* __restrict__ creep_flag,
-                                                         const uint8_t* __restrict__ slide,
-                                                         double* __restrict__ partials, int* __restrict__ status) {
+// The FP32-pair iteration (239 -> 88.5 ms at 128^3 with 134M particles, from start-based integrals, a
+// node table and shared 64-bit atomics before): G(v^p) for every particle, creeping ones listed for k_local (as in
+// k_push_cell), the e_v partial sums, and the orbit current of v^{p+1} = G(v^p) into Jnext.
+template <bool CELLS>
+__global__ void __launch_bounds__(THREADS, DF_MINB) k_push_df(ParamsDF pd, const double* __restrict__ xi,
+                                                               const double* __restrict__ v,
+                                                               const double* __restrict__ P,
+                                                               const double* __restrict__ vit,
+                                                               const float4* __restrict__ table,
+                                                               double* __restrict__ vnew, double* __restrict__ Jnext,
+                                                               int32_t* __restrict__ creep_list,
+                                                               int* __restrict__ creep_count,
+                                                               const uint8_t* __restrict__ slide,
+                                                               double* __restrict__ partials,
+                                                               int* __restrict__ status) {
     __shared__ double sm[32];
-    __shared__ int order[THREADS];
-    __shared__ int wcount[THREADS / 32][PIECE_CLASSES];
-    __shared__ int sbox[9 * 32 + 9];
-    __shared__ long long jt[3 * DF_TILE_CAP];
+    extern __shared__ __align__(16) unsigned char dyn[];
+    ChunkOrder& co = *reinterpret_cast<ChunkOrder*>(dyn);
+    long long* tile = reinterpret_cast<long long*>(dyn + sizeof(ChunkOrder)) + (threadIdx.x >> 5) * DEPOSIT_TILE;
     const StepParams& p = pd.p;
     const int64_t np = p.np, nchunks = (np + THREADS - 1) / THREADS;
-    double ev_num = 0.0, ev_den = 0.0, pieces_push = 0.0, pieces_scatter = 0.0;
+    double ev_num = 0.0, ev_den = 0.0;
+    long long pieces_push = 0, pieces_scatter = 0;
     for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-        const int64_t base = ch * THREADS;
-        {
-            const int64_t j = base + threadIdx.x;
-            const int cls = j < np ? piece_class(p, xi, v, vit, j) : PIECE_CLASSES - 1;
-            order[stable_class_rank(cls, wcount)] = threadIdx.x;
+        const int64_t base = ch * THREADS, j = base + threadIdx.x;
+        double x0[3], vs[3], v2[3];
+        CellStart<double> st;
+        if (j < np) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                x0[a] = xi[a * np + j];
+                v2[a] = vit[a * np + j] + v[a * np + j];
+            }
         }
-        __syncthreads();
-        const int64_t i = base + order[threadIdx.x];
-        int ref[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) ref[a] = min(max((int)::floor(xi[a * np + base]), 0), p.m.n[a] - 1);
-        // the particle's push; `scat` is set when its next orbit is scattered here
-        bool scat = false;
-        int c0[3] = {0, 0, 0}, co[3] = {0, 0, 0}, lo[3] = {INT_MAX, INT_MAX, INT_MAX}, hi[3] = {INT_MIN, INT_MIN, INT_MIN};
-        float amax[3] = {0.f, 0.f, 0.f};
-        DF off[3], beta2[3], w2[3];
+        const int64_t i = chunk_exchange(p, co, base, j < np, x0, v2, st, vs);
+        bool scat = false;               // this lane's next orbit is scattered here
+        double bn[3] = {0.0, 0.0, 0.0}, w[3] = {0.0, 0.0, 0.0};
         if (i < np) {
-            double x0[3], vn[3], vi[3], Pn[3];
-            DF vb[3], beta[3];
+            DF kick[3];
+            {
+                CellStart<DF> sd;
+                DF vd[3], beta[3], acc[3], Ae[3];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                x0[a] = xi[a * np + i];
-                vn[a] = v[a * np + i];
-                vi[a] = vit[a * np + i];
-                Pn[a] = P[a * np + i];
-                const double cf = ::floor(x0[a]);
-                c0[a] = (int)cf;
-                off[a] = df_of(x0[a] - cf);              // exact in FP64, then to a pair
-                vb[a] = df_of(0.5 * (vi[a] + vn[a]));
-                beta[a] = vb[a] * pd.dt_invH[a];
-            }
-            DF gphi[3], F[3];
-            const int nseg = for_each_segment(off, beta, true, [&](const Segment<DF>& sg) {
-                push_piece_df(pd, sg, c0, beta, vb, table, gphi, F);
-            });
-            if (nseg < 0) atomicOr(status, DEV_ERR_SEGMENTS);
-            pieces_push += (double)nseg;
-            // x^{n+1} in the cells of the start, A_h^{n+1}(x^{n+1}) by the point interpolant
-            DF xe[3], r[3];
-            int ce[3];
+                for (int a = 0; a < 3; ++a) {
+                    sd.f[a] = df_bits(st.f[a]);
+                    sd.c[a] = st.c[a];
+                    vd[a] = df_bits(vs[a]);
+                    beta[a] = pd.cb[a] * vd[a];
+                }
+                const int nseg = for_each_piece(sd, beta, p.m, [&](DF h, DF sc, const DF mid[3], const int c[3]) {
+                    piece_impulse(h, sc, mid, beta, vd, pd.ihs, PairLoad<CELLS>(table, c, p.m), acc);
+                });
+                if (nseg < 0) atomicOr(status, DEV_ERR_SEGMENTS);
+                pieces_push += nseg;
+                cell_A1(sd.f, PairLoad<CELLS>(table, sd.c, p.m), Ae);
+                // P^{n+1} - P^n - q A_h^{n+1}(x^{n+1}) (Eqs. (orbit-P-update), (orbit-v-update))
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                xe[a] = off[a] + beta[a];
-                const DF f = floor(xe[a]);
-                ce[a] = c0[a] + (int)f;
-                r[a] = xe[a] - f;
+                for (int a = 0; a < 3; ++a) kick[a] = mad(pd.dtq, acc[a], -(pd.q * Ae[a]));
             }
-            int64_t ge[8];
-            cell_nodes(ce, p.m, ge);
-            DF Ae[3];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const DF wx = (k & 1) ? r[0] : DF(1) - r[0];
-                const DF wy = (k & 2) ? r[1] : DF(1) - r[1];
-                const DF wz = (k & 4) ? r[2] : DF(1) - r[2];
-                const DF wk = wx * wy * wz;
-                const NodeDF n = load_node(table, ge[k]);
-                Ae[0] += wk * n.A1[0];
-                Ae[1] += wk * n.A1[1];
-                Ae[2] += wk * n.A1[2];
-            }
-            double vw[3];
+            double vw[3], d[3], vn[3], vi[3], beta[3];
             bool finite = true;
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                const double Pw = Pn[a] + dbl_of(pd.dt_q * (F[a] - gphi[a]));   // Eq. (orbit-P-update)
-                vw[a] = (Pw - dbl_of(pd.q * Ae[a])) * p.inv_mass;              // Eq. (orbit-v-update)
+                vw[a] = (P[a * np + i] + dbl_of(kick[a])) * p.inv_mass;
                 finite = finite && isfinite(vw[a]);
+                vi[a] = vit[a * np + i];
+                vn[a] = v[a * np + i];
+                d[a] = vw[a] - vi[a];
+                beta[a] = p.cb[a] * vs[a];
             }
             if (!finite) atomicOr(status, DEV_ERR_NONFINITE);
-            // the local-solve gate of k_push, in FP64
-            double beta_it[3];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) beta_it[a] = p.dt * 0.5 * (vi[a] + vn[a]) * p.invH[a];
-            const double xk[3] = {x0[0] - p.koff, x0[1] - p.koff, x0[2] - p.koff};
+            // the local-solve gate of k_push_cell, in FP64
             bool slow = false;
             if (p.hist) {
-                double dn = 0.0, dold = 0.0;
+                double dold = 0.0;
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    dn = fmax(dn, ::fabs(vw[a] - vi[a]));
-                    dold = fmax(dold, ::fabs(vi[a] - vnew[a * np + i]));
-                }
-                const double spd = sqrt(vi[0] * vi[0] + vi[1] * vi[1] + vi[2] * vi[2]);
-                slow = dn > SLOW_RATIO * dold && dn > pd.p.slow_floor * spd;
+                for (int a = 0; a < 3; ++a) dold = max_pos(dold, ::fabs(vi[a] - vnew[a * np + i]));
+                const double dn = max_pos(max_pos(::fabs(d[0]), ::fabs(d[1])), ::fabs(d[2]));
+                if (less_pos(SLOW_RATIO * dold, dn))
+                    slow = dn > p.slow_floor * sqrt(vi[0] * vi[0] + vi[1] * vi[1] + vi[2] * vi[2]);
             }
-            const bool creep = p.accel && (is_creeping(xk, beta_it) || (slide[i] & SLIDE_CREPT) || slow);
-            if (creep_flag) creep_flag[i] = creep ? 1 : 0;
+            const bool creep = p.accel && (is_creeping_cell(st.f, beta) || (slide[i] & SLIDE_CREPT) || slow);
 #pragma unroll
             for (int a = 0; a < 3; ++a) vnew[a * np + i] = vw[a];
             if (creep) {
-                if (!creep_flag) {
-                    const int k = atomicAdd(creep_count, 1);
-                    creep_list[k] = (int32_t)i;
-                }
+                const int k = atomicAdd(creep_count, 1);
+                creep_list[k] = (int32_t)i;
             } else {
-                double dnum = 0.0, dden = 0.0;
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const double d = vw[a] - vi[a];
-                    dnum += d * d;
-                    dden += vw[a] * vw[a];
-                    const DF vb2 = df_of(0.5 * (vw[a] + vn[a]));
-                    beta2[a] = vb2 * pd.dt_invH[a];
-                    w2[a] = vb2 * pd.q_dV;
-                    amax[a] = fabsf(w2[a].hi);
-                }
-                ev_num += dnum;
-                ev_den += dden;
                 scat = true;
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
-                    co[a] = rel_cell_df(c0[a], ref[a], p.m.n[a]);
-                    const DF xe2 = off[a] + beta2[a];
-                    const int e0 = (int)floor(fmin(off[a], xe2)), e1 = (int)floor(fmax(off[a], xe2));
-                    lo[a] = co[a] + e0;
-                    hi[a] = co[a] + e1 + 1;
+                    ev_num += d[a] * d[a];
+                    ev_den += vw[a] * vw[a];
+                    const double v2n = vw[a] + vn[a];
+                    bn[a] = p.cb[a] * v2n;
+                    w[a] = p.q_dV_half * v2n;
                 }
             }
         }
-        // the chunk's node box of the next orbits, and its fixed-point scales
-        block_box_df(lo, hi, amax, sbox);
-        TileDF tl;
-        int64_t vol = 1;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            tl.lo[a] = lo[a];
-            tl.ext[a] = hi[a] - lo[a] + 1;
-            vol *= tl.ext[a] > 0 ? tl.ext[a] : 0;
-            int e = 0;
-            frexpf(amax[a], &e);                    // amax < 2^e: a contribution maps below 2^52
-            tl.scale[a] = ldexpf(1.f, 52 - max(e, -60));
-        }
-        const bool tiled = vol > 0 && vol <= DF_TILE_CAP;
-        tl.vol = tiled ? (int)vol : 0;
-        tl.jt = jt;
-        if (tiled) {
-            for (int l = threadIdx.x; l < 3 * DF_TILE_CAP; l += blockDim.x) jt[l] = 0;
-            __syncthreads();
-        }
-        if (scat) {
-            const int ns = scatter_df(pd, tl, tiled, c0, co, off, beta2, w2, Jnext);
-            if (ns < 0) atomicOr(status, DEV_ERR_SEGMENTS);
-            pieces_scatter += (double)ns;
-        }
-        if (tiled) {
-            __syncthreads();
-            const int64_t N = p.m.ncell;
-            const int ex = tl.ext[0], exy = tl.ext[0] * tl.ext[1];
-            for (int l = threadIdx.x; l < tl.vol; l += blockDim.x) {
-                const int lz = l / exy, rr = l - lz * exy, ly = rr / ex, lx = rr - ly * ex;
-                const int64_t g = node_index(wrapi(ref[0] + tl.lo[0] + lx, p.m.n[0]),
-                                             wrapi(ref[1] + tl.lo[1] + ly, p.m.n[1]),
-                                             wrapi(ref[2] + tl.lo[2] + lz, p.m.n[2]), p.m);
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const long long s = jt[a * DF_TILE_CAP + l];
-                    if (s != 0) atomicAdd(Jnext + a * N + g, (double)s / (double)tl.scale[a]);
-                }
-            }
-        }
-        __syncthreads();   // order[] and the tile are rewritten by the next chunk
+        const int ns = scatter_warp(p.m, scat, st, bn, w, tile, 0, p.acc, Jnext);
+        if (ns < 0) atomicOr(status, DEV_ERR_SEGMENTS);
+        pieces_scatter += ns;
+        __syncthreads();   // the hand-over buffers are rewritten by the next chunk
     }
     write_partial<double>(partials, S_EV_NUM, ev_num, sm, false);
     write_partial<double>(partials, S_EV_DEN, ev_den, sm, false);
-    write_partial<double>(partials, S_PIECES_PUSH, pieces_push, sm, false);
-    write_partial<double>(partials, S_PIECES_SCATTER, pieces_scatter, sm, false);
+    write_partial<double>(partials, S_PIECES_PUSH, (double)pieces_push, sm, false);
+    write_partial<double>(partials, S_PIECES_SCATTER, (double)pieces_scatter, sm, false);
+}
+
+__device__ __forceinline__ float4 pairs_of(double a, double b) {
+    const float ah = (float)a, bh = (float)b;
+    return make_float4(ah, (float)(a - (double)ah), bh, (float)(b - (double)bh));
+}
+
+// FP64 cell table -> pair cell table, entry by entry.
+__global__ void k_cells_df(int64_t n, const double2* __restrict__ t64, float4* __restrict__ tdf) {
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+        const double2 q = t64[k];
+        tdf[k] = pairs_of(q.x, q.y);
+    }
 }
 
 // FP64 gather table (12 doubles per node) -> pair table (A^n, A^{n+1}, grad phi as pairs).
 __global__ void k_table_df(int64_t N, const double* __restrict__ t64, float4* __restrict__ tdf) {
     for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < N; g += (int64_t)gridDim.x * blockDim.x) {
-        float f[20];
+        const double* t = t64 + 12 * g;
 #pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            const double d = t64[12 * g + k];
-            const float h = (float)d;
-            f[2 * k] = h;
-            f[2 * k + 1] = (float)(d - (double)h);
-        }
-        f[18] = f[19] = 0.f;
-#pragma unroll
-        for (int q = 0; q < DF_NODE4; ++q) tdf[DF_NODE4 * g + q] = make_float4(f[4 * q], f[4 * q + 1], f[4 * q + 2], f[4 * q + 3]);
+        for (int q = 0; q < DF_NODE / 2; ++q) tdf[(DF_NODE / 2) * g + q] = pairs_of(t[2 * q], q < 4 ? t[2 * q + 1] : 0.0);
     }
 }
 
@@ -414,32 +230,46 @@ ParamsDF make_params_df(const Ctx& c) {
     pd.p = make_params(c);
     pd.p.hist = c.cfg.picard_accel && c.run.hist;
     for (int a = 0; a < 3; ++a) {
-        pd.dth[a] = pair_of(0.5 * c.cfg.dt / c.H[a]);
-        pd.dt_invH[a] = pair_of(c.cfg.dt / c.H[a]);
-        pd.invH[a] = pair_of(c.invH[a]);
+        pd.cb[a] = pair_of(pd.p.cb[a]);
+        pd.ihs[a] = pair_of(pd.p.ihs[a]);
     }
-    pd.dt_q = pair_of(c.cfg.dt * c.q);
+    pd.dtq = pair_of(pd.p.dtq);
     pd.q = pair_of(c.q);
-    pd.q_dV = pair_of(c.q / c.dV);
     return pd;
 }
 
 }  // namespace
 
+bool setup_pair_kernels() {
+    const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    return cudaFuncSetAttribute(k_push_df<true>, at, (int)CHUNK_SMEM) == cudaSuccess &&
+           cudaFuncSetAttribute(k_push_df<false>, at, (int)CHUNK_SMEM) == cudaSuccess;
+}
+
 void launch_table_df(Ctx& c) {
-    k_table_df<<<mesh_blocks(c), THREADS, 0, c.stream>>>(c.m.ncell, c.table, reinterpret_cast<float4*>(c.table_pair));
+    float4* t = reinterpret_cast<float4*>(c.table_pair);
+    if (c.pair_cells) {
+        const int64_t n = CELL_VALUES / 2 * c.m.ncell;
+        const int nb = (int)std::max<int64_t>(1, std::min<int64_t>((n + THREADS - 1) / THREADS, (int64_t)c.sms * 16));
+        k_cells_df<<<nb, THREADS, 0, c.stream>>>(n, reinterpret_cast<const double2*>(c.ctab), t);
+    } else {
+        k_table_df<<<mesh_blocks(c), THREADS, 0, c.stream>>>(c.m.ncell, c.table, t);
+    }
     ++c.launches;
 }
 
 void launch_push_df(Ctx& c, const double* vit, double* vnew, double* Jnext) {
-    const bool det = c.cfg.deterministic != 0;
     cudaMemsetAsync(c.creep_count, 0, 2 * sizeof(int), c.stream);   // count, k_local queue head
     int nb = (int)std::max<int64_t>(1, std::min<int64_t>((c.np + THREADS - 1) / THREADS, (int64_t)c.sms * c.push_bps));
     nb = std::min(nb, MAX_BLOCKS);
-    k_push_df<<<nb, THREADS, 0, c.stream>>>(make_params_df(c), c.xi, c.v, c.P, vit,
-                                            reinterpret_cast<const float4*>(c.table_pair), vnew, Jnext, c.creep_list,
-                                            c.creep_count, det ? c.creep_flag : nullptr, c.slide, c.partials,
-                                            c.dev_status);
+    const float4* t = reinterpret_cast<const float4*>(c.table_pair);
+#define PIC_PUSH_DF(T)                                                                                            \
+    k_push_df<T><<<nb, THREADS, CHUNK_SMEM, c.stream>>>(make_params_df(c), c.xi, c.v, c.P, vit, t, vnew, Jnext,     \
+                                                        c.creep_list, c.creep_count, c.slide, c.partials,          \
+                                                        c.dev_status)
+    if (c.pair_cells) PIC_PUSH_DF(true);
+    else PIC_PUSH_DF(false);
+#undef PIC_PUSH_DF
     ++c.launches;
 }
 

@@ -58,6 +58,7 @@ bool drop_cell_table(pic_ctx* ctx) {
         break;
     }
     c.ctab = nullptr;
+    c.pair_cells = false;   // its buffer is large enough for the pairs of the gather table
     return true;
 }
 
@@ -294,7 +295,7 @@ constexpr size_t CELL_TABLE_MAX_BYTES = (size_t)16 << 30;
 
 pic_status allocate(pic_ctx* ctx) {
     Ctx& c = ctx->c;
-    if (!setup_particle_kernels()) return check_cuda(ctx, "particle kernels");
+    if (!setup_particle_kernels() || !setup_pair_kernels()) return check_cuda(ctx, "particle kernels");
     const int64_t np3 = 3 * std::max<int64_t>(c.np, 1), N = c.m.ncell;
     ALLOC(c.xi, double, np3);
     ALLOC(c.v, double, np3);
@@ -348,7 +349,6 @@ pic_status allocate(pic_ctx* ctx) {
             if (reinterpret_cast<uintptr_t>(q) % 16 != 0)
                 return fail(ctx, PIC_ERR_ARG, "the allocator returned a pointer that is not 16-byte aligned");
         ALLOC(c.table32, float, 12 * N);
-        if (c.cfg.mixed_pair_max > 0 && !c.cfg.deterministic) ALLOC(c.table_pair, float, 20 * N);
     }
     if (c.cfg.deterministic) {
         ALLOC(c.acc_hi, long long, 3 * N);
@@ -428,6 +428,13 @@ pic_status allocate(pic_ctx* ctx) {
     if (c.cfg.quadrature == PIC_QUAD_CLOSED && c.np >= CELL_TABLE_MIN_PPC * N && cells <= CELL_TABLE_MAX_BYTES) {
         c.ctab = (double*)dev_alloc_once(ctx, cells);
         if (c.ctab && reinterpret_cast<uintptr_t>(c.ctab) % 16 != 0) drop_cell_table(ctx);
+    }
+    if (c.cfg.precision == PIC_MIXED && c.cfg.mixed_pair_max > 0 && !c.cfg.deterministic) {
+        if (c.ctab) c.table_pair = (float*)dev_alloc_once(ctx, cells);
+        c.pair_cells = c.table_pair != nullptr;
+        if (!c.table_pair) ALLOC(c.table_pair, float, 20 * N);
+        if (reinterpret_cast<uintptr_t>(c.table_pair) % 16 != 0)
+            return fail(ctx, PIC_ERR_ARG, "the allocator returned a pointer that is not 16-byte aligned");
     }
     cudaMemsetAsync(c.partials, 0, sizeof(double) * (size_t)NSLOT * MAX_BLOCKS, c.stream);
     cudaMemsetAsync(c.results, 0, sizeof(double) * NSLOT, c.stream);

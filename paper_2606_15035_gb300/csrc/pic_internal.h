@@ -181,7 +181,9 @@ struct Ctx {
     int32_t* cell32 = nullptr;
     float *off32 = nullptr, *v32 = nullptr, *vit32 = nullptr, *vnew32 = nullptr;   // iterates: increments
     float* table32 = nullptr;            // 12 * ncell
-    float* table_pair = nullptr;         // 20 * ncell: A^n, A^{n+1}, grad phi as FP32 pairs (+ pad)
+    float* table_pair = nullptr;         // FP32 pairs: the cell table (2 CELL_VALUES * ncell), or of the
+                                         // gather table (20 * ncell: A^n, A^{n+1}, grad phi, pad)
+    bool pair_cells = false;             // which of the two
 
     // reductions and status
     double *partials = nullptr, *results = nullptr;
@@ -320,6 +322,7 @@ int cheb_schedule(double lmin, double lmax, double eps, double* alpha, double* b
 StepParams make_params(const Ctx& c);
 
 bool setup_particle_kernels();
+bool setup_pair_kernels();
 int particle_blocks(const Ctx& c);
 int local_blocks(const Ctx& c);
 int mesh_blocks(const Ctx& c);
