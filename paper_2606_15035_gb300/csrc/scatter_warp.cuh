@@ -64,8 +64,10 @@ __device__ __forceinline__ int scatter_warp(const MeshDims& m, bool act, const C
         // 64: the unit 2^(top - 1079) stays a normal number
         top[a] = max((int)__reduce_max_sync(full, (unsigned)e), 64);
     }
-    if (max(max(top[0], top[1]), top[2]) == 0x7ff) {
-        // a weight that is not finite: the plain deposit, which hands it on to J
+    if (det || max(max(top[0], top[1]), top[2]) == 0x7ff) {
+        // Deterministic mode: each deposit goes to the exact accumulators by itself (the warp's unit
+        // would depend on which particles share it, and with that on the order a state was restored
+        // in).  A weight that is not finite: the plain deposit hands it on to J.
         if (!act) return 0;
         CellStart<double> s = st;
         return for_each_piece(s, beta, m, [&](double h, double, const double mid[3], const int c[3]) {
@@ -156,10 +158,7 @@ __device__ __forceinline__ int scatter_warp(const MeshDims& m, bool act, const C
 #pragma unroll
                 for (int a = 0; a < 3; ++a)
                     if ((lane >> a) & 1) c[a] = next_cell(c[a], m.n[a]);
-                const int64_t at = comp * N + cell_row(c, m);
-                const double v = (double)s * unit;
-                if (det) exact_add(acc, at, v);
-                else atomicAdd(J + at, v);
+                atomicAdd(J + comp * N + cell_row(c, m), (double)s * unit);
             }
         }
         __syncwarp();   // the tile is rewritten by the next pieces
