@@ -17,15 +17,14 @@
 //   3. the particles' derivative pass: each particle's scalar
 //         Phi = lam_gphibar . gphibar + lam_F . (D A)^T vbar + lam_Aend . A_h^{n+1}(x + beta)
 //             + lam_x' . (x + beta) + sum_g lam_J[g] . J_g(particle)
-//      is differentiated with respect to its start position and displacement beta by
-//      forward-mode dual numbers through the same closed-form orbit integrals (dual.cuh), six
-//      directions, with the mesh adjoints and fields held fixed.  beta = dt (v* + v^n) / (2 H)
-//      gives the adjoints of v* and v^n.
+//      is differentiated with respect to its start position and displacement beta in reverse
+//      through the closed-form orbit integrals, with the mesh adjoints and fields held fixed.
+//      beta = dt (v* + v^n) / (2 H) gives the adjoints of v* and v^n.
 // The transposed fixed point (I - K) mu = b0, g(mu) = K mu + b0 being step 3's adjoint of v*,
 // is solved by restarted GMRES with right preconditioning.  The preconditioner is the transpose
 // of the forward iteration's own splitting: a particle that the step solved locally (its
 // slide byte's SLIDE_CREPT bit) gets its 3 x 3 block (I - B^T)^{-1}, B = dG_i / dv*_i with the
-// fields fixed (from the same dual passes); every other particle gets the identity, as the plain
+// fields fixed (dual numbers, dual.cuh); every other particle gets the identity, as the plain
 // Picard update treats it.  The stationary iteration with this splitting is the transposed
 // linearisation of the forward solve, so its spectral radius is that of the forward iteration
 // at the accepted step (below one, since the step converged), and the preconditioned operator's
@@ -47,7 +46,7 @@
 #include <string>
 
 #include "pic_internal.h"
-#include "particle_common.cuh"
+#include "chunk.cuh"
 #include "dual.cuh"
 
 namespace pic {
@@ -330,126 +329,296 @@ __global__ void k_adj_mesh_out(AdjParams ap, const double* __restrict__ y, const
 }
 
 // ---- step 3: the particles' derivative pass --------------------------------------------------------
+//
+// Each particle's scalar Phi (file comment) is differentiated with respect to its start coordinate
+// and displacement in reverse, by hand, piece by piece in the centred form of orbit_cell.cuh.  With
+// f_j = lam_F,j / (2 H_j), a piece contributes h X,
+//     X = sum_k a_k abar_k + cc_k cbar_k + sum_T K_T M_T,
+// where a_k and cc_k are the table's A columns contracted with v (k = subsets of the axes), M_T the
+// moments, abar_k and cbar_k the moments that multiply them in sum_j f_j F_j, and K_T the adjoint-
+// weighted coefficients of -grad phi and of J's adjoint.  X is multilinear in the midpoint m, in
+// kappa = h^2 / 12 (through e = kappa beta and k_pq = kappa beta_p beta_q) and in v, so every partial
+// is one more contraction of the same loaded values; the limits s0, s1 = (knot - x) / beta of the
+// piece pass theirs on to the axis that crosses.  About 300 FP64 operations a piece, where the same
+// derivatives by six dual-number evaluations of the push took 13.6 ms a sweep at 32^3 with 524,288
+// particles.
 
-// Phi of one particle for start x0 and displacement beta (cell units), with the scalar type T.
-template <typename T>
-__device__ __forceinline__ T particle_phi(const AdjParams& ap, const T x0[3], const T beta[3], const double lg[3],
-                                          const double lF[3], const double lAe[3], const double lxe[3],
-                                          const double* __restrict__ table, const double* __restrict__ lJ, T gphi[3],
-                                          T F[3], T Ae[3]) {
+template <bool CELLS>
+__global__ void __launch_bounds__(THREADS, 2) k_adj_derivs(AdjParams ap, const double* __restrict__ xi,
+                                                           const double* __restrict__ v,
+                                                           const double* __restrict__ vstar,
+                                                           const double* __restrict__ table,
+                                                           const double* __restrict__ lJ,
+                                                           const double* __restrict__ lam_P,
+                                                           const double* __restrict__ lam_v,
+                                                           const double* __restrict__ lam_xe,
+                                                           const double* __restrict__ mu,
+                                                           const uint8_t* __restrict__ slide,
+                                                           double* __restrict__ lam_xi, double* __restrict__ gout,
+                                                           double* __restrict__ lvn, double* __restrict__ lPn,
+                                                           int* __restrict__ status) {
+    __shared__ ChunkOrder co;
     const StepParams& p = ap.p;
-    const int64_t N = p.m.ncell;
-    T vb[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        vb[a] = beta[a] * T(p.H[a] / p.dt);
-        gphi[a] = T(0);
-        F[a] = T(0);
-    }
-    T phi = T(0);
-    for_each_segment(x0, beta, true, [&](const Segment<T>& sg) {
-        push_piece_t(p, sg, beta, vb, table, gphi, F);
-        // this particle's orbit current q vbar Sbar / dV against the adjoint of J
-        T I[8];
-        weights_from_ints(piece_integrals(sg, beta, false), I);
-        Segment<double> sd;
-        sd.cell[0] = sg.cell[0];
-        sd.cell[1] = sg.cell[1];
-        sd.cell[2] = sg.cell[2];
-        int64_t g[8];
-        segment_nodes8(sd, p.m, g);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const T s = vb[0] * lJ[g[k]] + vb[1] * lJ[N + g[k]] + vb[2] * lJ[2 * N + g[k]];
-            phi += T(p.q_dV) * I[k] * s;
-        }
-    });
-    T xe[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) xe[a] = wrap_t(x0[a] + beta[a], (double)p.m.n[a]);
-    point_A1_t(p, xe, table, Ae);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        phi += T(lg[a]) * gphi[a] + T(lF[a]) * F[a] + T(lAe[a]) * Ae[a];
-        phi += T(lxe[a]) * (x0[a] + beta[a]);
-    }
-    return phi;
-}
-
-// Per particle: the adjoints of the start position (lam_xi) and of v* (g = dt/(2H) dPhi/dbeta,
-// which is also the adjoint of v^n), and the block B = dG_i/dv*_i (9, row-major) of the
-// transposed solve's preconditioner (zero outside the particles the step solved locally).
-// lam_xe: adjoint of the end position x^{n+1} in cell units.
-__global__ void __launch_bounds__(THREADS) k_adj_derivs(AdjParams ap, const double* __restrict__ xi,
-                                                        const double* __restrict__ v, const double* __restrict__ vstar,
-                                                        const double* __restrict__ table, const double* __restrict__ lJ,
-                                                        const double* __restrict__ lam_P, const double* __restrict__ lam_v,
-                                                        const double* __restrict__ lam_xe, const double* __restrict__ mu,
-                                                        const uint8_t* __restrict__ slide, double* __restrict__ lam_xi,
-                                                        double* __restrict__ gout, double* __restrict__ lvn,
-                                                        double* __restrict__ lPn, double* __restrict__ Bout,
-                                                        int* __restrict__ status) {
-    const StepParams& p = ap.p;
-    const int64_t np = p.np;
-    ADJ_LOOP(i, np) {
-        double x0[3], beta[3], lg[3], lF[3], lAe[3], lxe[3], lP1[3];
-        const uint8_t sb = slide[i];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            x0[a] = xi[a * np + i];
-            beta[a] = p.dt * 0.5 * (vstar[a * np + i] + v[a * np + i]) * p.invH[a];
-            out_adjoints(p, (sb >> a) & 1u, lam_v[a * np + i], lam_P[a * np + i], mu[a * np + i], lP1[a], lAe[a], lg[a],
-                         lF[a]);
-            lxe[a] = lam_xe[a * np + i];
-        }
-        double dB[3][3];
-        bool ok = true;
-        for (int dir = 0; dir < 6; ++dir) {
-            Dual xd[3], bd[3], gphi[3], F[3], Ae[3];
+    const int64_t np = p.np, N = p.m.ncell, nchunks = (np + THREADS - 1) / THREADS;
+    for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
+        const int64_t base = ch * THREADS, j = base + threadIdx.x;
+        double x0[3], v2[3], vs[3];
+        CellStart<double> st;
+        if (j < np) {
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                xd[a] = Dual(x0[a], dir == a ? 1.0 : 0.0);
-                bd[a] = Dual(beta[a], dir == 3 + a ? 1.0 : 0.0);
+                x0[a] = xi[a * np + j];
+                v2[a] = vstar[a * np + j] + v[a * np + j];
             }
-            const Dual phi = particle_phi(ap, xd, bd, lg, lF, lAe, lxe, table, lJ, gphi, F, Ae);
-            ok = ok && isfinite(phi.d);
-            if (dir < 3) {
-                lam_xi[dir * np + i] = phi.d;
-            } else {
-                const int d = dir - 3;
-                const double c = p.dt * 0.5 * p.invH[d];   // d beta_d / d v*_d
-                gout[d * np + i] = c * phi.d;
+        }
+        const int64_t i = chunk_exchange(p, co, base, j < np, x0, v2, st, vs);
+        if (i < np) {
+            const uint8_t sb = slide[i];
+            double beta[3], f[3], ng[3], xbar[3], bbar[3], vbar[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                double lP1, lAe, lg, lF;
+                out_adjoints(p, (sb >> a) & 1u, lam_v[a * np + i], lam_P[a * np + i], mu[a * np + i], lP1, lAe, lg, lF);
+                beta[a] = p.cb[a] * vs[a];
+                f[a] = lF * p.ihs[a];
+                ng[a] = -lg;              // the table holds -grad phi
+                xbar[a] = bbar[a] = vbar[a] = 0.0;
+            }
+            PieceWalk<double> wk(st, beta, p.m);
+            int axis = -1;                // the axis of the crossing that opened the piece
+            double pend = 0.0;            // what the piece before it passed on to that crossing's s
+            for (int it = 0; it < MAX_SEGMENTS; ++it) {
+                const double s0 = wk.s0, s1 = wk.upcoming();
+                double s1bar = 0.0;
+                if (less_pos(s0, s1)) {
+                    const double h = s1 - s0, sm = 0.5 * (s0 + s1), nms = sm - 1.0;
+                    double m[3];
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) m[a] = wk.fd[a] + sm * beta[a];
+                    const PieceMoments<double> q = piece_moments(h, m, beta);
+                    // abar_k and cbar_k
+                    double ab[8], cb[8];
+                    ab[1] = f[0];
+                    ab[2] = f[1];
+                    ab[4] = f[2];
+                    ab[3] = f[0] * m[1] + f[1] * m[0];
+                    ab[5] = f[0] * m[2] + f[2] * m[0];
+                    ab[6] = f[1] * m[2] + f[2] * m[1];
+                    ab[7] = f[0] * q.Pyz + f[1] * q.Pxz + f[2] * q.Pxy;
+                    cb[1] = cb[2] = cb[4] = 0.0;
+                    cb[3] = f[0] * q.e[1] + f[1] * q.e[0];
+                    cb[5] = f[0] * q.e[2] + f[2] * q.e[0];
+                    cb[6] = f[1] * q.e[2] + f[2] * q.e[1];
+                    cb[7] = f[0] * (m[1] * q.e[2] + m[2] * q.e[1]) + f[1] * (m[0] * q.e[2] + m[2] * q.e[0]) +
+                            f[2] * (m[0] * q.e[1] + m[1] * q.e[0]);
+                    double K[8], vb[3], X = 0.0, smx = 0.0, eb[3];
+                    // the adjoint of J: contracted with q v / dV per node, then to mixed differences
+                    {
+                        double W[8];
+                        int64_t g[8];
+                        node_weights(q, W);
+                        cell_nodes8(wk.c, p.m, g);
+                        double w[3];
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) {
+                            w[a] = p.q_dV_half * vs[a];
+                            vb[a] = 0.0;
+                        }
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            const double l0 = lJ[g[k]], l1 = lJ[N + g[k]], l2 = lJ[2 * N + g[k]];
+                            K[k] = w[0] * l0 + w[1] * l1 + w[2] * l2;
+                            vb[0] += W[k] * l0;
+                            vb[1] += W[k] * l1;
+                            vb[2] += W[k] * l2;
+                        }
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) vb[a] *= p.q_dV_half;
+#pragma unroll
+                        for (int bit = 1; bit < 8; bit <<= 1)
+#pragma unroll
+                            for (int k = 0; k < 8; ++k)
+                                if (k & bit) K[k] -= K[k ^ bit];
+                    }
+                    const FieldLoad<CELLS> ld(table, wk.c, p.m);
+                    double a3 = 0.0, a5 = 0.0, a6 = 0.0, a7 = 0.0, c3 = 0.0, c5 = 0.0, c6 = 0.0, c7 = 0.0;
+#pragma unroll
+                    for (int pr = 0; pr < 4; ++pr) {
+                        double C[3][2], A[3][2], G[3][2];
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) {
+                            ld(pr, c, A[c][0], A[c][1]);
+                            ld(pr, 3 + c, C[c][0], C[c][1]);
+                            ld(pr, 6 + c, G[c][0], G[c][1]);
+                        }
+#pragma unroll
+                        for (int o = 0; o < 2; ++o) {
+                            const int k = 2 * pr + o;
+                            K[k] += ng[0] * G[0][o] + ng[1] * G[1][o] + ng[2] * G[2][o];
+                            if (k == 0) continue;
+                            const double cc = C[0][o] * vs[0] + C[1][o] * vs[1] + C[2][o] * vs[2];
+                            const double aa = A[0][o] * vs[0] + A[1][o] * vs[1] + A[2][o] * vs[2] + nms * cc;
+                            const double t = nms * ab[k] + cb[k];
+#pragma unroll
+                            for (int c = 0; c < 3; ++c) vb[c] += ab[k] * A[c][o] + t * C[c][o];
+                            smx += ab[k] * cc;
+                            X += aa * ab[k] + cc * cb[k];
+                            if (k == 3) a3 = aa, c3 = cc;
+                            if (k == 5) a5 = aa, c5 = cc;
+                            if (k == 6) a6 = aa, c6 = cc;
+                            if (k == 7) a7 = aa, c7 = cc;
+                        }
+                    }
+                    X += K[0] + K[1] * m[0] + K[2] * m[1] + K[3] * q.Pxy + K[4] * m[2] + K[5] * q.Pxz + K[6] * q.Pyz +
+                         K[7] * q.S;
+                    // what F adds to the coefficients of the moments
+                    K[1] += f[1] * a3 + f[2] * a5;
+                    K[2] += f[0] * a3 + f[2] * a6;
+                    K[4] += f[0] * a5 + f[1] * a6;
+                    K[3] += f[2] * a7;
+                    K[5] += f[1] * a7;
+                    K[6] += f[0] * a7;
+                    const double mb[3] = {K[1] + K[3] * m[1] + K[5] * m[2] + K[7] * q.Pyz + c7 * cb[6],
+                                          K[2] + K[3] * m[0] + K[6] * m[2] + K[7] * q.Pxz + c7 * cb[5],
+                                          K[4] + K[5] * m[0] + K[6] * m[1] + K[7] * q.Pxy + c7 * cb[3]};
+                    eb[0] = c3 * f[1] + c5 * f[2] + c7 * ab[6];
+                    eb[1] = c3 * f[0] + c6 * f[2] + c7 * ab[5];
+                    eb[2] = c5 * f[0] + c6 * f[1] + c7 * ab[3];
+                    const double kxy = K[3] + K[7] * m[2], kxz = K[5] + K[7] * m[1], kyz = K[6] + K[7] * m[0];
+                    const double t[3] = {eb[0] + kxy * beta[1] + kxz * beta[2], eb[1] + kxy * beta[0] + kyz * beta[2],
+                                         eb[2] + kxz * beta[0] + kyz * beta[1]};
+                    const double h2 = h * h, kap = h2 * (1.0 / 12.0);
+                    double kb = 0.0, mbb = 0.0;   // adjoint of kappa; mb . beta
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        kb += 0.5 * beta[a] * (eb[a] + t[a]);
+                        mbb += mb[a] * beta[a];
+                        xbar[a] += h * mb[a];
+                        bbar[a] += h * (sm * mb[a] + kap * t[a]);
+                        vbar[a] += h * vb[a];
+                    }
+                    const double hbar = X + h2 * (1.0 / 6.0) * kb, half = 0.5 * h * (smx + mbb);
+                    s1bar = half + hbar;
+                    const double sbar = pend + (half - hbar);
+#pragma unroll
+                    for (int a = 0; a < 3; ++a)
+                        if (a == axis) {
+                            const double r = sbar / beta[a];
+                            xbar[a] -= r;
+                            bbar[a] -= r * s0;
+                        }
+                } else {
+                    s1bar = pend;   // a second axis at the same breakpoint
+                }
+                if (same_bits(s1, 1.0)) break;
+                pend = s1bar;
+#pragma unroll
+                for (int a = 2; a >= 0; --a)
+                    if (same_bits(wk.sn[a], s1)) axis = a;
+                wk.cross(s1, beta, p.m);
+            }
+            // the end point: A_h^{n+1}(x + beta) and x + beta themselves
+            double g[3], lP1[3];
+            {
+                double lAe[3], KA[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
-                    // v1 = (P + dt q (-gphibar + F) - q A_end) / m
-                    const double dv1 = (p.dt * p.q * (F[a].d - gphi[a].d) - p.q * Ae[a].d) * p.inv_mass;
-                    dB[a][d] = c * dv1;
+                    double lg, lF;
+                    out_adjoints(p, (sb >> a) & 1u, lam_v[a * np + i], lam_P[a * np + i], mu[a * np + i], lP1[a],
+                                 lAe[a], lg, lF);
+                }
+                const FieldLoad<CELLS> ld(table, wk.c, p.m);
+#pragma unroll
+                for (int pr = 0; pr < 4; ++pr)
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        double e0, e1;
+                        ld(pr, c, e0, e1);
+                        KA[2 * pr] += lAe[c] * e0;
+                        KA[2 * pr + 1] += lAe[c] * e1;
+                    }
+                const double x = wk.te[0], y = wk.te[1], z = wk.te[2];
+                const double r[3] = {KA[1] + KA[3] * y + z * (KA[5] + KA[7] * y),
+                                     KA[2] + KA[3] * x + z * (KA[6] + KA[7] * x),
+                                     KA[4] + KA[5] * x + y * (KA[6] + KA[7] * x)};
+                bool ok = true;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const double e = r[a] + lam_xe[a * np + i];
+                    xbar[a] += e;
+                    g[a] = p.cb[a] * (bbar[a] + e) + vbar[a];   // the orbit's adjoint of v*_a, also of v^n_a
+                    ok = ok && isfinite(xbar[a]) && isfinite(g[a]);
+                }
+                if (!ok) atomicOr(status, DEV_ERR_NONFINITE);
+            }
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                if ((sb >> a) & 1u) {
+                    // nu_a: the direct adjoint of v*_a (its velocity and momentum outputs) plus the
+                    // orbit's; v*_a = 2 d_a H_a / dt - v^n_a with d_a = knot - xi_a
+                    const double nu = lam_v[a * np + i] + p.mass * lam_P[a * np + i] + g[a];
+                    lam_xi[a * np + i] = xbar[a] - nu * 2.0 * p.H[a] / p.dt;
+                    lvn[a * np + i] = g[a] - nu;
+                    lPn[a * np + i] = 0.0;
+                    gout[a * np + i] = 0.0;                  // no fixed-point equation: mu_a = 0
+                } else {
+                    lam_xi[a * np + i] = xbar[a];
+                    lvn[a * np + i] = g[a];
+                    lPn[a * np + i] = lP1[a];
+                    gout[a * np + i] = g[a];
                 }
             }
         }
-        if (!ok) atomicOr(status, DEV_ERR_NONFINITE);
+        __syncthreads();   // the hand-over buffers are rewritten by the next chunk
+    }
+}
+
+// The blocks B = dG_i/dv*_i (9, row-major) of the transposed solve's preconditioner for the particles
+// that the step solved locally, by dual numbers along the three displacements; the caller zeroes the
+// others'.  They depend on the step alone, so once per solve.  Each block lists its share's few such
+// particles first, so that its warps work on full ones.
+constexpr int BLOCKS_SPAN = 4096;
+
+__global__ void __launch_bounds__(THREADS) k_adj_blocks(AdjParams ap, const double* __restrict__ xi,
+                                                        const double* __restrict__ v, const double* __restrict__ vstar,
+                                                        const double* __restrict__ table,
+                                                        const uint8_t* __restrict__ slide, double* __restrict__ Bout) {
+    __shared__ int list[BLOCKS_SPAN];
+    __shared__ int count;
+    const StepParams& p = ap.p;
+    const int64_t np = p.np, nspans = (np + BLOCKS_SPAN - 1) / BLOCKS_SPAN;
+    for (int64_t sp = blockIdx.x; sp < nspans; sp += gridDim.x) {
+        if (threadIdx.x == 0) count = 0;
+        __syncthreads();
+        for (int k = threadIdx.x; k < BLOCKS_SPAN && sp * BLOCKS_SPAN + k < np; k += blockDim.x)
+            if (slide[sp * BLOCKS_SPAN + k] & SLIDE_CREPT) list[atomicAdd(&count, 1)] = k;
+        __syncthreads();
+        for (int t = threadIdx.x; t < 3 * count; t += blockDim.x) {
+            const int64_t i = sp * BLOCKS_SPAN + list[t / 3];
+            const int d = t % 3;
+            const uint8_t sb = slide[i];
+            Dual x0[3], beta[3], vb[3], gphi[3], F[3], xe[3], Ae[3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const bool sl = (sb >> a) & 1u;
-            const double g = gout[a * np + i];          // the orbit's adjoint of v*_a (also of v^n_a)
-            if (sl) {
-                // nu_a: the direct adjoint of v*_a (its velocity and momentum outputs) plus the
-                // orbit's; v*_a = 2 d_a H_a / dt - v^n_a with d_a = knot - xi_a
-                const double nu = lam_v[a * np + i] + p.mass * lam_P[a * np + i] + g;
-                lam_xi[a * np + i] -= nu * 2.0 * p.H[a] / p.dt;
-                lvn[a * np + i] = g - nu;
-                lPn[a * np + i] = 0.0;
-                gout[a * np + i] = 0.0;                  // no fixed-point equation: mu_a = 0
-            } else {
-                lvn[a * np + i] = g;
-                lPn[a * np + i] = lP1[a];
+            for (int a = 0; a < 3; ++a) {
+                x0[a] = Dual(xi[a * np + i], 0.0);
+                beta[a] = Dual(p.dt * 0.5 * (vstar[a * np + i] + v[a * np + i]) * p.invH[a], a == d ? 1.0 : 0.0);
+                vb[a] = beta[a] * Dual(p.H[a] / p.dt);
             }
+            for_each_segment(x0, beta, true,
+                             [&](const Segment<Dual>& sg) { push_piece_t(p, sg, beta, vb, table, gphi, F); });
 #pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                const bool drop = sl || ((sb >> d) & 1u) || !(sb & SLIDE_CREPT);
-                Bout[(3 * a + d) * np + i] = drop ? 0.0 : dB[a][d];
+            for (int a = 0; a < 3; ++a) xe[a] = wrap_t(x0[a] + beta[a], (double)p.m.n[a]);
+            point_A1_t(p, xe, table, Ae);
+            const double c = d == 0 ? p.cb[0] : (d == 1 ? p.cb[1] : p.cb[2]);   // d beta_d / d v*_d
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                // v1 = (P + dt q (-gphibar + F) - q A_end) / m; sliding components have no equation
+                const double dv1 = (p.dtq * (F[a].d - gphi[a].d) - p.q * Ae[a].d) * p.inv_mass;
+                const bool drop = ((sb >> a) & 1u) || ((sb >> d) & 1u);
+                Bout[(3 * a + d) * np + i] = drop ? 0.0 : c * dv1;
             }
         }
+        __syncthreads();   // the list is rewritten by the next span
     }
 }
 
@@ -652,10 +821,22 @@ void launch_adj_mesh_out(Ctx& c, const double* y, const double* pn, const double
 
 void launch_adj_derivs(Ctx& c, const double* xi, const double* v, const double* vstar, const double* lJ,
                        const double* lam_P, const double* lam_v, const double* lam_xe, const double* mu,
-                       double* lam_xi, double* g, double* lvn, double* lPn, double* B) {
-    k_adj_derivs<<<adj_blocks(c, c.np), THREADS, 0, c.stream>>>(adj_params(c), xi, v, vstar, c.table, lJ, lam_P,
-                                                                 lam_v, lam_xe, mu, c.slide, lam_xi, g, lvn, lPn, B,
-                                                                 c.dev_status);
+                       double* lam_xi, double* g, double* lvn, double* lPn) {
+    const int nb = adj_blocks(c, c.np);
+#define PIC_DERIVS(T, TAB)                                                                                        \
+    k_adj_derivs<T><<<nb, THREADS, 0, c.stream>>>(adj_params(c), xi, v, vstar, TAB, lJ, lam_P, lam_v, lam_xe, mu,    \
+                                                  c.slide, lam_xi, g, lvn, lPn, c.dev_status)
+    if (c.ctab) PIC_DERIVS(true, c.ctab);
+    else PIC_DERIVS(false, c.table);
+#undef PIC_DERIVS
+    ++c.launches;
+}
+
+void launch_adj_block_rows(Ctx& c, const double* xi, const double* v, const double* vstar, double* B) {
+    cudaMemsetAsync(B, 0, sizeof(double) * 9 * c.np, c.stream);
+    const int64_t spans = (c.np + BLOCKS_SPAN - 1) / BLOCKS_SPAN;
+    const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(spans, (int64_t)c.sms * 2));
+    k_adj_blocks<<<nb, THREADS, 0, c.stream>>>(adj_params(c), xi, v, vstar, c.table, c.slide, B);
     ++c.launches;
 }
 

@@ -1328,7 +1328,7 @@ void mesh_out(Ctx& c, const double* src, double* dst, cudaMemcpyKind kind, int64
 }
 
 // One transposed sweep at (level n, v*) for the velocity-output adjoint lam_v + mu: the mesh
-// adjoints (adj_F0, adj_W0, adj_rho0, adj_J), and per particle adj_xi, adj_g, adj_B.
+// adjoints (adj_F0, adj_W0, adj_rho0, adj_J), and per particle adj_xi, adj_g, adj_vn, adj_Pn.
 void adj_sweep(Ctx& c, const double* xi_n, const double* v_n, const double* vstar) {
     const int64_t N = c.m.ncell;
     const double a = 0.25 * c.cfg.kappa * c.cfg.kappa * c.cfg.dt * c.cfg.dt;
@@ -1340,8 +1340,9 @@ void adj_sweep(Ctx& c, const double* xi_n, const double* v_n, const double* vsta
     double* ys = c.adj_ys;
     launch_helmholtz(c, c.adj_t, 1.0, a, 4, c.cheb_iters, c.cheb_alpha, c.cheb_beta, &y, &ys);
     launch_adj_mesh_out(c, y, c.adj_pn, c.adj_W1, c.adj_rho1, c.adj_F0, c.adj_W0, c.adj_rho0, c.adj_J);
-    launch_adj_derivs(c, xi_n, v_n, vstar, c.adj_J, c.adj_P, c.adj_v, c.adj_xe, c.adj_mu, c.adj_xi, c.adj_g, c.adj_vn,
-                      c.adj_Pn, c.adj_B);
+    if (c.np > 0)
+        launch_adj_derivs(c, xi_n, v_n, vstar, c.adj_J, c.adj_P, c.adj_v, c.adj_xe, c.adj_mu, c.adj_xi, c.adj_g,
+                          c.adj_vn, c.adj_Pn);
 }
 
 // The transposed fixed point (I - K) mu = b0 (g(mu) = K mu + b0 is a sweep's adjoint of v*) by
@@ -1363,6 +1364,7 @@ pic_status adj_solve(pic_ctx* ctx, const double* xi_n, const double* v_n, const 
         return sync_results(ctx, "pic_step_vjp");
     };
     int sweeps = 0;
+    launch_adj_block_rows(c, xi_n, v_n, vstar, c.adj_B);
     cudaMemsetAsync(c.adj_mu, 0, vb, c.stream);
     adj_sweep(c, xi_n, v_n, vstar);
     ++sweeps;

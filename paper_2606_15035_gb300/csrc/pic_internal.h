@@ -260,7 +260,8 @@ void launch_adj_mesh_out(Ctx& c, const double* y, const double* pn, const double
                          double* lF0, double* lW0, double* lrho0, double* lJ);
 void launch_adj_derivs(Ctx& c, const double* xi, const double* v, const double* vstar, const double* lJ,
                        const double* lam_P, const double* lam_v, const double* lam_xe, const double* mu,
-                       double* lam_xi, double* g, double* lvn, double* lPn, double* B);
+                       double* lam_xi, double* g, double* lvn, double* lPn);
+void launch_adj_block_rows(Ctx& c, const double* xi, const double* v, const double* vstar, double* B);
 void launch_adj_precond(Ctx& c, const double* B, const double* r, double* z);
 void launch_adj_apply(Ctx& c, int64_t n, const double* z, const double* g, const double* b0, double* w);
 void launch_adj_mdot(Ctx& c, int64_t n, const double* w, const double* V, int64_t ldv, int nv, double* part,
