@@ -14,13 +14,16 @@
 
 namespace pic {
 
-__constant__ double c_gauss_t[16];
-__constant__ double c_gauss_w[16];
+// The Gauss--Legendre rules of 1 .. 16 points on [0, 1], rule nq at nq (nq - 1) / 2 (a place for each,
+// so that contexts of different rules do not share one).
+constexpr int GAUSS_MAX = 16;
+__constant__ double c_gauss_t[GAUSS_MAX * (GAUSS_MAX + 1) / 2];
+__constant__ double c_gauss_w[GAUSS_MAX * (GAUSS_MAX + 1) / 2];
 
-// Gauss-Legendre nodes on [0, 1] by Newton's method on the Legendre polynomial P_nq
-// (three-term recurrence), weights 1 / ((1 - x^2) P'(x)^2) mapped from [-1, 1].
+// Nodes by Newton's method on the Legendre polynomial P_nq (three-term recurrence), weights
+// 1 / ((1 - x^2) P'(x)^2) mapped from [-1, 1].
 void set_gauss_rule(int nq) {
-    double t[16] = {0}, w[16] = {0};
+    double t[GAUSS_MAX] = {0}, w[GAUSS_MAX] = {0};
     for (int k = 0; k < nq; ++k) {
         double x = std::cos(M_PI * (k + 0.75) / (nq + 0.5));
         double dp = 1.0;
@@ -41,8 +44,9 @@ void set_gauss_rule(int nq) {
         t[k] = 0.5 * (1.0 - x);
         w[k] = 1.0 / ((1.0 - x * x) * dp * dp);  // = 0.5 * 2 / ((1 - x^2) P'^2)
     }
-    cudaMemcpyToSymbol(c_gauss_t, t, sizeof(t));
-    cudaMemcpyToSymbol(c_gauss_w, w, sizeof(w));
+    const size_t at = sizeof(double) * (size_t)(nq * (nq - 1) / 2);
+    cudaMemcpyToSymbol(c_gauss_t, t, sizeof(double) * nq, at);
+    cudaMemcpyToSymbol(c_gauss_w, w, sizeof(double) * nq, at);
 }
 
 namespace {
@@ -76,14 +80,14 @@ __device__ __forceinline__ int scatter_closed(const StepParams& p, CellStart<dou
     });
 }
 
-// Same with an n_q-point Gauss rule on each piece (split) or on the whole path (unsplit).
+// Same with an n_q-point Gauss rule on the whole path (unsplit).
 __device__ __forceinline__ int scatter_gauss(const StepParams& p, const double x0[3], const double beta[3],
                                              const double w[3], double* __restrict__ J) {
     const int64_t N = p.m.ncell;
-    return for_each_segment(x0, beta, p.split != 0, [&](const Segment<double>& sg) {
+    return for_each_segment(x0, beta, false, [&](const Segment<double>& sg) {
         for (int qd = 0; qd < p.nq; ++qd) {
-            double s = sg.s0 + sg.h * c_gauss_t[qd];
-            double wq = sg.h * c_gauss_w[qd];
+            double s = sg.s0 + sg.h * c_gauss_t[p.rule + qd];
+            double wq = sg.h * c_gauss_w[p.rule + qd];
             double xq[3] = {x0[0] + s * beta[0], x0[1] + s * beta[1], x0[2] + s * beta[2]};
             int64_t g[8];
             double S[8];
@@ -170,17 +174,15 @@ __device__ __forceinline__ void for_each_node(const StepParams& p, const Basis1<
     }
 }
 
-// The orbit current with an n_q-point Gauss rule on each piece between the knots of the
-// degree-R shape (split) or on the whole path (unsplit).
+// The orbit current of the degree-R shape with an n_q-point Gauss rule on the whole path (unsplit).
 template <int R>
 __device__ __forceinline__ int scatter_gauss_r(const StepParams& p, const double x0[3], const double beta[3],
                                                const double w[3], double* __restrict__ J) {
     const int64_t N = p.m.ncell;
-    const double xs[3] = {x0[0] - p.koff, x0[1] - p.koff, x0[2] - p.koff};
-    return for_each_segment(xs, beta, p.split != 0, [&](const Segment<double>& sg) {
+    return for_each_segment(x0, beta, false, [&](const Segment<double>& sg) {
         for (int qd = 0; qd < p.nq; ++qd) {
-            const double s = sg.s0 + sg.h * c_gauss_t[qd];
-            const double wq = sg.h * c_gauss_w[qd];
+            const double s = sg.s0 + sg.h * c_gauss_t[p.rule + qd];
+            const double wq = sg.h * c_gauss_w[p.rule + qd];
             const double xq[3] = {x0[0] + s * beta[0], x0[1] + s * beta[1], x0[2] + s * beta[2]};
             Basis1<R> b[3];
             basis3<R>(p, xq, b);
@@ -200,6 +202,132 @@ __device__ __forceinline__ int scatter_gauss_r(const StepParams& p, const double
     });
 }
 
+// ---- pieces of split orbits with a Gauss rule, any degree ----------------------------------
+//
+// On a piece between the knots of the degree-R shape the stencil does not change, so the rule's nq
+// points share its (R + 1)^3 nodes: each node is loaded and contracted with v once per piece, and
+// the points are summed in the tensor product's order (rows of R + 1 nodes along x, then y and z),
+// which takes 18 operations per row and point at R = 2 where the pointwise form took 20 per node
+// and point.  Bound by the FP64 pipe; measured at R = 2, nq = 4 with 442,368 particles (36 x 32 x 24):
+// iterate 4.91 -> 2.32 ms, first scatter 1.35 -> 0.55 ms (a quarter of the L2 reductions).
+
+// The start on the knot lattice of the shape (knots at the integers or half-integers).
+__device__ __forceinline__ void knot_start(const StepParams& p, const double x0[3], CellStart<double>& st) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double xs = x0[a] - p.koff, fl = floor(xs);
+        st.f[a] = xs - fl;
+        const int c = (int)fl;
+        st.c[a] = c < 0 ? p.m.n[a] - 1 : min(c, p.m.n[a] - 1);
+    }
+}
+
+// Values and derivatives (per cell) of the R + 1 splines at coordinate t of their knot interval.
+template <int R>
+__device__ __forceinline__ void splines(double t, double w[R + 1], double d[R + 1]) {
+    const double u = 1.0 - t;
+    if constexpr (R == 1) {
+        w[0] = u;
+        w[1] = t;
+        d[0] = -1.0;
+        d[1] = 1.0;
+    } else if constexpr (R == 2) {
+        w[0] = 0.5 * u * u;
+        w[1] = 0.5 + t * u;
+        w[2] = 0.5 * t * t;
+        d[0] = -u;
+        d[1] = u - t;
+        d[2] = t;
+    } else {
+        const double t2 = t * t, u2 = u * u;
+        w[0] = u2 * u * (1.0 / 6.0);
+        w[1] = (3.0 * t - 6.0) * t2 * (1.0 / 6.0) + 4.0 / 6.0;
+        w[2] = (3.0 * u - 6.0) * u2 * (1.0 / 6.0) + 4.0 / 6.0;
+        w[3] = t2 * t * (1.0 / 6.0);
+        d[0] = -0.5 * u2;
+        d[1] = 1.5 * t2 - 2.0 * t;
+        d[2] = 2.0 * u - 1.5 * u2;
+        d[3] = 0.5 * t2;
+    }
+}
+
+// A piece's splines at its points: per point and axis the values and derivatives, those of z times
+// the point's weight (points in local memory, read back through L1).  A split orbit's rule has at
+// most the points that integrate the degree exactly (setup_geometry).
+template <int R>
+struct PiecePoints {
+    static constexpr int MAX = (3 * R + 2) / 2;
+    double w[MAX][3][R + 1], d[MAX][3][R + 1];
+
+    __device__ __forceinline__ PiecePoints(const StepParams& p, double h, const double mid[3], const double beta[3],
+                                           bool derivs) {
+        for (int q = 0; q < p.nq; ++q) {
+            const double hu = h * (c_gauss_t[p.rule + q] - 0.5), wq = c_gauss_w[p.rule + q];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                double v[R + 1], e[R + 1];
+                splines<R>(mid[a] + hu * beta[a], v, e);
+#pragma unroll
+                for (int k = 0; k <= R; ++k) {
+                    w[q][a][k] = a == 2 ? wq * v[k] : v[k];
+                    if (derivs) d[q][a][k] = a == 2 ? wq * e[k] : e[k];
+                }
+            }
+        }
+    }
+};
+
+// The stencil's first node per axis, and node rows along x.
+template <int R>
+struct Stencil {
+    int x[R + 1], first[3];
+    __device__ __forceinline__ Stencil(const int c[3], const MeshDims& m) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) first[a] = wrapi(c[a] - (R - 1) / 2, m.n[a]);
+        x[0] = first[0];
+#pragma unroll
+        for (int k = 1; k <= R; ++k) x[k] = next_cell(x[k - 1], m.n[0]);
+    }
+};
+
+// J_c[g] += w_c Sbar of the orbit's pieces.
+template <int R>
+__device__ __forceinline__ int scatter_pieces(const StepParams& p, const double x0[3], const double beta[3],
+                                              const double w[3], double* __restrict__ J) {
+    const int64_t N = p.m.ncell;
+    CellStart<double> st;
+    knot_start(p, x0, st);
+    return for_each_piece(st, beta, p.m, [&](double h, double, const double mid[3], const int c[3]) {
+        const PiecePoints<R> pt(p, h, mid, beta, false);
+        const Stencil<R> sl(c, p.m);
+        const double wh[3] = {h * w[0], h * w[1], h * w[2]};
+        int gz = sl.first[2];
+        for (int kz = 0; kz <= R; ++kz, gz = next_cell(gz, p.m.n[2])) {
+            int gy = sl.first[1];
+            for (int ky = 0; ky <= R; ++ky, gy = next_cell(gy, p.m.n[1])) {
+                const int64_t row = (int64_t)p.m.n[0] * ((int64_t)gy + (int64_t)p.m.n[1] * gz);
+                double M[R + 1];
+#pragma unroll
+                for (int k = 0; k <= R; ++k) M[k] = 0.0;
+                for (int q = 0; q < p.nq; ++q) {
+                    const double wyz = pt.w[q][1][ky] * pt.w[q][2][kz];
+#pragma unroll
+                    for (int k = 0; k <= R; ++k) M[k] += wyz * pt.w[q][0][k];
+                }
+#pragma unroll
+                for (int k = 0; k <= R; ++k) {
+                    const int64_t g = row + sl.x[k];
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        if (p.det) exact_add(p.acc, a * N + g, wh[a] * M[k]);
+                        else atomicAdd(J + a * N + g, wh[a] * M[k]);
+                    }
+                }
+            }
+        }
+    });
+}
+
 template <int QUAD>
 __device__ __forceinline__ int scatter_orbit(const StepParams& p, const double x0[3], const double beta[3],
                                              const double w[3], double* J) {
@@ -208,6 +336,11 @@ __device__ __forceinline__ int scatter_orbit(const StepParams& p, const double x
         cell_start(x0, p.m, st);
         return scatter_closed(p, st, beta, w, J);
     } else {
+        if (p.split) {
+            if (p.order == 2) return scatter_pieces<2>(p, x0, beta, w, J);
+            if (p.order == 3) return scatter_pieces<3>(p, x0, beta, w, J);
+            return scatter_pieces<1>(p, x0, beta, w, J);
+        }
         if (p.order == 2) return scatter_gauss_r<2>(p, x0, beta, w, J);
         if (p.order == 3) return scatter_gauss_r<3>(p, x0, beta, w, J);
         return scatter_gauss(p, x0, beta, w, J);
@@ -302,8 +435,8 @@ __device__ __forceinline__ void push_piece_gauss(const StepParams& p, const Segm
                                                  const double beta[3], const double vb[3],
                                                  const double* __restrict__ table, PushAcc& acc) {
     for (int qd = 0; qd < p.nq; ++qd) {
-        const double s = sg.s0 + sg.h * c_gauss_t[qd];
-        const double wq = sg.h * c_gauss_w[qd];
+        const double s = sg.s0 + sg.h * c_gauss_t[p.rule + qd];
+        const double wq = sg.h * c_gauss_w[p.rule + qd];
         double xq[3] = {x0[0] + s * beta[0], x0[1] + s * beta[1], x0[2] + s * beta[2]};
         int c[3];
         double r[3];
@@ -356,8 +489,8 @@ __device__ __forceinline__ void push_piece_gauss_r(const StepParams& p, const Se
                                                    const double beta[3], const double vb[3],
                                                    const double* __restrict__ table, PushAcc& acc) {
     for (int qd = 0; qd < p.nq; ++qd) {
-        const double s = sg.s0 + sg.h * c_gauss_t[qd];
-        const double wq = sg.h * c_gauss_w[qd];
+        const double s = sg.s0 + sg.h * c_gauss_t[p.rule + qd];
+        const double wq = sg.h * c_gauss_w[p.rule + qd];
         const double xq[3] = {x0[0] + s * beta[0], x0[1] + s * beta[1], x0[2] + s * beta[2]};
         Basis1<R> b[3];
         basis3<R>(p, xq, b);
@@ -385,6 +518,80 @@ __device__ __forceinline__ void push_piece_gauss_r(const StepParams& p, const Se
             }
         });
     }
+}
+
+// One piece of a split orbit (see scatter_pieces): the impulse's two integrals and, with DIAG, the
+// orbit gathers of the chain-rule and power tests.
+template <int R, bool DIAG>
+__device__ __forceinline__ void push_piece_points(const StepParams& p, double h, double sm, const double mid[3],
+                                                  const int c[3], const double beta[3], const double vb[3],
+                                                  const double* __restrict__ table, PushAcc& acc) {
+    const PiecePoints<R> pt(p, h, mid, beta, true);
+    const Stencil<R> sl(c, p.m);
+    double F[3] = {0.0, 0.0, 0.0}, g3[3] = {0.0, 0.0, 0.0}, U3[3] = {0.0, 0.0, 0.0}, D3[3] = {0.0, 0.0, 0.0}, pu = 0.0;
+    const double vh[3] = {vb[0] * p.invH[0], vb[1] * p.invH[1], vb[2] * p.invH[2]};
+    int gz = sl.first[2];
+    for (int kz = 0; kz <= R; ++kz, gz = next_cell(gz, p.m.n[2])) {
+        int gy = sl.first[1];
+        for (int ky = 0; ky <= R; ++ky, gy = next_cell(gy, p.m.n[1])) {
+            const double* row = table + 12 * (int64_t)p.m.n[0] * ((int64_t)gy + (int64_t)p.m.n[1] * gz);
+            double a1[R + 1], cc[R + 1], M[R + 1];
+#pragma unroll
+            for (int k = 0; k <= R; ++k) {
+                const double* t = row + 12 * sl.x[k];
+                a1[k] = t[3] * vb[0] + t[4] * vb[1] + t[5] * vb[2];                  // A^{n+1}_g . vbar
+                cc[k] = a1[k] - (t[0] * vb[0] + t[1] * vb[1] + t[2] * vb[2]);        // its change over the step
+                M[k] = 0.0;
+            }
+            for (int q = 0; q < p.nq; ++q) {
+                const double wz = pt.w[q][2][kz], wy = pt.w[q][1][ky];
+                const double wyz = wy * wz, dyz = pt.d[q][1][ky] * wz, ydz = wy * pt.d[q][2][kz];
+                const double nms = sm + h * (c_gauss_t[p.rule + q] - 0.5) - 1.0;    // s - 1
+                double tw = 0.0, td = 0.0;
+#pragma unroll
+                for (int k = 0; k <= R; ++k) {
+                    const double as = a1[k] + nms * cc[k];                          // A_g(s) . vbar
+                    tw += as * pt.w[q][0][k];
+                    td += as * pt.d[q][0][k];
+                    M[k] += wyz * pt.w[q][0][k];
+                }
+                F[0] += td * wyz;
+                F[1] += tw * dyz;
+                F[2] += tw * ydz;
+                if constexpr (DIAG) {
+                    const double vx = vh[0] * wyz, vyz = vh[1] * dyz + vh[2] * ydz;
+#pragma unroll
+                    for (int k = 0; k <= R; ++k) {
+                        const double* t = row + 12 * sl.x[k];
+                        const double vdW = vx * pt.d[q][0][k] + vyz * pt.w[q][0][k];
+#pragma unroll
+                        for (int l = 0; l < 3; ++l) D3[l] += (t[3 + l] + nms * (t[3 + l] - t[l])) * vdW;
+                    }
+                }
+            }
+#pragma unroll
+            for (int k = 0; k <= R; ++k) {
+                const double* t = row + 12 * sl.x[k];
+#pragma unroll
+                for (int l = 0; l < 3; ++l) g3[l] += M[k] * t[6 + l];
+                if constexpr (DIAG) {
+#pragma unroll
+                    for (int l = 0; l < 3; ++l) U3[l] += M[k] * t[9 + l];
+                    pu += M[k];
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+        acc.F[l] += h * p.invH[l] * F[l];
+        acc.gphi[l] += h * g3[l];
+        if constexpr (DIAG) {
+            acc.Ubar[l] += h * U3[l];
+            acc.DAv[l] += h * D3[l];
+        }
+    }
+    if constexpr (DIAG) acc.pu += h * pu;
 }
 
 // Point interpolant of columns [col, col+3) of the table at a wrapped position.
@@ -552,13 +759,21 @@ __device__ __forceinline__ void push_eval(const StepParams& p, const double x0[3
             push_piece_closed<DIAG>(p, sg, beta, vb, table, acc);
         });
     } else {
-        // pieces between the knots of the shape's degree (shifted by 1/2 for even degrees)
-        const double xs[3] = {x0[0] - p.koff, x0[1] - p.koff, x0[2] - p.koff};
-        o.nseg = for_each_segment(xs, beta, p.split != 0, [&](const Segment<double>& sg) {
-            if (p.order == 2) push_piece_gauss_r<2, DIAG>(p, sg, x0, beta, vb, table, acc);
-            else if (p.order == 3) push_piece_gauss_r<3, DIAG>(p, sg, x0, beta, vb, table, acc);
-            else push_piece_gauss<DIAG>(p, sg, x0, beta, vb, table, acc);
-        });
+        if (p.split) {
+            CellStart<double> st;
+            knot_start(p, x0, st);
+            o.nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
+                if (p.order == 2) push_piece_points<2, DIAG>(p, h, sm, mid, c, beta, vb, table, acc);
+                else if (p.order == 3) push_piece_points<3, DIAG>(p, h, sm, mid, c, beta, vb, table, acc);
+                else push_piece_points<1, DIAG>(p, h, sm, mid, c, beta, vb, table, acc);
+            });
+        } else {
+            o.nseg = for_each_segment(x0, beta, false, [&](const Segment<double>& sg) {
+                if (p.order == 2) push_piece_gauss_r<2, DIAG>(p, sg, x0, beta, vb, table, acc);
+                else if (p.order == 3) push_piece_gauss_r<3, DIAG>(p, sg, x0, beta, vb, table, acc);
+                else push_piece_gauss<DIAG>(p, sg, x0, beta, vb, table, acc);
+            });
+        }
     }
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -1524,7 +1739,8 @@ StepParams make_params(const Ctx& c) {
     p.q_dV_half = 0.5 * p.q_dV;
     p.np = c.np;
     p.split = c.cfg.split_orbit_at_knots;
-    p.nq = c.cfg.nq;
+    p.nq = c.nq;
+    p.rule = c.nq * (c.nq - 1) / 2;
     p.accel = c.cfg.picard_accel;
     p.hist = 0;
     p.slow_floor = c.run.after32 ? SLOW_FLOOR_AFTER32 : SLOW_FLOOR;
@@ -1577,7 +1793,7 @@ void launch_point_deposit(Ctx& c) {
 void launch_first_scatter(Ctx& c, double* J, const double* v_iter_or_null) {
     StepParams p = make_params(c);
     int nb = particle_blocks(c);
-    if (c.cfg.quadrature == PIC_QUAD_CLOSED)
+    if (c.closed)
         k_first_scatter_cell<<<nb, THREADS, CHUNK_SMEM, c.stream>>>(p, c.xi, c.v, c.vprev, v_iter_or_null, c.vit, J, c.partials,
                                                            c.dev_status);
     else
@@ -1592,7 +1808,7 @@ void launch_push(Ctx& c, const double* vit, double* vnew, double* Jnext, bool co
     p.hist = !commit && c.cfg.picard_accel && c.run.hist;
     int nb = particle_blocks(c);
     const bool det = c.cfg.deterministic && !commit;
-    const bool closed = c.cfg.quadrature == PIC_QUAD_CLOSED;
+    const bool closed = c.closed;
     if (!commit) cudaMemsetAsync(c.creep_count, 0, 2 * sizeof(int), c.stream);   // count, k_local queue head
 #define PIC_PUSH(Q, C, D)                                                                                        \
     k_push<Q, C, D><<<nb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.P, vit, c.table, vnew, Jnext, c.xi_new, c.P_new, \
@@ -1634,7 +1850,7 @@ void launch_local(Ctx& c, const double* vit, double* vnew, double* Jnext) {
     k_local<Q, T><<<lb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.P, vit, TAB, vnew, c.gsave, Jnext, c.creep_list,   \
                                                 c.creep_count, det ? c.creep_flag : nullptr, c.slide,              \
                                                 c.creep_count + 1, c.partials, c.dev_status)
-    if (c.cfg.quadrature != PIC_QUAD_CLOSED) PIC_LOCAL(1, false, c.table);
+    if (!c.closed) PIC_LOCAL(1, false, c.table);
     else if (c.ctab) PIC_LOCAL(0, true, c.ctab);
     else PIC_LOCAL(0, false, c.table);
 #undef PIC_LOCAL

@@ -266,6 +266,18 @@ void setup_geometry(Ctx& c) {
         c.volume *= c.cfg.L[a];
     }
     c.dV = c.H[0] * c.H[1] * c.H[2];
+    // On a piece between knots the integrands of a split orbit are polynomials of degree 3 r in s
+    // (shapes: 3 r; a shape differentiated along one axis times A, linear in s: 3 r), which a rule with
+    // 2 nq - 1 >= 3 r points integrates exactly.  More points give the same integrals, so the fewest
+    // that do run; for linear shapes those integrals are the closed forms.  Measured, two steps at 16^3
+    // with 131,072 particles and nq = 16: 24.7 ms with all points, 4.7 with the closed forms.
+    const int exact = (3 * c.cfg.shape_order + 2) / 2;
+    c.closed = c.cfg.quadrature == PIC_QUAD_CLOSED;
+    c.nq = c.cfg.nq;
+    if (!c.closed && c.cfg.split_orbit_at_knots && c.cfg.nq >= exact) {
+        c.nq = exact;
+        c.closed = c.cfg.shape_order == 1;
+    }
     // CN Helmholtz operator I - a Delta_h: spectrum [1, 1 + a sum_a max sin^2 / H_a^2].
     double a = 0.25 * c.cfg.kappa * c.cfg.kappa * c.cfg.dt * c.cfg.dt;
     double lmax = 1.0;
@@ -425,7 +437,7 @@ pic_status allocate(pic_ctx* ctx) {
     // last, because it is optional: the closed forms' cell table, where there are particles enough to
     // repay building it and it stays a small part of the device's memory
     const size_t cells = sizeof(double) * CELL_VALUES * (size_t)N;
-    if (c.cfg.quadrature == PIC_QUAD_CLOSED && c.np >= CELL_TABLE_MIN_PPC * N && cells <= CELL_TABLE_MAX_BYTES) {
+    if (c.closed && c.np >= CELL_TABLE_MIN_PPC * N && cells <= CELL_TABLE_MAX_BYTES) {
         c.ctab = (double*)dev_alloc_once(ctx, cells);
         if (c.ctab && reinterpret_cast<uintptr_t>(c.ctab) % 16 != 0) drop_cell_table(ctx);
     }
@@ -1012,7 +1024,7 @@ pic_status pic_init(const pic_config* cfg, const pic_particles* particles, const
         delete ctx;
         return s;
     }
-    if (cfg->quadrature == PIC_QUAD_GAUSS) set_gauss_rule(cfg->nq);
+    if (!c.closed) set_gauss_rule(c.nq);
     const int64_t np = c.np, N = c.m.ncell;
     const cudaMemcpyKind kind = particles->on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     if (np > 0) {

@@ -69,7 +69,7 @@ struct StepParams {
     double cb[3], ihs[3], dtq, q_dV_half;   // dt / (2 H), 1 / (2 H), dt q, q / (2 dV): factors of v^{p} + v^n
     int64_t np;
     int split;                 // split orbits at knots
-    int nq;                    // Gauss points (Gauss quadrature only)
+    int nq, rule;              // Gauss points (Gauss quadrature only), and where their rule starts
     int accel;                 // particle-local solves for creeping particles
     int hist;                  // vnew holds v^{p-1} (slow particles are found against it)
     double slow_floor;         // a slow particle's change also exceeds this times its speed
@@ -124,6 +124,8 @@ struct Ctx {
     int push_bps = 8;     // grid of the FP64 particle kernels: blocks per SM (pic_autotune)
     int push32_bps = 16;  // grid of the FP32 chunk kernels: blocks per SM (pic_autotune)
     double H[3], invH[3], dV = 0, volume = 0;
+    bool closed = true;   // the closed-form particle kernels (configured, or equal to the Gauss rule)
+    int nq = 1;           // points of the Gauss rule that runs
     int64_t np = 0;
     double q = 0, mass = 0;
 

@@ -110,3 +110,35 @@ def test_deterministic_steps_do_not_depend_on_the_particle_order(sim, precision)
     for k in want:
         assert torch.equal(want[k], got[k]), k
     s.close()
+
+
+@pytest.mark.parametrize("order,nq", [(1, 1), (1, 2), (1, 16), (2, 3), (2, 4), (2, 16), (3, 4), (3, 5), (3, 11)])
+@pytest.mark.parametrize("n", [(8, 8, 8), (4, 5, 7)])
+def test_gauss_pieces_match_oracle(sim, n, order, nq):
+    """Split orbits with a Gauss rule: below the exact number of points, at it, and above it (where the
+    library runs the fewest that are exact, or the closed forms), from starts on knots too.  Same
+    tolerances; another context with another rule is alive, which must not change this one's."""
+    L = tuple(float(k) for k in n)
+    x, b = _edge_particles(np.asarray(n), 801, 60 + order)
+    x[100:200] = np.mod(x[100:200] + 0.5, np.asarray(n))      # on the half-integer knots of even degrees
+    v = 0.3 * b[::-1].copy()
+    v_it = 2.0 * b - v
+    q = -1e-3
+    kw = dict(n=n, L=L, dt=1.0, picard_tol=1e-13)
+    s = sim.PicSim(sim.pic_config_default(quadrature=1, nq=nq, shape_order=order, **kw), x, v, q, 1e-3)
+    other = sim.PicSim(sim.pic_config_default(quadrature=1, nq=3 if nq != 3 else 2, shape_order=2, **kw), x, v, q, 1e-3)
+    ocfg = opic.Config(quadrature="gauss", nq=nq, order=order, **kw)
+    o = opic.init(x, v, q, 1e-3, ocfg)
+    g = s.iterate(v_it)
+    it = opic.picard_iteration(o, v_it, ocfg, ocfg.grid())
+    s.close()
+    other.close()
+
+    def rel(a, r):
+        return np.linalg.norm(a - r) / max(np.linalg.norm(r), 1e-300)
+
+    assert rel(g["J"], it["J"]) <= 1e-13
+    for name in ("phi", "psi", "A", "U"):
+        assert rel(g[name], it[name]) <= 1e-12, (name, rel(g[name], it[name]))
+    assert rel(g["P"], it["P"]) <= 1e-13
+    assert rel(g["v"], it["v_new"]) <= 1e-13
