@@ -288,12 +288,17 @@ struct Stencil {
 #pragma unroll
         for (int k = 1; k <= R; ++k) x[k] = next_cell(x[k - 1], m.n[0]);
     }
+    // Index of the row of nodes (., ky, kz).
+    __device__ __forceinline__ int64_t row(int ky, int kz, const MeshDims& m) const {
+        return (int64_t)m.n[0] * ((int64_t)wrapi(first[1] + ky, m.n[1]) + (int64_t)m.n[1] * wrapi(first[2] + kz, m.n[2]));
+    }
 };
 
 // J_c[g] += w_c Sbar of the orbit's pieces.
+// Rows part, part + parts, ... of the stencil only (k_local shares a particle among lanes).
 template <int R>
 __device__ __forceinline__ int scatter_pieces(const StepParams& p, const double x0[3], const double beta[3],
-                                              const double w[3], double* __restrict__ J) {
+                                              const double w[3], double* __restrict__ J, int part = 0, int parts = 1) {
     const int64_t N = p.m.ncell;
     CellStart<double> st;
     knot_start(p, x0, st);
@@ -301,27 +306,24 @@ __device__ __forceinline__ int scatter_pieces(const StepParams& p, const double 
         const PiecePoints<R> pt(p, h, mid, beta, false);
         const Stencil<R> sl(c, p.m);
         const double wh[3] = {h * w[0], h * w[1], h * w[2]};
-        int gz = sl.first[2];
-        for (int kz = 0; kz <= R; ++kz, gz = next_cell(gz, p.m.n[2])) {
-            int gy = sl.first[1];
-            for (int ky = 0; ky <= R; ++ky, gy = next_cell(gy, p.m.n[1])) {
-                const int64_t row = (int64_t)p.m.n[0] * ((int64_t)gy + (int64_t)p.m.n[1] * gz);
-                double M[R + 1];
+        for (int r = part; r < (R + 1) * (R + 1); r += parts) {
+            const int kz = r / (R + 1), ky = r - kz * (R + 1);
+            const int64_t row = sl.row(ky, kz, p.m);
+            double M[R + 1];
 #pragma unroll
-                for (int k = 0; k <= R; ++k) M[k] = 0.0;
-                for (int q = 0; q < p.nq; ++q) {
-                    const double wyz = pt.w[q][1][ky] * pt.w[q][2][kz];
+            for (int k = 0; k <= R; ++k) M[k] = 0.0;
+            for (int q = 0; q < p.nq; ++q) {
+                const double wyz = pt.w[q][1][ky] * pt.w[q][2][kz];
 #pragma unroll
-                    for (int k = 0; k <= R; ++k) M[k] += wyz * pt.w[q][0][k];
-                }
+                for (int k = 0; k <= R; ++k) M[k] += wyz * pt.w[q][0][k];
+            }
 #pragma unroll
-                for (int k = 0; k <= R; ++k) {
-                    const int64_t g = row + sl.x[k];
+            for (int k = 0; k <= R; ++k) {
+                const int64_t g = row + sl.x[k];
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        if (p.det) exact_add(p.acc, a * N + g, wh[a] * M[k]);
-                        else atomicAdd(J + a * N + g, wh[a] * M[k]);
-                    }
+                for (int a = 0; a < 3; ++a) {
+                    if (p.det) exact_add(p.acc, a * N + g, wh[a] * M[k]);
+                    else atomicAdd(J + a * N + g, wh[a] * M[k]);
                 }
             }
         }
@@ -525,60 +527,58 @@ __device__ __forceinline__ void push_piece_gauss_r(const StepParams& p, const Se
 template <int R, bool DIAG>
 __device__ __forceinline__ void push_piece_points(const StepParams& p, double h, double sm, const double mid[3],
                                                   const int c[3], const double beta[3], const double vb[3],
-                                                  const double* __restrict__ table, PushAcc& acc) {
+                                                  const double* __restrict__ table, PushAcc& acc, int part = 0,
+                                                  int parts = 1) {
     const PiecePoints<R> pt(p, h, mid, beta, true);
     const Stencil<R> sl(c, p.m);
     double F[3] = {0.0, 0.0, 0.0}, g3[3] = {0.0, 0.0, 0.0}, U3[3] = {0.0, 0.0, 0.0}, D3[3] = {0.0, 0.0, 0.0}, pu = 0.0;
     const double vh[3] = {vb[0] * p.invH[0], vb[1] * p.invH[1], vb[2] * p.invH[2]};
-    int gz = sl.first[2];
-    for (int kz = 0; kz <= R; ++kz, gz = next_cell(gz, p.m.n[2])) {
-        int gy = sl.first[1];
-        for (int ky = 0; ky <= R; ++ky, gy = next_cell(gy, p.m.n[1])) {
-            const double* row = table + 12 * (int64_t)p.m.n[0] * ((int64_t)gy + (int64_t)p.m.n[1] * gz);
-            double a1[R + 1], cc[R + 1], M[R + 1];
+    for (int r = part; r < (R + 1) * (R + 1); r += parts) {
+        const int kz = r / (R + 1), ky = r - kz * (R + 1);
+        const double* row = table + 12 * sl.row(ky, kz, p.m);
+        double a1[R + 1], cc[R + 1], M[R + 1];
+#pragma unroll
+        for (int k = 0; k <= R; ++k) {
+            const double* t = row + 12 * sl.x[k];
+            a1[k] = t[3] * vb[0] + t[4] * vb[1] + t[5] * vb[2];                  // A^{n+1}_g . vbar
+            cc[k] = a1[k] - (t[0] * vb[0] + t[1] * vb[1] + t[2] * vb[2]);        // its change over the step
+            M[k] = 0.0;
+        }
+        for (int q = 0; q < p.nq; ++q) {
+            const double wz = pt.w[q][2][kz], wy = pt.w[q][1][ky];
+            const double wyz = wy * wz, dyz = pt.d[q][1][ky] * wz, ydz = wy * pt.d[q][2][kz];
+            const double nms = sm + h * (c_gauss_t[p.rule + q] - 0.5) - 1.0;    // s - 1
+            double tw = 0.0, td = 0.0;
 #pragma unroll
             for (int k = 0; k <= R; ++k) {
-                const double* t = row + 12 * sl.x[k];
-                a1[k] = t[3] * vb[0] + t[4] * vb[1] + t[5] * vb[2];                  // A^{n+1}_g . vbar
-                cc[k] = a1[k] - (t[0] * vb[0] + t[1] * vb[1] + t[2] * vb[2]);        // its change over the step
-                M[k] = 0.0;
+                const double as = a1[k] + nms * cc[k];                          // A_g(s) . vbar
+                tw += as * pt.w[q][0][k];
+                td += as * pt.d[q][0][k];
+                M[k] += wyz * pt.w[q][0][k];
             }
-            for (int q = 0; q < p.nq; ++q) {
-                const double wz = pt.w[q][2][kz], wy = pt.w[q][1][ky];
-                const double wyz = wy * wz, dyz = pt.d[q][1][ky] * wz, ydz = wy * pt.d[q][2][kz];
-                const double nms = sm + h * (c_gauss_t[p.rule + q] - 0.5) - 1.0;    // s - 1
-                double tw = 0.0, td = 0.0;
+            F[0] += td * wyz;
+            F[1] += tw * dyz;
+            F[2] += tw * ydz;
+            if constexpr (DIAG) {
+                const double vx = vh[0] * wyz, vyz = vh[1] * dyz + vh[2] * ydz;
 #pragma unroll
                 for (int k = 0; k <= R; ++k) {
-                    const double as = a1[k] + nms * cc[k];                          // A_g(s) . vbar
-                    tw += as * pt.w[q][0][k];
-                    td += as * pt.d[q][0][k];
-                    M[k] += wyz * pt.w[q][0][k];
-                }
-                F[0] += td * wyz;
-                F[1] += tw * dyz;
-                F[2] += tw * ydz;
-                if constexpr (DIAG) {
-                    const double vx = vh[0] * wyz, vyz = vh[1] * dyz + vh[2] * ydz;
+                    const double* t = row + 12 * sl.x[k];
+                    const double vdW = vx * pt.d[q][0][k] + vyz * pt.w[q][0][k];
 #pragma unroll
-                    for (int k = 0; k <= R; ++k) {
-                        const double* t = row + 12 * sl.x[k];
-                        const double vdW = vx * pt.d[q][0][k] + vyz * pt.w[q][0][k];
-#pragma unroll
-                        for (int l = 0; l < 3; ++l) D3[l] += (t[3 + l] + nms * (t[3 + l] - t[l])) * vdW;
-                    }
+                    for (int l = 0; l < 3; ++l) D3[l] += (t[3 + l] + nms * (t[3 + l] - t[l])) * vdW;
                 }
             }
+        }
 #pragma unroll
-            for (int k = 0; k <= R; ++k) {
-                const double* t = row + 12 * sl.x[k];
+        for (int k = 0; k <= R; ++k) {
+            const double* t = row + 12 * sl.x[k];
 #pragma unroll
-                for (int l = 0; l < 3; ++l) g3[l] += M[k] * t[6 + l];
-                if constexpr (DIAG) {
+            for (int l = 0; l < 3; ++l) g3[l] += M[k] * t[6 + l];
+            if constexpr (DIAG) {
 #pragma unroll
-                    for (int l = 0; l < 3; ++l) U3[l] += M[k] * t[9 + l];
-                    pu += M[k];
-                }
+                for (int l = 0; l < 3; ++l) U3[l] += M[k] * t[9 + l];
+                pu += M[k];
             }
         }
     }
@@ -1175,8 +1175,153 @@ __global__ void __launch_bounds__(THREADS, DIAG ? 1 : 2) k_push(StepParams p, co
 // and the commit push sets v^{n+1}_a to it with P_a from the canonical relation.  The energy
 // identities hold to the size of vbar_a = d H / dt < D_KNOT H / dt.  The plain image G(v^p)
 // is saved in gsave (diagnostics), then the orbit current of the result is scattered.
+//
+// Eight lanes share a particle.  A solve is a serial chain of evaluations (up to 34, two on average),
+// and on the FP64 pipe a warp instruction takes 64 clocks of its scheduler whether one lane is active
+// or 32, so what bounds the launch is the length of that chain.  Lanes 0 .. 2 hold one component each
+// (state and step logic), lane k evaluates table entry k of a piece (subset k of the axes; rows k and
+// k + 8 of a Gauss piece's nodes) and the sums meet in three exchanges per evaluation: 55 FP64
+// instructions a piece for 130, and only the step that is taken is computed.  Groups take particles
+// from a queue four to a warp (deterministic mode: in index order from the warp's own share of the
+// flags, so that every partial sum is reproducible), the first warps of all blocks first.
+// With one particle per lane (13 of 32 lanes active on average, the particles on the blocks that came
+// first) the mean launch of two steps at 32^3 with 2,097,152 particles took 377 us, now 108; a
+// deterministic step at 24^3 with 442,368 376, now 147; quadratic shapes 800, now 307.
+constexpr int LOCAL_LANES = 8;
+constexpr int LOCAL_MINB = 1;   // blocks per SM: 2 (128 registers, 480 bytes of spills) measured 114 us
+
+// v[k] of an 8-array held in registers.
+__device__ __forceinline__ double pick8(const double v[8], int k) {
+    const double a0 = (k & 1) ? v[1] : v[0], a1 = (k & 1) ? v[3] : v[2];
+    const double a2 = (k & 1) ? v[5] : v[4], a3 = (k & 1) ? v[7] : v[6];
+    const double b0 = (k & 2) ? a1 : a0, b1 = (k & 2) ? a3 : a2;
+    return (k & 4) ? b1 : b0;
+}
+
+// Lane k's share of piece_impulse: acc_j += its terms (summed over the 8 lanes they are the piece's).
+template <bool CELLS>
+__device__ __forceinline__ void piece_impulse_share(const StepParams& p, int k, double h, double sm, const double mid[3],
+                                                    const double beta[3], const double vs[3], const int c[3],
+                                                    const double* __restrict__ table, double acc[3]) {
+    const PieceMoments<double> q = piece_moments(h, mid, beta);
+    const double M[8] = {1.0, mid[0], mid[1], q.Pxy, mid[2], q.Pxz, q.Pyz, q.S};
+    const double E[8] = {0.0, q.e[0], q.e[1], mid[0] * q.e[1] + mid[1] * q.e[0],
+                         q.e[2], mid[0] * q.e[2] + mid[2] * q.e[0], mid[1] * q.e[2] + mid[2] * q.e[1], 0.0};
+    const FieldLoad<CELLS> ld(table, c, p.m);
+    double col[CELL_COLS];
+#pragma unroll
+    for (int t = 0; t < CELL_COLS; ++t) {
+        double e0, e1;
+        ld(k >> 1, t, e0, e1);
+        col[t] = (k & 1) ? e1 : e0;
+    }
+    const double cc = col[3] * vs[0] + col[4] * vs[1] + col[5] * vs[2];
+    const double a = col[0] * vs[0] + col[1] * vs[1] + col[2] * vs[2] + (sm - 1.0) * cc;
+    const double m = pick8(M, k);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const bool in = (k >> j) & 1;
+        const double F = a * pick8(M, k ^ (1 << j)) + cc * pick8(E, k ^ (1 << j));
+        acc[j] += h * (col[6 + j] * m + (in ? p.ihs[j] * F : 0.0));
+    }
+}
+
+// A_h^{n+1} at a wrapped position, rows part, part + parts, ... of the stencil.
+template <int R>
+__device__ __forceinline__ void point_A1_rows(const StepParams& p, const double x[3], const double* __restrict__ table,
+                                              int part, int parts, double out[3]) {
+    Basis1<R> b[3];
+    basis3<R>(p, x, b);
+    for (int r = part; r < (R + 1) * (R + 1); r += parts) {
+        const int kz = r / (R + 1), ky = r - kz * (R + 1);
+        const int gy = wrapi(b[1].first + ky, p.m.n[1]), gz = wrapi(b[2].first + kz, p.m.n[2]);
+        const double wyz = b[1].w[ky] * b[2].w[kz];
+#pragma unroll
+        for (int k = 0; k <= R; ++k) {
+            const double* t = table + 12 * node_index(wrapi(b[0].first + k, p.m.n[0]), gy, gz, p.m) + 3;
+            const double w = wyz * b[0].w[k];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) out[a] += w * t[a];
+        }
+    }
+}
+
+// Basis1 of the linear shape (degrees 2 and 3: basis1).
+template <>
+__device__ __forceinline__ void basis1<1>(double x, double invH, Basis1<1>& b) {
+    const double f = floor(x), t = x - f;
+    b.first = (int)f;
+    b.w[0] = 1.0 - t;
+    b.w[1] = t;
+    b.dw[0] = -invH;
+    b.dw[1] = invH;
+}
+
+// G(u) of the particle that 8 lanes share, u = vs - v^n: every lane gets the component `comp` of
+// v^{n+1}.  Every lane of the warp calls it (inactive groups with any valid start).
 template <int QUAD, bool CELLS>
-__global__ void __launch_bounds__(THREADS) k_local(StepParams p, const double* __restrict__ xi,
+__device__ __forceinline__ double push_eval_shared(const StepParams& p, int k, int comp, const double x0[3],
+                                                   const CellStart<double>& start, const double vs[3], double Pn,
+                                                   const double* __restrict__ table, int& nseg) {
+    double beta[3], acc[3] = {0.0, 0.0, 0.0}, Ae[3] = {0.0, 0.0, 0.0};
+    CellStart<double> st = start;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) beta[a] = p.cb[a] * vs[a];
+    if constexpr (QUAD == 0) {
+        nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
+            piece_impulse_share<CELLS>(p, k, h, sm, mid, beta, vs, c, table, acc);
+        });
+        const FieldLoad<CELLS> ld(table, st.c, p.m);
+        double e = (k & 1) ? st.f[0] : 1.0;
+        if (k & 2) e *= st.f[1];
+        if (k & 4) e *= st.f[2];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            double e0, e1;
+            ld(k >> 1, a, e0, e1);
+            Ae[a] = e * ((k & 1) ? e1 : e0);
+        }
+    } else {
+        PushAcc pa{};
+        const double vb[3] = {0.5 * vs[0], 0.5 * vs[1], 0.5 * vs[2]};
+        if (p.split) {
+            nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
+                if (p.order == 2) push_piece_points<2, false>(p, h, sm, mid, c, beta, vb, table, pa, k, LOCAL_LANES);
+                else if (p.order == 3) push_piece_points<3, false>(p, h, sm, mid, c, beta, vb, table, pa, k, LOCAL_LANES);
+                else push_piece_points<1, false>(p, h, sm, mid, c, beta, vb, table, pa, k, LOCAL_LANES);
+            });
+        } else {
+            nseg = for_each_segment(x0, beta, false, [&](const Segment<double>& sg) {
+                if (p.order == 2) push_piece_gauss_r<2, false>(p, sg, x0, beta, vb, table, pa);
+                else if (p.order == 3) push_piece_gauss_r<3, false>(p, sg, x0, beta, vb, table, pa);
+                else push_piece_gauss<false>(p, sg, x0, beta, vb, table, pa);
+            });
+        }
+        const bool mine = p.split || k == 0;   // the whole path's points are not shared out
+        double xe[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            acc[a] = mine ? pa.F[a] - pa.gphi[a] : 0.0;
+            xe[a] = wrap_pos(x0[a] + beta[a], (double)p.m.n[a]);
+        }
+        if (p.order == 2) point_A1_rows<2>(p, xe, table, k, LOCAL_LANES, Ae);
+        else if (p.order == 3) point_A1_rows<3>(p, xe, table, k, LOCAL_LANES, Ae);
+        else point_A1_rows<1>(p, xe, table, k, LOCAL_LANES, Ae);
+    }
+    __syncwarp();
+    double kick = 0.0;   // P^{n+1} - P^n - q A_h^{n+1}(x^{n+1}) of this lane's component
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        double t = p.dtq * acc[a] - p.q * Ae[a];
+#pragma unroll
+        for (int o = 1; o < LOCAL_LANES; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (a == comp) kick = t;
+    }
+    return (Pn + kick) * p.inv_mass;
+}
+
+template <int QUAD, bool CELLS>
+__global__ void __launch_bounds__(THREADS, LOCAL_MINB) k_local(StepParams p, const double* __restrict__ xi,
                                                    const double* __restrict__ v, const double* __restrict__ P,
                                                    const double* __restrict__ vit, const double* __restrict__ table,
                                                    double* __restrict__ vnew, double* __restrict__ gsave,
@@ -1186,79 +1331,108 @@ __global__ void __launch_bounds__(THREADS) k_local(StepParams p, const double* _
                                                    int* __restrict__ queue_head, double* __restrict__ partials,
                                                    int* __restrict__ status) {
     __shared__ double sm[32];
+    const unsigned full = 0xffffffffu;
     const int64_t np = p.np;
-    // The creeping particles: a list in arrival order, taken from a shared queue by whichever
-    // lane is free; or (deterministic mode) flags in index order, each thread walking its own
-    // fixed stride, so that the assignment (and every partial sum) is reproducible.
-    const int64_t count = creep_flag ? np : (int64_t)*creep_count;
-    const int64_t T = (int64_t)gridDim.x * blockDim.x;
-    int64_t next_static = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int k = lane & (LOCAL_LANES - 1), comp = min(k, 2), gbase = lane & ~(LOCAL_LANES - 1);
+    // this warp's share of the flags (deterministic mode), or of the queue
+    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    const int64_t share = (np + nwarps - 1) / nwarps, wid = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
+    int64_t pos = wid * share, word = 0;
+    const int64_t end = min(pos + share, np);
+    unsigned bits = 0;
+    const int64_t count = creep_flag ? 0 : (int64_t)*creep_count;
+    // few particles: the warps that the others' SMs can do without stay out
+    const int64_t per = (int64_t)gridDim.x * (32 / LOCAL_LANES);
+    bool active = false, exhausted = !creep_flag && count <= per * warp;
     double ev_num = 0.0, ev_den = 0.0;
     // One particle's solve is a sequence of push evaluations: sliding probes (phase 0: just
     // short of the knot, phase 1: just past it, per probed axis), the first evaluation
-    // (phase 2), then up to LOCAL_STEPS - 1 iteration steps (phase 3).  Every round, each lane
-    // with a particle makes its next evaluation together with the others, and a lane whose
-    // particle is done takes a new one: the warp's evaluations stay full even when particles
-    // need very different numbers of them.
-    bool active = false, exhausted = false;
+    // (phase 2), then up to LOCAL_STEPS - 1 iteration steps (phase 3).  Every round, each group
+    // with a particle makes its next evaluation, and one whose particle is done takes a new one.
     int64_t i = 0;
-    int phase = 0, paxis = 0, nstep = 0;
-    double x0[3], vn[3], Pn[3], u0[3], r0[3], u1[3], r1[3], bu[3];
-    double ua[3], ga[3], ub[3], gb[3], side[3], fac[3], uland[3], dk[3], ue[3], blim[3];
-    bool brk[3], secok[3], sl[3], probe[3];
-    int nrep[3];
+    int phase = 2, paxis = 0, nstep = 0, probes = 0, nrep = 0;
+    double x0[3] = {0.0, 0.0, 0.0}, xa = 0.0, vn = 0.0, Pn = 0.0, u0 = 0.0, r0 = 0.0, u1 = 0.0, r1 = 0.0, bu = 0.0;
+    double ua = 0.0, ga = 0.0, ub = 0.0, gb = 0.0, side = 0.0, fac = 2.0, uland = 0.0, dk = 0.0, blim = 0.0;
+    bool brk = false, secok = false, sl = false;
+    CellStart<double> st{};
     double tol = 0.0, spd = 0.0, gm = 0.0, brs = 0.0;
     double nsolve = 0.0, neval = 0.0, nfail = 0.0, nfail_free = 0.0;
+    const double Ha = comp == 0 ? p.H[0] : (comp == 1 ? p.H[1] : p.H[2]);
+    const double cba = comp == 0 ? p.cb[0] : (comp == 1 ? p.cb[1] : p.cb[2]);   // beta = cba (u + v^n), in cells
+    const double ha = 2.0 * Ha / p.dt;                                          // u + v^n = ha beta
+    auto of = [&](double x, int a) { return __shfl_sync(full, x, gbase + a); };
+    auto max3 = [&](double x) { return fmax(fmax(of(x, 0), of(x, 1)), of(x, 2)); };
+    auto bits3 = [&](bool f) { return (int)(__ballot_sync(full, f) >> gbase) & 7; };
     while (true) {
-        if (!active && !exhausted) {
-            int64_t k = -1;
-            if (creep_flag) {
-                while (next_static < count && !creep_flag[next_static]) next_static += T;
-                if (next_static < count) {
-                    k = next_static;
-                    next_static += T;
-                }
+        // groups without a particle take one
+        const bool want = !active && !exhausted;
+        const unsigned asking = __ballot_sync(full, want && k == 0);
+        if (asking) {
+            const int rank = __popc(asking & ((1u << gbase) - 1u));
+            int64_t got = -1;
+            if (!creep_flag) {
+                int first = 0;
+                if (lane == 0) first = atomicAdd(queue_head, __popc(asking));
+                first = __shfl_sync(full, first, 0);
+                if (want && first + rank < count) got = creep_list[first + rank];
             } else {
-                const int q = atomicAdd(queue_head, 1);
-                k = q < count ? q : -1;
+                int taken = 0;
+                const int need = __popc(asking);
+                while (taken < need) {
+                    if (bits == 0) {
+                        if (pos >= end) break;
+                        const int64_t j = pos + lane;
+                        bits = __ballot_sync(full, j < end && creep_flag[j]);
+                        word = pos;
+                        pos += 32;
+                        continue;
+                    }
+                    if (want && rank == taken) got = word + __ffs(bits) - 1;
+                    bits &= bits - 1;
+                    ++taken;
+                }
             }
-            if (k < 0) {
-                exhausted = true;
-            } else {
-                i = creep_flag ? k : (int64_t)creep_list[k];
-                double nrm = 0.0;
+            if (want) {
+                if (got < 0) {
+                    exhausted = true;
+                } else {
+                    i = got;
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    x0[a] = xi[a * np + i];
-                    vn[a] = v[a * np + i];
-                    Pn[a] = P[a * np + i];
-                    u0[a] = vit[a * np + i];
-                    u1[a] = vnew[a * np + i];          // G(v^p) from k_push
-                    gsave[a * np + i] = u1[a];
-                    r0[a] = u1[a] - u0[a];
-                    nrm += u0[a] * u0[a];
-                    blim[a] = fabs(p.dt * 0.5 / p.H[a] * (u0[a] + vn[a])) + BETA_TRIAL;   // trial-orbit bound
-                    dk[a] = rint(x0[a] - p.koff) - (x0[a] - p.koff);   // signed distance to the nearest knot
-                    uland[a] = 2.0 * dk[a] * p.H[a] / p.dt - vn[a];
-                    sl[a] = (slide[i] >> a) & 1u;       // pinned earlier in this step: stays pinned
-                    probe[a] = !sl[a] && fabs(dk[a]) < D_KNOT;
+                    for (int a = 0; a < 3; ++a) x0[a] = xi[a * np + i];
+                    if constexpr (QUAD == 0) cell_start(x0, p.m, st);
+                    else knot_start(p, x0, st);
+                    xa = (comp == 0 ? x0[0] : (comp == 1 ? x0[1] : x0[2])) - p.koff;   // start on the knot lattice
+                    vn = v[comp * np + i];
+                    Pn = P[comp * np + i];
+                    u0 = vit[comp * np + i];
+                    u1 = vnew[comp * np + i];          // G(v^p) from k_push
+                    if (k < 3) gsave[comp * np + i] = u1;
+                    r0 = u1 - u0;
+                    blim = fabs(cba * (u0 + vn)) + BETA_TRIAL;   // trial-orbit bound
+                    dk = rint(xa) - xa;                // signed distance to the nearest knot
+                    uland = ha * dk - vn;
+                    sl = (slide[i] >> comp) & 1u;      // pinned earlier in this step: stays pinned
                 }
-                spd = fmax(sqrt(nrm), 1e-300);
+            }
+            const double un = u0 * u0;
+            const double nrm = sqrt(of(un, 0) + of(un, 1) + of(un, 2));
+            const int pm = bits3(!sl && fabs(dk) < D_KNOT);
+            if (want && got >= 0) {
+                spd = fmax(nrm, 1e-300);
                 tol = LOCAL_TOL * spd;
+                probes = pm;
                 paxis = 0;
-                while (paxis < 3 && !probe[paxis]) ++paxis;
+                while (paxis < 3 && !((probes >> paxis) & 1)) ++paxis;
                 phase = paxis < 3 ? 0 : 2;
-                if (phase == 2) {
-#pragma unroll
-                    for (int a = 0; a < 3; ++a)
-                        if (sl[a]) u1[a] = uland[a];
-                }
+                if (phase == 2 && sl) u1 = uland;
                 nstep = 0;
                 active = true;
             }
         }
-        if (!__any_sync(0xffffffffu, active)) break;
+        if (!__any_sync(full, active)) break;
         // the evaluation point of this round
+        double ue = u1;
         if (active) {
             if (phase <= 1) {
                 // Sliding probes: a component starting within D_KNOT of a knot (signed distance
@@ -1266,190 +1440,149 @@ __global__ void __launch_bounds__(THREADS) k_local(StepParams p, const double* _
                 // SLIDE_FAR |d|) past it, where the path beyond the knot carries most of the
                 // orbit average; if both sides push onto the knot, the root lies within that
                 // hair, unresolved in double precision, and the component lands on the knot.
-#pragma unroll
-                for (int a = 0; a < 3; ++a) ue[a] = u1[a];
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-                    if (a == paxis) {
-                        const double d = dk[a], far = fmax(SLIDE_PROBE, SLIDE_FAR * fabs(d));
-                        ue[a] = phase == 0 ? 2.0 * (d - (d > 0.0 ? SLIDE_PROBE : far)) * p.H[a] / p.dt - vn[a]
-                                           : 2.0 * (d + (d > 0.0 ? far : SLIDE_PROBE)) * p.H[a] / p.dt - vn[a];
-                    }
-            } else if (phase == 2) {
-#pragma unroll
-                for (int a = 0; a < 3; ++a) ue[a] = u1[a];
-            } else {
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const double c = p.dt * 0.5 / p.H[a];   // beta = c (u + v^n), in cells
-                    const double xk = x0[a] - p.koff;        // start on the knot lattice
-                    double fp = ub[a] - gb[a] * (ub[a] - ua[a]) / (gb[a] - ga[a]);
-                    {
+                if (comp == paxis) {
+                    const double far = fmax(SLIDE_PROBE, SLIDE_FAR * fabs(dk));
+                    ue = phase == 0 ? ha * (dk - (dk > 0.0 ? SLIDE_PROBE : far)) - vn
+                                    : ha * (dk + (dk > 0.0 ? far : SLIDE_PROBE)) - vn;
+                }
+            } else if (phase == 3) {
+                // the knot landing strictly inside the bracket (the highest one, if several)
+                const double lo = fmin(ua, ub), hi = fmax(ua, ub);
+                const double bland = (ceil(xa + cba * (hi + vn)) - 1.0) - xa;
+                const double usplit = ha * bland - vn;
+                double fp = NAN;
+                if (sl) {
+                    ue = uland;                          // pinned: lands on the knot
+                } else if (brk && bland > cba * (lo + vn) && usplit > lo && usplit < hi) {
+                    ue = usplit;                         // split the bracket where G kinks
+                } else {
+                    if (brk) {
+                        fp = ub - gb * (ub - ua) / (gb - ga);
                         // Both ends past the same last knot (landing beta_L): on that knot-free
                         // piece the image G in cells is close to A + B w, w = beta_L / beta, steep
                         // near the knot and flat far past it; solve beta = A + B w exactly for the
                         // line through the two ends (D beta^2 - c1 beta - e = 0, root in bracket).
-                        const double ba = c * (ua[a] + vn[a]), bb = c * (ub[a] + vn[a]);
-                        const double la = ba > 0.0 ? floor(xk + ba) - xk : ceil(xk + ba) - xk;
-                        const double lb = bb > 0.0 ? floor(xk + bb) - xk : ceil(xk + bb) - xk;
-                        const double Ga = c * ga[a] + ba, Gb = c * gb[a] + bb;
-                        const double wa = la / ba, wb = la / bb;
-                        const double D = wb - wa;
-                        const double c1 = Ga * D - (Gb - Ga) * wa;
-                        const double e = (Gb - Ga) * la;
-                        const double disc = c1 * c1 + 4.0 * D * e;
-                        const double qq = 0.5 * (c1 + copysign(sqrt(fmax(disc, 0.0)), c1));
-                        const double x1 = qq / D, x2 = -e / qq;
-                        const double bl = fmin(ba, bb), bh = fmax(ba, bb);
-                        const bool in1 = x1 > bl && x1 < bh, in2 = x2 > bl && x2 < bh;
-                        const double fpm = 2.0 * (in1 ? x1 : x2) * p.H[a] / p.dt - vn[a];
-                        if (la == lb && la != 0.0 && la * ba > 0.0 && la * bb > 0.0 && disc >= 0.0 && (in1 || in2) &&
-                            isfinite(fpm))
-                            fp = fpm;
+                        const double ba = cba * (ua + vn), bb = cba * (ub + vn);
+                        const double la = ba > 0.0 ? floor(xa + ba) - xa : ceil(xa + ba) - xa;
+                        const double lb = bb > 0.0 ? floor(xa + bb) - xa : ceil(xa + bb) - xa;
+                        if (la == lb && la != 0.0 && la * ba > 0.0 && la * bb > 0.0) {
+                            const double Ga = cba * ga + ba, Gb = cba * gb + bb;
+                            const double wa = la / ba, wb = la / bb;
+                            const double D = wb - wa;
+                            const double c1 = Ga * D - (Gb - Ga) * wa;
+                            const double e = (Gb - Ga) * la;
+                            const double disc = c1 * c1 + 4.0 * D * e;
+                            const double qq = 0.5 * (c1 + copysign(sqrt(fmax(disc, 0.0)), c1));
+                            const double x1 = qq / D, x2 = -e / qq;
+                            const double bl = fmin(ba, bb), bh = fmax(ba, bb);
+                            const bool in1 = x1 > bl && x1 < bh, in2 = x2 > bl && x2 < bh;
+                            const double fpm = ha * (in1 ? x1 : x2) - vn;
+                            if (disc >= 0.0 && (in1 || in2) && isfinite(fpm)) fp = fpm;
+                        }
                     }
-                    double sec = -(u1[a] - u0[a]) / (r1[a] - r0[a]);
-                    sec = isfinite(sec) ? fmin(fmax(sec, -OMEGA_MAX), OMEGA_MAX) : 1.0;
-                    // the knot landing strictly inside the bracket (the highest one, if several)
-                    const double lo = fmin(ua[a], ub[a]), hi = fmax(ua[a], ub[a]);
-                    const double blo = c * (lo + vn[a]), bhi = c * (hi + vn[a]);
-                    const double bland = (ceil(xk + bhi) - 1.0) - xk;
-                    const double usplit = 2.0 * bland * p.H[a] / p.dt - vn[a];
-                    if (sl[a]) {
-                        ue[a] = uland[a];                    // pinned: lands on the knot
-                    } else if (brk[a] && bland > blo && usplit > lo && usplit < hi) {
-                        ue[a] = usplit;                      // split the bracket where G kinks
-                    } else if (brk[a] && isfinite(fp)) {
-                        ue[a] = fp;                          // bracketed step
-                    } else if (!brk[a] && !secok[a]) {
-                        ue[a] = u1[a] + fac[a] * r1[a];      // grow along g until g changes sign
-                        fac[a] *= 2.0;
+                    if (brk && isfinite(fp)) {
+                        ue = fp;                             // bracketed step
+                    } else if (!brk && !secok) {
+                        ue = u1 + fac * r1;                  // grow along g until g changes sign
+                        fac *= 2.0;
                     } else {
-                        ue[a] = u1[a] + sec * r1[a];         // secant while it converges
+                        double sec = -(u1 - u0) / (r1 - r0);
+                        sec = isfinite(sec) ? fmin(fmax(sec, -OMEGA_MAX), OMEGA_MAX) : 1.0;
+                        ue = u1 + sec * r1;                  // secant while it converges
                     }
-                    // trial orbits stay within BETA_TRIAL cells beyond the iterate's own orbit, per
-                    // axis (the growing steps along g would otherwise run past any neighbourhood
-                    // of the root)
-                    ue[a] = fmin(fmax(ue[a], -blim[a] / c - vn[a]), blim[a] / c - vn[a]);
                 }
+                // trial orbits stay within BETA_TRIAL cells beyond the iterate's own orbit, per
+                // axis (the growing steps along g would otherwise run past any neighbourhood
+                // of the root)
+                ue = fmin(fmax(ue, -blim / cba - vn), blim / cba - vn);
             }
         }
-        PushOut o;
-        if (active) {
-            if constexpr (QUAD == 0) {
-                CellStart<double> st;
-                CellOut co;
-                double vs[3];
-                cell_start(x0, p.m, st);
-#pragma unroll
-                for (int a = 0; a < 3; ++a) vs[a] = ue[a] + vn[a];
-                push_eval_cell<CELLS>(p, st, vs, Pn, table, co);
-                o.nseg = co.nseg;
-#pragma unroll
-                for (int a = 0; a < 3; ++a) o.vw[a] = co.vw[a];
-            } else {
-                PushAcc acc;
-                push_eval<QUAD, false>(p, x0, vn, Pn, ue, table, acc, o);
-            }
-            if (phase >= 2 && o.nseg < 0) atomicOr(status, DEV_ERR_SEGMENTS);
-            neval += 1.0;
-        }
-        if (!active) continue;
+        const double vsa = active ? ue + vn : 0.0;
+        const double vs[3] = {of(vsa, 0), of(vsa, 1), of(vsa, 2)};
+        int nseg = 0;
+        const double vw = push_eval_shared<QUAD, CELLS>(p, k, comp, x0, st, vs, Pn, table, nseg);
+        const double res = vw - ue;                          // g of this lane's component
+        const double gp = of(res, paxis < 3 ? paxis : 0);
+        const double a0 = max3(sl ? 0.0 : fabs(r0)), a1 = max3(sl ? 0.0 : fabs(res));
         bool done = false;
-        if (phase == 0) {
-            gm = o.vw[paxis] - ue[paxis];
-            phase = 1;
-        } else if (phase == 1) {
-            const double gp = o.vw[paxis] - ue[paxis];
-            sl[paxis] = gm > 0.0 && gp < 0.0;
-            ++paxis;
-            while (paxis < 3 && !probe[paxis]) ++paxis;
-            if (paxis < 3) {
-                phase = 0;
+        if (active) {
+            if (phase >= 2 && nseg < 0) atomicOr(status, DEV_ERR_SEGMENTS);
+            if (k == 0) neval += 1.0;
+            if (phase == 0) {
+                gm = gp;
+                phase = 1;
+            } else if (phase == 1) {
+                if (comp == paxis) sl = gm > 0.0 && gp < 0.0;
+                ++paxis;
+                while (paxis < 3 && !((probes >> paxis) & 1)) ++paxis;
+                if (paxis < 3) {
+                    phase = 0;
+                } else {
+                    if (sl) u1 = uland;
+                    phase = 2;
+                }
+            } else if (phase == 2) {
+                r1 = sl ? 0.0 : res;
+                if (sl) r0 = 0.0;
+                brk = !sl && r0 * r1 < 0.0;
+                ua = u0;
+                ga = r0;
+                ub = u1;
+                gb = r1;
+                side = 0.0;
+                secok = fabs(r1) <= 0.5 * fabs(r0);
+                fac = 2.0;
+                nrep = 0;
+                // the best evaluation so far, whole (the components are coupled): the smallest
+                // largest-component |g|; pinned components land on their knot
+                bu = sl ? uland : (a1 < a0 ? u1 : u0);
+                brs = fmin(a0, a1);
+                phase = 3;
+                done = nstep >= LOCAL_STEPS - 1 || brs <= tol;
             } else {
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-                    if (sl[a]) u1[a] = uland[a];
-                phase = 2;
-            }
-        } else if (phase == 2) {
-            double m0 = 0.0, m1 = 0.0;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                r1[a] = sl[a] ? 0.0 : o.vw[a] - u1[a];
-                if (sl[a]) r0[a] = 0.0;
-                m0 = fmax(m0, fabs(r0[a]));
-                m1 = fmax(m1, fabs(r1[a]));
-                brk[a] = !sl[a] && r0[a] * r1[a] < 0.0;
-                ua[a] = u0[a];
-                ga[a] = r0[a];
-                ub[a] = u1[a];
-                gb[a] = r1[a];
-                side[a] = 0.0;
-                secok[a] = fabs(r1[a]) <= 0.5 * fabs(r0[a]);
-                fac[a] = 2.0;
-                nrep[a] = 0;
-            }
-            // the best evaluation so far, whole (the components are coupled): the smallest
-            // largest-component |g|; pinned components land on their knot
-            const bool take1 = m1 < m0;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) bu[a] = sl[a] ? uland[a] : (take1 ? u1[a] : u0[a]);
-            brs = fmin(m0, m1);
-            phase = 3;
-            done = nstep >= LOCAL_STEPS - 1 || brs <= tol;
-        } else {
-            double r2v[3], m2 = 0.0;
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                r2v[a] = sl[a] ? 0.0 : o.vw[a] - ue[a];
-                m2 = fmax(m2, fabs(r2v[a]));
-            }
-            if (m2 < brs) {
-                brs = m2;
-#pragma unroll
-                for (int a = 0; a < 3; ++a) bu[a] = ue[a];
-            }
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const double r2 = r2v[a];
-                secok[a] = secok[a] && fabs(r2) <= 0.5 * fabs(r1[a]);
-                if (brk[a]) {
-                    if (r2 * gb[a] > 0.0) {            // replaces the b end
-                        nrep[a] = side[a] > 0.0 ? nrep[a] + 1 : 1;
-                        ub[a] = ue[a];
-                        gb[a] = r2;
-                        side[a] = 1.0;
+                const double r2 = sl ? 0.0 : res;
+                if (a1 < brs) {
+                    brs = a1;
+                    bu = ue;
+                }
+                secok = secok && fabs(r2) <= 0.5 * fabs(r1);
+                if (brk) {
+                    if (r2 * gb > 0.0) {               // replaces the b end
+                        nrep = side > 0.0 ? nrep + 1 : 1;
+                        ub = ue;
+                        gb = r2;
+                        side = 1.0;
                     } else {                           // replaces the a end
-                        nrep[a] = side[a] < 0.0 ? nrep[a] + 1 : 1;
-                        ua[a] = ue[a];
-                        ga[a] = r2;
-                        side[a] = -1.0;
+                        nrep = side < 0.0 ? nrep + 1 : 1;
+                        ua = ue;
+                        ga = r2;
+                        side = -1.0;
                     }
                     // the same end replaced twice running: the kept end is stale (its g was
                     // taken before the other components moved) or regula falsi stagnates;
                     // released, the next step is a secant one from two fresh points
-                    if (nrep[a] >= 2) {
-                        brk[a] = false;
-                        secok[a] = true;
-                        nrep[a] = 0;
-                        side[a] = 0.0;
+                    if (nrep >= 2) {
+                        brk = false;
+                        secok = true;
+                        nrep = 0;
+                        side = 0.0;
                     }
-                } else if (!sl[a] && r2 * r1[a] < 0.0) {
-                    brk[a] = true;
-                    ua[a] = u1[a];
-                    ga[a] = r1[a];
-                    ub[a] = ue[a];
-                    gb[a] = r2;
+                } else if (!sl && r2 * r1 < 0.0) {
+                    brk = true;
+                    ua = u1;
+                    ga = r1;
+                    ub = ue;
+                    gb = r2;
                 }
-                u0[a] = u1[a];
-                r0[a] = r1[a];
-                u1[a] = ue[a];
-                r1[a] = r2;
+                u0 = u1;
+                r0 = r1;
+                u1 = ue;
+                r1 = r2;
+                ++nstep;
+                done = nstep >= LOCAL_STEPS - 1 || brs <= tol;
             }
-            ++nstep;
-            done = nstep >= LOCAL_STEPS - 1 || brs <= tol;
         }
-        if (!done) continue;
+        if (!__any_sync(full, done)) continue;
         // the particle's solve is over: its best iterate, sliding marks, e_v terms and current.
         // A solve that ends above the tolerance on the landing of its nearest knot, or that
         // fails (best residual above FAIL_RES of the speed) with a component starting within
@@ -1458,40 +1591,62 @@ __global__ void __launch_bounds__(THREADS) k_local(StepParams p, const double* _
         // defect is then bounded by vbar_a = d H / dt times its residual, where it would
         // otherwise be the whole velocity times that residual; below FAIL_RES the residual
         // itself costs less.
-        {
-            const bool failed = brs > FAIL_RES * spd;
-            bool pinned = false;
+        const bool failed = brs > FAIL_RES * spd;
+        const bool hair = failed && fabs(dk) < D_FALLBACK;
+        if (done && ((brs > tol && bu == uland) || hair)) sl = true;
+        const int pinned = bits3(hair), slides = bits3(sl);
+        if (done && sl) bu = uland;
+        const double v2 = bu + vn;
+        const double v2n[3] = {of(v2, 0), of(v2, 1), of(v2, 2)};
+        if (done) {
+            if (!isfinite(bu)) atomicOr(status, DEV_ERR_NONFINITE);
+            if (k < 3) {
+                const double d = bu - vit[comp * np + i];
+                ev_num += d * d;
+                ev_den += bu * bu;
+                vnew[comp * np + i] = bu;
+            }
+            if (k == 0) {
+                slide[i] = (uint8_t)(slides | SLIDE_CREPT);
+                nsolve += 1.0;
+                nfail += failed ? 1.0 : 0.0;
+                nfail_free += (failed && !pinned) ? 1.0 : 0.0;
+            }
+            double beta[3], w[3];
+            int ns;
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                if ((brs > tol && bu[a] == uland[a]) || (failed && fabs(dk[a]) < D_FALLBACK)) sl[a] = true;
-                pinned = pinned || (failed && fabs(dk[a]) < D_FALLBACK);
+                beta[a] = p.cb[a] * v2n[a];
+                w[a] = p.q_dV_half * v2n[a];
             }
-            nfail += failed ? 1.0 : 0.0;
-            nfail_free += (failed && !pinned) ? 1.0 : 0.0;
-        }
-        uint8_t sb = 0;
+            if constexpr (QUAD == 0) {
+                const int64_t N = p.m.ncell;
+                CellStart<double> s = st;
+                ns = for_each_piece(s, beta, p.m, [&](double h, double, const double mid[3], const int c[3]) {
+                    double W[8];
+                    node_weights(piece_moments(h, mid, beta), W);
+                    int cn[3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
-            if (sl[a]) {
-                bu[a] = uland[a];
-                sb |= (uint8_t)(1u << a);
+                    for (int a = 0; a < 3; ++a) cn[a] = ((k >> a) & 1) ? next_cell(c[a], p.m.n[a]) : c[a];
+                    const int64_t g = cell_row(cn, p.m);
+                    const double Wk = h * pick8(W, k);
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        if (p.det) exact_add(p.acc, a * N + g, w[a] * Wk);
+                        else atomicAdd(Jnext + a * N + g, w[a] * Wk);
+                    }
+                });
+            } else if (p.split) {
+                if (p.order == 2) ns = scatter_pieces<2>(p, x0, beta, w, Jnext, k, LOCAL_LANES);
+                else if (p.order == 3) ns = scatter_pieces<3>(p, x0, beta, w, Jnext, k, LOCAL_LANES);
+                else ns = scatter_pieces<1>(p, x0, beta, w, Jnext, k, LOCAL_LANES);
+            } else {
+                ns = k == 0 ? scatter_orbit<QUAD>(p, x0, beta, w, Jnext) : 0;
             }
-        slide[i] = sb | SLIDE_CREPT;
-        double wv[3], bet2[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            if (!isfinite(bu[a])) atomicOr(status, DEV_ERR_NONFINITE);
-            const double d = bu[a] - vit[a * np + i];
-            ev_num += d * d;
-            ev_den += bu[a] * bu[a];
-            vnew[a * np + i] = bu[a];
-            const double vb2 = 0.5 * (bu[a] + vn[a]);
-            bet2[a] = p.dt * vb2 * p.invH[a];
-            wv[a] = p.q_dV * vb2;
+            if (ns < 0) atomicOr(status, DEV_ERR_SEGMENTS);
+            active = false;
         }
-        if (scatter_orbit<QUAD>(p, x0, bet2, wv, Jnext) < 0) atomicOr(status, DEV_ERR_SEGMENTS);
-        nsolve += 1.0;
-        active = false;
+        __syncwarp();
     }
     write_partial<double>(partials, S_EVL_NUM, ev_num, sm, false);
     write_partial<double>(partials, S_EVL_DEN, ev_den, sm, false);
@@ -1761,7 +1916,10 @@ bool setup_particle_kernels() {
            cudaFuncSetAttribute(k_push_cell<false, false>, at, bytes) == cudaSuccess;
 }
 
-int local_blocks(const Ctx& c) { return std::max(1, std::min(particle_blocks(c), c.sms * 2)); }
+int local_blocks(const Ctx& c) {
+    const int64_t b = (c.np * LOCAL_LANES + THREADS - 1) / THREADS;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)c.sms * LOCAL_MINB));
+}
 
 int particle_blocks(const Ctx& c) {
     int64_t b = (c.np + THREADS - 1) / THREADS;
