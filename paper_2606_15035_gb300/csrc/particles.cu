@@ -1176,18 +1176,24 @@ __global__ void __launch_bounds__(THREADS, DIAG ? 1 : 2) k_push(StepParams p, co
 // identities hold to the size of vbar_a = d H / dt < D_KNOT H / dt.  The plain image G(v^p)
 // is saved in gsave (diagnostics), then the orbit current of the result is scattered.
 //
-// Eight lanes share a particle.  A solve is a serial chain of evaluations (up to 34, two on average),
-// and on the FP64 pipe a warp instruction takes 64 clocks of its scheduler whether one lane is active
-// or 32, so what bounds the launch is the length of that chain.  Lanes 0 .. 2 hold one component each
-// (state and step logic), lane k evaluates table entry k of a piece (subset k of the axes; rows k and
-// k + 8 of a Gauss piece's nodes) and the sums meet in three exchanges per evaluation: 55 FP64
-// instructions a piece for 130, and only the step that is taken is computed.  Groups take particles
-// from a queue four to a warp (deterministic mode: in index order from the warp's own share of the
-// flags, so that every partial sum is reproducible), the first warps of all blocks first.
+// Four lanes share a particle (eight with a Gauss rule).  A solve is a serial chain of evaluations (up
+// to 34, two on average), and on the FP64 pipe a warp instruction takes 64 clocks of its scheduler
+// whether one lane is active or 32, so what bounds the launch is the length of that chain, or, with
+// many particles, the instructions a warp spends on each.  Lanes 0 .. 2 hold one component each (state
+// and step logic), lane k evaluates table entries k and k + 4 of a piece (subsets of the axes; rows k,
+// k + 8 of a Gauss piece's nodes) and the sums meet in two exchanges per evaluation, and only the step
+// that is taken is computed.  Groups take particles from a queue, a warp's groups together
+// (deterministic mode: in index order from the warp's own share of the flags, so that every partial
+// sum is reproducible), the first warps of all blocks first.
 // With one particle per lane (13 of 32 lanes active on average, the particles on the blocks that came
-// first) the mean launch of two steps at 32^3 with 2,097,152 particles took 377 us, now 108; a
-// deterministic step at 24^3 with 442,368 376, now 147; quadratic shapes 800, now 307.
-constexpr int LOCAL_LANES = 8;
+// first) the mean launch of two steps at 32^3 with 2,097,152 particles took 377 us, now 113; two
+// diagnosed steps at 50 x 35 x 22 with 539,000 particles, one in ten of them solved here, 454, now 247;
+// quadratic shapes 800, now 294.  With eight lanes the closed forms measured 110, 327, and 5.3 ms
+// where four take 3.5 at 128^3 with 134M particles; quadratic shapes with four 348.
+template <int QUAD>
+constexpr int local_lanes() {
+    return QUAD == 0 ? 4 : 8;
+}
 constexpr int LOCAL_MINB = 1;   // blocks per SM: 2 (128 registers, 480 bytes of spills) measured 114 us
 
 // v[k] of an 8-array held in registers.
@@ -1198,9 +1204,10 @@ __device__ __forceinline__ double pick8(const double v[8], int k) {
     return (k & 4) ? b1 : b0;
 }
 
-// Lane k's share of piece_impulse: acc_j += its terms (summed over the 8 lanes they are the piece's).
-template <bool CELLS>
-__device__ __forceinline__ void piece_impulse_share(const StepParams& p, int k, double h, double sm, const double mid[3],
+// Lane r's share of piece_impulse: acc_j += its terms, those of the subsets r, r + LANES, ... (summed
+// over the lanes they are the piece's).
+template <bool CELLS, int LANES>
+__device__ __forceinline__ void piece_impulse_share(const StepParams& p, int r, double h, double sm, const double mid[3],
                                                     const double beta[3], const double vs[3], const int c[3],
                                                     const double* __restrict__ table, double acc[3]) {
     const PieceMoments<double> q = piece_moments(h, mid, beta);
@@ -1208,21 +1215,27 @@ __device__ __forceinline__ void piece_impulse_share(const StepParams& p, int k, 
     const double E[8] = {0.0, q.e[0], q.e[1], mid[0] * q.e[1] + mid[1] * q.e[0],
                          q.e[2], mid[0] * q.e[2] + mid[2] * q.e[0], mid[1] * q.e[2] + mid[2] * q.e[1], 0.0};
     const FieldLoad<CELLS> ld(table, c, p.m);
-    double col[CELL_COLS];
+    const double hi[3] = {h * p.ihs[0], h * p.ihs[1], h * p.ihs[2]};
 #pragma unroll
-    for (int t = 0; t < CELL_COLS; ++t) {
-        double e0, e1;
-        ld(k >> 1, t, e0, e1);
-        col[t] = (k & 1) ? e1 : e0;
-    }
-    const double cc = col[3] * vs[0] + col[4] * vs[1] + col[5] * vs[2];
-    const double a = col[0] * vs[0] + col[1] * vs[1] + col[2] * vs[2] + (sm - 1.0) * cc;
-    const double m = pick8(M, k);
+    for (int s = 0; s < 8 / LANES; ++s) {
+        const int k = r + s * LANES;
+        double col[CELL_COLS];
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        const bool in = (k >> j) & 1;
-        const double F = a * pick8(M, k ^ (1 << j)) + cc * pick8(E, k ^ (1 << j));
-        acc[j] += h * (col[6 + j] * m + (in ? p.ihs[j] * F : 0.0));
+        for (int t = 0; t < CELL_COLS; ++t) {
+            double e0, e1;
+            ld(k >> 1, t, e0, e1);
+            col[t] = (k & 1) ? e1 : e0;
+        }
+        const double cc = col[3] * vs[0] + col[4] * vs[1] + col[5] * vs[2];
+        const double a = col[0] * vs[0] + col[1] * vs[1] + col[2] * vs[2] + (sm - 1.0) * cc;
+        const double m = h * pick8(M, k);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const bool in = (k >> j) & 1;
+            const double F = a * pick8(M, k ^ (1 << j)) + cc * pick8(E, k ^ (1 << j));
+            acc[j] += col[6 + j] * m;
+            acc[j] += in ? hi[j] * F : 0.0;
+        }
     }
 }
 
@@ -1257,38 +1270,43 @@ __device__ __forceinline__ void basis1<1>(double x, double invH, Basis1<1>& b) {
     b.dw[1] = invH;
 }
 
-// G(u) of the particle that 8 lanes share, u = vs - v^n: every lane gets the component `comp` of
+// G(u) of the particle that a group of lanes shares, u = vs - v^n: every lane gets the component `comp` of
 // v^{n+1}.  Every lane of the warp calls it (inactive groups with any valid start).
 template <int QUAD, bool CELLS>
 __device__ __forceinline__ double push_eval_shared(const StepParams& p, int k, int comp, const double x0[3],
                                                    const CellStart<double>& start, const double vs[3], double Pn,
                                                    const double* __restrict__ table, int& nseg) {
+    constexpr int LANES = local_lanes<QUAD>();
     double beta[3], acc[3] = {0.0, 0.0, 0.0}, Ae[3] = {0.0, 0.0, 0.0};
     CellStart<double> st = start;
 #pragma unroll
     for (int a = 0; a < 3; ++a) beta[a] = p.cb[a] * vs[a];
     if constexpr (QUAD == 0) {
         nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
-            piece_impulse_share<CELLS>(p, k, h, sm, mid, beta, vs, c, table, acc);
+            piece_impulse_share<CELLS, LANES>(p, k, h, sm, mid, beta, vs, c, table, acc);
         });
         const FieldLoad<CELLS> ld(table, st.c, p.m);
-        double e = (k & 1) ? st.f[0] : 1.0;
-        if (k & 2) e *= st.f[1];
-        if (k & 4) e *= st.f[2];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            double e0, e1;
-            ld(k >> 1, a, e0, e1);
-            Ae[a] = e * ((k & 1) ? e1 : e0);
+        for (int s = 0; s < 8 / LANES; ++s) {
+            const int kk = k + s * LANES;
+            double e = (kk & 1) ? st.f[0] : 1.0;
+            if (kk & 2) e *= st.f[1];
+            if (kk & 4) e *= st.f[2];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                double e0, e1;
+                ld(kk >> 1, a, e0, e1);
+                Ae[a] += e * ((kk & 1) ? e1 : e0);
+            }
         }
     } else {
         PushAcc pa{};
         const double vb[3] = {0.5 * vs[0], 0.5 * vs[1], 0.5 * vs[2]};
         if (p.split) {
             nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
-                if (p.order == 2) push_piece_points<2, false>(p, h, sm, mid, c, beta, vb, table, pa, k, LOCAL_LANES);
-                else if (p.order == 3) push_piece_points<3, false>(p, h, sm, mid, c, beta, vb, table, pa, k, LOCAL_LANES);
-                else push_piece_points<1, false>(p, h, sm, mid, c, beta, vb, table, pa, k, LOCAL_LANES);
+                if (p.order == 2) push_piece_points<2, false>(p, h, sm, mid, c, beta, vb, table, pa, k, LANES);
+                else if (p.order == 3) push_piece_points<3, false>(p, h, sm, mid, c, beta, vb, table, pa, k, LANES);
+                else push_piece_points<1, false>(p, h, sm, mid, c, beta, vb, table, pa, k, LANES);
             });
         } else {
             nseg = for_each_segment(x0, beta, false, [&](const Segment<double>& sg) {
@@ -1304,9 +1322,9 @@ __device__ __forceinline__ double push_eval_shared(const StepParams& p, int k, i
             acc[a] = mine ? pa.F[a] - pa.gphi[a] : 0.0;
             xe[a] = wrap_pos(x0[a] + beta[a], (double)p.m.n[a]);
         }
-        if (p.order == 2) point_A1_rows<2>(p, xe, table, k, LOCAL_LANES, Ae);
-        else if (p.order == 3) point_A1_rows<3>(p, xe, table, k, LOCAL_LANES, Ae);
-        else point_A1_rows<1>(p, xe, table, k, LOCAL_LANES, Ae);
+        if (p.order == 2) point_A1_rows<2>(p, xe, table, k, LANES, Ae);
+        else if (p.order == 3) point_A1_rows<3>(p, xe, table, k, LANES, Ae);
+        else point_A1_rows<1>(p, xe, table, k, LANES, Ae);
     }
     __syncwarp();
     double kick = 0.0;   // P^{n+1} - P^n - q A_h^{n+1}(x^{n+1}) of this lane's component
@@ -1314,7 +1332,7 @@ __device__ __forceinline__ double push_eval_shared(const StepParams& p, int k, i
     for (int a = 0; a < 3; ++a) {
         double t = p.dtq * acc[a] - p.q * Ae[a];
 #pragma unroll
-        for (int o = 1; o < LOCAL_LANES; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        for (int o = 1; o < LANES; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
         if (a == comp) kick = t;
     }
     return (Pn + kick) * p.inv_mass;
@@ -1331,10 +1349,11 @@ __global__ void __launch_bounds__(THREADS, LOCAL_MINB) k_local(StepParams p, con
                                                    int* __restrict__ queue_head, double* __restrict__ partials,
                                                    int* __restrict__ status) {
     __shared__ double sm[32];
+    constexpr int LANES = local_lanes<QUAD>();
     const unsigned full = 0xffffffffu;
     const int64_t np = p.np;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int k = lane & (LOCAL_LANES - 1), comp = min(k, 2), gbase = lane & ~(LOCAL_LANES - 1);
+    const int k = lane & (LANES - 1), comp = min(k, 2), gbase = lane & ~(LANES - 1);
     // this warp's share of the flags (deterministic mode), or of the queue
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
     const int64_t share = (np + nwarps - 1) / nwarps, wid = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
@@ -1343,7 +1362,7 @@ __global__ void __launch_bounds__(THREADS, LOCAL_MINB) k_local(StepParams p, con
     unsigned bits = 0;
     const int64_t count = creep_flag ? 0 : (int64_t)*creep_count;
     // few particles: the warps that the others' SMs can do without stay out
-    const int64_t per = (int64_t)gridDim.x * (32 / LOCAL_LANES);
+    const int64_t per = (int64_t)gridDim.x * (32 / LANES);
     bool active = false, exhausted = !creep_flag && count <= per * warp;
     double ev_num = 0.0, ev_den = 0.0;
     // One particle's solve is a sequence of push evaluations: sliding probes (phase 0: just
@@ -1625,21 +1644,25 @@ __global__ void __launch_bounds__(THREADS, LOCAL_MINB) k_local(StepParams p, con
                 ns = for_each_piece(s, beta, p.m, [&](double h, double, const double mid[3], const int c[3]) {
                     double W[8];
                     node_weights(piece_moments(h, mid, beta), W);
-                    int cn[3];
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) cn[a] = ((k >> a) & 1) ? next_cell(c[a], p.m.n[a]) : c[a];
-                    const int64_t g = cell_row(cn, p.m);
-                    const double Wk = h * pick8(W, k);
+                    for (int t = 0; t < 8 / LANES; ++t) {
+                        const int kk = k + t * LANES;
+                        int cn[3];
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        if (p.det) exact_add(p.acc, a * N + g, w[a] * Wk);
-                        else atomicAdd(Jnext + a * N + g, w[a] * Wk);
+                        for (int a = 0; a < 3; ++a) cn[a] = ((kk >> a) & 1) ? next_cell(c[a], p.m.n[a]) : c[a];
+                        const int64_t g = cell_row(cn, p.m);
+                        const double Wk = h * pick8(W, kk);
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) {
+                            if (p.det) exact_add(p.acc, a * N + g, w[a] * Wk);
+                            else atomicAdd(Jnext + a * N + g, w[a] * Wk);
+                        }
                     }
                 });
             } else if (p.split) {
-                if (p.order == 2) ns = scatter_pieces<2>(p, x0, beta, w, Jnext, k, LOCAL_LANES);
-                else if (p.order == 3) ns = scatter_pieces<3>(p, x0, beta, w, Jnext, k, LOCAL_LANES);
-                else ns = scatter_pieces<1>(p, x0, beta, w, Jnext, k, LOCAL_LANES);
+                if (p.order == 2) ns = scatter_pieces<2>(p, x0, beta, w, Jnext, k, LANES);
+                else if (p.order == 3) ns = scatter_pieces<3>(p, x0, beta, w, Jnext, k, LANES);
+                else ns = scatter_pieces<1>(p, x0, beta, w, Jnext, k, LANES);
             } else {
                 ns = k == 0 ? scatter_orbit<QUAD>(p, x0, beta, w, Jnext) : 0;
             }
@@ -1917,7 +1940,7 @@ bool setup_particle_kernels() {
 }
 
 int local_blocks(const Ctx& c) {
-    const int64_t b = (c.np * LOCAL_LANES + THREADS - 1) / THREADS;
+    const int64_t b = (c.np * 8 + THREADS - 1) / THREADS;
     return (int)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)c.sms * LOCAL_MINB));
 }
 
