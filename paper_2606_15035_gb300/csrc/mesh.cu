@@ -178,26 +178,41 @@ __global__ void k_rhs0(MeshParams p, const double* __restrict__ F0, const double
 // Continuity (Eq. (cn-continuity)) and the CN sources; e_J partial sums.
 __global__ void k_source(MeshParams p, const double* __restrict__ J, const double* __restrict__ Jprev,
                          const double* __restrict__ rho0, const double* __restrict__ rhs0, double* __restrict__ rho1,
-                         double* __restrict__ rhs, double* __restrict__ partials) {
+                         double* __restrict__ rhs, const double* __restrict__ start, int* __restrict__ top,
+                         double* __restrict__ partials) {
     __shared__ double sm[32];
     const int64_t N = p.m.ncell;
     double num = 0.0, den = 0.0;
+    int e[4] = {0, 0, 0, 0};   // largest exponents of the right-hand sides and the solve's start
     GRID_LOOP(g, N) {
         Nb b = decompose(g, p.m);
         double divJ = dcen(J, b, 0, p.m, p.invH) + dcen(J + N, b, 1, p.m, p.invH) + dcen(J + 2 * N, b, 2, p.m, p.invH);
         double r0 = rho0[g];
         double r1 = r0 - p.dt * divJ;
         rho1[g] = r1;
-        rhs[g] = rhs0[g] + p.c_rho * 0.5 * (r1 + r0);
+        double rh[4];
+        rh[0] = rhs0[g] + p.c_rho * 0.5 * (r1 + r0);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             double j = J[c * N + g];
-            rhs[(1 + c) * N + g] = rhs0[(1 + c) * N + g] + p.c_J * j;
+            rh[1 + c] = rhs0[(1 + c) * N + g] + p.c_J * j;
             den += j * j;
             if (Jprev) {
                 double d = j - Jprev[c * N + g];
                 num += d * d;
             }
+        }
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            rhs[f * N + g] = rh[f];
+            if (top) e[f] = max(e[f], max((__double2hiint(rh[f]) >> 20) & 0x7ff, (__double2hiint(start[f * N + g]) >> 20) & 0x7ff));
+        }
+    }
+    if (top) {
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+            const int t = (int)__reduce_max_sync(0xffffffffu, (unsigned)e[f]);
+            if ((threadIdx.x & 31) == 0) atomicMax(top + f, t);
         }
     }
     put_partial(partials, S_EJ_NUM, num, sm, false);
@@ -336,8 +351,10 @@ __global__ void __launch_bounds__(THREADS) k_cheb_all(MeshParams p, double* xa, 
 }
 
 __global__ void k_backsub_table(MeshParams p, const double* __restrict__ F0, const double* __restrict__ W0,
-                                const double* __restrict__ F1, double* __restrict__ W1, double* __restrict__ table) {
+                                const double* __restrict__ F1, double* __restrict__ W1, double* __restrict__ table,
+                                int* __restrict__ top) {
     const int64_t N = p.m.ncell;
+    if (top && blockIdx.x == 0 && threadIdx.x < 4) top[threadIdx.x] = 0;   // for the next k_source
     GRID_LOOP(g, N) {
         Nb b = decompose(g, p.m);
         double w1[4];
@@ -539,7 +556,7 @@ void launch_rhs0(Ctx& c) {
 
 void launch_source(Ctx& c, const double* Jcur, const double* Jprev) {
     k_source<<<mesh_blocks(c), THREADS, 0, c.stream>>>(mesh_params(c), Jcur, Jprev, c.rho0, c.rhs0, c.rho1, c.rhs,
-                                                       c.partials);
+                                                       c.F1, c.helm_top, c.partials);
     ++c.launches;
 }
 
@@ -618,7 +635,8 @@ int cheb_coop_capacity(const Ctx& c) {
 }
 
 void launch_backsub_table(Ctx& c, bool) {
-    k_backsub_table<<<mesh_blocks(c), THREADS, 0, c.stream>>>(mesh_params(c), c.F0, c.W0, c.F1, c.W1, c.table);
+    k_backsub_table<<<mesh_blocks(c), THREADS, 0, c.stream>>>(mesh_params(c), c.F0, c.W0, c.F1, c.W1, c.table,
+                                                            c.helm_top);
     ++c.launches;
 }
 

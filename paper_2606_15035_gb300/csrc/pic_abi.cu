@@ -292,6 +292,16 @@ void setup_geometry(Ctx& c) {
     c.cheb_rate = (c.cheb_iters > 1 && rho > 0.0) ? 1.0 / std::log(1.0 / rho) : 0.0;
 }
 
+// PIC_MIXED: the fields of an FP32 iteration need no more accuracy than its iterate has
+// (e_v >= ~1e-9), and those of an FP64 refinement iteration no more than a thousandth of
+// mixed_tol64; the final sweep's mesh phase, which the committed step uses, keeps
+// helmholtz_tol.
+constexpr double MESH_TOL32 = 1e-10;
+
+// More corrections than this (lmax above 40,000: a time step of many light crossings of a cell) and the
+// Helmholtz solves go through FP64 transforms.
+constexpr int HELM_MAX_CORRECTIONS = 8;
+
 // Rule of the cell table (576 B per cell, orbit_cell.cuh): from one particle per cell on.  Three
 // FP64 steps measured with the table | without it: 64^3 at 1 per cell 11.18 | 11.19 ms a step, at 4
 // 15.0 | 17.9, at 16 32.6 | 45.7; 128^3 at 1 68.7 | 72.8, at 16 314 | 454; 32^3 at 1 4.34 | 4.53.
@@ -398,6 +408,28 @@ pic_status allocate(pic_ctx* ctx) {
         c.helm_fft = ok;
     }
     if (c.helm_fft) {
+        // Corrections that bring an error of one below `to`: the FP32 transforms leave about 2^-22 of
+        // the residual, which is at most lmax times the error: 3 at 32^3 and 64^3 of the standard box,
+        // 4 at 128^3 (lmax 29), 6 at lmax 3000; the fields then match an exact FP64 update to 5e-16.
+        const double q = 2.5e-7 * c.cheb_lmax;
+        auto corrections = [&](double to) { return (int)std::ceil(std::log(to) / std::log(q)); };
+        c.helm_corrections = q < 1.0 ? corrections(1e-16) : HELM_MAX_CORRECTIONS + 1;
+        if (c.helm_corrections > HELM_MAX_CORRECTIONS) c.helm_corrections = 0;   // the FP64 transforms
+        else c.helm_corrections32 = std::max(1, corrections(MESH_TOL32));
+    }
+    if (c.helm_corrections > 0) {
+        std::vector<float2> tw;
+        std::vector<float> s2;
+        helm32_tables(c, tw, s2);
+        ALLOC(c.helm_z, float2, 2 * N);
+        ALLOC(c.helm_tw, float2, tw.size());
+        ALLOC(c.helm_s2f, float, s2.size());
+        ALLOC(c.helm_top, int, 8);
+        cudaMemcpyAsync(c.helm_tw, tw.data(), sizeof(float2) * tw.size(), cudaMemcpyHostToDevice, c.stream);
+        cudaMemcpyAsync(c.helm_s2f, s2.data(), sizeof(float) * s2.size(), cudaMemcpyHostToDevice, c.stream);
+        cudaMemsetAsync(c.helm_top, 0, 8 * sizeof(int), c.stream);
+        if (cudaStreamSynchronize(c.stream) != cudaSuccess) return check_cuda(ctx, "helmholtz tables");
+    } else if (c.helm_fft) {
         ALLOC(c.helm_spec, double2, 4 * N);
         ALLOC(c.helm_s2, double, c.m.n[0] + c.m.n[1] + c.m.n[2]);
         std::vector<double> s2;
@@ -416,7 +448,7 @@ pic_status allocate(pic_ctx* ctx) {
         ALLOC(c.specR, double2, 3 * N);
         ALLOC(c.spec_gphi, double, 3 * N);
     }
-    if (c.cfg.ops == PIC_OPS_SPECTRAL || c.helm_fft) {
+    if (c.cfg.ops == PIC_OPS_SPECTRAL || c.helm_spec) {
         for (int a = 0; a < 3; ++a) {
             fft_factor(c.m.n[a], c.fft_radix[a], c.fft_nst[a]);
             std::vector<double2> tw;
@@ -543,7 +575,10 @@ void mesh_phase(Ctx& c, const double* Jcur, const double* Jprev, double tol = 0.
         launch_spec_mesh_phase(c, Jcur, Jprev);
     } else {
         launch_source(c, Jcur, Jprev);
-        if (c.helm_fft) {
+        if (c.helm_corrections > 0) {
+            // to roundoff, but for the FP32 iterations' fields
+            launch_helm32(c, c.rhs, c.F1, c.helm_top, tol >= MESH_TOL32 ? c.helm_corrections32 : c.helm_corrections);
+        } else if (c.helm_fft) {
             launch_helmholtz_fft_refined(c, c.F1);   // to roundoff: the tolerance does not apply
         } else {
             launch_helmholtz_cn(c, &c.F1, &c.F1b, tol > 0.0 ? std::max(tol, c.cfg.helmholtz_tol) : c.cfg.helmholtz_tol);
@@ -553,11 +588,6 @@ void mesh_phase(Ctx& c, const double* Jcur, const double* Jprev, double tol = 0.
     if (cells && c.ctab) launch_cell_table(c);
 }
 
-// PIC_MIXED: the fields of an FP32 iteration need no more accuracy than its iterate has
-// (e_v >= ~1e-9), and those of an FP64 refinement iteration no more than a thousandth of
-// mixed_tol64; the final sweep's mesh phase, which the committed step uses, keeps
-// helmholtz_tol.
-constexpr double MESH_TOL32 = 1e-10;
 
 // ---- one time step as a sequence of issue / finish phases --------------------------------
 //
@@ -1350,7 +1380,12 @@ void adj_sweep(Ctx& c, const double* xi_n, const double* v_n, const double* vsta
     cudaMemsetAsync(c.adj_y, 0, sizeof(double) * 4 * N, c.stream);
     double* y = c.adj_y;
     double* ys = c.adj_ys;
-    launch_helmholtz(c, c.adj_t, 1.0, a, 4, c.cheb_iters, c.cheb_alpha, c.cheb_beta, &y, &ys);
+    if (c.helm_corrections > 0) {
+        launch_helm_exponents(c, c.adj_t, c.helm_top + 4);
+        launch_helm32(c, c.adj_t, y, c.helm_top + 4, c.helm_corrections);
+    } else {
+        launch_helmholtz(c, c.adj_t, 1.0, a, 4, c.cheb_iters, c.cheb_alpha, c.cheb_beta, &y, &ys);
+    }
     launch_adj_mesh_out(c, y, c.adj_pn, c.adj_W1, c.adj_rho1, c.adj_F0, c.adj_W0, c.adj_rho0, c.adj_J);
     if (c.np > 0)
         launch_adj_derivs(c, xi_n, v_n, vstar, c.adj_J, c.adj_P, c.adj_v, c.adj_xe, c.adj_mu, c.adj_xi, c.adj_g,

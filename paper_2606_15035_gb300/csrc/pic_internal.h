@@ -172,6 +172,13 @@ struct Ctx {
     bool helm_fft = false;
     double2* helm_spec = nullptr;
     double* helm_s2 = nullptr;
+    // ... by FP32 transforms and refinement (helm32.cu): corrections to roundoff and to the FP32
+    // iterations' accuracy (0: FP64 transforms), 2 N complex scratch, twiddles and symbols of the three
+    // axes, largest exponents of the right-hand sides (mesh phase | adjoint)
+    int helm_corrections = 0, helm_corrections32 = 0;
+    float2 *helm_z = nullptr, *helm_tw = nullptr;
+    float* helm_s2f = nullptr;
+    int* helm_top = nullptr;
     // deterministic mode: exact deposit accumulators (3 N each), their scales, creeping flags,
     // and the radix-sort work arrays
     long long *acc_hi = nullptr, *acc_lo = nullptr;
@@ -289,6 +296,10 @@ void launch_spec_energy(Ctx& c, const double* F, const double* W, int slot);
 void launch_spec_diag(Ctx& c, const double* Jfinal);
 void launch_spec_poisson(Ctx& c);
 void launch_helmholtz_fft(Ctx& c, const double* b, double* x, int nf, double a);
+// helm32.cu
+void helm32_tables(const Ctx& c, std::vector<float2>& tw, std::vector<float>& s2);
+void launch_helm_exponents(Ctx& c, const double* b, int* top);
+void launch_helm32(Ctx& c, const double* b, double* x, const int* top, int corrections);
 int radix_tiles(int64_t np);
 int push32_blocks(const Ctx& c);   // grid of the FP32 chunk kernels (partials per block)
 void launch_table32(Ctx& c);
