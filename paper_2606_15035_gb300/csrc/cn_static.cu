@@ -4,7 +4,7 @@
 // a fixed, pre-committed memory budget, host threads that must not enter the CUDA
 // allocator (it can synchronise the device), or plugins whose host application owns all
 // device allocations.  They pass device buffers for the inputs and outputs only; the
-// working storage (right-hand sides, Chebyshev iterates and directions) lives in one
+// working storage (right-hand sides, iterates, directions or transforms) lives in one
 // file-scope __device__ array of fixed size, which every device that loads this library
 // holds until the process exits.
 #include <cmath>
@@ -20,58 +20,71 @@ constexpr int STATIC_MAX_STEPS = 1024;   // Chebyshev steps one call may run
 static __device__ __align__(256) double g_cn_scratch[4 * 4 * STATIC_MAX_CELLS];
 
 struct Dims {
-    int n[3];
-    int64_t N;
+    int n[3], N;
     double invH[3];
 };
 
-__device__ __forceinline__ int wrap_index(int c, int n) {
-    int r = c % n;
-    return r < 0 ? r + n : r;
+// i + k wrapped onto [0, n) for |k| <= 2 (two conditional steps also cover n = 1)
+__device__ __forceinline__ int wrap2(int i, int n) {
+    if (i >= n) i -= n;
+    if (i >= n) i -= n;
+    if (i < 0) i += n;
+    if (i < 0) i += n;
+    return i;
 }
 
-__device__ __forceinline__ int64_t at(const Dims& d, int ix, int iy, int iz) {
-    return (int64_t)wrap_index(ix, d.n[0]) + (int64_t)d.n[0] * ((int64_t)wrap_index(iy, d.n[1]) +
-                                                                 (int64_t)d.n[1] * wrap_index(iz, d.n[2]));
-}
-
-// Delta_h f = sum_a (f[+2] - 2 f + f[-2]) / (4 H_a^2) at node (ix, iy, iz).
-__device__ __forceinline__ double lap_at(const double* __restrict__ f, const Dims& d, int ix, int iy, int iz) {
-    const double c = f[at(d, ix, iy, iz)];
-    return 0.25 * d.invH[0] * d.invH[0] * (f[at(d, ix + 2, iy, iz)] - 2.0 * c + f[at(d, ix - 2, iy, iz)]) +
-           0.25 * d.invH[1] * d.invH[1] * (f[at(d, ix, iy + 2, iz)] - 2.0 * c + f[at(d, ix, iy - 2, iz)]) +
-           0.25 * d.invH[2] * d.invH[2] * (f[at(d, ix, iy, iz + 2)] - 2.0 * c + f[at(d, ix, iy, iz - 2)]);
+// Delta_h f = sum_a (f[+2] - 2 f + f[-2]) / (4 H_a^2) at node g.
+__device__ __forceinline__ double lap_at(const double* __restrict__ f, const Dims& d, int g) {
+    const int t = (unsigned)g / (unsigned)d.n[0], ix = g - t * d.n[0];
+    const int iz = (unsigned)t / (unsigned)d.n[1], iy = t - iz * d.n[1];
+    const int sy = d.n[0], sz = d.n[0] * d.n[1];
+    const double c = f[g];
+    const double fx = f[g + wrap2(ix + 2, d.n[0]) - ix] - 2.0 * c + f[g + wrap2(ix - 2, d.n[0]) - ix];
+    const double fy = f[g + sy * (wrap2(iy + 2, d.n[1]) - iy)] - 2.0 * c + f[g + sy * (wrap2(iy - 2, d.n[1]) - iy)];
+    const double fz = f[g + sz * (wrap2(iz + 2, d.n[2]) - iz)] - 2.0 * c + f[g + sz * (wrap2(iz - 2, d.n[2]) - iz)];
+    return 0.25 * d.invH[0] * d.invH[0] * fx + 0.25 * d.invH[1] * d.invH[1] * fy + 0.25 * d.invH[2] * d.invH[2] * fz;
 }
 
 struct Fields4 {
     const double* f[4];
 };
 
-// rhs_f = (I + a Delta_h) F_f + dt W_f + c_f src_f and the warm start x_f = F_f.
+// rhs_f = (I + a Delta_h) F_f + dt W_f + c_f src_f and the warm start x_f = F_f.  With tw (the solve by
+// transforms): also the axes' twiddles and symbols, and top_f, the largest exponents of rhs_f and x_f.
 __global__ void k_static_rhs(Dims d, Fields4 F, Fields4 W, Fields4 src, double a, double dt, double c_rho, double c_J,
-                             double* __restrict__ rhs, double* __restrict__ x) {
-    const int f = blockIdx.y;
+                             double* __restrict__ rhs, double* __restrict__ x, float2* __restrict__ tw,
+                             float* __restrict__ s2, int* __restrict__ top) {
+    const int f = blockIdx.y, first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
     const double cf = f == 0 ? c_rho : c_J;
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < d.N; g += (int64_t)gridDim.x * blockDim.x) {
-        const int ix = (int)(g % d.n[0]);
-        const int64_t t = g / d.n[0];
-        const int iy = (int)(t % d.n[1]), iz = (int)(t / d.n[1]);
+    int e = 0;
+    for (int g = first; g < d.N; g += step) {
         const double u = F.f[f][g];
-        rhs[f * d.N + g] = u + a * lap_at(F.f[f], d, ix, iy, iz) + dt * W.f[f][g] + cf * src.f[f][g];
+        const double r = u + a * lap_at(F.f[f], d, g) + dt * W.f[f][g] + cf * src.f[f][g];
+        rhs[f * d.N + g] = r;
         x[f * d.N + g] = u;
+        e = max(e, max((__double2hiint(r) >> 20) & 0x7ff, (__double2hiint(u) >> 20) & 0x7ff));
     }
+    if (!tw) return;
+    e = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
+    if ((threadIdx.x & 31) == 0) atomicMax(top + f, e);
+    if (f == 0)
+        for (int t = first; t < d.n[0] + d.n[1] + d.n[2]; t += step) {
+            const int ax = t < d.n[0] ? 0 : (t < d.n[0] + d.n[1] ? 1 : 2);
+            const int i = t - (ax > 0 ? d.n[0] : 0) - (ax > 1 ? d.n[1] : 0);
+            double s, c;
+            sincospi(2.0 * i / d.n[ax], &s, &c);
+            tw[t] = make_float2((float)c, (float)-s);
+            s2[t] = (float)(s * s * d.invH[ax] * d.invH[ax]);
+        }
 }
 
 // One Chebyshev step of (I - a Delta_h) x = rhs (the recurrence of the library's solver).
 __global__ void k_static_cheb(Dims d, const double* __restrict__ x, double* __restrict__ xout, double* __restrict__ dir,
                               const double* __restrict__ rhs, double a, double alpha, double beta) {
-    const int64_t off = blockIdx.y * d.N;
+    const int off = blockIdx.y * d.N;
     const double* xf = x + off;
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < d.N; g += (int64_t)gridDim.x * blockDim.x) {
-        const int ix = (int)(g % d.n[0]);
-        const int64_t t = g / d.n[0];
-        const int iy = (int)(t % d.n[1]), iz = (int)(t / d.n[1]);
-        const double r = rhs[off + g] - (xf[g] - a * lap_at(xf, d, ix, iy, iz));
+    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < d.N; g += gridDim.x * blockDim.x) {
+        const double r = rhs[off + g] - (xf[g] - a * lap_at(xf, d, g));
         const double dn = (alpha == 0.0 ? 0.0 : alpha * dir[off + g]) + beta * r;
         dir[off + g] = dn;
         xout[off + g] = xf[g] + dn;
@@ -82,9 +95,9 @@ __global__ void k_static_cheb(Dims d, const double* __restrict__ x, double* __re
 __global__ void k_static_backsub(Dims d, Fields4 F, Fields4 W, const double* __restrict__ x, double dt, double* phi1,
                                  double* psi1, double* A1, double* U1) {
     const int f = blockIdx.y;
-    double* Fo = f == 0 ? phi1 : A1 + (int64_t)(f - 1) * d.N;
-    double* Wo = f == 0 ? psi1 : U1 + (int64_t)(f - 1) * d.N;
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < d.N; g += (int64_t)gridDim.x * blockDim.x) {
+    double* Fo = f == 0 ? phi1 : A1 + (f - 1) * d.N;
+    double* Wo = f == 0 ? psi1 : U1 + (f - 1) * d.N;
+    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < d.N; g += gridDim.x * blockDim.x) {
         const double u1 = x[f * d.N + g];
         Fo[g] = u1;
         Wo[g] = 2.0 * (u1 - F.f[f][g]) / dt - W.f[f][g];
@@ -115,7 +128,7 @@ extern "C" pic_status pic_cn_update_static(const int32_t n[3], const double L[3]
     if (!(dt > 0.0) || !(kappa > 0.0) || !(sigma1 > 0.0) || !(sigma2 > 0.0) || !(helmholtz_tol > 0.0))
         return PIC_ERR_ARG;
     Dims d;
-    d.N = N;
+    d.N = (int)N;
     double lmax = 1.0;
     const double a = 0.25 * kappa * kappa * dt * dt;
     for (int ax = 0; ax < 3; ++ax) {
@@ -160,14 +173,46 @@ extern "C" pic_status pic_cn_update_static(const int32_t n[3], const double L[3]
     Fields4 src = {{rho_half, J, J + N, J + 2 * N}};
     const double c_rho = 0.5 * dt * dt * kappa * kappa * sigma1;
     const double c_J = 0.5 * dt * dt * kappa * kappa * sigma2;
-    k_static_rhs<<<grid, 256, 0, s>>>(d, F, W, src, a, dt, c_rho, c_J, rhs, xa);
+    // By transforms on 2^p 3^q meshes where they are cheaper than the Chebyshev steps: a correction
+    // (five launches) costs about five steps, 23 against 4.6 us at 32^3.  The whole call at 32^3 with
+    // helmholtz_tol = 1e-17: 326 us by 30 steps (8.2 us each with 64-bit index divisions), 122 by transforms.
+    bool fft = true;
+    for (int ax = 0; ax < 3; ++ax) {
+        int radix[pic::FFT_MAX_STAGES], nst = 0;
+        fft = fft && pic::fft_factor(n[ax], radix, nst);
+    }
+    const int corrections = fft ? pic::helm32_corrections(lmax, std::fmax(helmholtz_tol, 1e-16)) : 0;
+    fft = corrections > 0 && iters > 5 * corrections;
+    // the transforms' buffers: z in place of the second iterate, the tables and exponents in the
+    // directions' place
+    float2* tw = fft ? reinterpret_cast<float2*>(dir) : nullptr;
+    float* s2 = reinterpret_cast<float*>(dir + 3 * pic::FFT_MAX);
+    int* top = reinterpret_cast<int*>(dir + 6 * pic::FFT_MAX);
+    static_assert(6 * pic::FFT_MAX + 2 <= 4 * STATIC_MAX_CELLS, "the tables fit the directions' place");
+    if (fft) cudaMemsetAsync(top, 0, 4 * sizeof(int), s);
+    k_static_rhs<<<grid, 256, 0, s>>>(d, F, W, src, a, dt, c_rho, c_J, rhs, xa, tw, s2, top);
     double* x = xa;
-    double* spare = xb;
-    for (int k = 0; k < iters; ++k) {
-        k_static_cheb<<<grid, 256, 0, s>>>(d, x, spare, dir, rhs, a, alpha[k], beta[k]);
-        double* t = x;
-        x = spare;
-        spare = t;
+    if (fft) {
+        pic::HelmPlan plan;
+        plan.m.ncell = N;
+        for (int ax = 0; ax < 3; ++ax) {
+            plan.m.n[ax] = n[ax];
+            plan.invH[ax] = d.invH[ax];
+        }
+        plan.a = a;
+        plan.sms = sms;
+        plan.z = reinterpret_cast<float2*>(xb);
+        plan.tw = tw;
+        plan.s2 = s2;
+        pic::helm32_solve(plan, rhs, x, top, corrections, s);
+    } else {
+        double* spare = xb;
+        for (int k = 0; k < iters; ++k) {
+            k_static_cheb<<<grid, 256, 0, s>>>(d, x, spare, dir, rhs, a, alpha[k], beta[k]);
+            double* t = x;
+            x = spare;
+            spare = t;
+        }
     }
     k_static_backsub<<<grid, 256, 0, s>>>(d, F, W, x, dt, phi1, psi1, A1, U1);
     if (cudaGetLastError() != cudaSuccess) return PIC_ERR_CUDA;

@@ -231,12 +231,12 @@ __global__ void k_exponents(int64_t N, const double* __restrict__ b, int* __rest
 
 unsigned multiplier(int d) { return d <= 1 ? 0u : (unsigned)((((uint64_t)1 << 32) + d - 1) / d); }
 
-Axis32 make_axis32(const Ctx& c, int a) {
+Axis32 make_axis32(const HelmPlan& c, int a) {
     Axis32 ax{};
     ax.axis = a;
     ax.n = c.m.n[a];
     ax.stride = a == 0 ? 1 : (a == 1 ? c.m.n[0] : (int64_t)c.m.n[0] * c.m.n[1]);
-    ax.tw = c.helm_tw + (a == 0 ? 0 : (a == 1 ? c.m.n[0] : c.m.n[0] + c.m.n[1]));
+    ax.tw = c.tw + (a == 0 ? 0 : (a == 1 ? c.m.n[0] : c.m.n[0] + c.m.n[1]));
     const int64_t run = a == 0 ? c.m.ncell / ax.n : (a == 1 ? c.m.n[0] : (int64_t)c.m.n[0] * c.m.n[1]);
     ax.lb = (int)std::max<int64_t>(1, std::min<int64_t>(run, ELEMS / ax.n));
     // few lines: a block for each part of them, so that the launch spreads over the SMs
@@ -277,18 +277,25 @@ void launch_helm_exponents(Ctx& c, const double* b, int* top) {
     ++c.launches;
 }
 
-void launch_helm32(Ctx& c, const double* b, double* x, const int* top, int corrections) {
+int helm32_corrections(double lmax, double to) {
+    const double q = 2.5e-7 * lmax;
+    if (!(q < 1.0)) return 0;
+    const double k = std::ceil(std::log(to) / std::log(q));
+    return k > HELM_MAX_CORRECTIONS ? 0 : std::max(1, (int)k);
+}
+
+int helm32_solve(const HelmPlan& c, const double* b, double* x, const int* top, int corrections, cudaStream_t stream) {
     Helm32 h;
     h.m = c.m;
     for (int a = 0; a < 3; ++a) h.invH[a] = c.invH[a];
-    h.a = 0.25 * c.cfg.kappa * c.cfg.kappa * c.cfg.dt * c.cfg.dt;
-    h.af = (float)h.a;
+    h.a = c.a;
+    h.af = (float)c.a;
     h.invN = (float)(1.0 / (double)c.m.ncell);
     h.b = b;
     h.x = x;
     h.top = top;
-    h.z = c.helm_z;
-    h.s2 = c.helm_s2f;
+    h.z = c.z;
+    h.s2 = c.s2;
     const Axis32 ax = make_axis32(c, 0), ay = make_axis32(c, 1), az = make_axis32(c, 2);
     auto grid = [&](int64_t groups) { return dim3((unsigned)std::min<int64_t>(groups, (int64_t)c.sms * 16), 2); };
     auto smem = [](const Axis32& q) { return 2 * sizeof(float2) * (size_t)q.lb * q.n; };
@@ -297,13 +304,25 @@ void launch_helm32(Ctx& c, const double* b, double* x, const int* top, int corre
     const dim3 gz = grid(((int64_t)c.m.n[0] * c.m.n[1] + az.lb - 1) / az.lb);
     for (int k = 0; k < corrections; ++k) {
         h.up = 20 * k;   // each correction leaves a residual some 2^20 smaller
-        k_helm_x<false><<<gx, 256, smem(ax), c.stream>>>(h, ax);
-        if (ay.n > 1) k_helm_yz<false, false><<<gy, 256, smem(ay), c.stream>>>(h, ay);
-        k_helm_yz<false, true><<<gz, 256, smem(az), c.stream>>>(h, az);
-        if (ay.n > 1) k_helm_yz<true, false><<<gy, 256, smem(ay), c.stream>>>(h, ay);
-        k_helm_x<true><<<gx, 256, smem(ax), c.stream>>>(h, ax);
-        c.launches += ay.n > 1 ? 5 : 3;
+        k_helm_x<false><<<gx, 256, smem(ax), stream>>>(h, ax);
+        if (ay.n > 1) k_helm_yz<false, false><<<gy, 256, smem(ay), stream>>>(h, ay);
+        k_helm_yz<false, true><<<gz, 256, smem(az), stream>>>(h, az);
+        if (ay.n > 1) k_helm_yz<true, false><<<gy, 256, smem(ay), stream>>>(h, ay);
+        k_helm_x<true><<<gx, 256, smem(ax), stream>>>(h, ax);
     }
+    return corrections * (ay.n > 1 ? 5 : 3);
+}
+
+void launch_helm32(Ctx& c, const double* b, double* x, const int* top, int corrections) {
+    HelmPlan p;
+    p.m = c.m;
+    for (int a = 0; a < 3; ++a) p.invH[a] = c.invH[a];
+    p.a = 0.25 * c.cfg.kappa * c.cfg.kappa * c.cfg.dt * c.cfg.dt;
+    p.sms = c.sms;
+    p.z = c.helm_z;
+    p.tw = c.helm_tw;
+    p.s2 = c.helm_s2f;
+    c.launches += helm32_solve(p, b, x, top, corrections, c.stream);
 }
 
 }  // namespace pic

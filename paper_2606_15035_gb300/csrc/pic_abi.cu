@@ -298,10 +298,6 @@ void setup_geometry(Ctx& c) {
 // helmholtz_tol.
 constexpr double MESH_TOL32 = 1e-10;
 
-// More corrections than this (lmax above 40,000: a time step of many light crossings of a cell) and the
-// Helmholtz solves go through FP64 transforms.
-constexpr int HELM_MAX_CORRECTIONS = 8;
-
 // Rule of the cell table (576 B per cell, orbit_cell.cuh): from one particle per cell on.  Three
 // FP64 steps measured with the table | without it: 64^3 at 1 per cell 11.18 | 11.19 ms a step, at 4
 // 15.0 | 17.9, at 16 32.6 | 45.7; 128^3 at 1 68.7 | 72.8, at 16 314 | 454; 32^3 at 1 4.34 | 4.53.
@@ -408,14 +404,8 @@ pic_status allocate(pic_ctx* ctx) {
         c.helm_fft = ok;
     }
     if (c.helm_fft) {
-        // Corrections that bring an error of one below `to`: the FP32 transforms leave about 2^-22 of
-        // the residual, which is at most lmax times the error: 3 at 32^3 and 64^3 of the standard box,
-        // 4 at 128^3 (lmax 29), 6 at lmax 3000; the fields then match an exact FP64 update to 5e-16.
-        const double q = 2.5e-7 * c.cheb_lmax;
-        auto corrections = [&](double to) { return (int)std::ceil(std::log(to) / std::log(q)); };
-        c.helm_corrections = q < 1.0 ? corrections(1e-16) : HELM_MAX_CORRECTIONS + 1;
-        if (c.helm_corrections > HELM_MAX_CORRECTIONS) c.helm_corrections = 0;   // the FP64 transforms
-        else c.helm_corrections32 = std::max(1, corrections(MESH_TOL32));
+        c.helm_corrections = helm32_corrections(c.cheb_lmax, 1e-16);
+        c.helm_corrections32 = helm32_corrections(c.cheb_lmax, MESH_TOL32);
     }
     if (c.helm_corrections > 0) {
         std::vector<float2> tw;

@@ -300,6 +300,24 @@ void launch_helmholtz_fft(Ctx& c, const double* b, double* x, int nf, double a);
 void helm32_tables(const Ctx& c, std::vector<float2>& tw, std::vector<float>& s2);
 void launch_helm_exponents(Ctx& c, const double* b, int* top);
 void launch_helm32(Ctx& c, const double* b, double* x, const int* top, int corrections);
+// The same without a context: a solve's constants and device buffers (z: 2 N; tw, s2: n0 + n1 + n2).
+struct HelmPlan {
+    MeshDims m;
+    double invH[3], a;
+    int sms;
+    float2* z;
+    const float2* tw;
+    const float* s2;
+};
+// More corrections than this (lmax above 40,000: a time step of many light crossings of a cell) and the
+// Helmholtz solves go through FP64 transforms.
+constexpr int HELM_MAX_CORRECTIONS = 8;
+// Corrections that bring an error of one below `to` (0: more than HELM_MAX_CORRECTIONS).  The FP32
+// transforms leave about 2^-22 of the residual, which is at most lmax times the error: 3 to roundoff at
+// 32^3 and 64^3 of the standard box, 4 at 128^3 (lmax 29), 6 at lmax 3000; the fields then match an
+// exact FP64 update to 5e-16.
+int helm32_corrections(double lmax, double to);
+int helm32_solve(const HelmPlan& c, const double* b, double* x, const int* top, int corrections, cudaStream_t stream);
 int radix_tiles(int64_t np);
 int push32_blocks(const Ctx& c);   // grid of the FP32 chunk kernels (partials per block)
 void launch_table32(Ctx& c);
