@@ -14,7 +14,7 @@
 #include <algorithm>
 
 #include "pic_internal.h"
-#include "orbit_cell.cuh"
+#include "orbit_fixed.cuh"
 
 namespace pic {
 namespace {
@@ -377,17 +377,20 @@ __global__ void k_backsub_table(MeshParams p, const double* __restrict__ F0, con
 
 // Cell table (orbit_cell.cuh) from the gather table: one thread per cell and column takes the
 // column's 8 node values to their mixed differences.  Writes 576 B a cell, 18 doubles apart per
-// thread with a cell's columns on neighbouring threads.
-__global__ void k_cell_table(MeshDims m, const double* __restrict__ table, double2* __restrict__ ctab) {
-    const int64_t total = m.ncell * CELL_COLS;
-    GRID_LOOP(idx, total) {
-        const int64_t cell = idx / CELL_COLS;
+// thread with a cell's columns on neighbouring threads.  Also the largest exponents of the two groups
+// that the fixed-point table scales by: the differences of the A columns, and -grad phi (top, zero
+// before).
+__global__ void k_cell_table(MeshDims m, const double* __restrict__ table, double2* __restrict__ ctab,
+                             int* __restrict__ top) {
+    const unsigned total = (unsigned)m.ncell * CELL_COLS;
+    unsigned eA = 0, eG = 0;
+    for (unsigned idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
+        const unsigned cell = idx / CELL_COLS, t = cell / (unsigned)m.n[0];
         const int col = (int)(idx - cell * CELL_COLS);
         int c[3];
-        c[0] = (int)(cell % m.n[0]);
-        const int64_t t = cell / m.n[0];
-        c[1] = (int)(t % m.n[1]);
-        c[2] = (int)(t / m.n[1]);
+        c[0] = (int)(cell - t * (unsigned)m.n[0]);
+        c[2] = (int)(t / (unsigned)m.n[1]);
+        c[1] = (int)t - c[2] * m.n[1];
         int64_t g[8];
         cell_nodes8(c, m, g);
         double f[8];
@@ -401,9 +404,45 @@ __global__ void k_cell_table(MeshDims m, const double* __restrict__ table, doubl
 #pragma unroll
             for (int k = 0; k < 8; ++k)
                 if (k & bit) f[k] -= f[k ^ bit];
+        unsigned e = 0;
+#pragma unroll
+        for (int k = 1; k < 8; ++k) e = max(e, (unsigned)exponent_of(f[k]));
+        if (col < 6) eA = max(eA, e);
+        else eG = max(eG, max(e, (unsigned)exponent_of(f[0])));
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            ctab[cell * (CELL_VALUES / 2) + q * CELL_COLS + col] = make_double2(f[2 * q], f[2 * q + 1]);
+            ctab[(int64_t)cell * (CELL_VALUES / 2) + q * CELL_COLS + col] = make_double2(f[2 * q], f[2 * q + 1]);
+    }
+    if (!top) return;
+    __shared__ unsigned sA, sG;
+    if (threadIdx.x == 0) sA = sG = 0;
+    __syncthreads();
+    eA = __reduce_max_sync(0xffffffffu, eA);
+    eG = __reduce_max_sync(0xffffffffu, eG);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&sA, eA);
+        atomicMax(&sG, eG);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        atomicMax(top, (int)sA);
+        atomicMax(top + 1, (int)sG);
+    }
+}
+
+// FP64 cell table -> fixed-point cell table (orbit_fixed.cuh).  The entries k = 0 of the A columns are
+// not used there.
+__global__ void k_cells_fixed(unsigned n, const double2* __restrict__ t64, longlong2* __restrict__ tfx,
+                              const int* __restrict__ top) {
+    const int eA = max(top[0], 64), eG = max(top[1], 64);
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const unsigned r = i % (CELL_VALUES / 2), p = r / CELL_COLS, col = r - p * CELL_COLS;
+        const double2 q = t64[i];
+        const int e = col < 6 ? eA : eG;
+        longlong2 o;
+        o.x = (p == 0 && col < 6) ? 0 : fixed_of(q.x, e, FX_FIELD_UP);
+        o.y = fixed_of(q.y, e, FX_FIELD_UP);
+        tfx[i] = o;
     }
 }
 
@@ -640,10 +679,19 @@ void launch_backsub_table(Ctx& c, bool) {
     ++c.launches;
 }
 
-void launch_cell_table(Ctx& c) {
-    const int64_t b = (c.m.ncell * CELL_COLS + THREADS - 1) / THREADS;
-    const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(b, (int64_t)c.sms * 16));
-    k_cell_table<<<nb, THREADS, 0, c.stream>>>(c.m, c.table, reinterpret_cast<double2*>(c.ctab));
+void launch_cell_table(Ctx& c, bool fixed) {
+    auto blocks = [&](int64_t n) {
+        return (int)std::max<int64_t>(1, std::min<int64_t>((n + THREADS - 1) / THREADS, (int64_t)c.sms * 16));
+    };
+    fixed = fixed && c.fxtab;
+    if (fixed) cudaMemsetAsync(c.cell_top, 0, 2 * sizeof(int), c.stream);
+    k_cell_table<<<blocks(c.m.ncell * CELL_COLS), THREADS, 0, c.stream>>>(
+        c.m, c.table, reinterpret_cast<double2*>(c.ctab), fixed ? c.cell_top : nullptr);
+    ++c.launches;
+    if (!fixed) return;
+    const int64_t n = c.m.ncell * (CELL_VALUES / 2);
+    k_cells_fixed<<<blocks(n), THREADS, 0, c.stream>>>((unsigned)n, reinterpret_cast<const double2*>(c.ctab),
+                                                       reinterpret_cast<longlong2*>(c.fxtab), c.cell_top);
     ++c.launches;
 }
 

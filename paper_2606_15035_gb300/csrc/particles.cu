@@ -11,6 +11,7 @@
 #include "particle_common.cuh"
 #include "orbit_cell.cuh"
 #include "chunk.cuh"
+#include "orbit_fixed.cuh"
 
 namespace pic {
 
@@ -785,28 +786,58 @@ __device__ __forceinline__ void push_eval(const StepParams& p, const double x0[3
     for (int a = 0; a < 3; ++a) o.vw[a] = (o.Pw[a] - p.q * o.Ae[a]) * p.inv_mass;
 }
 
-// G(u) from the cell table (closed forms, no diagnostics): the push of push_eval in the centred
-// form of orbit_cell.cuh, from the start (cell, coordinate) and vs = u + v^n = 2 vbar.
+// G(u) of the closed forms without diagnostics, from the start (cell, coordinate) and vs = u + v^n =
+// 2 vbar: in fixed point from the cell tables (FIXED), or from the gather table in FP64.
 struct CellOut {
     double Pw[3], Ae[3], vw[3];
     int nseg;
 };
 
-template <bool CELLS>
+struct CellFields {
+    const double* t64;        // FP64 cell table, or (not FIXED) the gather table
+    const longlong2* tfx;
+    const int* top;           // largest exponents of the fixed table's groups
+};
+
+template <bool FIXED>
 __device__ __forceinline__ void push_eval_cell(const StepParams& p, CellStart<double> st, const double vs[3],
-                                               const double Pn[3], const double* __restrict__ ctab, CellOut& o) {
-    double beta[3], acc[3] = {0.0, 0.0, 0.0};
+                                               const double Pn[3], const CellFields& cf, CellOut& o) {
+    double beta[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) beta[a] = p.cb[a] * vs[a];
-    o.nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
-        piece_impulse(h, sm, mid, beta, vs, p.ihs, FieldLoad<CELLS>(ctab, c, p.m), acc);
-    });
-    cell_A1(st.f, FieldLoad<CELLS>(ctab, st.c, p.m), o.Ae);
+    if constexpr (FIXED) {
+        const int ev = max(max(exponent_of(vs[0]), exponent_of(vs[1])), max(exponent_of(vs[2]), 64));
+        const int eA = max(__ldg(cf.top), 64), eG = max(__ldg(cf.top + 1), 64);
+        Fx v[3];
+        long long accF[3] = {0, 0, 0}, accG[3] = {0, 0, 0}, A1[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        o.Pw[a] = Pn[a] + p.dtq * acc[a];
-        o.vw[a] = (o.Pw[a] - p.q * o.Ae[a]) * p.inv_mass;
+        for (int a = 0; a < 3; ++a) v[a] = fx_split(fixed_of(vs[a], ev, FX_V_UP));
+        o.nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
+            const double d[3] = {h * beta[0], h * beta[1], h * beta[2]};
+            piece_impulse_fixed(h, sm, mid, d, v, FixedLoad(cf.tfx, c, p.m), accF, accG);
+        });
+        cell_A1_fixed(st.f, FixedLoad(cf.tfx, st.c, p.m), A1);
+        // values that are not finite stay so
+        const bool ok = max(ev, max(eA, eG)) < 2047;
+        const double uF = ok ? p.dtq * pow2_biased(eA + ev - 1078) : NAN;
+        const double uG = ok ? p.dtq * pow2_biased(eG - 56) : NAN, uA = pow2_biased(eA - 56);
+        const double* low = cf.t64 + CELL_VALUES * cell_row(st.c, p.m);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            o.Ae[a] = __ldg(low + 2 * a) + uA * (double)A1[a];
+            o.Pw[a] = Pn[a] + (uG * (double)accG[a] + uF * p.ihs[a] * (double)accF[a]);
+        }
+    } else {
+        double acc[3] = {0.0, 0.0, 0.0};
+        o.nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
+            piece_impulse(h, sm, mid, beta, vs, p.ihs, FieldLoad<false>(cf.t64, c, p.m), acc);
+        });
+        cell_A1(st.f, FieldLoad<false>(cf.t64, st.c, p.m), o.Ae);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) o.Pw[a] = Pn[a] + p.dtq * acc[a];
     }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) o.vw[a] = (o.Pw[a] - p.q * o.Ae[a]) * p.inv_mass;
 }
 
 // Blocks per SM of the scatter: 3 (80 registers, a few spills) measured 43.6 ms at 128^3 with 134M
@@ -853,21 +884,21 @@ __global__ void __launch_bounds__(THREADS, SCATTER_MINB) k_first_scatter_cell(
     write_partial<double>(partials, S_JSCALE, jsc, sm, false);
 }
 
-// The Algorithm 1 push for the closed forms without diagnostics: as k_push (below), from the
-// cell table (CELLS) or the gather table.
+// The Algorithm 1 push for the closed forms without diagnostics: as k_push (below), in fixed point
+// from the cell tables (FIXED) or in FP64 from the gather table.
 //
-// Bound by the FP64 pipe (one warp instruction in 16 clocks per SM), so what counts is the number of
-// FP64 instructions: the centred moments and the cell's mixed differences take 120 a piece where
-// node weights took 270 (57 against 88 for the scatter), and the walk, the creeping test and the
-// piece count compare on the integer pipe.  Measured at 32^3 with 2,097,152 particles (1.31 pieces
-// each): iterate 3.52 -> 1.59 ms (1.43 with the fixed-point deposit), final sweep 2.40 -> 1.11 ms;
-// 25.6M FP64 warp instructions (22.7M) where there were 58.2M, the pipe 83% busy (88% in the final
-// sweep).  Two blocks per SM (128 registers).
-template <bool COMMIT, bool CELLS>
+// It was bound by the FP64 pipe (one warp instruction in 16 clocks per SM), so the steps that made it
+// faster take instructions off that pipe.  Measured at 32^3 with 2,097,152 particles (1.31 pieces
+// each), iterate and final sweep: 3.52 and 2.40 ms from start-based integrals and node weights (58.2M
+// FP64 warp instructions in the iterate); 1.59 and 1.11 with centred moments and the cell's mixed
+// differences (25.6M); 1.43 with the fixed-point deposit; 1.22 and 0.77 with the fixed-point pieces
+// (11.4M and 9.0M, the pipe 52% and 62% busy).  At 128^3 with 134M particles the final sweep took 225,
+// 102 and now 66 ms.
+template <bool COMMIT, bool FIXED>
 __global__ void __launch_bounds__(THREADS, 2) k_push_cell(StepParams p, const double* __restrict__ xi,
                                                           const double* __restrict__ v, const double* __restrict__ P,
                                                           const double* __restrict__ vit,
-                                                          const double* __restrict__ ctab, double* __restrict__ vnew,
+                                                          CellFields cf, double* __restrict__ vnew,
                                                           double* __restrict__ Jnext, double* __restrict__ xi_out,
                                                           double* __restrict__ P_out,
                                                           int32_t* __restrict__ creep_list,
@@ -903,7 +934,7 @@ __global__ void __launch_bounds__(THREADS, 2) k_push_cell(StepParams p, const do
 #pragma unroll
                 for (int a = 0; a < 3; ++a) Pn[a] = P[a * np + i];
                 CellOut o;
-                push_eval_cell<CELLS>(p, st, vs, Pn, ctab, o);
+                push_eval_cell<FIXED>(p, st, vs, Pn, cf, o);
                 if (o.nseg < 0) atomicOr(status, DEV_ERR_SEGMENTS);
                 pieces_push += o.nseg;
                 if (!(isfinite(o.vw[0]) && isfinite(o.vw[1]) && isfinite(o.vw[2]))) atomicOr(status, DEV_ERR_NONFINITE);
@@ -1996,16 +2027,17 @@ void launch_push(Ctx& c, const double* vit, double* vnew, double* Jnext, bool co
                                                   c.creep_list, c.creep_count, det ? c.creep_flag : nullptr,  \
                                                   c.slide,                                                    \
                                                   c.partials, c.dev_status)
+    const CellFields cf{c.fxtab ? c.ctab : c.table, reinterpret_cast<const longlong2*>(c.fxtab), c.cell_top};
 #define PIC_PUSH_CELL(C, T)                                                                                       \
-    k_push_cell<C, T><<<nb, THREADS, C ? sizeof(ChunkOrder) : CHUNK_SMEM, c.stream>>>(p, c.xi, c.v, c.P, vit, T ? c.ctab : c.table, vnew, Jnext,     \
+    k_push_cell<C, T><<<nb, THREADS, C ? sizeof(ChunkOrder) : CHUNK_SMEM, c.stream>>>(p, c.xi, c.v, c.P, vit, cf, vnew, Jnext,     \
                                                     c.xi_new, c.P_new, c.creep_list, c.creep_count,                \
                                                     det ? c.creep_flag : nullptr, c.slide, c.partials, c.dev_status)
     if (closed && !diag) {
         if (commit) {
-            if (c.ctab) PIC_PUSH_CELL(true, true);
+            if (c.fxtab) PIC_PUSH_CELL(true, true);
             else PIC_PUSH_CELL(true, false);
         } else {
-            if (c.ctab) PIC_PUSH_CELL(false, true);
+            if (c.fxtab) PIC_PUSH_CELL(false, true);
             else PIC_PUSH_CELL(false, false);
         }
     } else if (!commit) {

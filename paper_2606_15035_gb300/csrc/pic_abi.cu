@@ -45,19 +45,21 @@ void* dev_alloc_once(pic_ctx* ctx, size_t bytes) {
     return p;
 }
 
-// Give the optional cell table back (between calls: the kernels then read the gather table).
+// Give the optional cell tables back (between calls: the kernels then read the gather table).
 bool drop_cell_table(pic_ctx* ctx) {
     Ctx& c = ctx->c;
     if (!c.ctab) return false;
     cudaStreamSynchronize(c.stream);
-    for (size_t k = 0; k < ctx->allocs.size(); ++k) {
-        if (ctx->allocs[k].first != c.ctab) continue;
-        if (c.has_alloc) c.alloc.free(c.ctab, ctx->allocs[k].second, (void*)c.stream, c.alloc.user);
-        else cudaFree(c.ctab);
-        ctx->allocs.erase(ctx->allocs.begin() + (long)k);
-        break;
-    }
+    for (void* t : {(void*)c.ctab, (void*)c.fxtab})
+        for (size_t k = 0; t && k < ctx->allocs.size(); ++k) {
+            if (ctx->allocs[k].first != t) continue;
+            if (c.has_alloc) c.alloc.free(t, ctx->allocs[k].second, (void*)c.stream, c.alloc.user);
+            else cudaFree(t);
+            ctx->allocs.erase(ctx->allocs.begin() + (long)k);
+            break;
+        }
     c.ctab = nullptr;
+    c.fxtab = nullptr;
     c.pair_cells = false;   // its buffer is large enough for the pairs of the gather table
     return true;
 }
@@ -451,6 +453,7 @@ pic_status allocate(pic_ctx* ctx) {
     ALLOC(c.partials, double, (size_t)NSLOT * MAX_BLOCKS);
     ALLOC(c.results, double, NSLOT);
     ALLOC(c.dev_status, int, 1);
+    ALLOC(c.cell_top, int, 2);
     if (cudaMallocHost(&c.host_results, sizeof(double) * NSLOT) != cudaSuccess ||
         cudaMallocHost(&c.host_status, sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
@@ -461,7 +464,9 @@ pic_status allocate(pic_ctx* ctx) {
     const size_t cells = sizeof(double) * CELL_VALUES * (size_t)N;
     if (c.closed && c.np >= CELL_TABLE_MIN_PPC * N && cells <= CELL_TABLE_MAX_BYTES) {
         c.ctab = (double*)dev_alloc_once(ctx, cells);
-        if (c.ctab && reinterpret_cast<uintptr_t>(c.ctab) % 16 != 0) drop_cell_table(ctx);
+        if (c.ctab) c.fxtab = (long long*)dev_alloc_once(ctx, cells);
+        if (c.ctab && (!c.fxtab || (reinterpret_cast<uintptr_t>(c.ctab) | reinterpret_cast<uintptr_t>(c.fxtab)) % 16 != 0))
+            drop_cell_table(ctx);
     }
     if (c.cfg.precision == PIC_MIXED && c.cfg.mixed_pair_max > 0 && !c.cfg.deterministic) {
         if (c.ctab) c.table_pair = (float*)dev_alloc_once(ctx, cells);
@@ -575,7 +580,7 @@ void mesh_phase(Ctx& c, const double* Jcur, const double* Jprev, double tol = 0.
         }
         launch_backsub_table(c, false);
     }
-    if (cells && c.ctab) launch_cell_table(c);
+    if (cells && c.ctab) launch_cell_table(c, true);
 }
 
 

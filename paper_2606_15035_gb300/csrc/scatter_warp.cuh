@@ -11,6 +11,7 @@
 // transposed shared tile, turned into node weights by three exchanges, and added to J once.
 #pragma once
 
+#include "fixed.cuh"
 #include "orbit_cell.cuh"
 
 namespace pic {
@@ -18,31 +19,6 @@ namespace pic {
 constexpr int DEPOSIT_ROWS = 24;
 constexpr int DEPOSIT_STRIDE = 33;   // 33 x 8 B: a row's lanes and a column's rows miss each other's banks
 constexpr int DEPOSIT_TILE = DEPOSIT_ROWS * DEPOSIT_STRIDE;   // 64-bit words per warp
-
-// x times 2^s truncated to an integer, |x| 2^s < 2^63: `drop` is how far the exponent of x is below
-// the one whose mantissa is shifted left by `up`.
-__device__ __forceinline__ long long fixed_of(double x, int top, int up) {
-    const int hi = __double2hiint(x);
-    const int drop = min(max(top - ((hi >> 20) & 0x7ff), 0), 63);
-    const unsigned long long mant =
-        ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(x);
-    const long long r = (long long)((mant << up) >> drop);
-    return hi < 0 ? -r : r;
-}
-
-// A factor: its signed high word and the upper 31 bits of its low word.
-struct Fx {
-    int h, l;
-};
-
-__device__ __forceinline__ Fx fx_split(long long v) { return Fx{(int)(v >> 32), (int)((unsigned)v >> 1)}; }
-
-// a b 2^-62 from three 32 x 32 products; the constant stands for the mean of the dropped low product
-// and rounds (errors within about 2 units, mean below a quarter).
-__device__ __forceinline__ long long fx_mul(Fx a, Fx b) {
-    const long long u = (long long)a.h * b.l + ((long long)a.l * b.h + 912680550LL);   // 1.7 x 2^29
-    return (((long long)a.h * b.h) << 2) + (u >> 29);
-}
 
 // Measured at 32^3 with 2,097,152 particles (1.31 pieces each): the first scatter 0.82 -> 0.49 ms with
 // 4.5M L2 reduction requests where there were 67M; at 128^3 with 134M (2.2 pieces) 96 -> 44 ms.
