@@ -344,7 +344,7 @@ __global__ void k_adj_mesh_out(AdjParams ap, const double* __restrict__ y, const
 // particles.
 
 template <bool CELLS>
-__global__ void __launch_bounds__(THREADS, 2) k_adj_derivs(AdjParams ap, const double* __restrict__ xi,
+__global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_derivs(AdjParams ap, const double* __restrict__ xi,
                                                            const double* __restrict__ v,
                                                            const double* __restrict__ vstar,
                                                            const double* __restrict__ table,
@@ -357,22 +357,24 @@ __global__ void __launch_bounds__(THREADS, 2) k_adj_derivs(AdjParams ap, const d
                                                            double* __restrict__ lam_xi, double* __restrict__ gout,
                                                            double* __restrict__ lvn, double* __restrict__ lPn,
                                                            int* __restrict__ status) {
-    __shared__ ChunkOrder co;
+    __shared__ ChunkLarge co;
     const StepParams& p = ap.p;
-    const int64_t np = p.np, N = p.m.ncell, nchunks = (np + THREADS - 1) / THREADS;
+    const int64_t np = p.np, N = p.m.ncell, nchunks = (np + ChunkLarge::SIZE - 1) / ChunkLarge::SIZE;
     for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-        const int64_t base = ch * THREADS, j = base + threadIdx.x;
-        double x0[3], v2[3], vs[3];
-        CellStart<double> st;
-        if (j < np) {
+        const int64_t base = ch * ChunkLarge::SIZE;
+        chunk_exchange(p, co, base, [&](int64_t j, double x0[3], double v2[3]) {
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 x0[a] = xi[a * np + j];
                 v2[a] = vstar[a * np + j] + v[a * np + j];
             }
-        }
-        const int64_t i = chunk_exchange(p, co, base, j < np, x0, v2, st, vs);
-        if (i < np) {
+        });
+#pragma unroll 1
+        for (int item = 0; item < 2; ++item) {
+            CellStart<double> st;
+            double vs[3];
+            const int64_t i = co.take(item, base, st, vs);
+            if (i >= np) continue;
             const uint8_t sb = slide[i];
             double beta[3], f[3], ng[3], xbar[3], bbar[3], vbar[3];
 #pragma unroll
@@ -824,7 +826,7 @@ void launch_adj_derivs(Ctx& c, const double* xi, const double* v, const double* 
                        double* lam_xi, double* g, double* lvn, double* lPn) {
     const int nb = adj_blocks(c, c.np);
 #define PIC_DERIVS(T, TAB)                                                                                        \
-    k_adj_derivs<T><<<nb, THREADS, 0, c.stream>>>(adj_params(c), xi, v, vstar, TAB, lJ, lam_P, lam_v, lam_xe, mu,    \
+    k_adj_derivs<T><<<nb, ChunkLarge::THREADS_, 0, c.stream>>>(adj_params(c), xi, v, vstar, TAB, lJ, lam_P, lam_v, lam_xe, mu,    \
                                                   c.slide, lam_xi, g, lvn, lPn, c.dev_status)
     if (c.ctab) PIC_DERIVS(true, c.ctab);
     else PIC_DERIVS(false, c.table);

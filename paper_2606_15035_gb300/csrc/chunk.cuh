@@ -1,5 +1,5 @@
-// A chunk of THREADS cell-sorted particles in the closed-form particle kernels: their hand-over to the
-// threads in order of orbit-piece count, and the local-solve gates on cell coordinates.
+// A chunk of cell-sorted particles in the closed-form particle kernels: their hand-over to the threads
+// in order of orbit-piece count, and the local-solve gates on cell coordinates.
 #pragma once
 
 #include "orbit_cell.cuh"
@@ -8,54 +8,99 @@
 
 namespace pic {
 
-// Shared-memory hand-over of a chunk's particles to the threads in order of orbit-piece count:
-// what the ranking computed (cell, coordinate, v^{p} + v^n) travels with the particle.
+// Shared-memory hand-over of a chunk's particles to the threads in order of orbit-piece count, so that
+// the lanes of a warp run the same number of pieces: what the ranking computed (cell, coordinate, v^{p}
+// + v^n) travels with the particle.  A block of WARPS warps takes chunks of 32 WARPS ITEMS particles;
+// with two items a warp takes one group from each end of the order, so that the block's warps have
+// about equal work and wait little at the chunk's barriers (with one group of 32 per warp, eight warps
+// a block, barriers were the first stall reason).
+template <int WARPS, int ITEMS>
 struct ChunkOrder {
-    int order[THREADS];
-    int wcount[THREADS / 32][PIECE_CLASSES];
-    double f[3][THREADS], vs[3][THREADS];
-    int c[3][THREADS];
+    static constexpr int THREADS_ = 32 * WARPS, GROUPS = WARPS * ITEMS, SIZE = THREADS_ * ITEMS;
+    int order[SIZE];
+    int wcount[GROUPS][PIECE_CLASSES];
+    double f[3][SIZE], vs[3][SIZE];
+    int c[3][SIZE];
+
+    // Dynamic shared memory of a kernel that also deposits: the hand-over and one tile per warp.
+    static constexpr size_t smem() { return sizeof(ChunkOrder) + sizeof(long long) * DEPOSIT_TILE * WARPS; }
+    static __device__ __forceinline__ ChunkOrder& in(unsigned char* dyn) { return *reinterpret_cast<ChunkOrder*>(dyn); }
+    static __device__ __forceinline__ long long* tile(unsigned char* dyn) {
+        return reinterpret_cast<long long*>(dyn + sizeof(ChunkOrder)) + (threadIdx.x >> 5) * DEPOSIT_TILE;
+    }
+
+    // The place of this thread's item `it` in the order; its particle's data and index (>= np: none).
+    __device__ __forceinline__ int64_t take(int it, int64_t base, CellStart<double>& st, double v[3]) const {
+        const int w = threadIdx.x >> 5, s = 32 * (it == 0 ? w : GROUPS - 1 - w) + (threadIdx.x & 31);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            st.f[a] = f[a][s];
+            v[a] = vs[a][s];
+            st.c[a] = c[a][s];
+        }
+        return base + order[s];
+    }
 };
 
-// Dynamic shared memory of the kernels that also deposit: the hand-over and one tile per warp.
-constexpr size_t CHUNK_SMEM = sizeof(ChunkOrder) + sizeof(long long) * DEPOSIT_TILE * (THREADS / 32);
+// The chunk sizes: four warps with two groups each, or, for runs too small to fill the SMs that way,
+// one group per block.
+typedef ChunkOrder<4, 2> ChunkLarge;
+typedef ChunkOrder<1, 1> ChunkSmall;
 
 // Knots crossed by an axis whose orbit ends at te (relative to its start cell).
 __device__ __forceinline__ unsigned crossings(double te) {
     return (at_least_one(te) || below_zero(te)) ? min((unsigned)abs(__double2int_rd(te)), 3u) : 0u;
 }
 
-// Rank the chunk's particles by piece count and hand them over; ends with a barrier.  Returns the
-// index of this thread's particle (>= np: none).
-__device__ __forceinline__ int64_t chunk_exchange(const StepParams& p, ChunkOrder& co, int64_t base, bool valid,
-                                                  const double x0[3], const double v2[3], CellStart<double>& st,
-                                                  double vs[3]) {
-    int cls = PIECE_CLASSES - 1;
-    if (valid) {
-        cell_start(x0, p.m, st);
-        unsigned pieces = 1;
+// Rank the chunk's particles by piece count (a stable order) and hand them over; ends with a barrier.
+// load(j, x0, v2) gives particle j's position and v^{p} + v^n.
+template <int WARPS, int ITEMS, typename L>
+__device__ __forceinline__ void chunk_exchange(const StepParams& p, ChunkOrder<WARPS, ITEMS>& co, int64_t base,
+                                               L&& load) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    CellStart<double> st[ITEMS];
+    double v2[ITEMS][3];
+    int cls[ITEMS];
+    unsigned mine[ITEMS];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) pieces += crossings(st.f[a] + p.cb[a] * v2[a]);
-        cls = (int)min(pieces, (unsigned)(PIECE_CLASSES - 1)) - 1;
-    }
-    const int r = stable_class_rank(cls, co.wcount);
-    co.order[r] = threadIdx.x;
-    if (valid) {
+    for (int it = 0; it < ITEMS; ++it) {
+        const int64_t j = base + it * 32 * WARPS + threadIdx.x;
+        cls[it] = PIECE_CLASSES - 1;
+        mine[it] = 0;
+        if (j < p.np) {
+            double x0[3];
+            load(j, x0, v2[it]);
+            cell_start(x0, p.m, st[it]);
+            unsigned pieces = 1;
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            co.f[a][r] = st.f[a];
-            co.vs[a][r] = v2[a];
-            co.c[a][r] = st.c[a];
+            for (int a = 0; a < 3; ++a) pieces += crossings(st[it].f[a] + p.cb[a] * v2[it][a]);
+            cls[it] = (int)min(pieces, (unsigned)(PIECE_CLASSES - 1)) - 1;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < PIECE_CLASSES; ++c) {
+            const unsigned m = __ballot_sync(0xffffffffu, cls[it] == c);
+            if (lane == 0) co.wcount[it * WARPS + w][c] = __popc(m);
+            if (cls[it] == c) mine[it] = m;
         }
     }
     __syncthreads();
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        st.f[a] = co.f[a][threadIdx.x];
-        vs[a] = co.vs[a][threadIdx.x];
-        st.c[a] = co.c[a][threadIdx.x];
+    for (int it = 0; it < ITEMS; ++it) {
+        int r = __popc(mine[it] & ((1u << lane) - 1u));
+        for (int c = 0; c < cls[it]; ++c)
+#pragma unroll
+            for (int v = 0; v < WARPS * ITEMS; ++v) r += co.wcount[v][c];
+        for (int v = 0; v < it * WARPS + w; ++v) r += co.wcount[v][cls[it]];
+        co.order[r] = it * 32 * WARPS + threadIdx.x;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            co.f[a][r] = st[it].f[a];
+            co.vs[a][r] = v2[it][a];
+            co.c[a][r] = st[it].c[a];
+        }
     }
-    return base + co.order[threadIdx.x];
+    __syncthreads();
 }
 
 // is_creeping from the start's cell coordinate: on an axis with |beta| < BETA_CREEP, does twice

@@ -808,10 +808,10 @@ __device__ __forceinline__ void push_eval_cell(const StepParams& p, CellStart<do
     if constexpr (FIXED) {
         const int ev = max(max(exponent_of(vs[0]), exponent_of(vs[1])), max(exponent_of(vs[2]), 64));
         const int eA = max(__ldg(cf.top), 64), eG = max(__ldg(cf.top + 1), 64);
-        Fx v[3];
+        Fs v[3];
         long long accF[3] = {0, 0, 0}, accG[3] = {0, 0, 0}, A1[3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) v[a] = fx_split(fixed_of(vs[a], ev, FX_V_UP));
+        for (int a = 0; a < 3; ++a) v[a] = fs_of(fixed_of(vs[a], ev, FX_V_UP));
         o.nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
             const double d[3] = {h * beta[0], h * beta[1], h * beta[2]};
             piece_impulse_fixed(h, sm, mid, d, v, FixedLoad(cf.tfx, c, p.m), accF, accG);
@@ -819,8 +819,8 @@ __device__ __forceinline__ void push_eval_cell(const StepParams& p, CellStart<do
         cell_A1_fixed(st.f, FixedLoad(cf.tfx, st.c, p.m), A1);
         // values that are not finite stay so
         const bool ok = max(ev, max(eA, eG)) < 2047;
-        const double uF = ok ? p.dtq * pow2_biased(eA + ev - 1078) : NAN;
-        const double uG = ok ? p.dtq * pow2_biased(eG - 56) : NAN, uA = pow2_biased(eA - 56);
+        const double uF = ok ? p.dtq * pow2_biased(eA + ev - 1079) : NAN;
+        const double uG = ok ? p.dtq * pow2_biased(eG - 57) : NAN, uA = pow2_biased(eA - 57);
         const double* low = cf.t64 + CELL_VALUES * cell_row(st.c, p.m);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
@@ -840,26 +840,28 @@ __device__ __forceinline__ void push_eval_cell(const StepParams& p, CellStart<do
     for (int a = 0; a < 3; ++a) o.vw[a] = (o.Pw[a] - p.q * o.Ae[a]) * p.inv_mass;
 }
 
-// Blocks per SM of the scatter: 3 (80 registers, a few spills) measured 43.6 ms at 128^3 with 134M
-// particles, 2 (128 registers) 46.0, 4 (64) 48.5.
-constexpr int SCATTER_MINB = 3;
+// Warps per SM that the kernels are compiled for.  First scatter: 16 (128 registers) measured 37.2 ms at
+// 128^3 with 134M particles, 20 38.7, 24 42.3.  Push: 16 measured 1.13 ms (iterate, 32^3, 2,097,152
+// particles), 20 (102 registers, more spills) 1.26, 12 1.29.
+constexpr int SCATTER_WARPS = 16;
+constexpr int PUSH_WARPS = 16;
 
 // k_first_scatter for the closed forms.
-__global__ void __launch_bounds__(THREADS, SCATTER_MINB) k_first_scatter_cell(
+template <int WARPS, int ITEMS>
+__global__ void __launch_bounds__(32 * WARPS, SCATTER_WARPS / WARPS) k_first_scatter_cell(
     StepParams p, const double* __restrict__ xi, const double* __restrict__ v, const double* __restrict__ vprev,
     const double* __restrict__ vgiven, double* __restrict__ vit, double* __restrict__ J, double* __restrict__ partials,
     int* __restrict__ status) {
+    typedef ChunkOrder<WARPS, ITEMS> Chunk;
     __shared__ double sm[32];
     extern __shared__ __align__(16) unsigned char dyn[];
-    ChunkOrder& co = *reinterpret_cast<ChunkOrder*>(dyn);
-    long long* tile = reinterpret_cast<long long*>(dyn + sizeof(ChunkOrder)) + (threadIdx.x >> 5) * DEPOSIT_TILE;
-    const int64_t np = p.np, nchunks = (np + THREADS - 1) / THREADS;
+    Chunk& co = Chunk::in(dyn);
+    long long* tile = Chunk::tile(dyn);
+    const int64_t np = p.np, nchunks = (np + Chunk::SIZE - 1) / Chunk::SIZE;
     double jsc = 0.0;
     for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-        const int64_t base = ch * THREADS, j = base + threadIdx.x;
-        double x0[3], v2[3], vs[3];
-        CellStart<double> st;
-        if (j < np) {
+        const int64_t base = ch * Chunk::SIZE;
+        chunk_exchange(p, co, base, [&](int64_t j, double x0[3], double v2[3]) {
             double vn[3];
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
@@ -870,15 +872,19 @@ __global__ void __launch_bounds__(THREADS, SCATTER_MINB) k_first_scatter_cell(
                 v2[a] = vi + vn[a];
             }
             jsc += sqrt(vn[0] * vn[0] + vn[1] * vn[1] + vn[2] * vn[2]);
-        }
-        const int64_t i = chunk_exchange(p, co, base, j < np, x0, v2, st, vs);
-        double beta[3], w[3];
+        });
+#pragma unroll 1
+        for (int it = 0; it < ITEMS; ++it) {
+            CellStart<double> st;
+            double vs[3], beta[3], w[3];
+            const int64_t i = co.take(it, base, st, vs);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            beta[a] = p.cb[a] * vs[a];
-            w[a] = p.q_dV_half * vs[a];
+            for (int a = 0; a < 3; ++a) {
+                beta[a] = p.cb[a] * vs[a];
+                w[a] = p.q_dV_half * vs[a];
+            }
+            if (scatter_warp(p.m, i < np, st, beta, w, tile, p.det, p.acc, J) < 0) atomicOr(status, DEV_ERR_SEGMENTS);
         }
-        if (scatter_warp(p.m, i < np, st, beta, w, tile, p.det, p.acc, J) < 0) atomicOr(status, DEV_ERR_SEGMENTS);
         __syncthreads();   // the hand-over buffers are rewritten by the next chunk
     }
     write_partial<double>(partials, S_JSCALE, jsc, sm, false);
@@ -892,10 +898,10 @@ __global__ void __launch_bounds__(THREADS, SCATTER_MINB) k_first_scatter_cell(
 // each), iterate and final sweep: 3.52 and 2.40 ms from start-based integrals and node weights (58.2M
 // FP64 warp instructions in the iterate); 1.59 and 1.11 with centred moments and the cell's mixed
 // differences (25.6M); 1.43 with the fixed-point deposit; 1.22 and 0.77 with the fixed-point pieces
-// (11.4M and 9.0M, the pipe 52% and 62% busy).  At 128^3 with 134M particles the final sweep took 225,
-// 102 and now 66 ms.
-template <bool COMMIT, bool FIXED>
-__global__ void __launch_bounds__(THREADS, 2) k_push_cell(StepParams p, const double* __restrict__ xi,
+// (11.4M and 9.0M, the pipe 52% and 62% busy); 1.13 and 0.73 with chunks whose warps have equal work and
+// sums of products shifted once.  At 128^3 with 134M particles the final sweep took 225, 102, now 64 ms.
+template <bool COMMIT, bool FIXED, int WARPS, int ITEMS>
+__global__ void __launch_bounds__(32 * WARPS, PUSH_WARPS / WARPS) k_push_cell(StepParams p, const double* __restrict__ xi,
                                                           const double* __restrict__ v, const double* __restrict__ P,
                                                           const double* __restrict__ vit,
                                                           CellFields cf, double* __restrict__ vnew,
@@ -908,25 +914,26 @@ __global__ void __launch_bounds__(THREADS, 2) k_push_cell(StepParams p, const do
                                                           double* __restrict__ partials, int* __restrict__ status) {
     __shared__ double sm[32];
     extern __shared__ __align__(16) unsigned char dyn[];
-    ChunkOrder& co = *reinterpret_cast<ChunkOrder*>(dyn);
-    long long* tile = reinterpret_cast<long long*>(dyn + sizeof(ChunkOrder)) + (threadIdx.x >> 5) * DEPOSIT_TILE;
-    const int64_t np = p.np, nchunks = (np + THREADS - 1) / THREADS;
+    typedef ChunkOrder<WARPS, ITEMS> Chunk;
+    Chunk& co = Chunk::in(dyn);
+    long long* tile = Chunk::tile(dyn);
+    const int64_t np = p.np, nchunks = (np + Chunk::SIZE - 1) / Chunk::SIZE;
     double ev_num = 0.0, ev_den = 0.0;
     long long pieces_push = 0, pieces_scatter = 0;
     for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-        const int64_t base = ch * THREADS, j = base + threadIdx.x;
-        double x0[3], vs[3];
-        CellStart<double> st;
-        {
-            double v2[3];
-            if (j < np) {
+        const int64_t base = ch * Chunk::SIZE;
+        chunk_exchange(p, co, base, [&](int64_t j, double x0[3], double v2[3]) {
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    x0[a] = xi[a * np + j];
-                    v2[a] = vit[a * np + j] + v[a * np + j];
-                }
+            for (int a = 0; a < 3; ++a) {
+                x0[a] = xi[a * np + j];
+                v2[a] = vit[a * np + j] + v[a * np + j];
             }
-            const int64_t i = chunk_exchange(p, co, base, j < np, x0, v2, st, vs);
+        });
+#pragma unroll 1
+        for (int it = 0; it < ITEMS; ++it) {
+            CellStart<double> st;
+            double vs[3];
+            const int64_t i = co.take(it, base, st, vs);
             bool scat = false;               // this lane's next orbit is scattered here
             double bn[3] = {0.0, 0.0, 0.0}, w[3] = {0.0, 0.0, 0.0};
             if (i < np) {
@@ -1960,15 +1967,27 @@ StepParams make_params(const Ctx& c) {
     return p;
 }
 
-// Opt the depositing kernels in to their dynamic shared memory (above the 48 KB default; once per
-// context, on its device).
+// Opt the depositing kernels in to their dynamic shared memory (above the 48 KB default where the chunk
+// is large; once per context, on its device).
 bool setup_particle_kernels() {
-    const int bytes = (int)CHUNK_SMEM;
+    const int bytes = (int)ChunkLarge::smem();
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    return cudaFuncSetAttribute(k_first_scatter_cell, at, bytes) == cudaSuccess &&
-           cudaFuncSetAttribute(k_push_cell<false, true>, at, bytes) == cudaSuccess &&
-           cudaFuncSetAttribute(k_push_cell<false, false>, at, bytes) == cudaSuccess;
+    return cudaFuncSetAttribute(k_first_scatter_cell<4, 2>, at, bytes) == cudaSuccess &&
+           cudaFuncSetAttribute(k_push_cell<false, true, 4, 2>, at, bytes) == cudaSuccess &&
+           cudaFuncSetAttribute(k_push_cell<false, false, 4, 2>, at, bytes) == cudaSuccess;
 }
+
+// Chunks of one warp while they leave every scheduler at most two of them.
+bool small_chunks(const Ctx& c) { return c.np <= (int64_t)c.sms * 8 * ChunkSmall::SIZE; }
+
+// Grid of the kernels that walk chunks, and of the push of this context's kind (partials per block).
+int chunk_blocks(const Ctx& c) {
+    const int size = small_chunks(c) ? ChunkSmall::SIZE : ChunkLarge::SIZE;
+    const int64_t b = (c.np + size - 1) / size, cap = std::min<int64_t>((int64_t)c.sms * c.push_bps, MAX_BLOCKS);
+    return (int)std::max<int64_t>(1, std::min(b, std::max<int64_t>(cap, small_chunks(c) ? b : 1)));
+}
+
+int push_blocks(const Ctx& c) { return c.closed ? chunk_blocks(c) : particle_blocks(c); }
 
 int local_blocks(const Ctx& c) {
     const int64_t b = (c.np * 8 + THREADS - 1) / THREADS;
@@ -2005,9 +2024,12 @@ void launch_point_deposit(Ctx& c) {
 void launch_first_scatter(Ctx& c, double* J, const double* v_iter_or_null) {
     StepParams p = make_params(c);
     int nb = particle_blocks(c);
-    if (c.closed)
-        k_first_scatter_cell<<<nb, THREADS, CHUNK_SMEM, c.stream>>>(p, c.xi, c.v, c.vprev, v_iter_or_null, c.vit, J, c.partials,
-                                                           c.dev_status);
+    if (c.closed && small_chunks(c))
+        k_first_scatter_cell<1, 1><<<chunk_blocks(c), 32, ChunkSmall::smem(), c.stream>>>(
+            p, c.xi, c.v, c.vprev, v_iter_or_null, c.vit, J, c.partials, c.dev_status);
+    else if (c.closed)
+        k_first_scatter_cell<4, 2><<<chunk_blocks(c), 128, ChunkLarge::smem(), c.stream>>>(
+            p, c.xi, c.v, c.vprev, v_iter_or_null, c.vit, J, c.partials, c.dev_status);
     else
         k_first_scatter<1><<<nb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.vprev, v_iter_or_null, c.vit, J, c.partials,
                                                          c.dev_status);
@@ -2028,10 +2050,17 @@ void launch_push(Ctx& c, const double* vit, double* vnew, double* Jnext, bool co
                                                   c.slide,                                                    \
                                                   c.partials, c.dev_status)
     const CellFields cf{c.fxtab ? c.ctab : c.table, reinterpret_cast<const longlong2*>(c.fxtab), c.cell_top};
-#define PIC_PUSH_CELL(C, T)                                                                                       \
-    k_push_cell<C, T><<<nb, THREADS, C ? sizeof(ChunkOrder) : CHUNK_SMEM, c.stream>>>(p, c.xi, c.v, c.P, vit, cf, vnew, Jnext,     \
-                                                    c.xi_new, c.P_new, c.creep_list, c.creep_count,                \
-                                                    det ? c.creep_flag : nullptr, c.slide, c.partials, c.dev_status)
+    const bool small = small_chunks(c);
+#define PIC_PUSH_CELL_AS(C, T, W, I)                                                                              \
+    k_push_cell<C, T, W, I><<<chunk_blocks(c), 32 * W, C ? sizeof(ChunkOrder<W, I>) : ChunkOrder<W, I>::smem(),     \
+                              c.stream>>>(p, c.xi, c.v, c.P, vit, cf, vnew, Jnext, c.xi_new, c.P_new, c.creep_list, \
+                                          c.creep_count, det ? c.creep_flag : nullptr, c.slide, c.partials,        \
+                                          c.dev_status)
+#define PIC_PUSH_CELL(C, T)                \
+    do {                                   \
+        if (small) PIC_PUSH_CELL_AS(C, T, 1, 1); \
+        else PIC_PUSH_CELL_AS(C, T, 4, 2);       \
+    } while (0)
     if (closed && !diag) {
         if (commit) {
             if (c.fxtab) PIC_PUSH_CELL(true, true);
@@ -2050,6 +2079,7 @@ void launch_push(Ctx& c, const double* vit, double* vnew, double* Jnext, bool co
     }
 #undef PIC_PUSH
 #undef PIC_PUSH_CELL
+#undef PIC_PUSH_CELL_AS
     ++c.launches;
     // in deterministic mode the exact current is rounded once all of its deposits are in
     if (det && Jnext && !c.cfg.picard_accel) launch_exact_finish(c, Jnext, 3 * c.m.ncell, c.inv_u_J);

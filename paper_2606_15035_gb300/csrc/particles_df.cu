@@ -27,8 +27,8 @@
 namespace pic {
 namespace {
 
-// Blocks per SM: 2 (128 registers) measured 88.5 ms at 128^3 with 134M particles, 3 (85) 100.4.
-constexpr int DF_MINB = 2;
+// Blocks per SM: 16 warps (128 registers) measured 88.5 ms at 128^3 with 134M particles, 24 (85) 100.4.
+constexpr int DF_MINB = 4;
 
 struct ParamsDF {
     StepParams p;       // the FP64 parameters (creeping tests, residual sums, iterate I/O)
@@ -97,7 +97,7 @@ struct PairLoad<false> {
 // node table and shared 64-bit atomics before): G(v^p) for every particle, creeping ones listed for k_local (as in
 // k_push_cell), the e_v partial sums, and the orbit current of v^{p+1} = G(v^p) into Jnext.
 template <bool CELLS>
-__global__ void __launch_bounds__(THREADS, DF_MINB) k_push_df(ParamsDF pd, const double* __restrict__ xi,
+__global__ void __launch_bounds__(ChunkLarge::THREADS_, DF_MINB) k_push_df(ParamsDF pd, const double* __restrict__ xi,
                                                                const double* __restrict__ v,
                                                                const double* __restrict__ P,
                                                                const double* __restrict__ vit,
@@ -110,91 +110,94 @@ __global__ void __launch_bounds__(THREADS, DF_MINB) k_push_df(ParamsDF pd, const
                                                                int* __restrict__ status) {
     __shared__ double sm[32];
     extern __shared__ __align__(16) unsigned char dyn[];
-    ChunkOrder& co = *reinterpret_cast<ChunkOrder*>(dyn);
-    long long* tile = reinterpret_cast<long long*>(dyn + sizeof(ChunkOrder)) + (threadIdx.x >> 5) * DEPOSIT_TILE;
+    ChunkLarge& co = ChunkLarge::in(dyn);
+    long long* tile = ChunkLarge::tile(dyn);
     const StepParams& p = pd.p;
-    const int64_t np = p.np, nchunks = (np + THREADS - 1) / THREADS;
+    const int64_t np = p.np, nchunks = (np + ChunkLarge::SIZE - 1) / ChunkLarge::SIZE;
     double ev_num = 0.0, ev_den = 0.0;
     long long pieces_push = 0, pieces_scatter = 0;
     for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-        const int64_t base = ch * THREADS, j = base + threadIdx.x;
-        double x0[3], vs[3], v2[3];
-        CellStart<double> st;
-        if (j < np) {
+        const int64_t base = ch * ChunkLarge::SIZE;
+        chunk_exchange(p, co, base, [&](int64_t j, double x0[3], double v2[3]) {
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 x0[a] = xi[a * np + j];
                 v2[a] = vit[a * np + j] + v[a * np + j];
             }
-        }
-        const int64_t i = chunk_exchange(p, co, base, j < np, x0, v2, st, vs);
-        bool scat = false;               // this lane's next orbit is scattered here
-        double bn[3] = {0.0, 0.0, 0.0}, w[3] = {0.0, 0.0, 0.0};
-        if (i < np) {
-            DF kick[3];
-            {
-                CellStart<DF> sd;
-                DF vd[3], beta[3], acc[3], Ae[3];
+        });
+#pragma unroll 1
+        for (int it = 0; it < 2; ++it) {
+            CellStart<double> st;
+            double vs[3];
+            const int64_t i = co.take(it, base, st, vs);
+            bool scat = false;               // this lane's next orbit is scattered here
+            double bn[3] = {0.0, 0.0, 0.0}, w[3] = {0.0, 0.0, 0.0};
+            if (i < np) {
+                DF kick[3];
+                {
+                    CellStart<DF> sd;
+                    DF vd[3], beta[3], acc[3], Ae[3];
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) {
+                        sd.f[a] = df_bits(st.f[a]);
+                        sd.c[a] = st.c[a];
+                        vd[a] = df_bits(vs[a]);
+                        beta[a] = pd.cb[a] * vd[a];
+                    }
+                    const int nseg = for_each_piece(sd, beta, p.m, [&](DF h, DF sc, const DF mid[3], const int c[3]) {
+                        piece_impulse(h, sc, mid, beta, vd, pd.ihs, PairLoad<CELLS>(table, c, p.m), acc);
+                    });
+                    if (nseg < 0) atomicOr(status, DEV_ERR_SEGMENTS);
+                    pieces_push += nseg;
+                    cell_A1(sd.f, PairLoad<CELLS>(table, sd.c, p.m), Ae);
+                    // P^{n+1} - P^n - q A_h^{n+1}(x^{n+1}) (Eqs. (orbit-P-update), (orbit-v-update))
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) kick[a] = mad(pd.dtq, acc[a], -(pd.q * Ae[a]));
+                }
+                double vw[3], d[3], vn[3], vi[3], beta[3];
+                bool finite = true;
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
-                    sd.f[a] = df_bits(st.f[a]);
-                    sd.c[a] = st.c[a];
-                    vd[a] = df_bits(vs[a]);
-                    beta[a] = pd.cb[a] * vd[a];
+                    vw[a] = (P[a * np + i] + dbl_of(kick[a])) * p.inv_mass;
+                    finite = finite && isfinite(vw[a]);
+                    vi[a] = vit[a * np + i];
+                    vn[a] = v[a * np + i];
+                    d[a] = vw[a] - vi[a];
+                    beta[a] = p.cb[a] * vs[a];
                 }
-                const int nseg = for_each_piece(sd, beta, p.m, [&](DF h, DF sc, const DF mid[3], const int c[3]) {
-                    piece_impulse(h, sc, mid, beta, vd, pd.ihs, PairLoad<CELLS>(table, c, p.m), acc);
-                });
-                if (nseg < 0) atomicOr(status, DEV_ERR_SEGMENTS);
-                pieces_push += nseg;
-                cell_A1(sd.f, PairLoad<CELLS>(table, sd.c, p.m), Ae);
-                // P^{n+1} - P^n - q A_h^{n+1}(x^{n+1}) (Eqs. (orbit-P-update), (orbit-v-update))
+                if (!finite) atomicOr(status, DEV_ERR_NONFINITE);
+                // the local-solve gate of k_push_cell, in FP64
+                bool slow = false;
+                if (p.hist) {
+                    double dold = 0.0;
 #pragma unroll
-                for (int a = 0; a < 3; ++a) kick[a] = mad(pd.dtq, acc[a], -(pd.q * Ae[a]));
-            }
-            double vw[3], d[3], vn[3], vi[3], beta[3];
-            bool finite = true;
+                    for (int a = 0; a < 3; ++a) dold = max_pos(dold, ::fabs(vi[a] - vnew[a * np + i]));
+                    const double dn = max_pos(max_pos(::fabs(d[0]), ::fabs(d[1])), ::fabs(d[2]));
+                    if (less_pos(SLOW_RATIO * dold, dn))
+                        slow = dn > p.slow_floor * sqrt(vi[0] * vi[0] + vi[1] * vi[1] + vi[2] * vi[2]);
+                }
+                const bool creep = p.accel && (is_creeping_cell(st.f, beta) || (slide[i] & SLIDE_CREPT) || slow);
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                vw[a] = (P[a * np + i] + dbl_of(kick[a])) * p.inv_mass;
-                finite = finite && isfinite(vw[a]);
-                vi[a] = vit[a * np + i];
-                vn[a] = v[a * np + i];
-                d[a] = vw[a] - vi[a];
-                beta[a] = p.cb[a] * vs[a];
-            }
-            if (!finite) atomicOr(status, DEV_ERR_NONFINITE);
-            // the local-solve gate of k_push_cell, in FP64
-            bool slow = false;
-            if (p.hist) {
-                double dold = 0.0;
+                for (int a = 0; a < 3; ++a) vnew[a * np + i] = vw[a];
+                if (creep) {
+                    const int k = atomicAdd(creep_count, 1);
+                    creep_list[k] = (int32_t)i;
+                } else {
+                    scat = true;
 #pragma unroll
-                for (int a = 0; a < 3; ++a) dold = max_pos(dold, ::fabs(vi[a] - vnew[a * np + i]));
-                const double dn = max_pos(max_pos(::fabs(d[0]), ::fabs(d[1])), ::fabs(d[2]));
-                if (less_pos(SLOW_RATIO * dold, dn))
-                    slow = dn > p.slow_floor * sqrt(vi[0] * vi[0] + vi[1] * vi[1] + vi[2] * vi[2]);
-            }
-            const bool creep = p.accel && (is_creeping_cell(st.f, beta) || (slide[i] & SLIDE_CREPT) || slow);
-#pragma unroll
-            for (int a = 0; a < 3; ++a) vnew[a * np + i] = vw[a];
-            if (creep) {
-                const int k = atomicAdd(creep_count, 1);
-                creep_list[k] = (int32_t)i;
-            } else {
-                scat = true;
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    ev_num += d[a] * d[a];
-                    ev_den += vw[a] * vw[a];
-                    const double v2n = vw[a] + vn[a];
-                    bn[a] = p.cb[a] * v2n;
-                    w[a] = p.q_dV_half * v2n;
+                    for (int a = 0; a < 3; ++a) {
+                        ev_num += d[a] * d[a];
+                        ev_den += vw[a] * vw[a];
+                        const double v2n = vw[a] + vn[a];
+                        bn[a] = p.cb[a] * v2n;
+                        w[a] = p.q_dV_half * v2n;
+                    }
                 }
             }
+            const int ns = scatter_warp(p.m, scat, st, bn, w, tile, 0, p.acc, Jnext);
+            if (ns < 0) atomicOr(status, DEV_ERR_SEGMENTS);
+            pieces_scatter += ns;
         }
-        const int ns = scatter_warp(p.m, scat, st, bn, w, tile, 0, p.acc, Jnext);
-        if (ns < 0) atomicOr(status, DEV_ERR_SEGMENTS);
-        pieces_scatter += ns;
         __syncthreads();   // the hand-over buffers are rewritten by the next chunk
     }
     write_partial<double>(partials, S_EV_NUM, ev_num, sm, false);
@@ -242,8 +245,8 @@ ParamsDF make_params_df(const Ctx& c) {
 
 bool setup_pair_kernels() {
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    return cudaFuncSetAttribute(k_push_df<true>, at, (int)CHUNK_SMEM) == cudaSuccess &&
-           cudaFuncSetAttribute(k_push_df<false>, at, (int)CHUNK_SMEM) == cudaSuccess;
+    return cudaFuncSetAttribute(k_push_df<true>, at, (int)ChunkLarge::smem()) == cudaSuccess &&
+           cudaFuncSetAttribute(k_push_df<false>, at, (int)ChunkLarge::smem()) == cudaSuccess;
 }
 
 void launch_table_df(Ctx& c) {
@@ -260,11 +263,10 @@ void launch_table_df(Ctx& c) {
 
 void launch_push_df(Ctx& c, const double* vit, double* vnew, double* Jnext) {
     cudaMemsetAsync(c.creep_count, 0, 2 * sizeof(int), c.stream);   // count, k_local queue head
-    int nb = (int)std::max<int64_t>(1, std::min<int64_t>((c.np + THREADS - 1) / THREADS, (int64_t)c.sms * c.push_bps));
-    nb = std::min(nb, MAX_BLOCKS);
+    const int nb = chunk_blocks(c);
     const float4* t = reinterpret_cast<const float4*>(c.table_pair);
 #define PIC_PUSH_DF(T)                                                                                            \
-    k_push_df<T><<<nb, THREADS, CHUNK_SMEM, c.stream>>>(make_params_df(c), c.xi, c.v, c.P, vit, t, vnew, Jnext,     \
+    k_push_df<T><<<nb, ChunkLarge::THREADS_, ChunkLarge::smem(), c.stream>>>(make_params_df(c), c.xi, c.v, c.P, vit, t, vnew, Jnext,     \
                                                         c.creep_list, c.creep_count, c.slide, c.partials,          \
                                                         c.dev_status)
     if (c.pair_cells) PIC_PUSH_DF(true);

@@ -626,7 +626,7 @@ void step_begin(Ctx& c) {
             launch_first_scatter(c, c.J[r.cur], nullptr);
         }
     }
-    launch_finalize(c, S_JSCALE, 1, particle_blocks(c), false);
+    launch_finalize(c, S_JSCALE, 1, r.fp32 ? particle_blocks(c) : push_blocks(c), false);
 }
 
 // The trial final sweep (PIC_MIXED, see iter_finish): the final sweep of v* = v^{p+1} with
@@ -639,7 +639,7 @@ void trial_issue(Ctx& c) {
         ProfScope ps(c, PH_COMMIT);
         launch_push(c, c.vit, c.vnew, nullptr, true, false);
     }
-    launch_finalize(c, S_EV_NUM, 2, particle_blocks(c), false);
+    launch_finalize(c, S_EV_NUM, 2, push_blocks(c), false);
     queue_results(c);
 }
 
@@ -682,10 +682,10 @@ void iter_issue(Ctx& c) {
         }
         // the current fixed-point error of this update: J(v^{p+1}) against J(v^p)
         launch_jdiff(c, c.J[r.next], c.J[r.cur]);
-        launch_finalize(c, S_EV_NUM, 2, particle_blocks(c), false);
+        launch_finalize(c, S_EV_NUM, 2, push_blocks(c), false);
         if (c.cfg.picard_accel) launch_finalize(c, S_EVL_NUM, 2, local_blocks(c), false);
         launch_finalize(c, S_EJ_NUM, 2, mesh_blocks(c), false);
-        if (c.prof) launch_finalize(c, S_PIECES_PUSH, 2, particle_blocks(c), false);
+        if (c.prof) launch_finalize(c, S_PIECES_PUSH, 2, push_blocks(c), false);
         if (c.prof && c.cfg.picard_accel) launch_finalize(c, S_LOCAL_SOLVES, 4, local_blocks(c), false);
         c.last_v = c.vit;
         c.last_g = c.vnew;

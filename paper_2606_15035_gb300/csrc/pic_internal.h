@@ -359,6 +359,8 @@ StepParams make_params(const Ctx& c);
 bool setup_particle_kernels();
 bool setup_pair_kernels();
 int particle_blocks(const Ctx& c);
+int chunk_blocks(const Ctx& c);   // the closed forms' chunk kernels
+int push_blocks(const Ctx& c);    // the pushes without diagnostics and the first scatter
 int local_blocks(const Ctx& c);
 int mesh_blocks(const Ctx& c);
 
