@@ -182,7 +182,7 @@ extern "C" pic_status pic_cn_update_static(const int32_t n[3], const double L[3]
         fft = fft && pic::fft_factor(n[ax], radix, nst);
     }
     const int corrections = fft ? pic::helm32_corrections(lmax, std::fmax(helmholtz_tol, 1e-16)) : 0;
-    fft = corrections > 0 && iters > 5 * corrections;
+    fft = corrections > 0 && iters > 5 * corrections && pic::setup_helm_kernels();
     // the transforms' buffers: z in place of the second iterate, the tables and exponents in the
     // directions' place
     float2* tw = fft ? reinterpret_cast<float2*>(dir) : nullptr;

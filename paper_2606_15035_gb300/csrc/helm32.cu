@@ -12,7 +12,9 @@
 // Real fields travel in pairs, f + i g (the symbol is real and even, so the solve keeps them apart),
 // each scaled by a power of two near the inverse of its right-hand side's largest value, so that no
 // magnitude leaves the FP32 range and neither field of a pair drowns the other.  Five launches a
-// correction: residual and x transforms; y; z forward, division, z back; y; x and the addition.
+// correction: residual and x transforms; y; z forward, division, z back; y; x and the addition; or three
+// where a plane of y and z fits a block (a launch costs 1.3-3 us of gap here: the static update at 32^3
+// took 121.5 us with five, 106.5 with three).
 //
 // A mesh phase's solves measured against FP64 transforms with one refinement: 128^3 6.5 -> 1.8 ms (the
 // residuals 1.0 of it, FP64), 64^3 0.86 -> 0.25 ms, 32^3 0.17 -> 0.07 ms.
@@ -26,6 +28,7 @@ namespace pic {
 namespace {
 
 constexpr int ELEMS = 2048;   // complex elements of a block's lines
+constexpr int PLANE = 4096;   // ... of a block of whole y-z planes (64 KB of shared memory)
 
 struct Stage {
     int R, L, nb, tstep;      // radix, product of the radices before, n / R, n / (L R)
@@ -220,6 +223,50 @@ __global__ void __launch_bounds__(256) k_helm_yz(Helm32 h, Axis32 ax) {
     }
 }
 
+// k_helm_yz's three passes in one, where a plane of y and z fits a block's shared memory: lb adjacent x of
+// field blockIdx.y, y forward, z forward, division, z back, y back.
+__global__ void __launch_bounds__(512) k_helm_plane(Helm32 h, Axis32 ay, Axis32 az, int lb) {
+    extern __shared__ float2 buf[];
+    const int nx = h.m.n[0], ny = ay.n, nz = az.n, plane = ny * nz;
+    const int first = blockIdx.x * lb, xs = min(lb, nx - first), cnt = xs * plane;
+    float2* z = h.z + blockIdx.y * h.m.ncell + first;
+    float2* a = buf;
+    float2* b = buf + lb * plane;
+    // element (j, iz, iy) of the lines along y at (j nz + iz) ny + iy, of those along z at (j ny + iy) nz + iz
+    for (int e = threadIdx.x; e < lb * plane; e += blockDim.x) {
+        const int r = e / lb, j = e - r * lb, iz = quot(r, ay.mn), iy = r - iz * ny;
+        if (j < xs) a[(j * nz + iz) * ny + iy] = z[j + (int64_t)nx * r];
+    }
+    __syncthreads();
+    float2* r = lines_fft<false>(a, b, ay, xs * nz);
+    float2* o = r == a ? b : a;
+    for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
+        const int l = quot(e, ay.mn), iy = e - l * ny, j = quot(l, az.mn), iz = l - j * nz;
+        o[(j * ny + iy) * nz + iz] = r[e];
+    }
+    __syncthreads();
+    r = lines_fft<false>(o, r, az, xs * ny);
+    for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
+        const int l = quot(e, az.mn), iz = e - l * nz, j = quot(l, ay.mn), iy = l - j * ny;
+        const float s = __ldg(h.s2 + first + j) + __ldg(h.s2 + nx + iy) + __ldg(h.s2 + nx + ny + iz);
+        const float q = h.invN / (1.f + h.af * s);
+        r[e] = make_float2(r[e].x * q, r[e].y * q);
+    }
+    __syncthreads();
+    r = lines_fft<true>(r, r == a ? b : a, az, xs * ny);
+    o = r == a ? b : a;
+    for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
+        const int l = quot(e, az.mn), iz = e - l * nz, j = quot(l, ay.mn), iy = l - j * ny;
+        o[(j * nz + iz) * ny + iy] = r[e];
+    }
+    __syncthreads();
+    r = lines_fft<true>(o, r, ay, xs * nz);
+    for (int e = threadIdx.x; e < lb * plane; e += blockDim.x) {
+        const int q = e / lb, j = e - q * lb, iz = quot(q, ay.mn), iy = q - iz * ny;
+        if (j < xs) z[j + (int64_t)nx * q] = r[(j * nz + iz) * ny + iy];
+    }
+}
+
 // top[f] = max over field f of the biased exponents of b (top starts at zero).
 __global__ void k_exponents(int64_t N, const double* __restrict__ b, int* __restrict__ top) {
     int e = 0;
@@ -277,6 +324,11 @@ void launch_helm_exponents(Ctx& c, const double* b, int* top) {
     ++c.launches;
 }
 
+bool setup_helm_kernels() {
+    return cudaFuncSetAttribute(k_helm_plane, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                2 * (int)sizeof(float2) * PLANE) == cudaSuccess;
+}
+
 int helm32_corrections(double lmax, double to) {
     const double q = 2.5e-7 * lmax;
     if (!(q < 1.0)) return 0;
@@ -302,15 +354,27 @@ int helm32_solve(const HelmPlan& c, const double* b, double* x, const int* top, 
     const dim3 gx = grid((c.m.ncell / ax.n + ax.lb - 1) / ax.lb);
     const dim3 gy = grid((int64_t)((c.m.n[0] + ay.lb - 1) / ay.lb) * c.m.n[2]);
     const dim3 gz = grid(((int64_t)c.m.n[0] * c.m.n[1] + az.lb - 1) / az.lb);
+    // one launch for y and z where a plane fits (PLANE elements): lb adjacent x a block, fewer while the
+    // blocks do not fill the SMs
+    const int64_t plane = (int64_t)ay.n * az.n;
+    const bool fused = plane <= PLANE;
+    int lb = 4;
+    while (lb > 1 && (lb * plane > PLANE || 2 * ((c.m.n[0] + lb - 1) / lb) < c.sms / 2)) lb /= 2;
     for (int k = 0; k < corrections; ++k) {
         h.up = 20 * k;   // each correction leaves a residual some 2^20 smaller
         k_helm_x<false><<<gx, 256, smem(ax), stream>>>(h, ax);
+        if (fused) {
+            const int threads = (int)std::max<int64_t>(64, std::min<int64_t>(512, (lb * plane / 4 + 31) / 32 * 32));
+            k_helm_plane<<<dim3((c.m.n[0] + lb - 1) / lb, 2), threads, 2 * sizeof(float2) * lb * plane, stream>>>(h, ay, az, lb);
+            k_helm_x<true><<<gx, 256, smem(ax), stream>>>(h, ax);
+            continue;
+        }
         if (ay.n > 1) k_helm_yz<false, false><<<gy, 256, smem(ay), stream>>>(h, ay);
         k_helm_yz<false, true><<<gz, 256, smem(az), stream>>>(h, az);
         if (ay.n > 1) k_helm_yz<true, false><<<gy, 256, smem(ay), stream>>>(h, ay);
         k_helm_x<true><<<gx, 256, smem(ax), stream>>>(h, ax);
     }
-    return corrections * (ay.n > 1 ? 5 : 3);
+    return corrections * (fused || ay.n <= 1 ? 3 : 5);
 }
 
 void launch_helm32(Ctx& c, const double* b, double* x, const int* top, int corrections) {

@@ -319,6 +319,7 @@ constexpr int HELM_MAX_CORRECTIONS = 8;
 // 32^3 and 64^3 of the standard box, 4 at 128^3 (lmax 29), 6 at lmax 3000; the fields then match an
 // exact FP64 update to 5e-16.
 int helm32_corrections(double lmax, double to);
+bool setup_helm_kernels();   // their shared memory, on the current device
 int helm32_solve(const HelmPlan& c, const double* b, double* x, const int* top, int corrections, cudaStream_t stream);
 int radix_tiles(int64_t np);
 int push32_blocks(const Ctx& c);   // grid of the FP32 chunk kernels (partials per block)
