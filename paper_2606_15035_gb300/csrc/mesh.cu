@@ -352,12 +352,19 @@ __global__ void __launch_bounds__(THREADS) k_cheb_all(MeshParams p, double* xa, 
 
 __global__ void k_backsub_table(MeshParams p, const double* __restrict__ F0, const double* __restrict__ W0,
                                 const double* __restrict__ F1, double* __restrict__ W1, double* __restrict__ table,
-                                int* __restrict__ top) {
+                                int* __restrict__ top, int* __restrict__ cell_top, double* __restrict__ zero) {
     const int64_t N = p.m.ncell;
-    if (top && blockIdx.x == 0 && threadIdx.x < 4) top[threadIdx.x] = 0;   // for the next k_source
+    // cleared on the way for the kernels that follow: the next k_source's exponents, the cell tables',
+    // the next current
+    if (top && blockIdx.x == 0 && threadIdx.x < 4) top[threadIdx.x] = 0;
+    if (blockIdx.x == 0 && threadIdx.x < 2) cell_top[threadIdx.x] = 0;
     GRID_LOOP(g, N) {
         Nb b = decompose(g, p.m);
         double w1[4];
+        if (zero) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) zero[a * N + g] = 0.0;
+        }
 #pragma unroll
         for (int f = 0; f < 4; ++f) {
             w1[f] = 2.0 * (F1[f * N + g] - F0[f * N + g]) / p.dt - W0[f * N + g];
@@ -552,18 +559,27 @@ __global__ void k_add_const(double* __restrict__ f, int64_t n, double c) {
     GRID_LOOP(i, n) f[i] += c;
 }
 
-// Fold nblocks partials of each slot, in a fixed order, into results[slot].
-__global__ void k_finalize(const double* __restrict__ partials, double* __restrict__ results, int slot0, int nblocks,
-                           int is_max) {
+// Fold the queued slots' partials, each in a fixed order, into results and the host's copy (pinned
+// memory, which a stream synchronisation makes visible there); the first block also hands over the
+// status word.  One launch and no copies: three launches and two copies a Picard iteration before, some 20 us
+// of its latency.
+__global__ void k_finalize(const double* __restrict__ partials, double* __restrict__ results,
+                           double* __restrict__ host_results, FoldList folds, const int* __restrict__ status,
+                           int* __restrict__ host_status) {
     __shared__ double sm[32];
-    const int slot = slot0 + blockIdx.x;
+    if (host_status && blockIdx.x == 0 && threadIdx.x == 0) *host_status = *status;
+    if ((int)blockIdx.x >= folds.n) return;
+    const int slot = folds.slot[blockIdx.x], is_max = folds.is_max[blockIdx.x], nblocks = folds.blocks[blockIdx.x];
     double v = 0.0;
     for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
         double x = partials[slot * MAX_BLOCKS + b];
         v = is_max ? fmax(v, x) : v + x;
     }
     double r = is_max ? block_max(v, sm) : block_sum(v, sm);
-    if (threadIdx.x == 0) results[slot] = r;
+    if (threadIdx.x == 0) {
+        results[slot] = r;
+        host_results[slot] = r;
+    }
 }
 
 __global__ void k_fill(double* __restrict__ p, int64_t n, double v) {
@@ -673,9 +689,9 @@ int cheb_coop_capacity(const Ctx& c) {
     return per_sm * c.sms;
 }
 
-void launch_backsub_table(Ctx& c, bool) {
+void launch_backsub_table(Ctx& c, double* zero) {
     k_backsub_table<<<mesh_blocks(c), THREADS, 0, c.stream>>>(mesh_params(c), c.F0, c.W0, c.F1, c.W1, c.table,
-                                                            c.helm_top);
+                                                            c.helm_top, c.cell_top, zero);
     ++c.launches;
 }
 
@@ -684,7 +700,7 @@ void launch_cell_table(Ctx& c, bool fixed) {
         return (int)std::max<int64_t>(1, std::min<int64_t>((n + THREADS - 1) / THREADS, (int64_t)c.sms * 16));
     };
     fixed = fixed && c.fxtab;
-    if (fixed) cudaMemsetAsync(c.cell_top, 0, 2 * sizeof(int), c.stream);
+    if (fixed && c.cfg.ops == PIC_OPS_SPECTRAL) cudaMemsetAsync(c.cell_top, 0, 2 * sizeof(int), c.stream);
     k_cell_table<<<blocks(c.m.ncell * CELL_COLS), THREADS, 0, c.stream>>>(
         c.m, c.table, reinterpret_cast<double2*>(c.ctab), fixed ? c.cell_top : nullptr);
     ++c.launches;
@@ -705,6 +721,7 @@ void launch_null_project(Ctx& c, double* f, double add_const) {
     k_null_dots<<<nb, THREADS, 0, c.stream>>>(p, f, c.partials);
     ++c.launches;
     launch_finalize(c, S_PROJ0, 8, nb, false);
+    launch_folds(c, false);   // used on the device
     k_null_subtract<<<nb, THREADS, 0, c.stream>>>(p, f, c.results);
     ++c.launches;
 }
@@ -721,8 +738,24 @@ void launch_mesh_diag(Ctx& c, const double* Jfinal) {
 }
 
 void launch_finalize(Ctx& c, int slot0, int nslots, int nblocks, bool is_max) {
-    k_finalize<<<nslots, THREADS, 0, c.stream>>>(c.partials, c.results, slot0, nblocks, is_max ? 1 : 0);
+    for (int k = 0; k < nslots; ++k) {
+        if (c.folds.n == FoldList::MAX) launch_folds(c, false);
+        FoldList& f = c.folds;
+        int at = 0;   // a slot queued again (after a call that failed half-way) takes its old place
+        while (at < f.n && f.slot[at] != slot0 + k) ++at;
+        f.slot[at] = (short)(slot0 + k);
+        f.is_max[at] = is_max ? 1 : 0;
+        f.blocks[at] = nblocks;
+        f.n = std::max(f.n, at + 1);
+    }
+}
+
+void launch_folds(Ctx& c, bool status) {
+    if (c.folds.n == 0 && !status) return;
+    k_finalize<<<std::max(1, c.folds.n), THREADS, 0, c.stream>>>(c.partials, c.results, c.host_results, c.folds,
+                                                               c.dev_status, status ? c.host_status : nullptr);
     ++c.launches;
+    c.folds.n = 0;
 }
 
 void launch_fill(Ctx& c, double* p, int64_t n, double value) {

@@ -195,10 +195,10 @@ void prof_resolve(Ctx& c) {
 }
 
 // Copy results + status to the host and wait.
-// Queue the copy of the result slots and the status word to the pinned host buffers.
+// Queue the folds into the result slots and the hand-over of those and the status word to the pinned
+// host buffers.
 void queue_results(Ctx& c) {
-    cudaMemcpyAsync(c.host_results, c.results, sizeof(double) * NSLOT, cudaMemcpyDeviceToHost, c.stream);
-    cudaMemcpyAsync(c.host_status, c.dev_status, sizeof(int), cudaMemcpyDeviceToHost, c.stream);
+    launch_folds(c, true);
 }
 
 // Wait for the stream, then turn CUDA errors and device status bits into a status.
@@ -475,7 +475,10 @@ pic_status allocate(pic_ctx* ctx) {
         if (reinterpret_cast<uintptr_t>(c.table_pair) % 16 != 0)
             return fail(ctx, PIC_ERR_ARG, "the allocator returned a pointer that is not 16-byte aligned");
     }
+    std::memset(c.host_results, 0, sizeof(double) * NSLOT);
+    *c.host_status = 0;
     cudaMemsetAsync(c.partials, 0, sizeof(double) * (size_t)NSLOT * MAX_BLOCKS, c.stream);
+    cudaMemsetAsync(c.cell_top, 0, 2 * sizeof(int), c.stream);
     cudaMemsetAsync(c.results, 0, sizeof(double) * NSLOT, c.stream);
     cudaMemsetAsync(c.dev_status, 0, sizeof(int), c.stream);
     return check_cuda(ctx, "allocate");
@@ -564,10 +567,13 @@ void mesh_begin(Ctx& c) {
 // back-substitution and the gather table.
 // tol: the Chebyshev solve's relative accuracy (helmholtz_tol when not positive).
 // cells: also the cell table, for the FP64 closed-form kernels that follow.
-void mesh_phase(Ctx& c, const double* Jcur, const double* Jprev, double tol = 0.0, bool cells = true) {
+// zero: 3 N values to clear (the next current).
+void mesh_phase(Ctx& c, const double* Jcur, const double* Jprev, double tol = 0.0, bool cells = true,
+                double* zero = nullptr) {
     ProfScope ps(c, PH_MESH);
     if (c.cfg.ops == PIC_OPS_SPECTRAL) {
         launch_spec_mesh_phase(c, Jcur, Jprev);
+        if (zero) cudaMemsetAsync(zero, 0, sizeof(double) * 3 * c.m.ncell, c.stream);
     } else {
         launch_source(c, Jcur, Jprev);
         if (c.helm_corrections > 0) {
@@ -578,7 +584,7 @@ void mesh_phase(Ctx& c, const double* Jcur, const double* Jprev, double tol = 0.
         } else {
             launch_helmholtz_cn(c, &c.F1, &c.F1b, tol > 0.0 ? std::max(tol, c.cfg.helmholtz_tol) : c.cfg.helmholtz_tol);
         }
-        launch_backsub_table(c, false);
+        launch_backsub_table(c, zero);
     }
     if (cells && c.ctab) launch_cell_table(c, true);
 }
@@ -653,10 +659,9 @@ void iter_issue(Ctx& c) {
     const int64_t N = c.m.ncell;
     const double mesh_tol = r.fp32 ? MESH_TOL32
                             : (r.began32 && c.cfg.mixed_tol64 > 0.0 ? 1e-3 * c.cfg.mixed_tol64 : 0.0);
-    mesh_phase(c, c.J[r.cur], r.p > 0 ? c.J[r.prev] : nullptr, mesh_tol, !r.fp32);
+    mesh_phase(c, c.J[r.cur], r.p > 0 ? c.J[r.prev] : nullptr, mesh_tol, !r.fp32, c.J[r.next]);
     if (r.fp32) {
         launch_table32(c);
-        cudaMemsetAsync(c.J[r.next], 0, sizeof(double) * 3 * N, c.stream);
         {
             ProfScope ps(c, PH_PUSH32);
             launch_push32(c, c.J[r.next]);
@@ -665,7 +670,6 @@ void iter_issue(Ctx& c) {
         launch_finalize(c, S_EJ_NUM, 2, mesh_blocks(c), false);
         if (c.prof) launch_finalize(c, S_CHUNKS32, 2, push32_blocks(c), false);
     } else {
-        cudaMemsetAsync(c.J[r.next], 0, sizeof(double) * 3 * N, c.stream);
         r.pair_issued = r.pair;
         if (r.pair) {
             // PIC_MIXED refinement: the particle half in FP32 pairs from the pair table

@@ -82,6 +82,14 @@ struct StepParams {
 constexpr int FFT_MAX = 1024;       // largest mesh size per axis with spectral operators
 constexpr int FFT_MAX_STAGES = 16;
 
+// Slots whose per-block partials wait to be folded into results (and the host's copy of them).
+struct FoldList {
+    static constexpr int MAX = 48;
+    int n = 0;
+    short slot[MAX], is_max[MAX];
+    int blocks[MAX];
+};
+
 // Host-side state of the time step in progress (see step_begin / iter_issue / iter_finish).
 struct StepRun {
     int cur = 0, prev = 1, next = 2;   // J buffers: current iterate, previous, next
@@ -201,6 +209,7 @@ struct Ctx {
     int* dev_status = nullptr;
     double* host_results = nullptr;      // pinned, NSLOT
     int* host_status = nullptr;          // pinned
+    FoldList folds;                      // slots to fold at the next queue_results
 
     // Chebyshev schedule for the CN Helmholtz solve
     int cheb_iters = 0;
@@ -333,7 +342,7 @@ void launch_source(Ctx& c, const double* Jcur, const double* Jprev);
 void launch_jdiff(Ctx& c, const double* Jnew, const double* Jold);
 void launch_helmholtz(Ctx& c, const double* b, double c_id, double c_lap, int nfields, int iters,
                       const double* alpha, const double* beta, double** x_io, double** x_spare);
-void launch_backsub_table(Ctx& c, bool diag);
+void launch_backsub_table(Ctx& c, double* zero);   // zero (may be null): 3 ncell values to clear on the way
 // The cell tables of the FP64 closed-form particle kernels from the gather table (fixed: also the
 // fixed-point one, for the pushes).
 void launch_cell_table(Ctx& c, bool fixed);
@@ -343,7 +352,10 @@ int cheb_coop_capacity(const Ctx& c);
 void launch_null_project(Ctx& c, double* f, double add_const);
 void launch_mesh_energy(Ctx& c, const double* F, const double* W, int slot);
 void launch_mesh_diag(Ctx& c, const double* Jfinal);
+// Fold nblocks partials of each slot into results: queued, until launch_folds makes one launch of what
+// is queued and stores it, and with `status` the device status, to the host's pinned copies as well.
 void launch_finalize(Ctx& c, int slot0, int nslots, int nblocks, bool is_max);
+void launch_folds(Ctx& c, bool status);
 void launch_fill(Ctx& c, double* p, int64_t n, double value);
 void launch_scale_copy(Ctx& c, double* dst, const double* src, int64_t n, double s);
 
