@@ -90,9 +90,10 @@ typedef struct {
                                      mesh phase runs the fewest steps whose error bound is below
                                      helmholtz_tol times the solution's norm, from the warm start's
                                      residual (at most the schedule that reduces any start by it).
-                                     On a mesh whose sizes are all 2^p 3^q <= 1024 the central2
-                                     solve is by FFT instead, exact per mode (the wide Laplacian's
-                                     symbol), and this does not apply to it */
+                                     On a mesh whose sizes are all <= 1024 with no prime factor
+                                     above 127 the central2 solve is by FFT instead, to this
+                                     accuracy or better (to roundoff where all are 2^p 3^q, where
+                                     this does not apply) */
     double mixed_tol32;           /* PIC_MIXED: leave the FP32 iterations once e_v <= this */
     int32_t mixed_max32;          /* PIC_MIXED: at most this many FP32 iterations per step */
     int32_t deterministic;        /* 1: bitwise reproducible steps.  The particle sort is a stable
@@ -433,8 +434,8 @@ void pic_ensemble_destroy(pic_ensemble* e);
  * different update), (I - a Delta_h) F^{n+1} = (I + a Delta_h) F^n + dt W^n +
  * (dt^2 kappa^2 sigma / 2) src with a = kappa^2 dt^2 / 4 (src = rho_half for phi with sigma1,
  * J for A with sigma2), by the library's Chebyshev iteration (the fewest steps whose error
- * bound is below helmholtz_tol, at most 1024) or, where that is cheaper on a 2^p 3^q mesh, by FFT to
- * at least that accuracy, then W^{n+1} = 2 (F^{n+1} - F^n) / dt - W^n.
+ * bound is below helmholtz_tol, at most 1024) or, where that is cheaper (sizes <= 1024 with no prime factor
+ * above 127), by FFT to at least that accuracy, then W^{n+1} = 2 (F^{n+1} - F^n) / dt - W^n.
  *
  * Arguments: n, L: mesh nodes and box lengths (host); every array pointer is a DEVICE
  * pointer in the library's mesh layout (x-fastest; A, U, J component-major, 3 * ncell).

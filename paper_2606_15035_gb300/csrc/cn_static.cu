@@ -173,14 +173,11 @@ extern "C" pic_status pic_cn_update_static(const int32_t n[3], const double L[3]
     Fields4 src = {{rho_half, J, J + N, J + 2 * N}};
     const double c_rho = 0.5 * dt * dt * kappa * kappa * sigma1;
     const double c_J = 0.5 * dt * dt * kappa * kappa * sigma2;
-    // By transforms on 2^p 3^q meshes where they are cheaper than the Chebyshev steps: a correction
+    // By transforms where they take the mesh and are cheaper than the Chebyshev steps: a correction
     // (five launches) costs about five steps, 23 against 4.6 us at 32^3.  The whole call at 32^3 with
     // helmholtz_tol = 1e-17: 326 us by 30 steps (8.2 us each with 64-bit index divisions), 122 by transforms.
     bool fft = true;
-    for (int ax = 0; ax < 3; ++ax) {
-        int radix[pic::FFT_MAX_STAGES], nst = 0;
-        fft = fft && pic::fft_factor(n[ax], radix, nst);
-    }
+    for (int ax = 0; ax < 3; ++ax) fft = fft && pic::helm32_factor(n[ax]);
     const int corrections = fft ? pic::helm32_corrections(lmax, std::fmax(helmholtz_tol, 1e-16)) : 0;
     fft = corrections > 0 && iters > 5 * corrections && pic::setup_helm_kernels();
     // the transforms' buffers: z in place of the second iterate, the tables and exponents in the

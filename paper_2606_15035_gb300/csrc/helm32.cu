@@ -1,4 +1,4 @@
-// The Crank--Nicolson Helmholtz solve on 2^p 3^q meshes: FP64 residuals, FP32 transforms (sm_103a).
+// The Crank--Nicolson Helmholtz solve on meshes of small prime factors: FP64 residuals, FP32 transforms (sm_103a).
 //
 // (I - a Delta_h) x = b for the four potentials, by iterative refinement: the FP64 stencil residual
 // r = b - (I - a Delta_h) x of the warm start, its correction by an FFT solve in FP32 (the operator is
@@ -62,7 +62,21 @@ __device__ __forceinline__ float2* lines_fft(float2* x, float2* y, const Axis32&
     const int n = ax.n;
     for (int s = 0; s < ax.nst; ++s) {
         const Stage st = ax.st[s];
-        for (int e = threadIdx.x; e < lines * st.nb; e += blockDim.x) {
+        // a larger prime: a thread sums one output, input r rotated by r (k n / (L R) + q n / R) / n of a turn
+        for (int e = threadIdx.x; st.R > 4 && e < lines * n; e += blockDim.x) {
+            const int o = quot(e, st.mnb), q = o % st.R, line = o / st.R, j = e - o * st.nb;
+            const int jl = quot(j, st.mL), k = j - jl * st.L, step = k * st.tstep + q * st.nb;
+            const float2* in = x + line * n + j;
+            float2 a = in[0];
+            for (int r = 1, t = step; r < st.R; ++r) {
+                const float2 v = twiddle<INV>(in[r * st.nb], __ldg(ax.tw + t));
+                a = a + v;
+                t += step;
+                t -= t >= n ? n : 0;
+            }
+            y[line * n + jl * st.L * st.R + k + q * st.L] = a;
+        }
+        for (int e = threadIdx.x; st.R <= 4 && e < lines * st.nb; e += blockDim.x) {
             const int line = quot(e, st.mnb), j = e - line * st.nb;
             const int jl = quot(j, st.mL), k = j - jl * st.L;
             const float2* in = x + line * n + j;
@@ -83,7 +97,7 @@ __device__ __forceinline__ float2* lines_fft(float2* x, float2* y, const Axis32&
                 const float2 a = in[0], b = twiddle<INV>(in[st.nb], __ldg(ax.tw + t));
                 out[0] = a + b;
                 out[st.L] = a - b;
-            } else {
+            } else if (st.R == 3) {
                 const float s3 = INV ? 0.86602540378f : -0.86602540378f;
                 const float2 a = in[0];
                 const float2 b = twiddle<INV>(in[st.nb], __ldg(ax.tw + t));
@@ -294,7 +308,8 @@ Axis32 make_axis32(const HelmPlan& c, int a) {
     int L = 1, r = ax.n;
     while (r > 1) {
         Stage& s = ax.st[ax.nst++];
-        s.R = r % 4 == 0 ? 4 : (r % 2 == 0 ? 2 : 3);
+        s.R = r % 4 == 0 ? 4 : 2;
+        while (r % s.R) ++s.R;   // a prime from here on
         s.L = L;
         s.nb = ax.n / s.R;
         s.tstep = ax.n / (L * s.R);
@@ -327,6 +342,13 @@ void launch_helm_exponents(Ctx& c, const double* b, int* top) {
 bool setup_helm_kernels() {
     return cudaFuncSetAttribute(k_helm_plane, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 2 * (int)sizeof(float2) * PLANE) == cudaSuccess;
+}
+
+bool helm32_factor(int n) {
+    if (n < 1 || n > FFT_MAX) return false;
+    for (int p = 2; p <= HELM_MAX_RADIX; ++p)
+        while (n % p == 0) n /= p;
+    return n == 1;
 }
 
 int helm32_corrections(double lmax, double to) {

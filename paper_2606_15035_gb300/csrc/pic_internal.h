@@ -328,6 +328,10 @@ constexpr int HELM_MAX_CORRECTIONS = 8;
 // 32^3 and 64^3 of the standard box, 4 at 128^3 (lmax 29), 6 at lmax 3000; the fields then match an
 // exact FP64 update to 5e-16.
 int helm32_corrections(double lmax, double to);
+// Largest prime factor of an axis (its stage costs that many products a point): at 127^3 the transforms
+// still take a third of the Chebyshev steps' time.
+constexpr int HELM_MAX_RADIX = 127;
+bool helm32_factor(int n);   // whether the FP32 transforms take n: at most FFT_MAX, primes to HELM_MAX_RADIX
 bool setup_helm_kernels();   // their shared memory, on the current device
 int helm32_solve(const HelmPlan& c, const double* b, double* x, const int* top, int corrections, cudaStream_t stream);
 int radix_tiles(int64_t np);

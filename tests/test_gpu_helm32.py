@@ -1,6 +1,7 @@
 """The Crank--Nicolson update through FP32 transforms with FP64 residuals (helm32.cu), at mesh sizes
-where its line groups are ragged or degenerate, y-z planes that just fit a block and that do not, field magnitudes far from one, fields of a pair that
-differ by ten orders, and a time step whose operator needs the FP64 transforms.
+where its line groups are ragged or degenerate, y-z planes that just fit a block and that do not, prime
+factors at and above the transforms' limit, field magnitudes far from one, fields of a pair that differ by
+ten orders, and a time step whose operator needs the FP64 transforms.
 
 pic_iterate's fields against the oracle's exact per-mode update with the general parity tolerance:
 1e-12 of the field's norm (the solve itself ends at the rounding of its residual, a few 1e-16)."""
@@ -25,7 +26,9 @@ def sim(cuda_ok):
 @pytest.mark.parametrize("n,dt,amp", [
     ((1, 8, 9), 0.1, 1.0), ((8, 1, 4), 0.1, 1.0), ((6, 4, 1), 0.1, 1.0), ((2, 3, 4), 0.1, 1.0),
     ((27, 2, 16), 0.1, 1.0), ((1024, 2, 3), 0.1, 1.0), ((3, 768, 2), 0.1, 1.0), ((2, 3, 512), 0.1, 1.0),
-    ((48, 36, 54), 0.3, 1.0), ((6, 64, 64), 0.1, 1.0), ((4, 72, 64), 0.1, 1.0), ((16, 16, 16), 0.1, 1e-25), ((16, 16, 16), 0.1, 1e25), ((16, 12, 8), 60.0, 1.0),
+    ((48, 36, 54), 0.3, 1.0), ((6, 64, 64), 0.1, 1.0), ((4, 72, 64), 0.1, 1.0),
+    ((50, 35, 22), 0.1, 1.0), ((127, 5, 7), 0.1, 1.0), ((2, 113, 65), 0.1, 1.0), ((3, 11, 508), 0.1, 1.0),
+    ((127, 1, 1), 0.1, 1.0), ((131, 4, 5), 0.1, 1.0), ((16, 16, 16), 0.1, 1e-25), ((16, 16, 16), 0.1, 1e25), ((16, 12, 8), 60.0, 1.0),
 ])
 def test_fields_match_the_exact_update(sim, n, dt, amp):
     rng = np.random.default_rng(sum(n))
