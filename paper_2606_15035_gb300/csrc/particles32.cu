@@ -391,11 +391,9 @@ __global__ void k_to32(Params32 p, const double* __restrict__ xi, const double* 
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const double x = xi[a * np + i];
-            double c = floor(x);
-            if (c < 0.0) c = 0.0;
-            if (c > (double)(p.m.n[a] - 1)) c = (double)(p.m.n[a] - 1);
-            off[a * p.stride + i] = (float)(x - c);
-            packed |= ((int32_t)c & CELL_MASK) << (a * CELL_BITS);
+            const int c = min(max(__double2int_rd(x), 0), p.m.n[a] - 1);
+            off[a * p.stride + i] = (float)(x - (double)c);
+            packed |= (c & CELL_MASK) << (a * CELL_BITS);
             const double vv = v[a * np + i];
             v32[a * p.stride + i] = (float)vv;
             vit32[a * p.stride + i] = (float)(vv - vprev[a * np + i]);   // (2 v^n - v^{n-1}) - v^n
