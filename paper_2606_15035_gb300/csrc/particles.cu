@@ -55,32 +55,6 @@ namespace {
 
 // ---- orbit current scatter (Eq. (orbit-current)) -------------------------------------
 
-// J_c[g] += w_c * Sbar contribution of every piece (closed form, Appendix A), from the centred
-// moments of orbit_cell.cuh.
-__device__ __forceinline__ int scatter_closed(const StepParams& p, CellStart<double> st, const double beta[3],
-                                              const double w[3], double* __restrict__ J) {
-    const int64_t N = p.m.ncell;
-    return for_each_piece(st, beta, p.m, [&](double h, double, const double mid[3], const int c[3]) {
-        double W[8];
-        int64_t g[8];
-        node_weights(piece_moments(h, mid, beta), W);
-        cell_nodes8(c, p.m, g);
-        const double wh[3] = {h * w[0], h * w[1], h * w[2]};
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            if (p.det) {
-                exact_add(p.acc, g[k], wh[0] * W[k]);
-                exact_add(p.acc, N + g[k], wh[1] * W[k]);
-                exact_add(p.acc, 2 * N + g[k], wh[2] * W[k]);
-            } else {
-                atomicAdd(J + g[k], wh[0] * W[k]);
-                atomicAdd(J + N + g[k], wh[1] * W[k]);
-                atomicAdd(J + 2 * N + g[k], wh[2] * W[k]);
-            }
-        }
-    });
-}
-
 // Same with an n_q-point Gauss rule on the whole path (unsplit).
 __device__ __forceinline__ int scatter_gauss(const StepParams& p, const double x0[3], const double beta[3],
                                              const double w[3], double* __restrict__ J) {
@@ -331,23 +305,16 @@ __device__ __forceinline__ int scatter_pieces(const StepParams& p, const double 
     });
 }
 
-template <int QUAD>
 __device__ __forceinline__ int scatter_orbit(const StepParams& p, const double x0[3], const double beta[3],
                                              const double w[3], double* J) {
-    if constexpr (QUAD == 0) {
-        CellStart<double> st;
-        cell_start(x0, p.m, st);
-        return scatter_closed(p, st, beta, w, J);
-    } else {
-        if (p.split) {
-            if (p.order == 2) return scatter_pieces<2>(p, x0, beta, w, J);
-            if (p.order == 3) return scatter_pieces<3>(p, x0, beta, w, J);
-            return scatter_pieces<1>(p, x0, beta, w, J);
-        }
-        if (p.order == 2) return scatter_gauss_r<2>(p, x0, beta, w, J);
-        if (p.order == 3) return scatter_gauss_r<3>(p, x0, beta, w, J);
-        return scatter_gauss(p, x0, beta, w, J);
+    if (p.split) {
+        if (p.order == 2) return scatter_pieces<2>(p, x0, beta, w, J);
+        if (p.order == 3) return scatter_pieces<3>(p, x0, beta, w, J);
+        return scatter_pieces<1>(p, x0, beta, w, J);
     }
+    if (p.order == 2) return scatter_gauss_r<2>(p, x0, beta, w, J);
+    if (p.order == 3) return scatter_gauss_r<3>(p, x0, beta, w, J);
+    return scatter_gauss(p, x0, beta, w, J);
 }
 
 // ---- push (Eq. (orbit-push)) -------------------------------------------------------
@@ -359,79 +326,6 @@ struct PushAcc {
     double DAv[3];    // (D_i A) vbar, diagnostics only
     double pu;        // sum_g Sbar_ig, diagnostics only
 };
-
-template <bool DIAG>
-__device__ __forceinline__ void push_piece_closed(const StepParams& p, const Segment<double>& sg, const double beta[3],
-                                                  const double vb[3], const double* __restrict__ table, PushAcc& acc) {
-    double I[8];
-    int64_t g[8];
-    segment_weights8(sg, beta, I);
-    segment_nodes8(sg, p.m, g);
-    const double s = sg.s0, h = sg.h;
-    double am[8], cc[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const double* t = table + 12 * g[k];
-        double an = t[0] * vb[0] + t[1] * vb[1] + t[2] * vb[2];   // A^n_g . vbar
-        double a1 = t[3] * vb[0] + t[4] * vb[1] + t[5] * vb[2];   // A^{n+1}_g . vbar
-        am[k] = (1.0 - s) * an + s * a1;                          // A^{(m)}_nu . vbar
-        cc[k] = a1 - an;                                          // C^{(m)}_nu . vbar
-        acc.gphi[0] += I[k] * t[6];
-        acc.gphi[1] += I[k] * t[7];
-        acc.gphi[2] += I[k] * t[8];
-        if constexpr (DIAG) {
-            acc.Ubar[0] += I[k] * t[9];
-            acc.Ubar[1] += I[k] * t[10];
-            acc.Ubar[2] += I[k] * t[11];
-            acc.pu += I[k];
-        }
-    }
-    AxisPoly<double> px = axis_poly(sg.r[0], beta[0]);
-    AxisPoly<double> py = axis_poly(sg.r[1], beta[1]);
-    AxisPoly<double> pz = axis_poly(sg.r[2], beta[2]);
-    // transverse integrals T0, T1 per derivative direction j and transverse offsets
-    double t0x[4], t1x[4], t0y[4], t1y[4], t0z[4], t1z[4];
-#pragma unroll
-    for (int b = 0; b < 2; ++b)
-#pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            transverse_integrals(quad_product(py.L[a], py.M[a], pz.L[b], pz.M[b]), h, t0x[a + 2 * b], t1x[a + 2 * b]);
-            transverse_integrals(quad_product(px.L[a], px.M[a], pz.L[b], pz.M[b]), h, t0y[a + 2 * b], t1y[a + 2 * b]);
-            transverse_integrals(quad_product(px.L[a], px.M[a], py.L[b], py.M[b]), h, t0z[a + 2 * b], t1z[a + 2 * b]);
-        }
-    // [(D A)^T vbar]_j = sum_nu (sigma_{nu_j} / H_j) (A^{(m)}_nu.vbar T0 + C_nu.vbar T1)
-#pragma unroll
-    for (int b = 0; b < 2; ++b)
-#pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            int k;
-            k = 2 * a + 4 * b;  // nu = (0, a, b) vs (1, a, b)
-            acc.F[0] += p.invH[0] * (t0x[a + 2 * b] * (am[k + 1] - am[k]) + t1x[a + 2 * b] * (cc[k + 1] - cc[k]));
-            k = a + 4 * b;      // nu = (a, 0, b) vs (a, 1, b)
-            acc.F[1] += p.invH[1] * (t0y[a + 2 * b] * (am[k + 2] - am[k]) + t1y[a + 2 * b] * (cc[k + 2] - cc[k]));
-            k = a + 2 * b;      // nu = (a, b, 0) vs (a, b, 1)
-            acc.F[2] += p.invH[2] * (t0z[a + 2 * b] * (am[k + 4] - am[k]) + t1z[a + 2 * b] * (cc[k + 4] - cc[k]));
-        }
-    if constexpr (DIAG) {
-        // [(D A) vbar]_l = sum_nu (A^{(m)}_{l nu} G0_nu + C_{l nu} G1_nu),
-        // G_nu = sum_j sigma_{nu_j} vbar_j / H_j * T_j(transverse of nu)
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int nx = k & 1, ny = (k >> 1) & 1, nz = (k >> 2) & 1;
-            const double sx = nx ? 1.0 : -1.0, sy = ny ? 1.0 : -1.0, sz = nz ? 1.0 : -1.0;
-            double G0 = sx * p.invH[0] * vb[0] * t0x[ny + 2 * nz] + sy * p.invH[1] * vb[1] * t0y[nx + 2 * nz] +
-                        sz * p.invH[2] * vb[2] * t0z[nx + 2 * ny];
-            double G1 = sx * p.invH[0] * vb[0] * t1x[ny + 2 * nz] + sy * p.invH[1] * vb[1] * t1y[nx + 2 * nz] +
-                        sz * p.invH[2] * vb[2] * t1z[nx + 2 * ny];
-            const double* t = table + 12 * g[k];
-#pragma unroll
-            for (int l = 0; l < 3; ++l) {
-                double Am = (1.0 - s) * t[l] + s * t[3 + l];
-                acc.DAv[l] += Am * G0 + (t[3 + l] - t[l]) * G1;
-            }
-        }
-    }
-}
 
 template <bool DIAG>
 __device__ __forceinline__ void push_piece_gauss(const StepParams& p, const Segment<double>& sg, const double x0[3],
@@ -675,7 +569,6 @@ __global__ void k_point_deposit(StepParams p, const double* __restrict__ xi, dou
 
 // v^{n+1,0} = 2 v^n - v^{n-1} (Algorithm 1, extrapolated start) unless an iterate is given;
 // then the orbit current of that iterate, and sum_i |v^n_i| for the e_J floor.
-template <int QUAD>
 __global__ void k_first_scatter(StepParams p, const double* __restrict__ xi, const double* __restrict__ v,
                                 const double* __restrict__ vprev, const double* __restrict__ vgiven,
                                 double* __restrict__ vit, double* __restrict__ J, double* __restrict__ partials,
@@ -716,7 +609,7 @@ __global__ void k_first_scatter(StepParams p, const double* __restrict__ xi, con
                 beta[a] = p.dt * vb * p.invH[a];
                 w[a] = p.q_dV * vb;
             }
-            if (scatter_orbit<QUAD>(p, x0, beta, w, J) < 0) atomicOr(status, DEV_ERR_SEGMENTS);
+            if (scatter_orbit(p, x0, beta, w, J) < 0) atomicOr(status, DEV_ERR_SEGMENTS);
         }
         __syncthreads();   // order[] is rewritten by the next chunk
     }
@@ -744,7 +637,7 @@ struct PushOut {
 // G(u): the Algorithm 1 push of one particle for the end-of-step iterate u with the
 // current mesh table: orbit vbar = (u + v^n)/2, P^{n+1} (Eq. (orbit-P-update)),
 // x^{n+1} (Eq. (orbit-x-update)) and v^{n+1} = (P^{n+1} - q A_h^{n+1}(x^{n+1})) / m.
-template <int QUAD, bool DIAG>
+template <bool DIAG>
 __device__ __forceinline__ void push_eval(const StepParams& p, const double x0[3], const double vn[3],
                                           const double Pn[3], const double u[3], const double* __restrict__ table,
                                           PushAcc& acc, PushOut& o) {
@@ -755,26 +648,20 @@ __device__ __forceinline__ void push_eval(const StepParams& p, const double x0[3
         beta[a] = p.dt * vb[a] * p.invH[a];
     }
     acc = PushAcc{};
-    if constexpr (QUAD == 0) {
-        o.nseg = for_each_segment(x0, beta, true, [&](const Segment<double>& sg) {
-            push_piece_closed<DIAG>(p, sg, beta, vb, table, acc);
+    if (p.split) {
+        CellStart<double> st;
+        knot_start(p, x0, st);
+        o.nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
+            if (p.order == 2) push_piece_points<2, DIAG>(p, h, sm, mid, c, beta, vb, table, acc);
+            else if (p.order == 3) push_piece_points<3, DIAG>(p, h, sm, mid, c, beta, vb, table, acc);
+            else push_piece_points<1, DIAG>(p, h, sm, mid, c, beta, vb, table, acc);
         });
     } else {
-        if (p.split) {
-            CellStart<double> st;
-            knot_start(p, x0, st);
-            o.nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
-                if (p.order == 2) push_piece_points<2, DIAG>(p, h, sm, mid, c, beta, vb, table, acc);
-                else if (p.order == 3) push_piece_points<3, DIAG>(p, h, sm, mid, c, beta, vb, table, acc);
-                else push_piece_points<1, DIAG>(p, h, sm, mid, c, beta, vb, table, acc);
-            });
-        } else {
-            o.nseg = for_each_segment(x0, beta, false, [&](const Segment<double>& sg) {
-                if (p.order == 2) push_piece_gauss_r<2, DIAG>(p, sg, x0, beta, vb, table, acc);
-                else if (p.order == 3) push_piece_gauss_r<3, DIAG>(p, sg, x0, beta, vb, table, acc);
-                else push_piece_gauss<DIAG>(p, sg, x0, beta, vb, table, acc);
-            });
-        }
+        o.nseg = for_each_segment(x0, beta, false, [&](const Segment<double>& sg) {
+            if (p.order == 2) push_piece_gauss_r<2, DIAG>(p, sg, x0, beta, vb, table, acc);
+            else if (p.order == 3) push_piece_gauss_r<3, DIAG>(p, sg, x0, beta, vb, table, acc);
+            else push_piece_gauss<DIAG>(p, sg, x0, beta, vb, table, acc);
+        });
     }
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -786,7 +673,7 @@ __device__ __forceinline__ void push_eval(const StepParams& p, const double x0[3
     for (int a = 0; a < 3; ++a) o.vw[a] = (o.Pw[a] - p.q * o.Ae[a]) * p.inv_mass;
 }
 
-// G(u) of the closed forms without diagnostics, from the start (cell, coordinate) and vs = u + v^n =
+// G(u) of the closed forms, from the start (cell, coordinate) and vs = u + v^n =
 // 2 vbar: in fixed point from the cell tables (FIXED), or from the gather table in FP64.
 struct CellOut {
     double Pw[3], Ae[3], vw[3];
@@ -1028,6 +915,178 @@ __global__ void __launch_bounds__(32 * WARPS, PUSH_WARPS / WARPS) k_push_cell(St
     }
 }
 
+// One piece of an orbit for the final sweep with diagnostics: piece_impulse's two integrals apart, and
+// those of the identities, (D A) vbar and the gather of U, per particle.
+struct DiagAcc {
+    double F[3], g[3];        // (D_j A)^T vbar and -grad phi
+    double DAv[3], U[3], pu;  // (D A) vbar, U^{n+1/2}, sum of the weights
+};
+
+// vh_j = vbar_j / H_j; `ld` as for piece_impulse; U from the gather table's rows g (columns 9 to 11).
+template <typename L>
+__device__ __forceinline__ void piece_diag(double h, double sm, const double mid[3], const double beta[3],
+                                           const double vs[3], const double ihs[3], const double vh[3], L&& ld,
+                                           const double* __restrict__ table, const int64_t g[8], DiagAcc& acc) {
+    const PieceMoments<double> q = piece_moments(h, mid, beta);
+    const double nms = sm - 1.0;
+    {
+        double W[8], u[3] = {0.0, 0.0, 0.0}, sum = 0.0;
+        node_weights(q, W);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const double* t = table + 12 * g[k] + 9;
+            sum += W[k];
+#pragma unroll
+            for (int j = 0; j < 3; ++j) u[j] += W[k] * __ldg(t + j);
+        }
+        acc.pu += h * sum;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) acc.U[j] += h * u[j];
+    }
+    const double M[8] = {1.0, mid[0], mid[1], q.Pxy, mid[2], q.Pxz, q.Pyz, q.S};
+    const double E[8] = {0.0, q.e[0], q.e[1], mid[0] * q.e[1] + mid[1] * q.e[0],
+                         q.e[2], mid[0] * q.e[2] + mid[2] * q.e[0], mid[1] * q.e[2] + mid[2] * q.e[1], 0.0};
+    double F[3] = {0.0, 0.0, 0.0}, gg[3] = {0.0, 0.0, 0.0}, D[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        double x[3][2], d[3][2], y[3][2];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            ld(p, j, x[j][0], x[j][1]);
+            ld(p, 3 + j, d[j][0], d[j][1]);
+            ld(p, 6 + j, y[j][0], y[j][1]);
+        }
+#pragma unroll
+        for (int o = 0; o < 2; ++o) {
+            const int k = 2 * p + o;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) gg[j] += y[j][o] * M[k];
+            if (k == 0) continue;
+            double am[3], a = 0.0, cc = 0.0, dk = 0.0, ek = 0.0;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                am[j] = x[j][o] + nms * d[j][o];   // A_k at s_mid
+                a += am[j] * vs[j];
+                cc += d[j][o] * vs[j];
+                if ((k >> j) & 1) {
+                    dk += vh[j] * M[k ^ (1 << j)];
+                    if ((k ^ (1 << j)) != 0) ek += vh[j] * E[k ^ (1 << j)];
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                if ((k >> j) & 1) F[j] += a * M[k ^ (1 << j)] + cc * E[k ^ (1 << j)];
+                D[j] += am[j] * dk + d[j][o] * ek;
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        acc.F[j] += h * ihs[j] * F[j];
+        acc.g[j] += h * gg[j];
+        acc.DAv[j] += h * D[j];
+    }
+}
+
+// The closed forms' final sweep with the particle diagnostics, in the centred form of k_push_cell
+// (FP64; CELLS: from the cell table).  Bound by the FP64 pipe like that: some 240 operations a piece where
+// the integrals from the piece's start took some 700: 1.62 ms at 50 x 35 x 22 with 539,000 particles, now
+// 0.68.
+constexpr int DIAG_WARPS = 12;
+template <bool CELLS, int WARPS, int ITEMS>
+__global__ void __launch_bounds__(32 * WARPS, DIAG_WARPS / WARPS) k_commit_diag(
+    StepParams p, const double* __restrict__ xi, const double* __restrict__ v, const double* __restrict__ P,
+    const double* __restrict__ vit, const double* __restrict__ table, const double* __restrict__ ctab,
+    double* __restrict__ vnew, double* __restrict__ xi_out, double* __restrict__ P_out,
+    const uint8_t* __restrict__ slide, double* __restrict__ partials, int* __restrict__ status) {
+    __shared__ double sm[32];
+    extern __shared__ __align__(16) unsigned char dyn[];
+    typedef ChunkOrder<WARPS, ITEMS> Chunk;
+    Chunk& co = Chunk::in(dyn);
+    const int64_t np = p.np, nchunks = (np + Chunk::SIZE - 1) / Chunk::SIZE;
+    double ev_num = 0.0, ev_den = 0.0, k1 = 0.0, pwork = 0.0, ra_sq = 0.0, ra_max = 0.0, pu_max = 0.0;
+    for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
+        const int64_t base = ch * Chunk::SIZE;
+        chunk_exchange(p, co, base, [&](int64_t j, double x0[3], double v2[3]) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                x0[a] = xi[a * np + j];
+                v2[a] = vit[a * np + j] + v[a * np + j];
+            }
+        });
+#pragma unroll 1
+        for (int it = 0; it < ITEMS; ++it) {
+            CellStart<double> st;
+            double vs[3];
+            const int64_t i = co.take(it, base, st, vs);
+            if (i >= np) continue;
+            double beta[3], vh[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                beta[a] = p.cb[a] * vs[a];
+                vh[a] = vs[a] * p.ihs[a];
+            }
+            DiagAcc acc{};
+            const int nseg = for_each_piece(st, beta, p.m, [&](double h, double s, const double mid[3], const int c[3]) {
+                int64_t g[8];
+                cell_nodes8(c, p.m, g);
+                piece_diag(h, s, mid, beta, vs, p.ihs, vh, FieldLoad<CELLS>(CELLS ? ctab : table, c, p.m), table, g, acc);
+            });
+            if (nseg < 0) atomicOr(status, DEV_ERR_SEGMENTS);
+            double Ae[3], As[3], x0[3], ra2 = 0.0;
+            cell_A1(st.f, FieldLoad<CELLS>(CELLS ? ctab : table, st.c, p.m), Ae);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) x0[a] = xi[a * np + i];
+            {   // A_h^n(x^n)
+                double w[8];
+                int64_t g[8];
+                point_weights8(x0, p.m, g, w);
+                As[0] = As[1] = As[2] = 0.0;
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) As[a] += w[k] * __ldg(table + 12 * g[k] + a);
+            }
+            const uint8_t sb = slide ? slide[i] : 0;
+            bool finite = true;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                const double vi = vit[a * np + i];
+                double Pw = P[a * np + i] + p.dt * (p.q * acc.g[a] + p.q * acc.F[a]);
+                double vw = (Pw - p.q * Ae[a]) * p.inv_mass;
+                finite = finite && isfinite(vw);
+                // components sliding onto a knot, as in k_push_cell
+                if (sb & (1u << a)) {
+                    vw = vi;
+                    Pw = p.mass * vw + p.q * Ae[a];
+                }
+                vnew[a * np + i] = vw;
+                xi_out[a * np + i] = wrap_pos(x0[a] + beta[a], (double)p.m.n[a]);
+                P_out[a * np + i] = Pw;
+                const double d = vw - vi;
+                ev_num += d * d;
+                ev_den += vw * vw;
+                const double ra = Ae[a] - As[a] - p.dt * (acc.U[a] + acc.DAv[a]);        // Eq. (RA-test)
+                ra2 += ra * ra;
+                ra_max = fmax(ra_max, fabs(ra));
+                pwork += p.q * (0.5 * vs[a]) * (acc.g[a] - acc.U[a]);                     // q vbar . Ebar
+                k1 += 0.5 * p.mass * vw * vw;
+            }
+            if (!finite) atomicOr(status, DEV_ERR_NONFINITE);
+            ra_sq += ra2;
+            pu_max = fmax(pu_max, fabs(acc.pu - 1.0));
+        }
+        __syncthreads();   // the hand-over buffers are rewritten by the next chunk
+    }
+    write_partial<double>(partials, S_EV_NUM, ev_num, sm, false);
+    write_partial<double>(partials, S_EV_DEN, ev_den, sm, false);
+    write_partial<double>(partials, S_K1, k1, sm, false);
+    write_partial<double>(partials, S_PWORK, pwork, sm, false);
+    write_partial<double>(partials, S_RA_SQ, ra_sq, sm, false);
+    write_partial<double>(partials, S_RA_MAX, ra_max, sm, true);
+    write_partial<double>(partials, S_PU_MAX, pu_max, sm, true);
+}
+
 // The Algorithm 1 push for iterate vit, then either
 //   (iterate)  the next iterate and its orbit current into Jnext, plus the e_v partial sums.
 //              The next iterate is G(v^p); with p.accel, creeping particles are instead
@@ -1036,7 +1095,7 @@ __global__ void __launch_bounds__(32 * WARPS, PUSH_WARPS / WARPS) k_push_cell(St
 // Two resident blocks per SM (at most 128 registers, a few spills) hide more of the FP64
 // pipe's latency than one block at 178 registers (measured: 5% less push time at 32^3); the
 // diagnostics variant keeps one block, its larger state would spill far more.
-template <int QUAD, bool COMMIT, bool DIAG>
+template <bool COMMIT, bool DIAG>
 __global__ void __launch_bounds__(THREADS, DIAG ? 1 : 2) k_push(StepParams p, const double* __restrict__ xi,
                                                   const double* __restrict__ v, const double* __restrict__ P,
                                                   const double* __restrict__ vit, const double* __restrict__ table,
@@ -1076,7 +1135,7 @@ __global__ void __launch_bounds__(THREADS, DIAG ? 1 : 2) k_push(StepParams p, co
             }
             PushAcc acc;
             PushOut o;
-            push_eval<QUAD, DIAG>(p, x0, vn, Pn, vi, table, acc, o);
+            push_eval<DIAG>(p, x0, vn, Pn, vi, table, acc, o);
             if (o.nseg < 0) atomicOr(status, DEV_ERR_SEGMENTS);
             pieces_push += (double)o.nseg;
             if (!(isfinite(o.vw[0]) && isfinite(o.vw[1]) && isfinite(o.vw[2]))) atomicOr(status, DEV_ERR_NONFINITE);
@@ -1129,7 +1188,7 @@ __global__ void __launch_bounds__(THREADS, DIAG ? 1 : 2) k_push(StepParams p, co
                     }
                     ev_num += dnum;
                     ev_den += dden;
-                    int ns = scatter_orbit<QUAD>(p, x0, bet2, wv, Jnext);
+                    int ns = scatter_orbit(p, x0, bet2, wv, Jnext);
                     if (ns < 0) atomicOr(status, DEV_ERR_SEGMENTS);
                     pieces_scatter += (double)ns;
                 }
@@ -1702,7 +1761,7 @@ __global__ void __launch_bounds__(THREADS, LOCAL_MINB) k_local(StepParams p, con
                 else if (p.order == 3) ns = scatter_pieces<3>(p, x0, beta, w, Jnext, k, LANES);
                 else ns = scatter_pieces<1>(p, x0, beta, w, Jnext, k, LANES);
             } else {
-                ns = k == 0 ? scatter_orbit<QUAD>(p, x0, beta, w, Jnext) : 0;
+                ns = k == 0 ? scatter_orbit(p, x0, beta, w, Jnext) : 0;
             }
             if (ns < 0) atomicOr(status, DEV_ERR_SEGMENTS);
             active = false;
@@ -2031,7 +2090,7 @@ void launch_first_scatter(Ctx& c, double* J, const double* v_iter_or_null) {
         k_first_scatter_cell<4, 2><<<chunk_blocks(c), 128, ChunkLarge::smem(), c.stream>>>(
             p, c.xi, c.v, c.vprev, v_iter_or_null, c.vit, J, c.partials, c.dev_status);
     else
-        k_first_scatter<1><<<nb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.vprev, v_iter_or_null, c.vit, J, c.partials,
+        k_first_scatter<<<nb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.vprev, v_iter_or_null, c.vit, J, c.partials,
                                                          c.dev_status);
     ++c.launches;
     if (c.cfg.deterministic) launch_exact_finish(c, J, 3 * c.m.ncell, c.inv_u_J);
@@ -2044,8 +2103,8 @@ void launch_push(Ctx& c, const double* vit, double* vnew, double* Jnext, bool co
     const bool det = c.cfg.deterministic && !commit;
     const bool closed = c.closed;
     if (!commit) cudaMemsetAsync(c.creep_count, 0, 2 * sizeof(int), c.stream);   // count, k_local queue head
-#define PIC_PUSH(Q, C, D)                                                                                        \
-    k_push<Q, C, D><<<nb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.P, vit, c.table, vnew, Jnext, c.xi_new, c.P_new, \
+#define PIC_PUSH(C, D)                                                                                           \
+    k_push<C, D><<<nb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.P, vit, c.table, vnew, Jnext, c.xi_new, c.P_new, \
                                                   c.creep_list, c.creep_count, det ? c.creep_flag : nullptr,  \
                                                   c.slide,                                                    \
                                                   c.partials, c.dev_status)
@@ -2061,7 +2120,15 @@ void launch_push(Ctx& c, const double* vit, double* vnew, double* Jnext, bool co
         if (small) PIC_PUSH_CELL_AS(C, T, 1, 1); \
         else PIC_PUSH_CELL_AS(C, T, 4, 2);       \
     } while (0)
-    if (closed && !diag) {
+#define PIC_COMMIT_DIAG(T, W, I)                                                                                  \
+    k_commit_diag<T, W, I><<<chunk_blocks(c), 32 * W, sizeof(ChunkOrder<W, I>), c.stream>>>(                        \
+        p, c.xi, c.v, c.P, vit, c.table, c.ctab, vnew, c.xi_new, c.P_new, c.slide, c.partials, c.dev_status)
+    if (closed && diag) {   // (commit)
+        if (c.ctab && small) PIC_COMMIT_DIAG(true, 1, 1);
+        else if (c.ctab) PIC_COMMIT_DIAG(true, 4, 2);
+        else if (small) PIC_COMMIT_DIAG(false, 1, 1);
+        else PIC_COMMIT_DIAG(false, 4, 2);
+    } else if (closed) {
         if (commit) {
             if (c.fxtab) PIC_PUSH_CELL(true, true);
             else PIC_PUSH_CELL(true, false);
@@ -2070,13 +2137,13 @@ void launch_push(Ctx& c, const double* vit, double* vnew, double* Jnext, bool co
             else PIC_PUSH_CELL(false, false);
         }
     } else if (!commit) {
-        PIC_PUSH(1, false, false);
+        PIC_PUSH(false, false);
     } else if (!diag) {
-        PIC_PUSH(1, true, false);
+        PIC_PUSH(true, false);
     } else {
-        if (closed) PIC_PUSH(0, true, true);
-        else PIC_PUSH(1, true, true);
+        PIC_PUSH(true, true);
     }
+#undef PIC_COMMIT_DIAG
 #undef PIC_PUSH
 #undef PIC_PUSH_CELL
 #undef PIC_PUSH_CELL_AS

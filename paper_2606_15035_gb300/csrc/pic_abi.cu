@@ -918,8 +918,8 @@ void final_issue(Ctx& c) {
         launch_push(c, c.vit, c.vnew, nullptr, true, diag);
     }
     if (diag) {
-        launch_finalize(c, S_K1, 3, particle_blocks(c), false);   // K1, PWORK, RA_SQ
-        launch_finalize(c, S_RA_MAX, 2, particle_blocks(c), true);
+        launch_finalize(c, S_K1, 3, push_blocks(c), false);   // K1, PWORK, RA_SQ
+        launch_finalize(c, S_RA_MAX, 2, push_blocks(c), true);
         if (c.cfg.ops == PIC_OPS_SPECTRAL) launch_spec_diag(c, Jfin);
         else launch_mesh_diag(c, Jfin);
         launch_finalize(c, S_MWORK, 2, mesh_blocks(c), false);    // MWORK, W

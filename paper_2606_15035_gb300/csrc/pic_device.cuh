@@ -132,73 +132,6 @@ __device__ __forceinline__ int for_each_segment(const T xi0[3], const T beta[3],
     return -1;
 }
 
-// Per-axis linear weights on a piece: w_{a,0}(eta) = L0 + M0 eta, w_{a,1} = L1 + M1 eta,
-// with L0 = 1 - r, M0 = -beta, L1 = r, M1 = beta (Appendix A).
-template <typename T>
-struct AxisPoly {
-    T L[2], M[2];
-};
-
-template <typename T>
-__device__ __forceinline__ AxisPoly<T> axis_poly(T r, T beta) {
-    AxisPoly<T> p;
-    p.L[0] = T(1) - r;
-    p.M[0] = -beta;
-    p.L[1] = r;
-    p.M[1] = beta;
-    return p;
-}
-
-// Quadratic product (La + Ma eta)(Lb + Mb eta) = d0 + d1 eta + d2 eta^2.
-template <typename T>
-struct Quad {
-    T d0, d1, d2;
-};
-
-template <typename T>
-__device__ __forceinline__ Quad<T> quad_product(T La, T Ma, T Lb, T Mb) {
-    Quad<T> q;
-    q.d0 = La * Lb;
-    q.d1 = Ma * Lb + La * Mb;
-    q.d2 = Ma * Mb;
-    return q;
-}
-
-// I_nu = int_0^h (c0 + c1 eta + c2 eta^2 + c3 eta^3) d eta with the cubic being the
-// product of a quadratic (two axes) and a linear factor (third axis) (Appendix A).
-template <typename T>
-__device__ __forceinline__ T segment_weight(const Quad<T>& q, T L, T M, T h) {
-    T c0 = q.d0 * L;
-    T c1 = q.d1 * L + q.d0 * M;
-    T c2 = q.d2 * L + q.d1 * M;
-    T c3 = q.d2 * M;
-    return h * (c0 + h * (c1 * T(0.5) + h * (c2 * (T(1) / T(3)) + h * (c3 * T(0.25)))));
-}
-
-// The two bracketed integrals of I^D (Appendix B) for a transverse quadratic d:
-// T0 = int_0^h d(eta) d eta, T1 = int_0^h eta d(eta) d eta.
-template <typename T>
-__device__ __forceinline__ void transverse_integrals(const Quad<T>& q, T h, T& t0, T& t1) {
-    t0 = h * (q.d0 + h * (q.d1 * T(0.5) + h * (q.d2 * (T(1) / T(3)))));
-    t1 = h * h * (q.d0 * T(0.5) + h * (q.d1 * (T(1) / T(3)) + h * (q.d2 * T(0.25))));
-}
-
-// Eight closed-form weights I_nu of one piece, nu = nx + 2 ny + 4 nz (Appendix A).
-template <typename T>
-__device__ __forceinline__ void segment_weights8(const Segment<T>& sg, const T beta[3], T I[8]) {
-    AxisPoly<T> px = axis_poly(sg.r[0], beta[0]);
-    AxisPoly<T> py = axis_poly(sg.r[1], beta[1]);
-    AxisPoly<T> pz = axis_poly(sg.r[2], beta[2]);
-#pragma unroll
-    for (int ny = 0; ny < 2; ++ny)
-#pragma unroll
-        for (int nx = 0; nx < 2; ++nx) {
-            Quad<T> qxy = quad_product(px.L[nx], px.M[nx], py.L[ny], py.M[ny]);
-#pragma unroll
-            for (int nz = 0; nz < 2; ++nz) I[nx + 2 * ny + 4 * nz] = segment_weight(qxy, pz.L[nz], pz.M[nz], sg.h);
-        }
-}
-
 // Base integrals of one piece.  With w_a(eta) = r_a + beta_a eta the "upper" linear weight
 // of axis a (w_{a,1} of Appendix A; w_{a,0} = 1 - w_a):
 //   S1[a] = int_0^h w_a,   E1[a] = int_0^h eta w_a,

@@ -377,7 +377,7 @@ bool setup_particle_kernels();
 bool setup_pair_kernels();
 int particle_blocks(const Ctx& c);
 int chunk_blocks(const Ctx& c);   // the closed forms' chunk kernels
-int push_blocks(const Ctx& c);    // the pushes without diagnostics and the first scatter
+int push_blocks(const Ctx& c);    // the pushes and the first scatter
 int local_blocks(const Ctx& c);
 int mesh_blocks(const Ctx& c);
 

@@ -38,29 +38,34 @@ def _edge_particles(n, npart, seed):
     return x, np.clip(b, 0.5 - n, n - 0.5)                    # less than one box length
 
 
+def _refuse_cell_tables(sim, monkeypatch, n):
+    """Contexts get no cell tables from now on; the list of the requests refused."""
+    refused = []
+    want = 576 * n[0] * n[1] * n[2]
+    base = sim._TorchAllocator
+
+    class Refusing(base):
+        def __init__(self, device):
+            super().__init__(device)
+            inner = self._alloc_cb
+
+            def alloc(nbytes, stream, user):
+                if nbytes == want:
+                    refused.append(nbytes)
+                    return None
+                return inner(nbytes, stream, user)
+
+            self._outer_cb = sim._lib.ALLOC_FN(alloc)
+            self.struct = sim.PicAllocator(self._outer_cb, self._free_cb, None)
+
+    monkeypatch.setattr(sim, "_TorchAllocator", Refusing)
+    return refused
+
+
 @pytest.mark.parametrize("n", [(8, 8, 8), (2, 5, 3), (9, 2, 4)])
 @pytest.mark.parametrize("table", ["cells", "nodes"])
 def test_one_body_matches_oracle_at_the_edges(sim, monkeypatch, n, table):
-    refused = []
-    if table == "nodes":
-        want = 576 * n[0] * n[1] * n[2]
-        base = sim._TorchAllocator
-
-        class Refusing(base):
-            def __init__(self, device):
-                super().__init__(device)
-                inner = self._alloc_cb
-
-                def alloc(nbytes, stream, user):
-                    if nbytes == want:
-                        refused.append(nbytes)
-                        return None
-                    return inner(nbytes, stream, user)
-
-                self._outer_cb = sim._lib.ALLOC_FN(alloc)
-                self.struct = sim.PicAllocator(self._outer_cb, self._free_cb, None)
-
-        monkeypatch.setattr(sim, "_TorchAllocator", Refusing)
+    refused = _refuse_cell_tables(sim, monkeypatch, n) if table == "nodes" else []
     L = tuple(float(k) for k in n)
     x, b = _edge_particles(np.asarray(n), 1601, 40 + n[0])
     v = 0.3 * b[::-1].copy()
@@ -86,6 +91,37 @@ def test_one_body_matches_oracle_at_the_edges(sim, monkeypatch, n, table):
     d = g["x"] - it["xi"] * np.asarray(ocfg.grid().H)
     Lv = np.asarray(L)
     assert np.abs((d + 0.5 * Lv) % Lv - 0.5 * Lv).max() <= 1e-14 * Lv.max()
+
+
+@pytest.mark.parametrize("n,npart", [((8, 8, 8), 1601), ((9, 2, 4), 1601), ((6, 5, 4), 39169)])
+@pytest.mark.parametrize("table", ["cells", "nodes"])
+def test_diagnosed_step_at_the_edges(sim, monkeypatch, n, npart, table):
+    """The final sweep with diagnostics, by chunks of one warp and (from 38,913 particles on 152 SMs) of
+    four: the state of the step without them to 1e-12 (other kernels, the same formulas), the particles'
+    work and the mesh's, which are equal, to 100 times that (sums of terms of either sign), and the
+    identities' residuals at rounding: a few dozen terms an orbit, 1e-13 of A."""
+    refused = _refuse_cell_tables(sim, monkeypatch, n) if table == "nodes" else []
+    L = tuple(float(k) for k in n)
+    x, b = _edge_particles(np.asarray(n), npart, 70 + n[0])
+    q = -1e-3 / npart
+    out = []
+    for diagnostics in (0, 1):
+        s = sim.PicSim(sim.pic_config_default(n=n, L=L, dt=1.0, picard_tol=1e-13, diagnostics=diagnostics), x, b, q, 1e-3)
+        assert bool(refused) == (table == "nodes")
+        assert s.step(1).converged
+        out.append((s.get_state(), s.diagnostics() if diagnostics else None))
+        s.close()
+    (o, _), (st, d) = out
+
+    def rel(a, r):
+        return np.linalg.norm(a - r) / max(np.linalg.norm(r), 1e-300)
+
+    for name in ("P", "v", "phi", "psi", "A", "U"):
+        assert rel(getattr(st, name), getattr(o, name)) <= 1e-12, name
+    k1 = 0.5e-3 * np.sum(o.v ** 2)
+    assert abs(d.K1 - k1) <= 1e-12 * k1
+    assert abs(d.particle_work - d.mesh_work) <= 1e-10 * abs(d.mesh_work)
+    assert d.RA_max <= 1e-13 * np.abs(o.A).max() and d.partition_max <= 1e-14
 
 
 @pytest.mark.parametrize("precision", [0, 1])
