@@ -97,7 +97,7 @@ __device__ __forceinline__ double lap_s(const double* __restrict__ f, int64_t g,
 
 // ---- the particles' push, templated on the scalar type (double, or Dual for derivatives) -----
 //
-// The same formulas as the FP64 push (push_piece_fast, push_eval and scatter_closed): the
+// The formulas of the FP64 push from a piece's start (k_adj_blocks differentiates them by dual numbers): the
 // orbit gather of grad phi, (D_i A)^T vbar contracted with vbar first, the end point's
 // A_h^{n+1}, and the orbit weights of the current.  Positions are in cell units.
 
@@ -199,78 +199,195 @@ __device__ __forceinline__ void out_adjoints(const StepParams& p, bool sl, doubl
     }
 }
 
-__global__ void k_adj_scatter(AdjParams ap, const double* __restrict__ xi, const double* __restrict__ v,
-                              const double* __restrict__ vstar, const double* __restrict__ table,
-                              const double* __restrict__ lam_P, const double* __restrict__ lam_v,
-                              const double* __restrict__ mu, const uint8_t* __restrict__ slide,
-                              double* __restrict__ lam_tab) {
+// Per orbit piece the transposes of piece_impulse (orbit_cell.cuh) on the mixed differences of A^{n+1},
+// A^n and grad phi, 8 subsets of the axes and 3 components each, and of the interpolant of A^{n+1} at the
+// end point.  Every particle's 72 terms a piece went to the mesh by atomics, 96 L2 reductions a particle
+// and more, which bounded the kernel (0.80 ms at 32^3 with 524,288 particles).  As in scatter_warp the
+// warp's particles are summed per cell first, in 64-bit fixed point (values to 2^-57 of the warp's
+// largest), three tiles a piece, and turned into node values once per cell: 0.43 ms.
+__device__ __forceinline__ void plain_rows(double* __restrict__ col, const int c[3], const MeshDims& m, const double M[8],
+                                           const double w[3]) {
+    double W[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) W[k] = M[k];
+#pragma unroll
+    for (int bit = 1; bit < 8; bit <<= 1)
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (!(k & bit)) W[k] -= W[k | bit];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) atomicAdd(col + 9 * subset_node(c, k, m) + a, w[a] * W[k]);
+}
+
+__global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_scatter(
+    AdjParams ap, const double* __restrict__ xi, const double* __restrict__ v, const double* __restrict__ vstar,
+    const double* __restrict__ lam_P, const double* __restrict__ lam_v, const double* __restrict__ mu,
+    const uint8_t* __restrict__ slide, double* __restrict__ lam_tab) {
+    extern __shared__ __align__(16) unsigned char dyn[];
+    ChunkLarge& co = ChunkLarge::in(dyn);
+    long long* tile = ChunkLarge::tile(dyn);
     const StepParams& p = ap.p;
-    const int64_t np = p.np;
-    ADJ_LOOP(i, np) {
-        double x0[3], beta[3], vb[3], lP1[3], lAe[3], lg[3], lF[3];
-        const uint8_t sb = slide[i];
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, comp = min(lane >> 3, 2);
+    const int64_t np = p.np, nchunks = (np + ChunkLarge::SIZE - 1) / ChunkLarge::SIZE;
+    if (lane < DEPOSIT_ROWS) tile[lane * DEPOSIT_STRIDE + 32] = 0;
+    auto top_of = [&](double x) { return (int)__reduce_max_sync(full, (unsigned)exponent_of(x)); };
+    // the tile's sums per cell into column `col` of lam_tab, their unit 2^(e0 + e1 - 2046) as two factors
+    auto flush = [&](bool has, const int c[3], int col, int e0, int e1) {
+        const double u0 = pow2_biased(e0), u1 = pow2_biased(e1);
+        __syncwarp();
+        tile_sums(has, has ? (int)cell_row(c, p.m) : -1, c, tile, [&](long long sum, const int c0[3]) {
+            double x = (double)sum;
+#pragma unroll
+            for (int bit = 1; bit < 8; bit <<= 1) {
+                const double o = __shfl_xor_sync(full, x, bit);
+                if (!(lane & bit)) x -= o;
+            }
+            if (lane < DEPOSIT_ROWS) atomicAdd(lam_tab + 9 * subset_node(c0, lane, p.m) + col + comp, x * u0 * u1);
+        });
+        __syncwarp();
+    };
+    // rows (a, k) = w_a M_k, w given at 2^(-top - 56 + 1023), M at 2^-62
+    auto rows = [&](const long long w[3], const long long M[8]) {
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            x0[a] = xi[a * np + i];
-            vb[a] = 0.5 * (vstar[a * np + i] + v[a * np + i]);
-            beta[a] = p.dt * vb[a] * p.invH[a];
-            out_adjoints(p, (sb >> a) & 1u, lam_v[a * np + i], lam_P[a * np + i], mu[a * np + i], lP1[a], lAe[a], lg[a],
-                         lF[a]);
+            const Fx ws = fx_split(w[a]);
+            tile[8 * a * DEPOSIT_STRIDE + lane] = w[a];
+#pragma unroll
+            for (int k = 1; k < 8; ++k) tile[(8 * a + k) * DEPOSIT_STRIDE + lane] = fx_mul(ws, fx_split(M[k]));
         }
-        // the end point's interpolant of A^{n+1}, transposed
-        double xe[3];
+    };
+    for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
+        const int64_t base = ch * ChunkLarge::SIZE;
+        chunk_exchange(p, co, base, [&](int64_t j, double x0[3], double v2[3]) {
 #pragma unroll
-        for (int a = 0; a < 3; ++a) xe[a] = wrap_pos(x0[a] + beta[a], (double)p.m.n[a]);
-        {
-            int64_t g[8];
-            double w[8];
-            point_weights8(xe, p.m, g, w);
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-#pragma unroll
-                for (int a = 0; a < 3; ++a) atomicAdd(lam_tab + 9 * g[k] + 3 + a, w[k] * lAe[a]);
-        }
-        // the orbit gather and D_i A, transposed piece by piece
-        for_each_segment(x0, beta, true, [&](const Segment<double>& sg) {
-            const PieceInts<double> I = piece_integrals(sg, beta, true);
-            double W[8];
-            weights_from_ints(I, W);
-            int64_t g[8];
-            segment_nodes8(sg, p.m, g);
-            const double s = sg.s0, h = sg.h, hh2 = 0.5 * h * h;
-            double lam_am[8] = {0, 0, 0, 0, 0, 0, 0, 0}, lam_cc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-#pragma unroll
-            for (int j = 0; j < 3; ++j) {
-                const int pa = j == 0 ? 1 : 0, qa = j == 2 ? 1 : 2;
-                const int sp = j == 0 ? 2 : 1, sq = j == 2 ? 2 : 4;
-                const int sj = j == 0 ? 1 : (j == 1 ? 2 : 4);
-                const double f = p.invH[j] * lF[j];
-                // t0 = sum over transverse corners (a, b) of k0_ab (am[k_ab + sj] - am[k_ab])
-                const double k0[4] = {h - I.S1[pa] - I.S1[qa] + I.S2[j], I.S1[pa] - I.S2[j], I.S1[qa] - I.S2[j], I.S2[j]};
-                const double k1[4] = {hh2 - I.E1[pa] - I.E1[qa] + I.E2[j], I.E1[pa] - I.E2[j], I.E1[qa] - I.E2[j],
-                                      I.E2[j]};
-                const int kb[4] = {0, sp, sq, sp + sq};
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    lam_am[kb[c] + sj] += f * k0[c];
-                    lam_am[kb[c]] -= f * k0[c];
-                    lam_cc[kb[c] + sj] += f * k1[c];
-                    lam_cc[kb[c]] -= f * k1[c];
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const double lan = (1.0 - s) * lam_am[k] - lam_cc[k];   // am = (1-s) an + s a1, cc = a1 - an
-                const double la1 = s * lam_am[k] + lam_cc[k];
-                double* t = lam_tab + 9 * g[k];
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    atomicAdd(t + a, vb[a] * lan);                  // an = A^n . vbar
-                    atomicAdd(t + 3 + a, vb[a] * la1);              // a1 = A^{n+1} . vbar
-                    atomicAdd(t + 6 + a, W[k] * lg[a]);             // gphibar = sum W grad phi
-                }
+            for (int a = 0; a < 3; ++a) {
+                x0[a] = xi[a * np + j];
+                v2[a] = vstar[a * np + j] + v[a * np + j];
             }
         });
+#pragma unroll 1
+        for (int item = 0; item < 2; ++item) {
+            CellStart<double> st;
+            double vs[3], beta[3], bs[3], f[3] = {0.0, 0.0, 0.0}, lg[3] = {0.0, 0.0, 0.0}, lA[3] = {0.0, 0.0, 0.0};
+            const int64_t i = co.take(item, base, st, vs);
+            const bool act = i < np;
+            double fs = 0.0;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                if (act) {
+                    double lP1, lF;
+                    out_adjoints(p, (slide[i] >> a) & 1u, lam_v[a * np + i], lam_P[a * np + i], mu[a * np + i], lP1, lA[a],
+                                 lg[a], lF);
+                    f[a] = lF * p.ihs[a];
+                } else {
+                    vs[a] = 0.0;
+                }
+                beta[a] = p.cb[a] * vs[a];
+                bs[a] = 0.28867513459481288225 * beta[a];   // 1 / sqrt(12)
+                fs += fabs(f[a]);
+            }
+            // |a piece's sums| < 1.2 fs: an exponent above that of fs
+            const int tf = max(top_of(fs), 64) + 1;
+            const int tv = max(max(top_of(vs[0]), max(top_of(vs[1]), top_of(vs[2]))), 64);
+            const int tg = max(max(top_of(lg[0]), max(top_of(lg[1]), top_of(lg[2]))), 64);
+            const int tA = max(max(top_of(lA[0]), max(top_of(lA[1]), top_of(lA[2]))), 64);
+            const bool plain = max(max(tf, tv), max(tg, tA)) >= 0x7ff;   // a value that is not finite goes on as it is
+            Fx vf[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) vf[a] = fx_split(fixed_of(vs[a], tv, 9));
+            PieceWalk<double> wk(st, beta, p.m);
+            bool last = !act;
+            while (__any_sync(full, !last)) {
+                bool has = false;
+                int c[3] = {0, 0, 0};
+                double h = 0.0, sm = 0.0, m[3] = {0.0, 0.0, 0.0};
+                if (!last) has = wk.next(beta, p.m, h, sm, m, c, last);
+                double ab[8], x1[8];   // adjoints of A_k . vs at the piece's middle: all, and A^{n+1}'s share
+                double M[8];
+                if (has) {
+                    const PieceMoments<double> q = piece_moments(h, m, beta);
+                    const double hf[3] = {h * f[0], h * f[1], h * f[2]};
+                    ab[0] = x1[0] = 0.0;
+                    ab[1] = hf[0];
+                    ab[2] = hf[1];
+                    ab[4] = hf[2];
+                    ab[3] = hf[0] * m[1] + hf[1] * m[0];
+                    ab[5] = hf[0] * m[2] + hf[2] * m[0];
+                    ab[6] = hf[1] * m[2] + hf[2] * m[1];
+                    ab[7] = hf[0] * q.Pyz + hf[1] * q.Pxz + hf[2] * q.Pxy;
+                    x1[1] = sm * ab[1];
+                    x1[2] = sm * ab[2];
+                    x1[4] = sm * ab[4];
+                    x1[3] = sm * ab[3] + (hf[0] * q.e[1] + hf[1] * q.e[0]);
+                    x1[5] = sm * ab[5] + (hf[0] * q.e[2] + hf[2] * q.e[0]);
+                    x1[6] = sm * ab[6] + (hf[1] * q.e[2] + hf[2] * q.e[1]);
+                    x1[7] = sm * ab[7] + (hf[0] * (m[1] * q.e[2] + m[2] * q.e[1]) + hf[1] * (m[0] * q.e[2] + m[2] * q.e[0]) +
+                                          hf[2] * (m[0] * q.e[1] + m[1] * q.e[0]));
+                    M[0] = 1.0;
+                    M[1] = m[0];
+                    M[2] = m[1];
+                    M[3] = q.Pxy;
+                    M[4] = m[2];
+                    M[5] = q.Pxz;
+                    M[6] = q.Pyz;
+                    M[7] = q.S;
+                }
+                if (plain) {
+                    if (has) {
+                        double x0[8];
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) x0[k] = ab[k] - x1[k];
+                        plain_rows(lam_tab, c, p.m, x0, vs);
+                        plain_rows(lam_tab + 3, c, p.m, x1, vs);
+                        const double hl[3] = {h * lg[0], h * lg[1], h * lg[2]};
+                        plain_rows(lam_tab + 6, c, p.m, M, hl);
+                    }
+                    continue;
+                }
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    if (has) {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            const Fx e = fx_split(fixed_of(half == 0 ? ab[k] - x1[k] : x1[k], tf, 4));
+#pragma unroll
+                            for (int a = 0; a < 3; ++a)
+                                tile[(8 * a + k) * DEPOSIT_STRIDE + lane] = k == 0 ? 0 : fx_mul(vf[a], e);
+                        }
+                    }
+                    flush(has, c, 3 * half, tv - 28, tf - 27);
+                }
+                if (has) {
+                    long long w[3], Mf[8];
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) w[a] = fixed_of(h * lg[a], tg, 4);
+#pragma unroll
+                    for (int k = 1; k < 8; ++k) Mf[k] = fixed_of(M[k], 1023, 10);
+                    rows(w, Mf);
+                }
+                flush(has, c, 6, tg - 56, 1023);
+            }
+            // the end point's interpolant of A^{n+1}, transposed
+            const double M[8] = {1.0, wk.te[0], wk.te[1], wk.te[0] * wk.te[1], wk.te[2], wk.te[0] * wk.te[2],
+                                 wk.te[1] * wk.te[2], wk.te[0] * wk.te[1] * wk.te[2]};
+            if (plain) {
+                if (act) plain_rows(lam_tab + 3, wk.c, p.m, M, lA);
+                continue;
+            }
+            if (act) {
+                long long w[3], Mf[8];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) w[a] = fixed_of(lA[a], tA, 4);
+#pragma unroll
+                for (int k = 1; k < 8; ++k) Mf[k] = fixed_of(M[k], 1023, 10);
+                rows(w, Mf);
+            }
+            flush(act, wk.c, 3, tA - 56, 1023);
+        }
+        __syncthreads();   // the hand-over buffers are rewritten by the next chunk
     }
 }
 
@@ -802,10 +919,17 @@ int adj_blocks(const Ctx& c, int64_t n) {
     return (int)std::min<int64_t>(b, MAX_BLOCKS);
 }
 
+bool setup_adjoint_kernels() {
+    return cudaFuncSetAttribute(k_adj_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)ChunkLarge::smem()) == cudaSuccess;
+}
+
 void launch_adj_scatter(Ctx& c, const double* xi, const double* v, const double* vstar, const double* lam_P,
                         const double* lam_v, const double* mu, double* lam_tab) {
-    k_adj_scatter<<<adj_blocks(c, c.np), THREADS, 0, c.stream>>>(adj_params(c), xi, v, vstar, c.table, lam_P, lam_v,
-                                                                  mu, c.slide, lam_tab);
+    const int64_t chunks = (c.np + ChunkLarge::SIZE - 1) / ChunkLarge::SIZE;
+    const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(chunks, (int64_t)c.sms * 4));
+    k_adj_scatter<<<nb, ChunkLarge::THREADS_, ChunkLarge::smem(), c.stream>>>(adj_params(c), xi, v, vstar, lam_P, lam_v,
+                                                                           mu, c.slide, lam_tab);
     ++c.launches;
 }
 

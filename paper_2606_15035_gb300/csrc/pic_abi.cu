@@ -315,7 +315,7 @@ constexpr size_t CELL_TABLE_MAX_BYTES = (size_t)16 << 30;
 
 pic_status allocate(pic_ctx* ctx) {
     Ctx& c = ctx->c;
-    if (!setup_particle_kernels() || !setup_pair_kernels() || !setup_helm_kernels()) return check_cuda(ctx, "particle kernels");
+    if (!setup_particle_kernels() || !setup_pair_kernels() || !setup_adjoint_kernels() || !setup_helm_kernels()) return check_cuda(ctx, "particle kernels");
     const int64_t np3 = 3 * std::max<int64_t>(c.np, 1), N = c.m.ncell;
     ALLOC(c.xi, double, np3);
     ALLOC(c.v, double, np3);

@@ -273,6 +273,7 @@ void launch_table_df(Ctx& c);
 void launch_push_df(Ctx& c, const double* vit, double* vnew, double* Jnext);
 
 // ---- launchers (adjoint.cu) ----
+bool setup_adjoint_kernels();   // their shared memory, on the current device
 void launch_adj_scatter(Ctx& c, const double* xi, const double* v, const double* vstar, const double* lam_P,
                         const double* lam_v, const double* mu, double* lam_tab);
 void launch_adj_mesh_rhs(Ctx& c, const double* lam_tab, const double* lF1, const double* lW1, double* t, double* pn);

@@ -20,6 +20,46 @@ constexpr int DEPOSIT_ROWS = 24;
 constexpr int DEPOSIT_STRIDE = 33;   // 33 x 8 B: a row's lanes and a column's rows miss each other's banks
 constexpr int DEPOSIT_TILE = DEPOSIT_ROWS * DEPOSIT_STRIDE;   // 64-bit words per warp
 
+// The sums of the warp's tile over the lanes of each distinct cell (row, its coordinates pc; lanes with
+// `has`): add(sum, cell) on every lane, lane r < DEPOSIT_ROWS with the sum of row r.
+template <typename F>
+__device__ __forceinline__ void tile_sums(bool has, int row, const int pc[3], const long long* tile, F&& add) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    unsigned rest = __ballot_sync(full, has);
+    while (rest) {
+        const int lead = __ffs(rest) - 1;
+        const int r = __shfl_sync(full, row, lead);
+        const unsigned group = __ballot_sync(full, row == r);
+        rest &= ~group;
+        int c[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) c[a] = __shfl_sync(full, pc[a], lead);
+        long long s = 0;
+        if (lane < DEPOSIT_ROWS) {
+            const long long* rowp = tile + lane * DEPOSIT_STRIDE;
+            for (unsigned g = group; g;) {   // four loads in flight; the zero column pads the last ones
+                long long v[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    v[k] = rowp[min((unsigned)(__ffs(g) - 1), 32u)];
+                    g &= g - 1;
+                }
+                s += (v[0] + v[1]) + (v[2] + v[3]);
+            }
+        }
+        add(s, c);
+    }
+}
+
+// Row of the node of a cell that the lowest three bits of k name.
+__device__ __forceinline__ int64_t subset_node(const int c0[3], int k, const MeshDims& m) {
+    int c[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) c[a] = ((k >> a) & 1) ? next_cell(c0[a], m.n[a]) : c0[a];
+    return cell_row(c, m);
+}
+
 // Measured at 32^3 with 2,097,152 particles (1.31 pieces each): the first scatter 0.82 -> 0.49 ms with
 // 4.5M L2 reduction requests where there were 67M; at 128^3 with 134M (2.2 pieces) 96 -> 44 ms.
 // In the push it takes 46 FP64 instructions a piece off the pipe that bounds it (1.59 -> 1.43 ms).
@@ -102,41 +142,16 @@ __device__ __forceinline__ int scatter_warp(const MeshDims& m, bool act, const C
             }
         }
         __syncwarp();
-        unsigned rest = __ballot_sync(full, has);
-        while (rest) {
-            const int lead = __ffs(rest) - 1;
-            const int r = __shfl_sync(full, row, lead);
-            const unsigned group = __ballot_sync(full, row == r);
-            rest &= ~group;
-            int c[3];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) c[a] = __shfl_sync(full, pc[a], lead);
-            long long s = 0;
-            if (lane < DEPOSIT_ROWS) {
-                const long long* rowp = tile + lane * DEPOSIT_STRIDE;
-                for (unsigned g = group; g;) {   // four loads in flight; the zero column pads the last ones
-                    long long v[4];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        v[k] = rowp[min((unsigned)(__ffs(g) - 1), 32u)];
-                        g &= g - 1;
-                    }
-                    s += (v[0] + v[1]) + (v[2] + v[3]);
-                }
-            }
+        tile_sums(has, row, pc, tile, [&](long long sum, const int c0[3]) {
             // moments of the subsets -> weights of the nodes (inclusion--exclusion, axis by axis)
 #pragma unroll
             for (int bit = 1; bit < 8; bit <<= 1) {
-                const long long o = __shfl_xor_sync(full, s, bit);
-                if (!(lane & bit)) s -= o;
+                const long long o = __shfl_xor_sync(full, sum, bit);
+                if (!(lane & bit)) sum -= o;
             }
-            if (lane < DEPOSIT_ROWS && s != 0) {
-#pragma unroll
-                for (int a = 0; a < 3; ++a)
-                    if ((lane >> a) & 1) c[a] = next_cell(c[a], m.n[a]);
-                atomicAdd(J + comp * N + cell_row(c, m), (double)s * unit);
-            }
-        }
+            if (lane < DEPOSIT_ROWS && sum != 0)
+                atomicAdd(J + comp * N + subset_node(c0, lane, m), (double)sum * unit);
+        });
         __syncwarp();   // the tile is rewritten by the next pieces
     }
     return act ? wk.count : 0;

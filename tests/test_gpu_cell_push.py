@@ -178,3 +178,51 @@ def test_gauss_pieces_match_oracle(sim, n, order, nq):
         assert rel(g[name], it[name]) <= 1e-12, (name, rel(g[name], it[name]))
     assert rel(g["P"], it["P"]) <= 1e-13
     assert rel(g["v"], it["v_new"]) <= 1e-13
+
+
+@pytest.mark.parametrize("npart", [1, 33, 256, 257, 1037])
+def test_vjp_of_orbits_across_cells_matches_directional_differences(sim, npart):
+    """The transposed deposits (per warp and cell, in chunks of 256) with partial warps and chunks, orbits
+    across several cells and adjoints of very different size.  The difference quotient's own error,
+    h^2 = 1e-8 relative and 1e-16 / 1e-7 of rounding, stays below the 1e-6 of the one-step test."""
+    import torch
+    rng = np.random.default_rng(npart)
+    n, L = (6, 5, 4), (1.2, 1.0, 0.8)
+    x = rng.uniform(0, 1, size=(npart, 3)) * L
+    v = rng.normal(scale=0.3, size=x.shape)                    # dt v: up to three cells a step
+    q = -1e-3 / npart
+    s = sim.PicSim(sim.pic_config_default(n=n, L=L, dt=0.8, picard_tol=1e-14, picard_max=32), x, v, q, 1e-3 / npart)
+    s.step(2)
+    base = s.get_state_device()
+    gen = torch.Generator(device="cuda").manual_seed(npart)
+    keys = ("x", "v", "P", "phi", "psi", "rho", "A", "U")
+    m = 1e-3 / npart
+    d = {k: 1e-3 * (m if k == "P" else 1.0) * torch.randn(t.shape, generator=gen, device="cuda", dtype=torch.float64)
+         for k, t in base.items()}
+    lam = {k: torch.randn(t.shape, generator=gen, device="cuda", dtype=torch.float64) for k, t in base.items()}
+    for k in ("x", "v", "P"):
+        lam[k] *= (1.0 / m if k == "P" else 1.0) * 10.0 ** torch.randint(-3, 1, lam[k].shape, generator=gen, device="cuda")
+    d["vprev"].zero_()
+    lam["vprev"].zero_()
+    Lv = torch.tensor(L, dtype=torch.float64, device="cuda")
+
+    def step_from(st):
+        s.set_state_device(st)
+        assert s.step(1).converged
+        return s.get_state_device()
+
+    h = 1e-4
+    plus = step_from({k: base[k] + h * d[k] for k in base})
+    minus = step_from({k: base[k] - h * d[k] for k in base})
+    diff = {k: plus[k] - minus[k] for k in base}
+    dx = diff["x"].reshape(3, -1)
+    diff["x"] = (((dx + 0.5 * Lv[:, None]) % Lv[:, None]) - 0.5 * Lv[:, None]).reshape(-1)   # minimal image
+    dot = lambda a, b: sum(float((a[k] * b[k]).sum()) for k in keys)
+    fd = dot(lam, diff) / (2 * h)
+    s.set_state_device(base)
+    assert s.step(1).converged
+    lam_prev, info = s.step_vjp(lam)
+    adj = dot(lam_prev, d)
+    s.close()
+    assert info.residual <= 1e-11
+    assert abs(adj - fd) <= 1e-6 * max(abs(fd), float(sum((lam[k] * diff[k] / (2 * h)).abs().sum() for k in keys)) * 1e-2)
