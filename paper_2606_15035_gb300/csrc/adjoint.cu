@@ -235,10 +235,10 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_scatter(
     if (lane < DEPOSIT_ROWS) tile[lane * DEPOSIT_STRIDE + 32] = 0;
     auto top_of = [&](double x) { return (int)__reduce_max_sync(full, (unsigned)exponent_of(x)); };
     // the tile's sums per cell into column `col` of lam_tab, their unit 2^(e0 + e1 - 2046) as two factors
-    auto flush = [&](bool has, const int c[3], int col, int e0, int e1) {
+    auto flush = [&](const TileOrder& order, bool has, const int c[3], int col, int e0, int e1) {
         const double u0 = pow2_biased(e0), u1 = pow2_biased(e1);
         __syncwarp();
-        tile_sums(has, has ? (int)cell_row(c, p.m) : -1, c, tile, [&](long long sum, const int c0[3]) {
+        order.sums(has, c, tile, [&](long long sum, const int c0[3]) {
             double x = (double)sum;
 #pragma unroll
             for (int bit = 1; bit < 8; bit <<= 1) {
@@ -250,13 +250,13 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_scatter(
         __syncwarp();
     };
     // rows (a, k) = w_a M_k, w given at 2^(-top - 56 + 1023), M at 2^-62
-    auto rows = [&](const long long w[3], const long long M[8]) {
+    auto rows = [&](int col, const long long w[3], const long long M[8]) {
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             const Fx ws = fx_split(w[a]);
-            tile[8 * a * DEPOSIT_STRIDE + lane] = w[a];
+            tile[8 * a * DEPOSIT_STRIDE + col] = w[a];
 #pragma unroll
-            for (int k = 1; k < 8; ++k) tile[(8 * a + k) * DEPOSIT_STRIDE + lane] = fx_mul(ws, fx_split(M[k]));
+            for (int k = 1; k < 8; ++k) tile[(8 * a + k) * DEPOSIT_STRIDE + col] = fx_mul(ws, fx_split(M[k]));
         }
     };
     for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
@@ -347,6 +347,7 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_scatter(
                     }
                     continue;
                 }
+                const TileOrder order(has, has ? (int)cell_row(c, p.m) : -1);
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
                     if (has) {
@@ -355,10 +356,10 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_scatter(
                             const Fx e = fx_split(fixed_of(half == 0 ? ab[k] - x1[k] : x1[k], tf, 4));
 #pragma unroll
                             for (int a = 0; a < 3; ++a)
-                                tile[(8 * a + k) * DEPOSIT_STRIDE + lane] = k == 0 ? 0 : fx_mul(vf[a], e);
+                                tile[(8 * a + k) * DEPOSIT_STRIDE + order.col] = k == 0 ? 0 : fx_mul(vf[a], e);
                         }
                     }
-                    flush(has, c, 3 * half, tv - 28, tf - 27);
+                    flush(order, has, c, 3 * half, tv - 28, tf - 27);
                 }
                 if (has) {
                     long long w[3], Mf[8];
@@ -366,9 +367,9 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_scatter(
                     for (int a = 0; a < 3; ++a) w[a] = fixed_of(h * lg[a], tg, 4);
 #pragma unroll
                     for (int k = 1; k < 8; ++k) Mf[k] = fixed_of(M[k], 1023, 10);
-                    rows(w, Mf);
+                    rows(order.col, w, Mf);
                 }
-                flush(has, c, 6, tg - 56, 1023);
+                flush(order, has, c, 6, tg - 56, 1023);
             }
             // the end point's interpolant of A^{n+1}, transposed
             const double M[8] = {1.0, wk.te[0], wk.te[1], wk.te[0] * wk.te[1], wk.te[2], wk.te[0] * wk.te[2],
@@ -377,15 +378,16 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_scatter(
                 if (act) plain_rows(lam_tab + 3, wk.c, p.m, M, lA);
                 continue;
             }
+            const TileOrder order(act, act ? (int)cell_row(wk.c, p.m) : -1);
             if (act) {
                 long long w[3], Mf[8];
 #pragma unroll
                 for (int a = 0; a < 3; ++a) w[a] = fixed_of(lA[a], tA, 4);
 #pragma unroll
                 for (int k = 1; k < 8; ++k) Mf[k] = fixed_of(M[k], 1023, 10);
-                rows(w, Mf);
+                rows(order.col, w, Mf);
             }
-            flush(act, wk.c, 3, tA - 56, 1023);
+            flush(order, act, wk.c, 3, tA - 56, 1023);
         }
         __syncthreads();   // the hand-over buffers are rewritten by the next chunk
     }

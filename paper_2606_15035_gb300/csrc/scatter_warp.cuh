@@ -20,37 +20,56 @@ constexpr int DEPOSIT_ROWS = 24;
 constexpr int DEPOSIT_STRIDE = 33;   // 33 x 8 B: a row's lanes and a column's rows miss each other's banks
 constexpr int DEPOSIT_TILE = DEPOSIT_ROWS * DEPOSIT_STRIDE;   // 64-bit words per warp
 
-// The sums of the warp's tile over the lanes of each distinct cell (row, its coordinates pc; lanes with
-// `has`): add(sum, cell) on every lane, lane r < DEPOSIT_ROWS with the sum of row r.
-template <typename F>
-__device__ __forceinline__ void tile_sums(bool has, int row, const int pc[3], const long long* tile, F&& add) {
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    unsigned rest = __ballot_sync(full, has);
-    while (rest) {
-        const int lead = __ffs(rest) - 1;
-        const int r = __shfl_sync(full, row, lead);
-        const unsigned group = __ballot_sync(full, row == r);
-        rest &= ~group;
-        int c[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) c[a] = __shfl_sync(full, pc[a], lead);
-        long long s = 0;
-        if (lane < DEPOSIT_ROWS) {
-            const long long* rowp = tile + lane * DEPOSIT_STRIDE;
-            for (unsigned g = group; g;) {   // four loads in flight; the zero column pads the last ones
-                long long v[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    v[k] = rowp[min((unsigned)(__ffs(g) - 1), 32u)];
-                    g &= g - 1;
-                }
-                s += (v[0] + v[1]) + (v[2] + v[3]);
+// The lanes with `has` by cell: lanes of one row (its cell, -1 without) get adjacent columns of the tile.
+struct TileOrder {
+    unsigned group;   // lanes of this lane's cell
+    int col;          // this lane's column
+
+    __device__ __forceinline__ TileOrder(bool has, int row) : group(0), col(0) {
+        const unsigned full = 0xffffffffu, below = (1u << (threadIdx.x & 31)) - 1u;
+        int base = 0;
+        for (unsigned rest = __ballot_sync(full, has); rest;) {
+            const int r = __shfl_sync(full, row, __ffs(rest) - 1);
+            const unsigned g = __ballot_sync(full, row == r);
+            if (row == r) {
+                group = g;
+                col = base + __popc(g & below);
             }
+            base += __popc(g);
+            rest &= ~g;
         }
-        add(s, c);
     }
-}
+
+    // The tile's sums over the columns of each cell (coordinates pc of its lanes): add(sum, cell) on every
+    // lane, lane r < DEPOSIT_ROWS with the sum of row r.
+    template <typename F>
+    __device__ __forceinline__ void sums(bool has, const int pc[3], const long long* tile, F&& add) const {
+        const unsigned full = 0xffffffffu;
+        const int lane = threadIdx.x & 31;
+        int base = 0;
+        for (unsigned rest = __ballot_sync(full, has); rest;) {
+            const int lead = __ffs(rest) - 1;
+            const unsigned g = __shfl_sync(full, group, lead);
+            rest &= ~g;
+            int c[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) c[a] = __shfl_sync(full, pc[a], lead);
+            const int end = base + __popc(g);
+            long long s = 0;
+            if (lane < DEPOSIT_ROWS) {
+                const long long* rowp = tile + lane * DEPOSIT_STRIDE;
+                for (int j = base; j < end; j += 4) {   // four loads in flight; the zero column pads the last ones
+                    long long v[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) v[k] = rowp[j + k < end ? j + k : 32];
+                    s += (v[0] + v[1]) + (v[2] + v[3]);
+                }
+            }
+            base = end;
+            add(s, c);
+        }
+    }
+};
 
 // Row of the node of a cell that the lowest three bits of k name.
 __device__ __forceinline__ int64_t subset_node(const int c0[3], int k, const MeshDims& m) {
@@ -113,36 +132,37 @@ __device__ __forceinline__ int scatter_warp(const MeshDims& m, bool act, const C
     while (__any_sync(full, !last)) {
         bool has = false;
         int row = -1, pc[3] = {0, 0, 0};
+        double h = 0.0, sm, mid[3] = {0.0, 0.0, 0.0};
         if (!last) {
-            double h, sm, mid[3];
             has = wk.next(beta, m, h, sm, mid, pc, last);
-            if (has) {
-                row = (int)cell_row(pc, m);
-                long long M[8];
-                Fx q[3], d[3];
+            if (has) row = (int)cell_row(pc, m);
+        }
+        const TileOrder order(has, row);
+        if (has) {
+            long long M[8];
+            Fx q[3], d[3];
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    M[1 << a] = fixed_of(mid[a], 1023, 10);
-                    q[a] = fx_split(M[1 << a]);
-                    d[a] = fx_split(fixed_of(h * bs[a], 1023, 10));
-                }
-                const long long kxy = fx_mul(d[0], d[1]), kxz = fx_mul(d[0], d[2]), kyz = fx_mul(d[1], d[2]);
-                M[3] = fx_mul(q[0], q[1]) + kxy;
-                M[5] = fx_mul(q[0], q[2]) + kxz;
-                M[6] = fx_mul(q[1], q[2]) + kyz;
-                M[7] = fx_mul(q[0], fx_split(M[6])) + fx_mul(q[1], fx_split(kxz)) + fx_mul(q[2], fx_split(kxy));
+            for (int a = 0; a < 3; ++a) {
+                M[1 << a] = fixed_of(mid[a], 1023, 10);
+                q[a] = fx_split(M[1 << a]);
+                d[a] = fx_split(fixed_of(h * bs[a], 1023, 10));
+            }
+            const long long kxy = fx_mul(d[0], d[1]), kxz = fx_mul(d[0], d[2]), kyz = fx_mul(d[1], d[2]);
+            M[3] = fx_mul(q[0], q[1]) + kxy;
+            M[5] = fx_mul(q[0], q[2]) + kxz;
+            M[6] = fx_mul(q[1], q[2]) + kyz;
+            M[7] = fx_mul(q[0], fx_split(M[6])) + fx_mul(q[1], fx_split(kxz)) + fx_mul(q[2], fx_split(kxy));
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const long long wf = fixed_of(h * w[a], top[a], 4);
-                    const Fx ws = fx_split(wf);
-                    tile[(8 * a) * DEPOSIT_STRIDE + lane] = wf;
+            for (int a = 0; a < 3; ++a) {
+                const long long wf = fixed_of(h * w[a], top[a], 4);
+                const Fx ws = fx_split(wf);
+                tile[(8 * a) * DEPOSIT_STRIDE + order.col] = wf;
 #pragma unroll
-                    for (int k = 1; k < 8; ++k) tile[(8 * a + k) * DEPOSIT_STRIDE + lane] = fx_mul(ws, fx_split(M[k]));
-                }
+                for (int k = 1; k < 8; ++k) tile[(8 * a + k) * DEPOSIT_STRIDE + order.col] = fx_mul(ws, fx_split(M[k]));
             }
         }
         __syncwarp();
-        tile_sums(has, row, pc, tile, [&](long long sum, const int c0[3]) {
+        order.sums(has, pc, tile, [&](long long sum, const int c0[3]) {
             // moments of the subsets -> weights of the nodes (inclusion--exclusion, axis by axis)
 #pragma unroll
             for (int bit = 1; bit < 8; bit <<= 1) {
