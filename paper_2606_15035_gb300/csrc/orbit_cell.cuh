@@ -39,6 +39,11 @@ __device__ __forceinline__ bool less_pos(double a, double b) { return __double_a
 __device__ __forceinline__ bool same_bits(double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); }
 __device__ __forceinline__ bool at_least_one(double t) { return __double2hiint(t) >= 0x3ff00000; }
 __device__ __forceinline__ bool below_zero(double t) { return __double2hiint(t) < 0; }
+__device__ __forceinline__ bool less_pos(float a, float b) { return a < b; }
+__device__ __forceinline__ bool same_bits(float a, float b) { return a == b; }
+__device__ __forceinline__ bool at_least_one(float t) { return t >= 1.f; }
+__device__ __forceinline__ bool below_zero(float t) { return t < 0.f; }
+__device__ __forceinline__ bool is_zero(float t) { return t == 0.f; }
 __device__ __forceinline__ bool is_zero(double t) { return (__double_as_longlong(t) << 1) == 0; }
 
 // A particle's start: cell and coordinate in it.

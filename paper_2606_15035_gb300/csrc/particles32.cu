@@ -21,6 +21,7 @@
 #include <climits>
 #include <cmath>
 
+#include "orbit_cell.cuh"
 #include "pic_internal.h"
 
 namespace pic {
@@ -222,14 +223,32 @@ struct MeshView {
     }
 };
 
+// The pieces of an orbit that starts at offset x0 of cell co, by the walk of orbit_cell.cuh with cells
+// relative to the start's (no wrap): visit(h, s_mid, midpoint in the cell, cell).  Returns its count.
+template <typename F>
+__device__ __forceinline__ int pieces32(const int co[3], const float x0[3], const float beta[3], F&& visit) {
+    constexpr int MID = 1 << 24;   // (the walk's cells stay in [0, 2 MID))
+    CellStart<float> st;
+    MeshDims m;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        st.f[a] = x0[a];
+        st.c[a] = MID;
+        m.n[a] = 2 * MID;
+    }
+    return for_each_piece(st, beta, m, [&](float h, float sm, const float mid[3], const int cell[3]) {
+        const int c[3] = {co[0] + cell[0] - MID, co[1] + cell[1] - MID, co[2] + cell[2] - MID};
+        visit(h, sm, mid, c);
+    });
+}
+
 // Orbit current of one FP32 orbit (closed form, Appendix A): q v_bar S_bar / dV per node.
 template <bool TILED>
 __device__ __forceinline__ int scatter32(const MeshView<TILED>& mv, const int co[3], const float x0[3],
                                          const float beta[3], const float w[3]) {
-    return for_each_segment(x0, beta, true, [&](const Segment<float>& sg) {
+    return pieces32(co, x0, beta, [&](float h, float, const float mid[3], const int c[3]) {
         float I[8];
-        weights_from_ints(piece_integrals(sg, beta, false), I);
-        const int c[3] = {co[0] + sg.cell[0], co[1] + sg.cell[1], co[2] + sg.cell[2]};
+        node_weights(piece_moments(h, mid, beta), I);
         int g[8];
         int64_t gg[8];
         if (!mv.nodes8(c, g, gg)) return;
@@ -252,7 +271,7 @@ __device__ __forceinline__ int scatter32(const MeshView<TILED>& mv, const int co
             }
         }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) mv.add(g, gg, k, w[0] * I[k], w[1] * I[k], w[2] * I[k]);
+        for (int k = 0; k < 8; ++k) mv.add(g, gg, k, w[0] * (h * I[k]), w[1] * (h * I[k]), w[2] * (h * I[k]));
     });
 }
 
@@ -263,43 +282,47 @@ template <bool TILED>
 __device__ __forceinline__ int push32(const Params32& p, const MeshView<TILED>& mv, const int co[3], const float x0[3],
                                       const float beta[3], const float vb[3], float dv[3]) {
     float gphi[3] = {0.f, 0.f, 0.f}, F[3] = {0.f, 0.f, 0.f};
-    const int nseg = for_each_segment(x0, beta, true, [&](const Segment<float>& sg) {
-        const PieceInts<float> I = piece_integrals(sg, beta, true);
+    const int nseg = pieces32(co, x0, beta, [&](float h, float sm, const float m[3], const int c[3]) {
+        const PieceMoments<float> q = piece_moments(h, m, beta);
         float W[8];
-        weights_from_ints(I, W);
-        const int c[3] = {co[0] + sg.cell[0], co[1] + sg.cell[1], co[2] + sg.cell[2]};
+        node_weights(q, W);
         int g[8];
         int64_t gg[8];
         if (!mv.nodes8(c, g, gg)) return;
-        const float s = sg.s0, oms = 1.f - s, h = sg.h, hh2 = 0.5f * h * h;
-        float am[8], cc[8];
+        const float nms = sm - 1.f;
+        float am[8], cc[8], gp[3] = {0.f, 0.f, 0.f};   // A . vbar at s_mid, and its change over the step
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             const float4* t4 = mv.node(g, gg, k);
             const float4 a = t4[0], b = t4[1], c4 = t4[2];
             const float an = a.x * vb[0] + a.y * vb[1] + a.z * vb[2];
             const float a1 = a.w * vb[0] + b.x * vb[1] + b.y * vb[2];
-            am[k] = oms * an + s * a1;
             cc[k] = a1 - an;
-            gphi[0] += W[k] * b.z;
-            gphi[1] += W[k] * b.w;
-            gphi[2] += W[k] * c4.x;
+            am[k] = a1 + nms * cc[k];
+            gp[0] += W[k] * b.z;
+            gp[1] += W[k] * b.w;
+            gp[2] += W[k] * c4.x;
         }
+        // mixed differences, and their contraction as in piece_impulse
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const int pa = j == 0 ? 1 : 0, qa = j == 2 ? 1 : 2;
-            const int sp = j == 0 ? 2 : 1, sq = j == 2 ? 2 : 4;
-            const int sj = j == 0 ? 1 : (j == 1 ? 2 : 4);
-            const float D00 = am[sj] - am[0], D10 = am[sp + sj] - am[sp];
-            const float D01 = am[sq + sj] - am[sq], D11 = am[sp + sq + sj] - am[sp + sq];
-            const float C00 = cc[sj] - cc[0], C10 = cc[sp + sj] - cc[sp];
-            const float C01 = cc[sq + sj] - cc[sq], C11 = cc[sp + sq + sj] - cc[sp + sq];
-            const float t0 = D00 * h + (D10 - D00) * I.S1[pa] + (D01 - D00) * I.S1[qa] +
-                             (D11 - D10 - D01 + D00) * I.S2[j];
-            const float t1 = C00 * hh2 + (C10 - C00) * I.E1[pa] + (C01 - C00) * I.E1[qa] +
-                             (C11 - C10 - C01 + C00) * I.E2[j];
-            F[j] += p.invH[j] * (t0 + t1);
-        }
+        for (int bit = 1; bit < 8; bit <<= 1)
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (k & bit) {
+                    am[k] -= am[k ^ bit];
+                    cc[k] -= cc[k ^ bit];
+                }
+        const float F0 = am[1] + am[3] * m[1] + am[5] * m[2] + am[7] * q.Pyz + cc[3] * q.e[1] + cc[5] * q.e[2] +
+                         cc[7] * (m[1] * q.e[2] + m[2] * q.e[1]);
+        const float F1 = am[2] + am[3] * m[0] + am[6] * m[2] + am[7] * q.Pxz + cc[3] * q.e[0] + cc[6] * q.e[2] +
+                         cc[7] * (m[0] * q.e[2] + m[2] * q.e[0]);
+        const float F2 = am[4] + am[5] * m[0] + am[6] * m[1] + am[7] * q.Pxy + cc[5] * q.e[0] + cc[6] * q.e[1] +
+                         cc[7] * (m[0] * q.e[1] + m[1] * q.e[0]);
+        F[0] += h * (p.invH[0] * F0);
+        F[1] += h * (p.invH[1] * F1);
+        F[2] += h * (p.invH[2] * F2);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) gphi[j] += h * gp[j];
     });
     // dA = A_h^{n+1}(x^{n+1}) - A_h^n(x^n): point interpolants at the end and start points
     float dA[3] = {0.f, 0.f, 0.f};

@@ -226,3 +226,24 @@ def test_vjp_of_orbits_across_cells_matches_directional_differences(sim, npart):
     s.close()
     assert info.residual <= 1e-11
     assert abs(adj - fd) <= 1e-6 * max(abs(fd), float(sum((lam[k] * diff[k] / (2 * h)).abs().sum() for k in keys)) * 1e-2)
+
+
+@pytest.mark.parametrize("npart", [1, 255, 257, 2000])
+def test_fp32_iterations_end_near_the_fp64_fixed_point(sim, npart):
+    """FP32 pieces of orbits across several cells, some from knots (exactly) and one ending on one: the
+    first refinement of the FP32 iterate changes v by its rounding, 1e-7 times a few dozen terms of dv,
+    dv / v below 0.1: 1e-6.  A piece in the wrong cell or with a wrong weight shows at 1e-3."""
+    rng = np.random.default_rng(npart)
+    n, L = (6, 5, 4), (6.0, 5.0, 4.0)
+    x = rng.uniform(0, 1, size=(npart, 3)) * L
+    b = rng.normal(scale=0.9, size=x.shape)
+    x[: npart // 4] = np.floor(x[: npart // 4])
+    b[npart // 8: npart // 4] = np.round(b[npart // 8: npart // 4]) + 0.25
+    b = np.where(np.abs(b) < 0.1, 0.1, b)                       # (slow ones go to the local solves)
+    s = sim.PicSim(sim.pic_config_default(n=n, L=L, dt=1.0, precision=1, picard_tol=1e-13), x, b, -0.2 / npart, 0.5 / npart)
+    assert s.step(1).converged
+    e_v, _, kind = s.residual_history()
+    fp32 = [e for k, e in zip(kind, e_v) if k == 1]
+    rest = [e for k, e in zip(kind, e_v) if k != 1]
+    s.close()
+    assert len(fp32) >= 2 and fp32[0] > 1e-5 and rest[0] <= 1e-6, (kind, e_v)
