@@ -596,8 +596,18 @@ __global__ void k_add_to(double* __restrict__ dst, const double* __restrict__ sr
 
 }  // namespace
 
+// Threads of a block of the mesh kernels: no more than spread the mesh over the SMs (each kernel is one
+// chain of FP64 instructions a thread, and an SM's warps share that pipe: the back substitution took
+// 7.0 us at 8^3 in blocks of 256, 5.1 in blocks of 32; the spectral update at 16^3 20 and, with its divisions
+// replaced, 6.3).
+int mesh_threads(const Ctx& c) {
+    const int64_t warps = (c.m.ncell + 32 * (int64_t)c.sms - 1) / (32 * (int64_t)c.sms);
+    return 32 * (int)std::min<int64_t>(THREADS / 32, warps);
+}
+
 int mesh_blocks(const Ctx& c) {
-    int64_t b = (c.m.ncell + THREADS - 1) / THREADS;
+    const int threads = mesh_threads(c);
+    int64_t b = (c.m.ncell + threads - 1) / threads;
     int64_t cap = (int64_t)c.sms * 8;
     if (b > cap) b = cap;
     if (b < 1) b = 1;
@@ -605,18 +615,18 @@ int mesh_blocks(const Ctx& c) {
 }
 
 void launch_rhs0(Ctx& c) {
-    k_rhs0<<<mesh_blocks(c), THREADS, 0, c.stream>>>(mesh_params(c), c.F0, c.W0, c.rhs0);
+    k_rhs0<<<mesh_blocks(c), mesh_threads(c), 0, c.stream>>>(mesh_params(c), c.F0, c.W0, c.rhs0);
     ++c.launches;
 }
 
 void launch_source(Ctx& c, const double* Jcur, const double* Jprev) {
-    k_source<<<mesh_blocks(c), THREADS, 0, c.stream>>>(mesh_params(c), Jcur, Jprev, c.rho0, c.rhs0, c.rho1, c.rhs,
+    k_source<<<mesh_blocks(c), mesh_threads(c), 0, c.stream>>>(mesh_params(c), Jcur, Jprev, c.rho0, c.rhs0, c.rho1, c.rhs,
                                                        c.F1, c.helm_top, c.partials);
     ++c.launches;
 }
 
 void launch_jdiff(Ctx& c, const double* Jnew, const double* Jold) {
-    k_jdiff<<<mesh_blocks(c), THREADS, 0, c.stream>>>(3 * c.m.ncell, Jnew, Jold, c.partials);
+    k_jdiff<<<mesh_blocks(c), mesh_threads(c), 0, c.stream>>>(3 * c.m.ncell, Jnew, Jold, c.partials);
     ++c.launches;
 }
 
@@ -690,7 +700,7 @@ int cheb_coop_capacity(const Ctx& c) {
 }
 
 void launch_backsub_table(Ctx& c, double* zero) {
-    k_backsub_table<<<mesh_blocks(c), THREADS, 0, c.stream>>>(mesh_params(c), c.F0, c.W0, c.F1, c.W1, c.table,
+    k_backsub_table<<<mesh_blocks(c), mesh_threads(c), 0, c.stream>>>(mesh_params(c), c.F0, c.W0, c.F1, c.W1, c.table,
                                                             c.helm_top, c.cell_top, zero);
     ++c.launches;
 }
@@ -727,12 +737,12 @@ void launch_null_project(Ctx& c, double* f, double add_const) {
 }
 
 void launch_mesh_energy(Ctx& c, const double* F, const double* W, int slot) {
-    k_mesh_energy<<<mesh_blocks(c), THREADS, 0, c.stream>>>(mesh_params(c), F, W, c.partials, slot);
+    k_mesh_energy<<<mesh_blocks(c), mesh_threads(c), 0, c.stream>>>(mesh_params(c), F, W, c.partials, slot);
     ++c.launches;
 }
 
 void launch_mesh_diag(Ctx& c, const double* Jfinal) {
-    k_mesh_diag<<<mesh_blocks(c), THREADS, 0, c.stream>>>(mesh_params(c), c.F0, c.W0, c.rho0, c.F1, c.W1, c.rho1,
+    k_mesh_diag<<<mesh_blocks(c), mesh_threads(c), 0, c.stream>>>(mesh_params(c), c.F0, c.W0, c.rho0, c.F1, c.W1, c.rho1,
                                                           Jfinal, c.partials);
     ++c.launches;
 }

@@ -380,6 +380,7 @@ int particle_blocks(const Ctx& c);
 int chunk_blocks(const Ctx& c);   // the closed forms' chunk kernels
 int push_blocks(const Ctx& c);    // the pushes and the first scatter
 int local_blocks(const Ctx& c);
-int mesh_blocks(const Ctx& c);
+int mesh_blocks(const Ctx& c);    // with mesh_threads(c) threads each
+int mesh_threads(const Ctx& c);
 
 }  // namespace pic

@@ -22,12 +22,29 @@
 namespace pic {
 namespace {
 
+struct FftStage {
+    int R, L, nb, tstep;         // radix, product of the radices before, n / R, n / (L R)
+    unsigned mL, mnb;            // multipliers of the divisions by L and nb
+};
+
 struct FftAxis {
-    int axis, n, nst;
+    int axis, n, nst, lb;        // lb: lines of a block
     int64_t stride;              // element stride of a line along this axis
-    int radix[FFT_MAX_STAGES];
+    unsigned mn, mlb;
+    FftStage st[FFT_MAX_STAGES];
     const double2* tw;           // exp(-2 pi i t / n), t = 0 .. n-1
 };
+
+// Real fields that a pass reads or writes in place of the complex ones (null: complex).
+constexpr int SPEC_FIELDS = 12;
+struct RealFields {
+    double* f[SPEC_FIELDS] = {};
+    double scale = 1.0;
+};
+
+unsigned multiplier(int d) { return d <= 1 ? 0u : (unsigned)((((uint64_t)1 << 32) + d - 1) / d); }
+// x / d for x < 2^16 by m = ceil(2^32 / d) (d = 1: m = 0)
+__device__ __forceinline__ int quot(int x, unsigned m) { return m ? (int)__umulhi((unsigned)x, m) : x; }
 
 __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -46,68 +63,88 @@ __device__ __forceinline__ int64_t line_base(int axis, int64_t l, const MeshDims
 // Stockham autosort: stage s of radix R, with L = product of the previous radices, takes
 // v_r = x[j + r n/R] (j < n/R, k = j mod L), twiddles v_r by exp(-+2 pi i k r / (L R)),
 // applies the radix-R DFT and stores output s at (j div L) L R + k + s L.
-// A block transforms `lb` lines whose first elements are adjacent in memory (lines l0 .. l0 +
-// lb - 1 along y or z start at consecutive x, or consecutive x-y positions), so that the loads
-// and stores of a strided axis read lb consecutive complex values at a time; along x (stride 1)
-// lb is 1.  Shared memory holds the lb lines twice (ping-pong), line j at j n.
-__global__ void k_fft_axis(double2* __restrict__ data, MeshDims m, FftAxis ax, int inverse, int lb) {
+// A block transforms `lb` lines that are adjacent in memory (along x one after the other; along y and z
+// element by element, so that the loads and stores of a strided axis take lb consecutive values at a
+// time).  Shared memory holds the lb lines twice (ping-pong), line j at j n.  The first pass of a forward
+// transform reads the real fields, the last of an inverse one writes them.
+//
+// At small meshes the passes are bound by latency (index divisions, stages, launches): a mesh phase of 15
+// fields at 16^3 took 14 launches and 77 us of kernels with separate conversions and radix 2, now 9 and 47;
+// a pass at 36^3 19.6 us, now 14.1.
+__global__ void k_fft_axis(double2* __restrict__ data, MeshDims m, FftAxis ax, int inverse, RealFields rin,
+                           RealFields rout) {
     extern __shared__ double2 sbuf[];
-    const int n = ax.n;
-    const int64_t nlines = m.ncell / n;
-    const int64_t ngroups = nlines / lb;
+    const int n = ax.n, lb = ax.lb, tot = lb * n;
+    const int64_t ngroups = m.ncell / tot;
     double2* field = data + (int64_t)blockIdx.y * m.ncell;
+    const double* real_in = rin.f[blockIdx.y];
+    double* real_out = rout.f[blockIdx.y];
     const double sgn = inverse ? 1.0 : -1.0;
     const double s3 = sgn * 0.86602540378443864676;   // sin(2 pi / 3) with the transform's sign
-    const int tot = lb * n;
+    auto tw = [&](int t) {
+        double2 w = ax.tw[t];
+        if (inverse) w.y = -w.y;
+        return w;
+    };
+    // element t of line j: place in memory (from the first line's start) and in the buffer
+    auto place = [&](int e, int& at) {
+        if (ax.axis == 0) {
+            at = e;
+            return (int64_t)e;
+        }
+        const int t = quot(e, ax.mlb), j = e - t * lb;
+        at = j * n + t;
+        return j + (int64_t)t * ax.stride;
+    };
     for (int64_t gr = blockIdx.x; gr < ngroups; gr += gridDim.x) {
         double2* x = sbuf;
         double2* y = sbuf + tot;
-        double2* first = field + line_base(ax.axis, gr * lb, m);
-        // element t of line j sits at first + j + t stride (lb > 1 only where lines are adjacent)
+        const int64_t first = line_base(ax.axis, gr * lb, m);
         for (int e = threadIdx.x; e < tot; e += blockDim.x) {
-            const int j = e % lb, t = e / lb;
-            x[j * n + t] = lb > 1 ? first[j + (int64_t)t * ax.stride] : first[(int64_t)t * ax.stride];
+            int at;
+            const int64_t g = first + place(e, at);
+            x[at] = real_in ? make_double2(real_in[g], 0.0) : field[g];
         }
         __syncthreads();
-        int L = 1;
-        for (int st = 0; st < ax.nst; ++st) {
-            const int R = ax.radix[st];
-            const int nb = n / R, tstep = n / (L * R);
-            for (int e = threadIdx.x; e < lb * nb; e += blockDim.x) {
-                const int line = e / nb, j = e - line * nb;
-                const double2* xl = x + line * n;
-                double2* yl = y + line * n;
-                const int k = j % L;
-                const int out = (j / L) * L * R + k;
-                double2 v0 = xl[j], v1 = xl[j + nb];
-                double2 t1 = ax.tw[k * tstep];
-                if (inverse) t1.y = -t1.y;
-                v1 = cmul(v1, t1);
-                if (R == 2) {
-                    yl[out] = cadd(v0, v1);
-                    yl[out + L] = csub(v0, v1);
+        for (int si = 0; si < ax.nst; ++si) {
+            const FftStage st = ax.st[si];
+            for (int e = threadIdx.x; e < lb * st.nb; e += blockDim.x) {
+                const int line = quot(e, st.mnb), j = e - line * st.nb;
+                const int jl = quot(j, st.mL), k = j - jl * st.L;
+                const double2* in = x + line * n + j;
+                double2* out = y + line * n + jl * st.L * st.R + k;
+                const double2 v0 = in[0], v1 = cmul(in[st.nb], tw(k * st.tstep));
+                if (st.R == 2) {
+                    out[0] = cadd(v0, v1);
+                    out[st.L] = csub(v0, v1);
+                } else if (st.R == 4) {
+                    const double2 v2 = cmul(in[2 * st.nb], tw(2 * k * st.tstep));
+                    const double2 v3 = cmul(in[3 * st.nb], tw(3 * k * st.tstep));
+                    const double2 a = cadd(v0, v2), b = csub(v0, v2), c = cadd(v1, v3), d = csub(v1, v3);
+                    const double2 id = make_double2(-sgn * d.y, sgn * d.x);   // +- i d
+                    out[0] = cadd(a, c);
+                    out[st.L] = cadd(b, id);
+                    out[2 * st.L] = csub(a, c);
+                    out[3 * st.L] = csub(b, id);
                 } else {
-                    double2 v2 = xl[j + 2 * nb];
-                    double2 t2 = ax.tw[2 * k * tstep];
-                    if (inverse) t2.y = -t2.y;
-                    v2 = cmul(v2, t2);
+                    const double2 v2 = cmul(in[2 * st.nb], tw(2 * k * st.tstep));
                     const double2 sum = cadd(v1, v2), dif = csub(v1, v2);
                     const double2 mid = make_double2(v0.x - 0.5 * sum.x, v0.y - 0.5 * sum.y);
-                    yl[out] = cadd(v0, sum);
-                    yl[out + L] = make_double2(mid.x - s3 * dif.y, mid.y + s3 * dif.x);        // + i s3 dif
-                    yl[out + 2 * L] = make_double2(mid.x + s3 * dif.y, mid.y - s3 * dif.x);    // - i s3 dif
+                    out[0] = cadd(v0, sum);
+                    out[st.L] = make_double2(mid.x - s3 * dif.y, mid.y + s3 * dif.x);        // + i s3 dif
+                    out[2 * st.L] = make_double2(mid.x + s3 * dif.y, mid.y - s3 * dif.x);    // - i s3 dif
                 }
             }
             __syncthreads();
             double2* t = x;
             x = y;
             y = t;
-            L *= R;
         }
         for (int e = threadIdx.x; e < tot; e += blockDim.x) {
-            const int j = e % lb, t = e / lb;
-            if (lb > 1) first[j + (int64_t)t * ax.stride] = x[j * n + t];
-            else first[(int64_t)t * ax.stride] = x[j * n + t];
+            int at;
+            const int64_t g = first + place(e, at);
+            if (real_out) real_out[g] = x[at].x * rout.scale;
+            else field[g] = x[at];
         }
         __syncthreads();
     }
@@ -139,14 +176,6 @@ __device__ __forceinline__ double2 ik(double k, double2 z) { return make_double2
 
 #define SPEC_LOOP(g, N) for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < (N); g += (int64_t)gridDim.x * blockDim.x)
 
-__global__ void k_r2c(const double* __restrict__ in, double2* __restrict__ out, int64_t n) {
-    SPEC_LOOP(i, n) out[i] = make_double2(in[i], 0.0);
-}
-
-__global__ void k_c2r(const double2* __restrict__ in, double* __restrict__ out, int64_t n, double scale) {
-    SPEC_LOOP(i, n) out[i] = in[i].x * scale;
-}
-
 // Continuity and the CN update per mode.  In: J^ (3), level n: [phi, A (3) | psi, U (3) | rho].
 // Out: level n+1 [phi, A | psi, U | rho] and D phi^{n+1/2} (3).
 __global__ void k_spec_cn(SpecParams p, const double2* __restrict__ Jh, const double2* __restrict__ S0,
@@ -157,7 +186,12 @@ __global__ void k_spec_cn(SpecParams p, const double2* __restrict__ Jh, const do
         double k[3];
         mode_k(p, g, k);
         const double lam = -(k[0] * k[0] + k[1] * k[1] + k[2] * k[2]);
-        const double b = hdt * p.kappa2 * lam, det = 1.0 - hdt * b;
+        const double b = hdt * p.kappa2 * lam, det = 1.0 - hdt * b, inv = 1.0 / det;
+        // x / det by the reciprocal and one correction from the exact remainder (16 divisions bound the kernel)
+        auto over = [&](double x) {
+            const double q = x * inv;
+            return fma(fma(-q, det, x), inv, q);
+        };
         const double2 J[3] = {Jh[g], Jh[N + g], Jh[2 * N + g]};
         double2 divJ = cadd(cadd(ik(k[0], J[0]), ik(k[1], J[1])), ik(k[2], J[2]));
         const double2 r0 = S0[8 * N + g];
@@ -172,8 +206,8 @@ __global__ void k_spec_cn(SpecParams p, const double2* __restrict__ Jh, const do
             const double cs = p.dt * p.kappa2 * (f == 0 ? p.sigma1 : p.sigma2);
             const double2 q1 = make_double2(u0.x + hdt * w0.x, u0.y + hdt * w0.y);
             const double2 q2 = make_double2(w0.x + b * u0.x + cs * src.x, w0.y + b * u0.y + cs * src.y);
-            const double2 u1 = make_double2((q1.x + hdt * q2.x) / det, (q1.y + hdt * q2.y) / det);
-            const double2 w1 = make_double2((q2.x + b * q1.x) / det, (q2.y + b * q1.y) / det);
+            const double2 u1 = make_double2(over(q1.x + hdt * q2.x), over(q1.y + hdt * q2.y));
+            const double2 w1 = make_double2(over(q2.x + b * q1.x), over(q2.y + b * q1.y));
             S1[f * N + g] = u1;
             S1[(4 + f) * N + g] = w1;
             if (f == 0) phi1 = u1;
@@ -351,47 +385,76 @@ int spec_blocks(const Ctx& c, int64_t n) {
     return (int)std::max<int64_t>(b, 1);
 }
 
-FftAxis make_axis(const Ctx& c, int a) {
-    FftAxis ax;
+FftAxis make_axis(const Ctx& c, int a, int nf) {
+    FftAxis ax{};
     ax.axis = a;
     ax.n = c.m.n[a];
     ax.stride = a == 0 ? 1 : (a == 1 ? c.m.n[0] : (int64_t)c.m.n[0] * c.m.n[1]);
-    ax.nst = c.fft_nst[a];
-    for (int s = 0; s < FFT_MAX_STAGES; ++s) ax.radix[s] = s < ax.nst ? c.fft_radix[a][s] : 1;
     ax.tw = c.fft_tw[a];
+    // lines per block: as many as keep the two shared copies within 32 KB and divide the run of adjacent
+    // lines (all of them along x, the x extent for y, the x-y plane for z), while the blocks fill the SMs
+    const int64_t nlines = c.m.ncell / ax.n, run = a == 0 ? nlines : ax.stride;
+    ax.lb = 1;
+    while (ax.lb < 16 && 2 * (2 * ax.lb) * ax.n <= 2048 && run % (2 * ax.lb) == 0 &&
+           (ax.lb < (a == 0 ? 1 : 4) || nf * (nlines / (2 * ax.lb)) >= 2 * c.sms))
+        ax.lb *= 2;
+    ax.mn = multiplier(ax.n);
+    ax.mlb = multiplier(ax.lb);
+    for (int s = 0, L = 1; s < c.fft_nst[a]; ++s) {
+        FftStage& st = ax.st[ax.nst++];
+        st.R = c.fft_radix[a][s];
+        if (st.R == 2 && s + 1 < c.fft_nst[a]) {   // (the 3s come first)
+            st.R = 4;
+            ++s;
+        }
+        st.L = L;
+        st.nb = ax.n / st.R;
+        st.tstep = ax.n / (L * st.R);
+        st.mL = multiplier(L);
+        st.mnb = multiplier(st.nb);
+        L *= st.R;
+    }
     return ax;
 }
 
-// 3D transform of nf contiguous complex fields in place.
-void fft3(Ctx& c, double2* data, int nf, bool inverse) {
-    for (int a = 0; a < 3; ++a) {
-        const FftAxis ax = make_axis(c, a);
-        if (ax.n == 1) continue;
-        const int64_t nlines = c.m.ncell / ax.n;
-        // lines per block: 1 along x (contiguous); along y and z as many adjacent lines as keep
-        // the two shared copies within 32 KB and divide the run of adjacent line starts (the
-        // x extent for y, the x-y plane for z)
-        int lb = 1;
-        if (a > 0) {
-            const int64_t run = a == 1 ? c.m.n[0] : (int64_t)c.m.n[0] * c.m.n[1];
-            while (lb < 16 && 2 * (2 * lb) * ax.n <= 2048 && run % (2 * lb) == 0) lb *= 2;
-        }
-        int threads = std::min(256, std::max(32, ((lb * ax.n / 2 + 31) / 32) * 32));
-        const int64_t gx = std::min<int64_t>(nlines / lb, (int64_t)c.sms * 16);
+// 3D transform of nf contiguous complex fields, in place, or from (forward) or to (inverse) real ones.
+void fft3(Ctx& c, double2* data, int nf, bool inverse, const RealFields* real = nullptr) {
+    const RealFields none;
+    int first = 0, last = 2;
+    while (first < 2 && c.m.n[first] == 1) ++first;
+    while (last > first && c.m.n[last] == 1) --last;
+    for (int a = first; a <= last; ++a) {   // (one pass at least, which converts)
+        if (c.m.n[a] == 1 && first != last) continue;
+        const FftAxis ax = make_axis(c, a, nf);
+        const int threads = std::min(256, std::max(32, ((ax.lb * ax.n / 4 + 31) / 32) * 32));
+        const int64_t gx = std::min<int64_t>(c.m.ncell / (ax.lb * ax.n), (int64_t)c.sms * 16);
         dim3 grid((unsigned)gx, (unsigned)nf);
-        k_fft_axis<<<grid, threads, 2 * lb * ax.n * sizeof(double2), c.stream>>>(data, c.m, ax, inverse ? 1 : 0, lb);
+        k_fft_axis<<<grid, threads, 2 * ax.lb * ax.n * sizeof(double2), c.stream>>>(
+            data, c.m, ax, inverse ? 1 : 0, !inverse && real && a == first ? *real : none,
+            inverse && real && a == last ? *real : none);
         ++c.launches;
     }
 }
 
-void r2c(Ctx& c, const double* in, double2* out, int64_t n) {
-    k_r2c<<<spec_blocks(c, n), THREADS, 0, c.stream>>>(in, out, n);
-    ++c.launches;
+// The state's fields [phi, A (3) | psi, U (3) | rho | gphi (3)] as real fields (null ones left out at the end).
+RealFields state_fields(const Ctx& c, const double* F, const double* W, const double* rho = nullptr,
+                        const double* gphi = nullptr) {
+    const int64_t N = c.m.ncell;
+    RealFields r;
+    for (int f = 0; f < 4; ++f) {
+        r.f[f] = const_cast<double*>(F) + f * N;
+        r.f[4 + f] = const_cast<double*>(W) + f * N;
+    }
+    r.f[8] = const_cast<double*>(rho);
+    for (int f = 0; f < 3 && gphi; ++f) r.f[9 + f] = const_cast<double*>(gphi) + f * N;
+    return r;
 }
 
-void c2r(Ctx& c, const double2* in, double* out, int64_t n, double scale) {
-    k_c2r<<<spec_blocks(c, n), THREADS, 0, c.stream>>>(in, out, n, scale);
-    ++c.launches;
+RealFields fields_of(const Ctx& c, const double* x, int nf, double scale = 1.0) {
+    RealFields r;
+    for (int f = 0; f < nf; ++f) r.f[f] = const_cast<double*>(x) + f * c.m.ncell;
+    r.scale = scale;
+    return r;
 }
 
 }  // namespace
@@ -420,11 +483,8 @@ void spec_twiddles(int n, std::vector<double2>& tw) {
 
 // Start of a step: transforms of the level-n state [phi, A | psi, U | rho] into spec0.
 void launch_spec_begin(Ctx& c) {
-    const int64_t N = c.m.ncell;
-    r2c(c, c.F0, c.spec0, 4 * N);
-    r2c(c, c.W0, c.spec0 + 4 * N, 4 * N);
-    r2c(c, c.rho0, c.spec0 + 8 * N, N);
-    fft3(c, c.spec0, 9, false);
+    const RealFields in = state_fields(c, c.F0, c.W0, c.rho0);
+    fft3(c, c.spec0, 9, false, &in);
 }
 
 // The mesh half of an iteration with spectral operators: e_J partials, continuity and the
@@ -432,28 +492,24 @@ void launch_spec_begin(Ctx& c) {
 void launch_spec_mesh_phase(Ctx& c, const double* Jcur, const double* Jprev) {
     const int64_t N = c.m.ncell;
     const SpecParams p = spec_params(c);
-    k_spec_ej<<<mesh_blocks(c), THREADS, 0, c.stream>>>(N, Jcur, Jprev, c.partials);
+    k_spec_ej<<<mesh_blocks(c), mesh_threads(c), 0, c.stream>>>(N, Jcur, Jprev, c.partials);
     ++c.launches;
-    r2c(c, Jcur, c.specJ, 3 * N);
-    fft3(c, c.specJ, 3, false);
-    k_spec_cn<<<spec_blocks(c, N), THREADS, 0, c.stream>>>(p, c.specJ, c.spec0, c.spec1);
+    const RealFields J = fields_of(c, Jcur, 3);
+    fft3(c, c.specJ, 3, false, &J);
+    k_spec_cn<<<mesh_blocks(c), mesh_threads(c), 0, c.stream>>>(p, c.specJ, c.spec0, c.spec1);
     ++c.launches;
-    fft3(c, c.spec1, 12, true);
-    c2r(c, c.spec1, c.F1, 4 * N, p.invN);
-    c2r(c, c.spec1 + 4 * N, c.W1, 4 * N, p.invN);
-    c2r(c, c.spec1 + 8 * N, c.rho1, N, p.invN);
-    c2r(c, c.spec1 + 9 * N, c.spec_gphi, 3 * N, p.invN);
-    k_spec_table<<<mesh_blocks(c), THREADS, 0, c.stream>>>(N, c.F0, c.W0, c.F1, c.W1, c.spec_gphi, c.table);
+    RealFields out = state_fields(c, c.F1, c.W1, c.rho1, c.spec_gphi);
+    out.scale = p.invN;
+    fft3(c, c.spec1, 12, true, &out);
+    k_spec_table<<<mesh_blocks(c), mesh_threads(c), 0, c.stream>>>(N, c.F0, c.W0, c.F1, c.W1, c.spec_gphi, c.table);
     ++c.launches;
 }
 
 // Field energy of the state (F, W) into partial slot `slot` (spec1 is used as scratch).
 void launch_spec_energy(Ctx& c, const double* F, const double* W, int slot) {
-    const int64_t N = c.m.ncell;
-    r2c(c, F, c.spec1, 4 * N);
-    r2c(c, W, c.spec1 + 4 * N, 4 * N);
-    fft3(c, c.spec1, 8, false);
-    k_spec_energy<<<mesh_blocks(c), THREADS, 0, c.stream>>>(spec_params(c), c.spec1, c.partials, slot);
+    const RealFields in = state_fields(c, F, W);
+    fft3(c, c.spec1, 8, false, &in);
+    k_spec_energy<<<mesh_blocks(c), mesh_threads(c), 0, c.stream>>>(spec_params(c), c.spec1, c.partials, slot);
     ++c.launches;
 }
 
@@ -462,16 +518,14 @@ void launch_spec_diag(Ctx& c, const double* Jfinal) {
     const int64_t N = c.m.ncell;
     const SpecParams p = spec_params(c);
     // level n+1 in spectral form again (the mesh phase transformed spec1 back), its energy
-    r2c(c, c.F1, c.spec1, 4 * N);
-    r2c(c, c.W1, c.spec1 + 4 * N, 4 * N);
-    r2c(c, c.rho1, c.spec1 + 8 * N, N);
-    fft3(c, c.spec1, 9, false);
-    k_spec_energy<<<mesh_blocks(c), THREADS, 0, c.stream>>>(p, c.spec1, c.partials, S_W);
+    const RealFields in = state_fields(c, c.F1, c.W1, c.rho1);
+    fft3(c, c.spec1, 9, false, &in);
+    k_spec_energy<<<mesh_blocks(c), mesh_threads(c), 0, c.stream>>>(p, c.spec1, c.partials, S_W);
     ++c.launches;
-    k_spec_resid<<<spec_blocks(c, N), THREADS, 0, c.stream>>>(p, c.spec1, c.spec0, c.specJ, c.specR);
+    k_spec_resid<<<mesh_blocks(c), mesh_threads(c), 0, c.stream>>>(p, c.spec1, c.spec0, c.specJ, c.specR);
     ++c.launches;
     fft3(c, c.specR, 3, true);
-    k_spec_diag<<<mesh_blocks(c), THREADS, 0, c.stream>>>(p, Jfinal, c.spec_gphi, c.W0, c.W1, c.specR, c.partials);
+    k_spec_diag<<<mesh_blocks(c), mesh_threads(c), 0, c.stream>>>(p, Jfinal, c.spec_gphi, c.W0, c.W1, c.specR, c.partials);
     ++c.launches;
 }
 
@@ -479,24 +533,22 @@ void launch_spec_diag(Ctx& c, const double* Jfinal) {
 // (c.helm_spec: nf N complex scratch; c.helm_s2: the per-axis symbols).
 void launch_helmholtz_fft(Ctx& c, const double* b, double* x, int nf, double a) {
     const int64_t N = c.m.ncell;
-    r2c(c, b, c.helm_spec, nf * N);
-    fft3(c, c.helm_spec, nf, false);
+    const RealFields in = fields_of(c, b, nf), out = fields_of(c, x, nf);
+    fft3(c, c.helm_spec, nf, false, &in);
     k_helm_fft_divide<<<spec_blocks(c, N), THREADS, 0, c.stream>>>(c.m, c.helm_s2, a, 1.0 / (double)N, c.helm_spec,
                                                                    nf);
     ++c.launches;
-    fft3(c, c.helm_spec, nf, true);
-    c2r(c, c.helm_spec, x, nf * N, 1.0);
+    fft3(c, c.helm_spec, nf, true, &out);
 }
 
 // Initial potential: -Delta_h phi = sigma1 rho, zero on the null modes (§5.4).
 void launch_spec_poisson(Ctx& c) {
     const int64_t N = c.m.ncell;
-    r2c(c, c.rho0, c.specR, N);
-    fft3(c, c.specR, 1, false);
+    const RealFields in = fields_of(c, c.rho0, 1), out = fields_of(c, c.F0, 1, 1.0 / (double)N);
+    fft3(c, c.specR, 1, false, &in);
     k_spec_poisson<<<spec_blocks(c, N), THREADS, 0, c.stream>>>(spec_params(c), c.specR);
     ++c.launches;
-    fft3(c, c.specR, 1, true);
-    c2r(c, c.specR, c.F0, N, 1.0 / (double)N);
+    fft3(c, c.specR, 1, true, &out);
 }
 
 }  // namespace pic
