@@ -326,19 +326,22 @@ class PicSim:
 
     STATE_KEYS = ("x", "v", "P", "vprev", "phi", "psi", "rho", "A", "U")
 
+    def _state_tensors(self, make):
+        sizes = {"x": 3 * self.np, "v": 3 * self.np, "P": 3 * self.np, "vprev": 3 * self.np, "phi": self.ncell,
+                 "psi": self.ncell, "rho": self.ncell, "A": 3 * self.ncell, "U": 3 * self.ncell}
+        torch = _torch()
+        return {k: (make if n else torch.zeros)(max(n, 1), dtype=torch.float64, device="cuda") for k, n in sizes.items()}
+
     def state_zeros(self):
         """A dict of zero float64 CUDA tensors in the state layout: particles SoA (3 np),
         mesh x-fastest (ncell, or 3 ncell for A and U)."""
-        torch = _torch()
-        sizes = {"x": 3 * self.np, "v": 3 * self.np, "P": 3 * self.np, "vprev": 3 * self.np, "phi": self.ncell,
-                 "psi": self.ncell, "rho": self.ncell, "A": 3 * self.ncell, "U": 3 * self.ncell}
-        return {k: torch.zeros(max(n, 1), dtype=torch.float64, device="cuda") for k, n in sizes.items()}
+        return self._state_tensors(_torch().zeros)
 
     def _dview(self, d):
         return PicStateView(*[d[k].data_ptr() for k in self.STATE_KEYS], 1)
 
     def get_state_device(self):
-        d = self.state_zeros()
+        d = self._state_tensors(_torch().empty)   # (every element is written)
         pic_get_state(self.ctx, self._dview(d))
         return d
 
