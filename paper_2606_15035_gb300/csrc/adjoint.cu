@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_scatter(
 #pragma unroll 1
         for (int item = 0; item < 2; ++item) {
             CellStart<double> st;
-            double vs[3], beta[3], bs[3], f[3] = {0.0, 0.0, 0.0}, lg[3] = {0.0, 0.0, 0.0}, lA[3] = {0.0, 0.0, 0.0};
+            double vs[3], beta[3], f[3] = {0.0, 0.0, 0.0}, lg[3] = {0.0, 0.0, 0.0}, lA[3] = {0.0, 0.0, 0.0};
             const int64_t i = co.take(item, base, st, vs);
             const bool act = i < np;
             double fs = 0.0;
@@ -286,7 +286,6 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_scatter(
                     vs[a] = 0.0;
                 }
                 beta[a] = p.cb[a] * vs[a];
-                bs[a] = 0.28867513459481288225 * beta[a];   // 1 / sqrt(12)
                 fs += fabs(f[a]);
             }
             // |a piece's sums| < 1.2 fs: an exponent above that of fs

@@ -403,7 +403,19 @@ __device__ __forceinline__ void flush_jtile(const Params32& p, const Box& b, con
     }
 }
 
-// FP64 masters -> FP32 working set; first iterate v^{n+1,0} = 2 v^n - v^{n-1}, as an increment.
+// (float)x, round to nearest even, on the integer pipe in the normal range.
+__device__ __forceinline__ float to_float(double x) {
+    const int hi = __double2hiint(x), lo = __double2loint(x), e = (hi >> 20) & 0x7ff;
+    if (e < 897 || e > 1150) return (float)x;
+    unsigned b = ((unsigned)(e - 896) << 23) | ((unsigned)(hi & 0xfffff) << 3) | ((unsigned)lo >> 29);
+    const unsigned rest = (unsigned)lo & 0x1fffffffu;
+    b += (rest > 0x10000000u || (rest == 0x10000000u && (b & 1u))) ? 1u : 0u;
+    return __uint_as_float(b | ((unsigned)hi & 0x80000000u));
+}
+
+// FP64 masters -> FP32 working set; first iterate v^{n+1,0} = 2 v^n - v^{n-1}, as an increment.  At 128^3
+// with 134M particles 9.6 ms when its conversions and range tests ran on the FP64 pipe, now 5.8 (its bytes
+// would take 2.2; the square root remains).
 __global__ void k_to32(Params32 p, const double* __restrict__ xi, const double* __restrict__ v,
                        const double* __restrict__ vprev, int32_t* __restrict__ cell, float* __restrict__ off,
                        float* __restrict__ v32, float* __restrict__ vit32, double* __restrict__ partials) {
@@ -414,15 +426,15 @@ __global__ void k_to32(Params32 p, const double* __restrict__ xi, const double* 
         int32_t packed = 0;
         const double va = v[i], vb = v[np + i], vc = v[2 * np + i];
         jsc += sqrt(va * va + vb * vb + vc * vc);
+        CellStart<double> st;
+        const double x0[3] = {xi[i], xi[np + i], xi[2 * np + i]}, vn[3] = {va, vb, vc};
+        cell_start(x0, p.m, st);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            const double x = xi[a * np + i];
-            const int c = min(max(__double2int_rd(x), 0), p.m.n[a] - 1);
-            off[a * p.stride + i] = (float)(x - (double)c);
-            packed |= (c & CELL_MASK) << (a * CELL_BITS);
-            const double vv = v[a * np + i];
-            v32[a * p.stride + i] = (float)vv;
-            vit32[a * p.stride + i] = (float)(vv - vprev[a * np + i]);   // (2 v^n - v^{n-1}) - v^n
+            off[a * p.stride + i] = to_float(st.f[a]);
+            packed |= (st.c[a] & CELL_MASK) << (a * CELL_BITS);
+            v32[a * p.stride + i] = to_float(vn[a]);
+            vit32[a * p.stride + i] = to_float(vn[a] - vprev[a * np + i]);   // (2 v^n - v^{n-1}) - v^n
         }
         cell[i] = packed;
     }

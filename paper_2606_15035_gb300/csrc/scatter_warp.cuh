@@ -84,8 +84,7 @@ __device__ __forceinline__ int64_t subset_node(const int c0[3], int k, const Mes
 // In the push it takes 46 FP64 instructions a piece off the pipe that bounds it (1.59 -> 1.43 ms).
 //
 // Add the orbit currents q v_bar S_bar / dV (weights w, orbits st.f + s beta) of the lanes with `act`
-// to J.  Every lane of the warp calls it; `tile` is the warp's DEPOSIT_TILE words.  bs = beta /
-// sqrt(12).  Returns the lane's number of breakpoint intervals (-1: too many; 0: not active).
+// to J.  Every lane of the warp calls it; `tile` is the warp's DEPOSIT_TILE words.  Returns the lane's number of breakpoint intervals (-1: too many; 0: not active).
 __device__ __forceinline__ int scatter_warp(const MeshDims& m, bool act, const CellStart<double>& st,
                                             const double beta[3], const double w[3], long long* tile, int det,
                                             const ExactAcc& acc, double* __restrict__ J) {
@@ -123,10 +122,7 @@ __device__ __forceinline__ int scatter_warp(const MeshDims& m, bool act, const C
     // this lane's unit: component lane / 8 (lanes 24..31 sum nothing)
     const int comp = min(lane >> 3, 2);
     const double unit = __hiloint2double(((comp == 0 ? top[0] : (comp == 1 ? top[1] : top[2])) - 56) << 20, 0);
-    const double rs12 = 0.28867513459481288225;   // 1 / sqrt(12)
-    double bs[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) bs[a] = rs12 * beta[a];
+    const Fx c12 = fx_split(FX_ONE / 12);
     PieceWalk<double> wk(st, beta, m);
     bool last = !act;
     while (__any_sync(full, !last)) {
@@ -145,9 +141,10 @@ __device__ __forceinline__ int scatter_warp(const MeshDims& m, bool act, const C
             for (int a = 0; a < 3; ++a) {
                 M[1 << a] = fixed_of(mid[a], 1023, 10);
                 q[a] = fx_split(M[1 << a]);
-                d[a] = fx_split(fixed_of(h * bs[a], 1023, 10));
+                d[a] = fx_split(fixed_of(h * beta[a], 1023, 10));
             }
-            const long long kxy = fx_mul(d[0], d[1]), kxz = fx_mul(d[0], d[2]), kyz = fx_mul(d[1], d[2]);
+            const Fx dy = fx_split(fx_mul(d[1], c12)), dz = fx_split(fx_mul(d[2], c12));
+            const long long kxy = fx_mul(d[0], dy), kxz = fx_mul(d[0], dz), kyz = fx_mul(d[1], dz);
             M[3] = fx_mul(q[0], q[1]) + kxy;
             M[5] = fx_mul(q[0], q[2]) + kxz;
             M[6] = fx_mul(q[1], q[2]) + kyz;
