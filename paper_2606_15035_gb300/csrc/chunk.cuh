@@ -43,8 +43,14 @@ struct ChunkOrder {
 };
 
 // The chunk sizes: four warps with two groups each, or, for runs too small to fill the SMs that way,
-// one group per block.
+// one group per block.  The pushes, whose instruction stream passes the caches of an SM's schedulers (the
+// first stall reason with four warps a block: the blocks' warps are at different places of it), take eight
+// warps a block where each resident block gets two chunks or more: at 32^3 with 2,097,152 particles 1.03 ->
+// 0.96 ms (iterate) and 0.68 -> 0.65 (final sweep), in pairs 0.88 -> 0.81; at 128^3 with 134M 59.0 -> 53.9
+// and 82.8 -> 70.9; sixteen warps 1.04, 0.75, 0.87, 59.8 and 70.6.  With 131,072 particles four warps take
+// 63 us, eight 69.  The deposits by themselves prefer four (354 against 385 us).
 typedef ChunkOrder<4, 2> ChunkLarge;
+typedef ChunkOrder<8, 2> ChunkPush;
 typedef ChunkOrder<1, 1> ChunkSmall;
 
 // Knots crossed by an axis whose orbit ends at te (relative to its start cell).

@@ -1,5 +1,5 @@
-// Device helpers shared by the FP64 push (particles.cu) and the FP32-pair push
-// (particles_df.cu): the ordering of a chunk's particles by orbit-piece count, the per-particle
+// Device helpers shared by the particle kernels: the ordering of a block's particles by orbit-piece
+// count (Gauss rules; the closed forms order chunks, chunk.cuh), the per-particle
 // slide byte, the slow-particle gate of the particle-local solves, and the per-block partials.
 #pragma once
 

@@ -1,9 +1,10 @@
 // Particle kernels of the orbit-averaged PIC step (FP64, sm_103a).
 //
-// One particle per thread, grid-stride loops, particles in structure-of-arrays layout
-// (component c of particle i at c * np + i) and cell-sorted so that neighbouring
-// threads gather the same mesh nodes.  Mesh data for the gather come from a per-node
-// table of 12 doubles: A^n (3), A^{n+1,p} (3), grad_h phi^{n+1/2,p} (3), U^{n+1/2,p} (3).
+// Particles in structure-of-arrays layout (component c of particle i at c * np + i), cell-sorted
+// so that neighbouring threads gather the same mesh nodes.  The closed forms take one particle per thread
+// from chunks ordered by piece count (chunk.cuh) and the mesh fields from the cell tables (orbit_cell.cuh);
+// the Gauss rules, and the closed forms without cell tables, take them from a per-node table of 12 doubles:
+// A^n (3), A^{n+1,p} (3), grad_h phi^{n+1/2,p} (3), U^{n+1/2,p} (3).
 #include <algorithm>
 #include <cmath>
 
@@ -786,7 +787,9 @@ __global__ void __launch_bounds__(32 * WARPS, SCATTER_WARPS / WARPS) k_first_sca
 // FP64 warp instructions in the iterate); 1.59 and 1.11 with centred moments and the cell's mixed
 // differences (25.6M); 1.43 with the fixed-point deposit; 1.22 and 0.77 with the fixed-point pieces
 // (11.4M and 9.0M, the pipe 52% and 62% busy); 1.13 and 0.73 with chunks whose warps have equal work and
-// sums of products shifted once.  At 128^3 with 134M particles the final sweep took 225, 102, now 64 ms.
+// sums of products shifted once; 1.03 and 0.68 with the one-crossing walk (10.3M and 7.5M); 0.96 and 0.65 with
+// eight warps a block (chunk.cuh).  At 128^3 with 134M particles the final sweep took 225, 102, 64, now 54 ms.
+// What is left is latency (36% issue-active): fixed-latency waits, shared memory, the instruction cache.
 template <bool COMMIT, bool FIXED, int WARPS, int ITEMS>
 __global__ void __launch_bounds__(32 * WARPS, PUSH_WARPS / WARPS) k_push_cell(StepParams p, const double* __restrict__ xi,
                                                           const double* __restrict__ v, const double* __restrict__ P,
@@ -992,7 +995,7 @@ __device__ __forceinline__ void piece_diag(double h, double sm, const double mid
 // (FP64; CELLS: from the cell table).  Bound by the FP64 pipe like that: some 240 operations a piece where
 // the integrals from the piece's start took some 700: 1.62 ms at 50 x 35 x 22 with 539,000 particles, now
 // 0.68.
-constexpr int DIAG_WARPS = 12;
+constexpr int DIAG_WARPS = 16;   // 12 (168 registers): two steps at 16^3 2.77 ms, 16 2.69
 template <bool CELLS, int WARPS, int ITEMS>
 __global__ void __launch_bounds__(32 * WARPS, DIAG_WARPS / WARPS) k_commit_diag(
     StepParams p, const double* __restrict__ xi, const double* __restrict__ v, const double* __restrict__ P,
@@ -1092,9 +1095,9 @@ __global__ void __launch_bounds__(32 * WARPS, DIAG_WARPS / WARPS) k_commit_diag(
 //              The next iterate is G(v^p); with p.accel, creeping particles are instead
 //              appended to a list and solved locally by k_local (which also scatters them);
 //   (commit)   x^{n+1}, P^{n+1}, v^{n+1} and (optionally) the particle diagnostics.
-// Two resident blocks per SM (at most 128 registers, a few spills) hide more of the FP64
-// pipe's latency than one block at 178 registers (measured: 5% less push time at 32^3); the
-// diagnostics variant keeps one block, its larger state would spill far more.
+// For the Gauss rules; the closed forms run k_push_cell and k_commit_diag.  Two resident blocks per SM (128
+// registers, some spills): quadratic shapes at 36^3 2.26 ms, one block (255 registers) 2.40; the diagnostics
+// variant keeps one block, its larger state would spill far more.
 template <bool COMMIT, bool DIAG>
 __global__ void __launch_bounds__(THREADS, DIAG ? 1 : 2) k_push(StepParams p, const double* __restrict__ xi,
                                                   const double* __restrict__ v, const double* __restrict__ P,
@@ -2029,15 +2032,20 @@ StepParams make_params(const Ctx& c) {
 // Opt the depositing kernels in to their dynamic shared memory (above the 48 KB default where the chunk
 // is large; once per context, on its device).
 bool setup_particle_kernels() {
-    const int bytes = (int)ChunkLarge::smem();
+    const int bytes = (int)ChunkLarge::smem(), push = (int)ChunkPush::smem();
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
     return cudaFuncSetAttribute(k_first_scatter_cell<4, 2>, at, bytes) == cudaSuccess &&
            cudaFuncSetAttribute(k_push_cell<false, true, 4, 2>, at, bytes) == cudaSuccess &&
-           cudaFuncSetAttribute(k_push_cell<false, false, 4, 2>, at, bytes) == cudaSuccess;
+           cudaFuncSetAttribute(k_push_cell<false, false, 4, 2>, at, bytes) == cudaSuccess &&
+           cudaFuncSetAttribute(k_push_cell<false, true, 8, 2>, at, push) == cudaSuccess &&
+           cudaFuncSetAttribute(k_push_cell<false, false, 8, 2>, at, push) == cudaSuccess;
 }
 
 // Chunks of one warp while they leave every scheduler at most two of them.
 bool small_chunks(const Ctx& c) { return c.np <= (int64_t)c.sms * 8 * ChunkSmall::SIZE; }
+
+// The pushes' larger chunks (two blocks an SM) while each block gets at least two.
+bool wide_chunks(const Ctx& c) { return c.np >= 2 * (int64_t)c.sms * 2 * ChunkPush::SIZE; }
 
 // Grid of the kernels that walk chunks, and of the push of this context's kind (partials per block).
 int chunk_blocks(const Ctx& c) {
@@ -2109,7 +2117,7 @@ void launch_push(Ctx& c, const double* vit, double* vnew, double* Jnext, bool co
                                                   c.slide,                                                    \
                                                   c.partials, c.dev_status)
     const CellFields cf{c.fxtab ? c.ctab : c.table, reinterpret_cast<const longlong2*>(c.fxtab), c.cell_top};
-    const bool small = small_chunks(c);
+    const bool small = small_chunks(c), wide = wide_chunks(c);
 #define PIC_PUSH_CELL_AS(C, T, W, I)                                                                              \
     k_push_cell<C, T, W, I><<<chunk_blocks(c), 32 * W, C ? sizeof(ChunkOrder<W, I>) : ChunkOrder<W, I>::smem(),     \
                               c.stream>>>(p, c.xi, c.v, c.P, vit, cf, vnew, Jnext, c.xi_new, c.P_new, c.creep_list, \
@@ -2118,6 +2126,7 @@ void launch_push(Ctx& c, const double* vit, double* vnew, double* Jnext, bool co
 #define PIC_PUSH_CELL(C, T)                \
     do {                                   \
         if (small) PIC_PUSH_CELL_AS(C, T, 1, 1); \
+        else if (wide) PIC_PUSH_CELL_AS(C, T, 8, 2); \
         else PIC_PUSH_CELL_AS(C, T, 4, 2);       \
     } while (0)
 #define PIC_COMMIT_DIAG(T, W, I)                                                                                  \

@@ -27,8 +27,8 @@
 namespace pic {
 namespace {
 
-// Blocks per SM: 16 warps (128 registers) measured 88.5 ms at 128^3 with 134M particles, 24 (85) 100.4.
-constexpr int DF_MINB = 4;
+// Warps per SM: 16 (128 registers) measured 88.5 ms at 128^3 with 134M particles, 24 (85) 100.4.
+constexpr int DF_WARPS = 16;
 
 struct ParamsDF {
     StepParams p;       // the FP64 parameters (creeping tests, residual sums, iterate I/O)
@@ -94,10 +94,11 @@ struct PairLoad<false> {
 };
 
 // The FP32-pair iteration (239 -> 88.5 ms at 128^3 with 134M particles, from start-based integrals, a
-// node table and shared 64-bit atomics before): G(v^p) for every particle, creeping ones listed for k_local (as in
+// node table and shared 64-bit atomics before; 70.9 with the one-crossing walk, deposit columns by cell and
+// blocks of eight warps): G(v^p) for every particle, creeping ones listed for k_local (as in
 // k_push_cell), the e_v partial sums, and the orbit current of v^{p+1} = G(v^p) into Jnext.
-template <bool CELLS>
-__global__ void __launch_bounds__(ChunkLarge::THREADS_, DF_MINB) k_push_df(ParamsDF pd, const double* __restrict__ xi,
+template <bool CELLS, typename Chunk>
+__global__ void __launch_bounds__(Chunk::THREADS_, 32 * DF_WARPS / Chunk::THREADS_) k_push_df(ParamsDF pd, const double* __restrict__ xi,
                                                                const double* __restrict__ v,
                                                                const double* __restrict__ P,
                                                                const double* __restrict__ vit,
@@ -110,14 +111,14 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, DF_MINB) k_push_df(Param
                                                                int* __restrict__ status) {
     __shared__ double sm[32];
     extern __shared__ __align__(16) unsigned char dyn[];
-    ChunkLarge& co = ChunkLarge::in(dyn);
-    long long* tile = ChunkLarge::tile(dyn);
+    Chunk& co = Chunk::in(dyn);
+    long long* tile = Chunk::tile(dyn);
     const StepParams& p = pd.p;
-    const int64_t np = p.np, nchunks = (np + ChunkLarge::SIZE - 1) / ChunkLarge::SIZE;
+    const int64_t np = p.np, nchunks = (np + Chunk::SIZE - 1) / Chunk::SIZE;
     double ev_num = 0.0, ev_den = 0.0;
     long long pieces_push = 0, pieces_scatter = 0;
     for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-        const int64_t base = ch * ChunkLarge::SIZE;
+        const int64_t base = ch * Chunk::SIZE;
         chunk_exchange(p, co, base, [&](int64_t j, double x0[3], double v2[3]) {
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
@@ -245,8 +246,10 @@ ParamsDF make_params_df(const Ctx& c) {
 
 bool setup_pair_kernels() {
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    return cudaFuncSetAttribute(k_push_df<true>, at, (int)ChunkLarge::smem()) == cudaSuccess &&
-           cudaFuncSetAttribute(k_push_df<false>, at, (int)ChunkLarge::smem()) == cudaSuccess;
+    return cudaFuncSetAttribute(k_push_df<true, ChunkLarge>, at, (int)ChunkLarge::smem()) == cudaSuccess &&
+           cudaFuncSetAttribute(k_push_df<false, ChunkLarge>, at, (int)ChunkLarge::smem()) == cudaSuccess &&
+           cudaFuncSetAttribute(k_push_df<true, ChunkPush>, at, (int)ChunkPush::smem()) == cudaSuccess &&
+           cudaFuncSetAttribute(k_push_df<false, ChunkPush>, at, (int)ChunkPush::smem()) == cudaSuccess;
 }
 
 void launch_table_df(Ctx& c) {
@@ -265,12 +268,15 @@ void launch_push_df(Ctx& c, const double* vit, double* vnew, double* Jnext) {
     cudaMemsetAsync(c.creep_count, 0, 2 * sizeof(int), c.stream);   // count, k_local queue head
     const int nb = chunk_blocks(c);
     const float4* t = reinterpret_cast<const float4*>(c.table_pair);
-#define PIC_PUSH_DF(T)                                                                                            \
-    k_push_df<T><<<nb, ChunkLarge::THREADS_, ChunkLarge::smem(), c.stream>>>(make_params_df(c), c.xi, c.v, c.P, vit, t, vnew, Jnext,     \
-                                                        c.creep_list, c.creep_count, c.slide, c.partials,          \
-                                                        c.dev_status)
-    if (c.pair_cells) PIC_PUSH_DF(true);
-    else PIC_PUSH_DF(false);
+#define PIC_PUSH_DF(T, K)                                                                                           \
+    k_push_df<T, K><<<nb, K::THREADS_, K::smem(), c.stream>>>(make_params_df(c), c.xi, c.v, c.P, vit, t, vnew, Jnext, \
+                                                              c.creep_list, c.creep_count, c.slide, c.partials,    \
+                                                              c.dev_status)
+    const bool wide = wide_chunks(c);
+    if (c.pair_cells && wide) PIC_PUSH_DF(true, ChunkPush);
+    else if (c.pair_cells) PIC_PUSH_DF(true, ChunkLarge);
+    else if (wide) PIC_PUSH_DF(false, ChunkPush);
+    else PIC_PUSH_DF(false, ChunkLarge);
 #undef PIC_PUSH_DF
     ++c.launches;
 }

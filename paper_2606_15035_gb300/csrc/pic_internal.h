@@ -377,6 +377,7 @@ StepParams make_params(const Ctx& c);
 bool setup_particle_kernels();
 bool setup_pair_kernels();
 int particle_blocks(const Ctx& c);
+bool wide_chunks(const Ctx& c);
 int chunk_blocks(const Ctx& c);   // the closed forms' chunk kernels
 int push_blocks(const Ctx& c);    // the pushes and the first scatter
 int local_blocks(const Ctx& c);

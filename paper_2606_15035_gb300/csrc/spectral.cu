@@ -11,7 +11,7 @@
 // src = J_c^{n+1/2} (c = sigma2) for (A_c, U_c); continuity (Eq. (cn-continuity)) is
 // rho^{n+1} = rho^n - dt D . J in the same basis.
 //
-// Transforms: a batched, mixed-radix (2 and 3) Stockham FFT of complex FP64 lines, one line
+// Transforms: a batched, mixed-radix (4, 2 and 3) Stockham FFT of complex FP64 lines, up to 16 lines
 // per block in shared memory, applied along x, y and z; unnormalised forward transform and
 // a 1/N scale on the way back to real space.  Mesh sizes n_a = 2^p 3^q <= 1024.
 #include <cmath>

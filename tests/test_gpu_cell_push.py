@@ -247,3 +247,35 @@ def test_fp32_iterations_end_near_the_fp64_fixed_point(sim, npart):
     rest = [e for k, e in zip(kind, e_v) if k != 1]
     s.close()
     assert len(fp32) >= 2 and fp32[0] > 1e-5 and rest[0] <= 1e-6, (kind, e_v)
+
+
+@pytest.mark.parametrize("more", [-1, 3])
+def test_chunk_sizes_of_the_pushes(sim, more):
+    """On both sides of the particle count from which the pushes take chunks of 512 (two for each of two
+    blocks an SM), with a last chunk of one warp: one body against the oracle with the tolerances
+    above, and the FP32-pair iteration by the FP64 residual of what it leaves: 1e-9 is a hundred times
+    its 1e-15 of v over dv / v of 1e-4."""
+    import torch
+    npart = 2 * 2 * 512 * torch.cuda.get_device_properties(0).multi_processor_count + more
+    n, L = (8, 8, 8), (8.0, 8.0, 8.0)
+    rng = np.random.default_rng(5)
+    x = rng.uniform(0, 1, size=(npart, 3)) * L
+    v = rng.normal(scale=0.5, size=x.shape)
+    q = -1e-2 / npart
+    kw = dict(n=n, L=L, dt=1.0, picard_tol=1e-13)
+    s = sim.PicSim(sim.pic_config_default(**kw), x, v, q, 1.0 / npart)
+    ocfg = opic.Config(**kw)
+    g = s.iterate(v)
+    s.close()
+    it = opic.picard_iteration(opic.init(x, v, q, 1.0 / npart, ocfg), v, ocfg, ocfg.grid())
+
+    def rel(a, r):
+        return np.linalg.norm(a - r) / max(np.linalg.norm(r), 1e-300)
+
+    assert rel(g["J"], it["J"]) <= 1e-13 and rel(g["P"], it["P"]) <= 1e-13 and rel(g["v"], it["v_new"]) <= 1e-13
+    s = sim.PicSim(sim.pic_config_default(precision=1, **kw), x, v, q, 1.0 / npart)
+    assert s.step(1).converged
+    e_v, _, kind = s.residual_history()
+    s.close()
+    pair = [i for i, k in enumerate(kind) if k == 2]
+    assert pair and e_v[pair[-1] + 1] <= 1e-9, (kind, e_v)
