@@ -49,16 +49,20 @@ HBM_FALLBACK_GBS = 6800.0
 SUB_CELLS = 16            # the CPU oracle's sample: a periodic sub-box of SUB_CELLS^3 cells
 CPU_STEPS = 10            # timed oracle steps of the cpu_baseline leg
 
-# Algorithmic FP64 flops (add, mul = 1, FMA = 2; the scatter's atomic adds counted) of the
-# fused push + next-orbit scatter kernel, counted from the kernel source per particle and per
-# knot-free orbit piece:
-FLOPS_PER_PARTICLE = 190
-FLOPS_PER_PUSH_PIECE = 409
-FLOPS_PER_SCATTER_PIECE = 150
+# FP64 operations (add, mul, division = 1, FMA = 2) left on the FP64 pipe in the fused push +
+# next-orbit scatter kernel, counted from its source: per particle hand-over, displacement, end
+# point, momentum and velocity update and residual; per push piece the walk (12, and 5 a crossing);
+# per scatter piece the walk and weights (26) and the next orbit's setup (34).  The pieces'
+# moments, contractions and deposits, some 290 a piece, run in 64-bit fixed point on the integer pipe
+# and are not counted.
+FLOPS_PER_PARTICLE = 73
+FLOPS_PER_PUSH_PIECE = 17
+FLOPS_PER_SCATTER_PIECE = 60
 # The survey's lower estimate of the same work (its per-orbit count split into a per-particle part
 # and a per-piece part: weights 110, grad phi 24, A^(m) and C 72, contraction 48, transverse 72,
 # D sum 48 and scatter 24 per piece; point gather 36, push and orbit 30, next-orbit weights 20 per
-# particle), reported beside the source count so that both fractions are visible.
+# particle), reported beside the source count.  Its fraction of the FP64 peak passes 1: most of that
+# work is off the FP64 pipe.
 MIN_FLOPS_PER_PARTICLE = 86
 MIN_FLOPS_PER_PIECE = 398
 # Bytes per particle-iteration of the FP32 push (read cell 4, offset 12, v^n 12, increment 12;
@@ -68,12 +72,12 @@ BYTES32_PER_PARTICLE = 52
 # keyed by kernel and workload, with how the figure was obtained (absent: not captured for this
 # version).  The 128^3 run is too large for a multi-pass capture, so its k_push figure is the
 # 32^3 capture (2,097,152 particles, third Picard iteration) scaled by the particle count: the
-# kernel's traffic is its particle streams, 141.7 B per particle-iteration there.
+# kernel's traffic is its particle streams, 163 B per particle-iteration there.
 NCU_TRAFFIC = {
-    ("k_push", "twostream-32c-2M"): (297.07e6, "ncu capture, one launch (dram read 259.32 MB + write 37.75 MB)"),
-    ("k_push", "twostream-128c-134M"): (297.07e6 * 64, "the 32^3 capture scaled by particles (x 64)"),
-    ("k_push32", "twostream-32c-2M"): (96.43e6, "ncu capture, one launch (dram read 86.57 MB + write 9.86 MB)"),
-    ("k_push32", "twostream-128c-134M"): (96.43e6 * 64, "the 32^3 capture scaled by particles (x 64)"),
+    ("k_push", "twostream-32c-2M"): (342.53e6, "ncu capture, one launch (dram read 278.20 MB + write 64.33 MB)"),
+    ("k_push", "twostream-128c-134M"): (342.53e6 * 64, "the 32^3 capture scaled by particles (x 64)"),
+    ("k_push32", "twostream-32c-2M"): (96.59e6, "ncu capture, one launch (dram read 86.46 MB + write 10.13 MB)"),
+    ("k_push32", "twostream-128c-134M"): (96.59e6 * 64, "the 32^3 capture scaled by particles (x 64)"),
 }
 
 
@@ -443,10 +447,11 @@ def fp64_push_roofline(prof, workload):
     achieved_min = min_flops / (prof.push_ms / 1e3) / 1e12
     return {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
             "frac": achieved / FP64_PEAK_TFLOPS,
-            "flops_basis": "counted from the kernel source (add, mul = 1, FMA = 2): 190 per particle + 409 per push "
-                           "piece + 150 per scatter piece",
+            "flops_basis": "FP64 pipe only, from the kernel source (add, mul = 1, FMA = 2): 73 per particle + 17 per push "
+                           "piece + 60 per scatter piece; the pieces' contractions and deposits run on the integer pipe",
             "frac_survey_minimum": achieved_min / FP64_PEAK_TFLOPS,
-            "survey_minimum_basis": "86 per particle + 398 per orbit piece (the survey's per-orbit estimate)",
+            "survey_minimum_basis": "86 per particle + 398 per orbit piece (the survey's per-orbit estimate), over the FP64 "
+                                    "peak; above 1 where that work runs on the integer pipe",
             "traffic": NCU_TRAFFIC.get(("k_push", workload), (None, None))[0],
             "traffic_unit": "DRAM bytes per launch (ncu dram read + write)",
             "traffic_source": NCU_TRAFFIC.get(("k_push", workload), (None, "not captured"))[1],
@@ -469,10 +474,11 @@ def final_sweep_roofline(prof, workload, npart):
     min_flops = prof.commit_launches * npart * (MIN_FLOPS_PER_PARTICLE + MIN_FLOPS_PER_PIECE * msc)
     return {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
             "frac": achieved / FP64_PEAK_TFLOPS,
-            "flops_basis": "counted from the kernel source (add, mul = 1, FMA = 2): 190 per particle + 409 per push "
-                           "piece (no scatter in the final sweep)",
+            "flops_basis": "FP64 pipe only, from the kernel source (add, mul = 1, FMA = 2): 73 per particle + 17 per push "
+                           "piece (no scatter in the final sweep); the contractions run on the integer pipe",
             "frac_survey_minimum": min_flops / (prof.commit_ms / 1e3) / 1e12 / FP64_PEAK_TFLOPS,
-            "survey_minimum_basis": "86 per particle + 398 per orbit piece (the survey's per-orbit estimate)",
+            "survey_minimum_basis": "86 per particle + 398 per orbit piece (the survey's per-orbit estimate), over the FP64 "
+                                    "peak; above 1 where that work runs on the integer pipe",
             "traffic": None, "traffic_unit": "DRAM bytes per launch (ncu dram read + write)",
             "traffic_source": "not captured for the commit variant",
             "kernel": "k_push (FP64 final sweep: push of the accepted orbit, commit, residual sums)",
@@ -493,7 +499,7 @@ def pair_push_summary(prof, npart, step_ms):
     return {"kernel": "k_push_df (FP32-pair push + next-orbit current scatter)", "launches": int(prof.pushpair_launches),
             "ms_per_launch": ms_l, "share_of_step": prof.pushpair_ms / step_ms if step_ms > 0 else None,
             "fp64_equivalent_tflops": flops / (ms_l / 1e3) / 1e12,
-            "note": "FP32 pipes, four blocks per SM; the FP64 push's flop count for the same work, per launch time"}
+            "note": "FP32 pairs, 16 warps per SM; the flops the FP64 push has on its FP64 pipe, per launch time"}
 
 
 def fp32_push_roofline(prof, workload, npart, hbm_gbs, hbm_note):
