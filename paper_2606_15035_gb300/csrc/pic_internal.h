@@ -322,7 +322,7 @@ struct HelmPlan {
     const float* s2;
 };
 // More corrections than this (lmax above 40,000: a time step of many light crossings of a cell) and the
-// Helmholtz solves go through FP64 transforms.
+// Helmholtz solves go through FP64 transforms (2^p 3^q meshes) or Chebyshev steps.
 constexpr int HELM_MAX_CORRECTIONS = 8;
 // Corrections that bring an error of one below `to` (0: more than HELM_MAX_CORRECTIONS).  The FP32
 // transforms leave about 2^-22 of the residual, which is at most lmax times the error: 3 to roundoff at
