@@ -74,13 +74,15 @@ struct PieceWalk {
             c[a] = st.c[a];
             fd[a] = st.f[a];
             te[a] = fd[a] + beta[a];
-            if (below_zero(te[a]) && is_zero(fd[a])) {   // on a knot, moving down: the cell below
+            const bool down = below_zero(te[a]);
+            if (down && is_zero(fd[a])) {   // on a knot, moving down: the cell below
                 c[a] = prev_cell(c[a], m.n[a]);
                 fd[a] = T(1);
                 te[a] = T(1) + beta[a];
             }
             sn[a] = T(2);                          // 2: no crossing ahead
-            if (at_least_one(te[a]) || below_zero(te[a])) ahead |= 1u << a;
+            // (an end of one after a move down: 1 + beta rounds to one, the orbit stays below the knot)
+            if (below_zero(te[a]) || (!down && at_least_one(te[a]))) ahead |= 1u << a;
         }
         for (; ahead; ahead &= ahead - 1) {
             const int a = __ffs(ahead) - 1;
