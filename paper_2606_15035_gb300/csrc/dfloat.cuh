@@ -115,6 +115,7 @@ __device__ __forceinline__ DF ceil(DF a) {
 // order and range tests of the orbit walk (orbit_cell.cuh)
 __device__ __forceinline__ bool less_pos(DF a, DF b) { return a < b; }
 __device__ __forceinline__ bool same_bits(DF a, DF b) { return a == b; }
+__device__ __forceinline__ bool before_end(DF s) { return s < DF(1.f); }
 __device__ __forceinline__ bool at_least_one(DF t) { return t.hi > 1.f || (t.hi == 1.f && t.lo >= 0.f); }
 __device__ __forceinline__ bool below_zero(DF t) { return t.hi < 0.f || (t.hi == 0.f && t.lo < 0.f); }
 __device__ __forceinline__ bool is_zero(DF t) { return t.hi == 0.f && t.lo == 0.f; }

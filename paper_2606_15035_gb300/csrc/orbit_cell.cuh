@@ -43,6 +43,9 @@ __device__ __forceinline__ bool less_pos(float a, float b) { return a < b; }
 __device__ __forceinline__ bool same_bits(float a, float b) { return a == b; }
 __device__ __forceinline__ bool at_least_one(float t) { return t >= 1.f; }
 __device__ __forceinline__ bool below_zero(float t) { return t < 0.f; }
+// 0 <= s < 1 (not a NaN of either sign)
+__device__ __forceinline__ bool before_end(double s) { return in_box(s, 1.0); }
+__device__ __forceinline__ bool before_end(float s) { return s < 1.f; }
 __device__ __forceinline__ bool is_zero(float t) { return t == 0.f; }
 __device__ __forceinline__ bool is_zero(double t) { return (__double_as_longlong(t) << 1) == 0; }
 
@@ -109,7 +112,7 @@ struct PieceWalk {
     static __device__ __forceinline__ T crossing(T f, T t, T b) {
         const bool down = below_zero(t);
         const T s = (down ? f : T(1) - f) / (down ? -b : b);
-        return less_pos(s, T(1)) ? s : T(2);
+        return before_end(s) ? s : T(2);
     }
 
     // The next breakpoint (1: the end of the orbit).

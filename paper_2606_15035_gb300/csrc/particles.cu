@@ -705,8 +705,9 @@ __device__ __forceinline__ void push_eval_cell(const StepParams& p, CellStart<do
             piece_impulse_fixed(h, sm, mid, d, v, FixedLoad(cf.tfx, c, p.m), accF, accG);
         });
         cell_A1_fixed(st.f, FixedLoad(cf.tfx, st.c, p.m), A1);
-        // values that are not finite stay so
-        const bool ok = max(ev, max(eA, eG)) < 2047;
+        // values that are not finite stay so (the start's coordinate: the end's is its sum with beta)
+        const int ef = max(max(exponent_of(st.f[0]), exponent_of(st.f[1])), exponent_of(st.f[2]));
+        const bool ok = max(max(ev, ef), max(eA, eG)) < 2047;
         const double uF = ok ? p.dtq * pow2_biased(eA + ev - 1079) : NAN;
         const double uG = ok ? p.dtq * pow2_biased(eG - 57) : NAN, uA = pow2_biased(eA - 57);
         const double* low = cf.t64 + CELL_VALUES * cell_row(st.c, p.m);

@@ -93,16 +93,18 @@ __device__ __forceinline__ int scatter_warp(const MeshDims& m, bool act, const C
     const int lane = threadIdx.x & 31;
     const int64_t N = m.ncell;
     int top[3];
+    bool finite = true;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const int e = act ? (__double2hiint(w[a]) >> 20) & 0x7ff : 0;
+        const int e = act ? exponent_of(w[a]) : 0;
+        finite = finite && exponent_of(st.f[a]) < 0x7ff;
         // 64: the unit 2^(top - 1079) stays a normal number
         top[a] = max((int)__reduce_max_sync(full, (unsigned)e), 64);
     }
-    if (det || max(max(top[0], top[1]), top[2]) == 0x7ff) {
+    if (det || max(max(top[0], top[1]), top[2]) == 0x7ff || __any_sync(full, act && !finite)) {
         // Deterministic mode: each deposit goes to the exact accumulators by itself (the warp's unit
         // would depend on which particles share it, and with that on the order a state was restored
-        // in).  A weight that is not finite: the plain deposit hands it on to J.
+        // in).  A weight or a coordinate that is not finite: the plain deposit hands it on to J.
         if (!act) return 0;
         CellStart<double> s = st;
         return for_each_piece(s, beta, m, [&](double h, double, const double mid[3], const int c[3]) {
