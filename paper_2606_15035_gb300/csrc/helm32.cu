@@ -168,6 +168,9 @@ __global__ void __launch_bounds__(256) k_helm_x(Helm32 h, Axis32 ax) {
     float2* z = h.z + blockIdx.y * N;
     double* x0 = h.x + f * N;
     const int e0 = scale_exponent(h, f), e1 = scale_exponent(h, f + 1);
+    // a field with a value that is not finite is left out of the transforms, which would hand it on to the
+    // other field of the pair, and becomes NaN
+    const bool ok0 = __ldg(h.top + f) < 0x7ff, ok1 = __ldg(h.top + f + 1) < 0x7ff;
     for (int64_t gr = blockIdx.x; gr * ax.lb < nlines; gr += gridDim.x) {
         const int64_t l0 = gr * ax.lb;
         const int lines = (int)min((int64_t)ax.lb, nlines - l0), cnt = lines * n;
@@ -176,8 +179,8 @@ __global__ void __launch_bounds__(256) k_helm_x(Helm32 h, Axis32 ax) {
             for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
                 const int j = quot(e, ax.mn), ix = e - j * n;
                 const unsigned l = (unsigned)(l0 + j), iz = l / (unsigned)h.m.n[1], iy = l - iz * (unsigned)h.m.n[1];
-                buf[e] = make_float2((float)(s0 * residual(h, x0, h.b + f * N, ix, (int)iy, (int)iz)),
-                                     (float)(s1 * residual(h, x0 + N, h.b + (f + 1) * N, ix, (int)iy, (int)iz)));
+                buf[e] = make_float2(ok0 ? (float)(s0 * residual(h, x0, h.b + f * N, ix, (int)iy, (int)iz)) : 0.f,
+                                     ok1 ? (float)(s1 * residual(h, x0 + N, h.b + (f + 1) * N, ix, (int)iy, (int)iz)) : 0.f);
             }
         } else {
             for (int e = threadIdx.x; e < cnt; e += blockDim.x) buf[e] = z[l0 * n + e];
@@ -187,7 +190,7 @@ __global__ void __launch_bounds__(256) k_helm_x(Helm32 h, Axis32 ax) {
         if (!INV) {
             for (int e = threadIdx.x; e < cnt; e += blockDim.x) z[l0 * n + e] = r[e];
         } else {
-            const double s0 = pow2(2046 - e0), s1 = pow2(2046 - e1);
+            const double s0 = ok0 ? pow2(2046 - e0) : NAN, s1 = ok1 ? pow2(2046 - e1) : NAN;
             for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
                 const float2 v = r[e];
                 x0[l0 * n + e] += s0 * (double)v.x;
