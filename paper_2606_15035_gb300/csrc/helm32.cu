@@ -355,7 +355,7 @@ bool helm32_factor(int n) {
 }
 
 int helm32_corrections(double lmax, double to) {
-    const double q = 2.5e-7 * lmax;
+    const double q = 2.5e-7 * std::max(lmax, 2.0);
     if (!(q < 1.0)) return 0;
     const double k = std::ceil(std::log(to) / std::log(q));
     return k > HELM_MAX_CORRECTIONS ? 0 : std::max(1, (int)k);

@@ -327,7 +327,9 @@ constexpr int HELM_MAX_CORRECTIONS = 8;
 // Corrections that bring an error of one below `to` (0: more than HELM_MAX_CORRECTIONS).  The FP32
 // transforms leave about 2^-22 of the residual, which is at most lmax times the error: 3 to roundoff at
 // 32^3 and 64^3 of the standard box, 4 at 128^3 (lmax 29), 6 at lmax 3000; the fields then match an
-// exact FP64 update to 5e-16.
+// exact FP64 update to 5e-16.  At lmax near one a correction leaves 1.5e-7 (16 x 12 x 8) to 2.6e-7 (128^2 x
+// 64) of a random error on 2^p 3^q meshes, and up to 4.7e-7 with the prime 127, whose sums are the
+// longest: no less than 5e-7 is counted on.
 int helm32_corrections(double lmax, double to);
 // Largest prime factor of an axis (its stage costs that many products a point): at 127^3 the transforms
 // still take a third of the Chebyshev steps' time.
