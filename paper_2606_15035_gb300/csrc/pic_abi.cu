@@ -297,7 +297,7 @@ void setup_geometry(Ctx& c) {
 // PIC_MIXED: the fields of an FP32 iteration need no more accuracy than its iterate has
 // (e_v >= ~1e-9), and those of an FP64 refinement iteration no more than a thousandth of
 // mixed_tol64; the final sweep's mesh phase, which the committed step uses, keeps
-// helmholtz_tol.
+// helmholtz_tol.  (On 2^p 3^q meshes every solve goes to roundoff.)
 constexpr double MESH_TOL32 = 1e-10;
 
 // Rule of the cell table (576 B per cell, orbit_cell.cuh): from one particle per cell on.  Three
@@ -409,7 +409,7 @@ pic_status allocate(pic_ctx* ctx) {
         c.helm_fft = ok;
         if (ok32) {
             c.helm_corrections = helm32_corrections(c.cheb_lmax, ok ? 1e-16 : std::max(c.cfg.helmholtz_tol, 1e-16));
-            c.helm_corrections32 = helm32_corrections(c.cheb_lmax, MESH_TOL32);
+            c.helm_corrections32 = ok ? c.helm_corrections : helm32_corrections(c.cheb_lmax, MESH_TOL32);
         }
     }
     if (c.helm_fft && c.helm_corrections == 0) {
@@ -586,7 +586,7 @@ void mesh_phase(Ctx& c, const double* Jcur, const double* Jprev, double tol = 0.
     } else {
         launch_source(c, Jcur, Jprev);
         if (c.helm_corrections > 0) {
-            // to roundoff, but for the FP32 iterations' fields
+            // to roundoff, or, with other primes, to helmholtz_tol and the FP32 iterations' accuracy
             launch_helm32(c, c.rhs, c.F1, c.helm_top, tol >= MESH_TOL32 ? c.helm_corrections32 : c.helm_corrections);
         } else if (c.helm_fft) {
             launch_helmholtz_fft_refined(c, c.F1);   // to roundoff: the tolerance does not apply

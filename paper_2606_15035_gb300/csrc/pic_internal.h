@@ -182,8 +182,8 @@ struct Ctx {
     bool helm_fft = false;
     double2* helm_spec = nullptr;
     double* helm_s2 = nullptr;
-    // ... by FP32 transforms and refinement (helm32.cu): corrections to roundoff and to the FP32
-    // iterations' accuracy (0: FP64 transforms), 2 N complex scratch, twiddles and symbols of the three
+    // ... by FP32 transforms and refinement (helm32.cu): corrections of the solves and of those of
+    // the FP32 iterations (0: FP64 transforms), 2 N complex scratch, twiddles and symbols of the three
     // axes, largest exponents of the right-hand sides (mesh phase | adjoint)
     int helm_corrections = 0, helm_corrections32 = 0;
     float2 *helm_z = nullptr, *helm_tw = nullptr;
