@@ -451,12 +451,8 @@ pic_status allocate(pic_ctx* ctx) {
         return fail(ctx, PIC_ERR_OOM, "pinned host allocation failed");
     }
     if (c.helm_corrections > 0) {
-        // (a Chebyshev solve takes over where this memory is the last straw)
-        c.helm_z = (float2*)(c.helm_fft ? dev_alloc(ctx, sizeof(float2) * 2 * N) : dev_alloc_once(ctx, sizeof(float2) * 2 * N));
-        if (!c.helm_z && c.helm_fft) return fail(ctx, PIC_ERR_OOM, "device allocation of c.helm_z failed");
-        if (!c.helm_z) c.helm_corrections = 0;
-    }
-    if (c.helm_corrections > 0) {
+        // (the Chebyshev steps' directions, which no solve by transforms needs)
+        c.helm_z = reinterpret_cast<float2*>(c.cheb_d);
         std::vector<float2> tw;
         std::vector<float> s2;
         helm32_tables(c, tw, s2);
@@ -469,7 +465,7 @@ pic_status allocate(pic_ctx* ctx) {
         if (cudaStreamSynchronize(c.stream) != cudaSuccess) return check_cuda(ctx, "helmholtz tables");
     }
     // last, because it is optional: the closed forms' cell table, where there are particles enough to
-    // repay building it and it stays a small part of the device's memory
+    // repay building it and it stays a small part of the device's memory.
     const size_t cells = sizeof(double) * CELL_VALUES * (size_t)N;
     if (c.closed && c.np >= CELL_TABLE_MIN_PPC * N && cells <= CELL_TABLE_MAX_BYTES) {
         c.ctab = (double*)dev_alloc_once(ctx, cells);

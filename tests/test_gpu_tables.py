@@ -1,0 +1,72 @@
+"""The optional cell tables: deterministic bits do not depend on whether they fit, and a context that holds
+them gives them back to another one that needs the memory."""
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sim(cuda_ok):
+    from paper_2606_15035_gb300 import build
+    build.build()
+    from paper_2606_15035_gb300 import sim as s
+    return s
+
+
+class Limit:
+    """Device memory of `capacity` bytes for all contexts created while it is in place."""
+
+    def __init__(self, sim, monkeypatch, refuse=lambda nbytes: False):
+        self.live, self.capacity, self.refused = {}, float("inf"), 0
+        base = sim._TorchAllocator
+        limit = self
+
+        class Limited(base):
+            def __init__(self, device):
+                super().__init__(device)
+                inner_alloc, inner_free = self._alloc_cb, self._free_cb
+
+                def alloc(nbytes, stream, user):
+                    if refuse(nbytes) or limit.used() + nbytes > limit.capacity:
+                        limit.refused += 1
+                        return None
+                    ptr = inner_alloc(nbytes, stream, user)
+                    if ptr:
+                        limit.live[int(ptr)] = nbytes
+                    return ptr
+
+                def free(ptr, nbytes, stream, user):
+                    limit.live.pop(int(ptr), None)
+                    inner_free(ptr, nbytes, stream, user)
+
+                self._outer = (sim._lib.ALLOC_FN(alloc), sim._lib.FREE_FN(free))
+                self.struct = sim.PicAllocator(*self._outer, None)
+
+        monkeypatch.setattr(sim, "_TorchAllocator", Limited)
+
+    def used(self):
+        return sum(self.live.values())
+
+
+def particles(n, L, ppc, seed):
+    rng = np.random.default_rng(seed)
+    npart = ppc * int(np.prod(n))
+    x = rng.uniform(0, 1, size=(npart, 3)) * L
+    v = rng.normal(scale=5e-3, size=x.shape)
+    v[:, 0] += np.where(np.arange(npart) % 2 == 0, 0.2, -0.2)
+    q = -L[0] * L[1] * L[2] / npart
+    return x, v, q, -q
+
+
+@pytest.mark.parametrize("n", [(6, 5, 4), (11, 7, 5)])
+def test_the_transforms_need_no_memory_of_their_own(sim, monkeypatch, n):
+    """No request of the size of the Helmholtz transforms' scratch (16 bytes a cell), whose refusal would
+    change the solver, and with it the bits of a deterministic run."""
+    L, N = (1.2, 1.0, 0.8), int(np.prod(n))
+    x, v, q, m = particles(n, L, 17, 21)
+    limit = Limit(sim, monkeypatch, lambda b: b == 16 * N)
+    s = sim.PicSim(sim.pic_config_default(n=n, L=L, dt=0.1, deterministic=1), x, v, q, m)
+    assert s.step(1).converged and limit.refused == 0
+    s.close()
