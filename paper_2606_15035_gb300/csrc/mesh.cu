@@ -352,12 +352,10 @@ __global__ void __launch_bounds__(THREADS) k_cheb_all(MeshParams p, double* xa, 
 
 __global__ void k_backsub_table(MeshParams p, const double* __restrict__ F0, const double* __restrict__ W0,
                                 const double* __restrict__ F1, double* __restrict__ W1, double* __restrict__ table,
-                                int* __restrict__ top, int* __restrict__ cell_top, double* __restrict__ zero) {
+                                int* __restrict__ top, double* __restrict__ zero) {
     const int64_t N = p.m.ncell;
-    // cleared on the way for the kernels that follow: the next k_source's exponents, the cell tables',
-    // the next current
+    // cleared on the way for the kernels that follow: the next k_source's exponents, the next current
     if (top && blockIdx.x == 0 && threadIdx.x < 4) top[threadIdx.x] = 0;
-    if (blockIdx.x == 0 && threadIdx.x < 2) cell_top[threadIdx.x] = 0;
     GRID_LOOP(g, N) {
         Nb b = decompose(g, p.m);
         double w1[4];
@@ -382,74 +380,60 @@ __global__ void k_backsub_table(MeshParams p, const double* __restrict__ F0, con
     }
 }
 
-// Cell table (orbit_cell.cuh) from the gather table: one thread per cell and column takes the
-// column's 8 node values to their mixed differences.  Writes 576 B a cell, 18 doubles apart per
-// thread with a cell's columns on neighbouring threads.  Also the largest exponents of the two groups
-// that the fixed-point table scales by: the differences of the A columns, and -grad phi (top, zero
-// before).
-__global__ void k_cell_table(MeshDims m, const double* __restrict__ table, double2* __restrict__ ctab,
-                             int* __restrict__ top) {
-    const unsigned total = (unsigned)m.ncell * CELL_COLS;
-    unsigned eA = 0, eG = 0;
-    for (unsigned idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += gridDim.x * blockDim.x) {
-        const unsigned cell = idx / CELL_COLS, t = cell / (unsigned)m.n[0];
-        const int col = (int)(idx - cell * CELL_COLS);
-        int c[3];
-        c[0] = (int)(cell - t * (unsigned)m.n[0]);
-        c[2] = (int)(t / (unsigned)m.n[1]);
-        c[1] = (int)t - c[2] * m.n[1];
-        int64_t g[8];
-        cell_nodes8(c, m, g);
+// Cell tables from the gather table: FP64 (orbit_cell.cuh) and fixed point (orbit_fixed.cuh).  One thread per
+// cell and column takes the column's 8 node values to their mixed differences; the block's threads of a
+// cell share the largest exponents of its two groups, the differences of the A columns and -grad phi.
+// Bound by memory: 1,152 B written a cell, with a cell's columns on neighbouring threads.
+constexpr int TABLE_CELLS = 32;   // cells of a block
+__global__ void __launch_bounds__(TABLE_CELLS * CELL_COLS) k_cell_table(MeshDims m, const double* __restrict__ table,
+                                                                        double2* __restrict__ ctab,
+                                                                        longlong2* __restrict__ fxtab) {
+    __shared__ int top[TABLE_CELLS][2];
+    const int slot = threadIdx.x / CELL_COLS, col = threadIdx.x - slot * CELL_COLS, group = col < 6 ? 0 : 1;
+    const unsigned ncell = (unsigned)m.ncell;
+    for (unsigned first = blockIdx.x * TABLE_CELLS; first < ncell; first += gridDim.x * TABLE_CELLS) {
+        if (threadIdx.x < 2 * TABLE_CELLS) (&top[0][0])[threadIdx.x] = 64;   // (at least: the units stay normal)
+        __syncthreads();
+        const unsigned cell = first + slot;
         double f[8];
+        if (cell < ncell) {
+            const unsigned t = cell / (unsigned)m.n[0];
+            int c[3];
+            c[0] = (int)(cell - t * (unsigned)m.n[0]);
+            c[2] = (int)(t / (unsigned)m.n[1]);
+            c[1] = (int)t - c[2] * m.n[1];
+            int64_t g[8];
+            cell_nodes8(c, m, g);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const double* q = table + 12 * g[k];
-            f[k] = col < 3 ? q[3 + col] : (col < 6 ? q[col] - q[col - 3] : -q[col]);
+            for (int k = 0; k < 8; ++k) {
+                const double* q = table + 12 * g[k];
+                f[k] = col < 3 ? q[3 + col] : (col < 6 ? q[col] - q[col - 3] : -q[col]);
+            }
+#pragma unroll
+            for (int bit = 1; bit < 8; bit <<= 1)
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (k & bit) f[k] -= f[k ^ bit];
+            int e = group ? exponent_of(f[0]) : 0;
+#pragma unroll
+            for (int k = 1; k < 8; ++k) e = max(e, exponent_of(f[k]));
+            atomicMax(&top[slot][group], e);
         }
+        __syncthreads();
+        if (cell < ncell) {
+            const int e = top[slot][group];
+            const int64_t at = (int64_t)cell * (CELL_VALUES / 2) + col;
 #pragma unroll
-        for (int bit = 1; bit < 8; bit <<= 1)
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if (k & bit) f[k] -= f[k ^ bit];
-        unsigned e = 0;
-#pragma unroll
-        for (int k = 1; k < 8; ++k) e = max(e, (unsigned)exponent_of(f[k]));
-        if (col < 6) eA = max(eA, e);
-        else eG = max(eG, max(e, (unsigned)exponent_of(f[0])));
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            ctab[(int64_t)cell * (CELL_VALUES / 2) + q * CELL_COLS + col] = make_double2(f[2 * q], f[2 * q + 1]);
-    }
-    if (!top) return;
-    __shared__ unsigned sA, sG;
-    if (threadIdx.x == 0) sA = sG = 0;
-    __syncthreads();
-    eA = __reduce_max_sync(0xffffffffu, eA);
-    eG = __reduce_max_sync(0xffffffffu, eG);
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(&sA, eA);
-        atomicMax(&sG, eG);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        atomicMax(top, (int)sA);
-        atomicMax(top + 1, (int)sG);
-    }
-}
-
-// FP64 cell table -> fixed-point cell table (orbit_fixed.cuh).  The entries k = 0 of the A columns are
-// not used there.
-__global__ void k_cells_fixed(unsigned n, const double2* __restrict__ t64, longlong2* __restrict__ tfx,
-                              const int* __restrict__ top) {
-    const int eA = max(top[0], 64), eG = max(top[1], 64);
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const unsigned r = i % (CELL_VALUES / 2), p = r / CELL_COLS, col = r - p * CELL_COLS;
-        const double2 q = t64[i];
-        const int e = col < 6 ? eA : eG;
-        longlong2 o;
-        o.x = (p == 0 && col < 6) ? 0 : fixed_of(q.x, e, FX_FIELD_UP);
-        o.y = fixed_of(q.y, e, FX_FIELD_UP);
-        tfx[i] = o;
+            for (int q = 0; q < 4; ++q) {
+                longlong2 o;
+                o.x = fixed_of(f[2 * q], e, FX_FIELD_UP);
+                o.y = fixed_of(f[2 * q + 1], e, FX_FIELD_UP);
+                if (q == 0 && !group) o.x = col < 2 ? top[slot][col] : 0;
+                ctab[at + q * CELL_COLS] = make_double2(f[2 * q], f[2 * q + 1]);
+                fxtab[at + q * CELL_COLS] = o;
+            }
+        }
+        __syncthreads();   // the exponents are cleared for the next cells
     }
 }
 
@@ -701,23 +685,14 @@ int cheb_coop_capacity(const Ctx& c) {
 
 void launch_backsub_table(Ctx& c, double* zero) {
     k_backsub_table<<<mesh_blocks(c), mesh_threads(c), 0, c.stream>>>(mesh_params(c), c.F0, c.W0, c.F1, c.W1, c.table,
-                                                            c.helm_top, c.cell_top, zero);
+                                                            c.helm_top, zero);
     ++c.launches;
 }
 
-void launch_cell_table(Ctx& c, bool fixed) {
-    auto blocks = [&](int64_t n) {
-        return (int)std::max<int64_t>(1, std::min<int64_t>((n + THREADS - 1) / THREADS, (int64_t)c.sms * 16));
-    };
-    fixed = fixed && c.fxtab;
-    if (fixed && c.cfg.ops == PIC_OPS_SPECTRAL) cudaMemsetAsync(c.cell_top, 0, 2 * sizeof(int), c.stream);
-    k_cell_table<<<blocks(c.m.ncell * CELL_COLS), THREADS, 0, c.stream>>>(
-        c.m, c.table, reinterpret_cast<double2*>(c.ctab), fixed ? c.cell_top : nullptr);
-    ++c.launches;
-    if (!fixed) return;
-    const int64_t n = c.m.ncell * (CELL_VALUES / 2);
-    k_cells_fixed<<<blocks(n), THREADS, 0, c.stream>>>((unsigned)n, reinterpret_cast<const double2*>(c.ctab),
-                                                       reinterpret_cast<longlong2*>(c.fxtab), c.cell_top);
+void launch_cell_table(Ctx& c) {
+    const int64_t groups = (c.m.ncell + TABLE_CELLS - 1) / TABLE_CELLS;
+    k_cell_table<<<(int)std::min<int64_t>(groups, (int64_t)c.sms * 16), TABLE_CELLS * CELL_COLS, 0, c.stream>>>(
+        c.m, c.table, reinterpret_cast<double2*>(c.ctab), reinterpret_cast<longlong2*>(c.fxtab));
     ++c.launches;
 }
 

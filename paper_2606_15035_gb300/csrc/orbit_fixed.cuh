@@ -6,9 +6,13 @@
 //
 // Formats: coordinates, moments and piece lengths at 2^-62; v^p + v^n at 2^(ev - 1084), ev the largest
 // biased exponent of its components; the table's mixed differences (A^{n+1} and its change together,
-// and -grad phi) at 2^(e - 1080), e the largest exponent of that group over the mesh: 58 bits of the
-// largest difference, and sums of up to eight of them stay in range.  The end point's A_h^{n+1} adds the
-// differences to the cell's lowest node value in FP64.
+// and -grad phi) at 2^(e - 1080), e the largest exponent of that group in the cell: sums of up to eight of
+// them stay in range.  A factor of a product is its upper 60 (velocities) or 56 bits (differences), so that a
+// piece's integrals carry an error of a few 2^-55 of the cell's largest difference times the largest
+// velocity component, where FP64 rounds each product at 2^-53 of itself: small components beside large ones
+// of the same cell are held to that absolute bound.  Pieces are summed in FP64.  (With one exponent for the
+// whole mesh, a field of 2^-20 of its peak elsewhere was left with 35 bits.)  The end point's A_h^{n+1} adds
+// the differences to the cell's lowest node value in FP64.
 #pragma once
 
 #include "fixed.cuh"
@@ -19,6 +23,8 @@ namespace pic {
 constexpr int FX_FIELD_UP = 5;   // fixed_of's shift for the table: 58 bits
 constexpr int FX_V_UP = 9;       // ... for velocities: 62 bits
 
+// Loader of a cell's entries.  The entries k = 0 of the A columns are not used; two of them hold the
+// exponents of the cell's groups.
 struct FixedLoad {
     const longlong2* t;
     __device__ __forceinline__ FixedLoad(const longlong2* table, const int c[3], const MeshDims& m)
@@ -28,13 +34,19 @@ struct FixedLoad {
         a = q.x;
         b = q.y;
     }
+    __device__ __forceinline__ int top_A() const { return (int)__ldg(&t[0].x); }
+    __device__ __forceinline__ int top_g() const { return (int)__ldg(&t[1].x); }
 };
 
-// accF_j += int (D_j A)^T v and accG_j -= int d_j phi of one piece (h, s_mid, midpoint, displacement
-// d = h beta), in the formats above.
+// The unit 2^e' of a sum, e' = e - 1023, of quantities whose largest biased exponent is `top`: NaN where that
+// is not finite.
+__device__ __forceinline__ double fixed_unit(int e, int top) { return top < 0x7ff ? pow2_biased(e) : NAN; }
+
+// accF_j += int (D_j A)^T v, the difference along j per cell, and accG_j -= int d_j phi of one piece (h, s_mid,
+// midpoint, displacement d = h beta), v in the format above.
+template <typename L>
 __device__ __forceinline__ void piece_impulse_fixed(double h, double sm, const double mid[3], const double d[3],
-                                                    const Fs v[3], const FixedLoad& ld, long long accF[3],
-                                                    long long accG[3]) {
+                                                    const Fs v[3], int ev, const L& ld, double accF[3], double accG[3]) {
     const Fs hf = fs_of(fixed_of(h, 1023, 10));
     const Fs nms = fs_of(fixed_of(sm, 1023, 10) - FX_ONE);   // s_mid - 1
     Fs m[3], e[3], Pxy, Pxz, Pyz, S, E3, E5, E6;
@@ -112,15 +124,18 @@ __device__ __forceinline__ void piece_impulse_fixed(double h, double sm, const d
             g[j].add(fs_of(g1), p == 0 ? m[0] : (p == 1 ? Pxy : (p == 2 ? Pxz : S)));
         }
     }
+    const int eA = ld.top_A(), eG = ld.top_g();
+    const double uF = fixed_unit(eA + ev - 1079, max(eA, ev)), uG = fixed_unit(eG - 57, eG);
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        accF[j] += fx_sum(hf, F[j].factor()).value();
-        accG[j] += fx_sum(hf, g[j].factor()).value();
+        accF[j] = fma(uF, (double)fx_sum(hf, F[j].factor()).value(), accF[j]);
+        accG[j] = fma(uG, (double)fx_sum(hf, g[j].factor()).value(), accG[j]);
     }
 }
 
 // A^{n+1} at coordinate r of the cell less its lowest node's value, in the table's format.
-__device__ __forceinline__ void cell_A1_fixed(const double r[3], const FixedLoad& ld, long long out[3]) {
+template <typename L>
+__device__ __forceinline__ void cell_A1_fixed(const double r[3], const L& ld, long long out[3]) {
     Fs q[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) q[a] = fs_of(fixed_of(r[a], 1023, 10));

@@ -682,9 +682,8 @@ struct CellOut {
 };
 
 struct CellFields {
-    const double* t64;        // FP64 cell table, or (not FIXED) the gather table
-    const longlong2* tfx;
-    const int* top;           // largest exponents of the fixed table's groups
+    const double* table;      // gather table
+    const longlong2* tfx;     // fixed-point cell table (FIXED)
 };
 
 template <bool FIXED>
@@ -695,33 +694,33 @@ __device__ __forceinline__ void push_eval_cell(const StepParams& p, CellStart<do
     for (int a = 0; a < 3; ++a) beta[a] = p.cb[a] * vs[a];
     if constexpr (FIXED) {
         const int ev = max(max(exponent_of(vs[0]), exponent_of(vs[1])), max(exponent_of(vs[2]), 64));
-        const int eA = max(__ldg(cf.top), 64), eG = max(__ldg(cf.top + 1), 64);
         Fs v[3];
-        long long accF[3] = {0, 0, 0}, accG[3] = {0, 0, 0}, A1[3];
+        double accF[3] = {0.0, 0.0, 0.0}, accG[3] = {0.0, 0.0, 0.0};
 #pragma unroll
         for (int a = 0; a < 3; ++a) v[a] = fs_of(fixed_of(vs[a], ev, FX_V_UP));
         o.nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
             const double d[3] = {h * beta[0], h * beta[1], h * beta[2]};
-            piece_impulse_fixed(h, sm, mid, d, v, FixedLoad(cf.tfx, c, p.m), accF, accG);
+            piece_impulse_fixed(h, sm, mid, d, v, ev, FixedLoad(cf.tfx, c, p.m), accF, accG);
         });
-        cell_A1_fixed(st.f, FixedLoad(cf.tfx, st.c, p.m), A1);
+        const FixedLoad ld(cf.tfx, st.c, p.m);
+        long long A1[3];
+        cell_A1_fixed(st.f, ld, A1);
         // values that are not finite stay so (the start's coordinate: the end's is its sum with beta)
         const int ef = max(max(exponent_of(st.f[0]), exponent_of(st.f[1])), exponent_of(st.f[2]));
-        const bool ok = max(max(ev, ef), max(eA, eG)) < 2047;
-        const double uF = ok ? p.dtq * pow2_biased(eA + ev - 1079) : NAN;
-        const double uG = ok ? p.dtq * pow2_biased(eG - 57) : NAN, uA = pow2_biased(eA - 57);
-        const double* low = cf.t64 + CELL_VALUES * cell_row(st.c, p.m);
+        const double dtq = max(ev, ef) < 0x7ff ? p.dtq : NAN;
+        const double uA = pow2_biased(ld.top_A() - 57);
+        const double* low = cf.table + 12 * cell_row(st.c, p.m) + 3;   // A^{n+1} at the cell's lowest node
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            o.Ae[a] = __ldg(low + 2 * a) + uA * (double)A1[a];
-            o.Pw[a] = Pn[a] + (uG * (double)accG[a] + uF * p.ihs[a] * (double)accF[a]);
+            o.Ae[a] = __ldg(low + a) + uA * (double)A1[a];
+            o.Pw[a] = Pn[a] + dtq * (accG[a] + p.ihs[a] * accF[a]);
         }
     } else {
         double acc[3] = {0.0, 0.0, 0.0};
         o.nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
-            piece_impulse(h, sm, mid, beta, vs, p.ihs, FieldLoad<false>(cf.t64, c, p.m), acc);
+            piece_impulse(h, sm, mid, beta, vs, p.ihs, FieldLoad<false>(cf.table, c, p.m), acc);
         });
-        cell_A1(st.f, FieldLoad<false>(cf.t64, st.c, p.m), o.Ae);
+        cell_A1(st.f, FieldLoad<false>(cf.table, st.c, p.m), o.Ae);
 #pragma unroll
         for (int a = 0; a < 3; ++a) o.Pw[a] = Pn[a] + p.dtq * acc[a];
     }
@@ -2117,7 +2116,7 @@ void launch_push(Ctx& c, const double* vit, double* vnew, double* Jnext, bool co
                                                   c.creep_list, c.creep_count, det ? c.creep_flag : nullptr,  \
                                                   c.slide,                                                    \
                                                   c.partials, c.dev_status)
-    const CellFields cf{c.fxtab ? c.ctab : c.table, reinterpret_cast<const longlong2*>(c.fxtab), c.cell_top};
+    const CellFields cf{c.table, reinterpret_cast<const longlong2*>(c.fxtab)};
     const bool small = small_chunks(c), wide = wide_chunks(c);
 #define PIC_PUSH_CELL_AS(C, T, W, I)                                                                              \
     k_push_cell<C, T, W, I><<<chunk_blocks(c), 32 * W, C ? sizeof(ChunkOrder<W, I>) : ChunkOrder<W, I>::smem(),     \

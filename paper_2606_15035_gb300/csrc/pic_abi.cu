@@ -444,7 +444,6 @@ pic_status allocate(pic_ctx* ctx) {
     ALLOC(c.partials, double, (size_t)NSLOT * MAX_BLOCKS);
     ALLOC(c.results, double, NSLOT);
     ALLOC(c.dev_status, int, 1);
-    ALLOC(c.cell_top, int, 2);
     if (cudaMallocHost(&c.host_results, sizeof(double) * NSLOT) != cudaSuccess ||
         cudaMallocHost(&c.host_status, sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
@@ -483,7 +482,6 @@ pic_status allocate(pic_ctx* ctx) {
     std::memset(c.host_results, 0, sizeof(double) * NSLOT);
     *c.host_status = 0;
     cudaMemsetAsync(c.partials, 0, sizeof(double) * (size_t)NSLOT * MAX_BLOCKS, c.stream);
-    cudaMemsetAsync(c.cell_top, 0, 2 * sizeof(int), c.stream);
     cudaMemsetAsync(c.results, 0, sizeof(double) * NSLOT, c.stream);
     cudaMemsetAsync(c.dev_status, 0, sizeof(int), c.stream);
     return check_cuda(ctx, "allocate");
@@ -591,7 +589,7 @@ void mesh_phase(Ctx& c, const double* Jcur, const double* Jprev, double tol = 0.
         }
         launch_backsub_table(c, zero);
     }
-    if (cells && c.ctab) launch_cell_table(c, true);
+    if (cells && c.ctab) launch_cell_table(c);
 }
 
 

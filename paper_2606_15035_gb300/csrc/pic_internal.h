@@ -161,8 +161,7 @@ struct Ctx {
     double *J[3] = {nullptr, nullptr, nullptr};
     double* table = nullptr;             // 12 * ncell gather table
     double* ctab = nullptr;              // closed forms: CELL_VALUES * ncell cell table (orbit_cell.cuh)
-    long long* fxtab = nullptr;          // ... in fixed point (orbit_fixed.cuh), and its groups' largest
-    int* cell_top = nullptr;             // exponents (both or neither of the two tables)
+    long long* fxtab = nullptr;          // ... in fixed point (orbit_fixed.cuh; both or neither)
 
     // FP32 working set of the mixed path (allocated only for PIC_MIXED)
     std::vector<double> hist_ev, hist_eJ;   // residuals of the last step's iterations
@@ -350,9 +349,8 @@ void launch_jdiff(Ctx& c, const double* Jnew, const double* Jold);
 void launch_helmholtz(Ctx& c, const double* b, double c_id, double c_lap, int nfields, int iters,
                       const double* alpha, const double* beta, double** x_io, double** x_spare);
 void launch_backsub_table(Ctx& c, double* zero);   // zero (may be null): 3 ncell values to clear on the way
-// The cell tables of the FP64 closed-form particle kernels from the gather table (fixed: also the
-// fixed-point one, for the pushes).
-void launch_cell_table(Ctx& c, bool fixed);
+// The cell tables of the closed-form particle kernels from the gather table.
+void launch_cell_table(Ctx& c);
 void launch_helmholtz_cn(Ctx& c, double** x_io, double** x_spare, double tol);
 void launch_helmholtz_fft_refined(Ctx& c, double* x);
 int cheb_coop_capacity(const Ctx& c);

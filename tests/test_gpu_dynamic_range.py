@@ -1,0 +1,51 @@
+"""Quantities of very different size side by side: what the fixed-point sums hold is relative to the cell
+and the particles at hand, not to the largest value of the mesh or of the warp."""
+
+import numpy as np
+import pytest
+
+from oracle import mesh as omesh
+from oracle import pic as opic
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sim(cuda_ok):
+    from paper_2606_15035_gb300 import build
+    build.build()
+    from paper_2606_15035_gb300 import sim as s
+    return s
+
+
+@pytest.mark.parametrize("ppc", [4, 64])
+def test_push_ahead_of_a_localised_pulse(sim, ppc):
+    """A field of order one in a few cells and 1e-9 elsewhere: the momenta of the particles elsewhere,
+    from zero, against the oracle's push in the fields that the library returns.  A momentum is a sum of
+    a few dozen products of the fields around its particle: 1e-13 of that size and a digit of margin."""
+    rng = np.random.default_rng(3)
+    n, dt, q, m = (16, 4, 5), 0.05, 1e-6, 1.0
+    L = tuple(map(float, n))
+    x = rng.uniform(0, 1, size=(ppc * int(np.prod(n)), 3)) * L
+    v = rng.normal(scale=8.0, size=x.shape)
+    s = sim.PicSim(sim.pic_config_default(n=n, L=L, dt=dt), x, v, q, m)
+    st = s.get_state()
+    for name in ("phi", "psi", "A", "U", "rho"):
+        a = 1e-9 * rng.normal(size=getattr(st, name).shape)
+        if name in ("phi", "A"):
+            a[..., 7:9, :, :] *= 1e9
+        setattr(st, name, a)
+    st.P[:] = 0.0
+    s.set_state(st)
+    got = s.iterate(v)
+    s.close()
+    ocfg = opic.Config(n=n, L=L, dt=dt)
+    grid = ocfg.grid()
+    xi = st.x / np.asarray(grid.H)
+    want = opic.push_particles(xi, st.v, st.P, v, q, m, st.A, got["A"], omesh.grad(0.5 * (got["phi"] + st.phi), grid),
+                               0.5 * (got["U"] + st.U), ocfg, grid)["P"]
+    # (the update's tail falls by a / 4 H^2 = 1.6e-4 every two cells)
+    far = (np.abs(xi[:, 0] - 8.0) > 6.0)
+    size = np.sqrt(np.mean(want[far] ** 2))
+    assert size <= 1e-3 * np.abs(want).max()
+    assert np.abs(got["P"] - want)[far].max() <= 1e-12 * size
