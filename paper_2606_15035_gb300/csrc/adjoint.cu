@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_scatter(
     auto flush = [&](const TileOrder& order, bool has, const int c[3], int col, int e0, int e1) {
         const double u0 = pow2_biased(e0), u1 = pow2_biased(e1);
         __syncwarp();
-        order.sums(has, c, tile, [&](long long sum, const int c0[3]) {
+        order.sums(has, c, tile, [&](long long sum, const int c0[3], int) {
             double x = (double)sum;
 #pragma unroll
             for (int bit = 1; bit < 8; bit <<= 1) {
@@ -346,7 +346,9 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_scatter(
                     }
                     continue;
                 }
-                const TileOrder order(has, has ? (int)cell_row(c, p.m) : -1);
+                const int e0[1] = {0};
+                int top0[1] = {0};
+                const TileOrder order(has, has ? (int)cell_row(c, p.m) : -1, e0, top0);
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
                     if (has) {
@@ -377,7 +379,9 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_scatter(
                 if (act) plain_rows(lam_tab + 3, wk.c, p.m, M, lA);
                 continue;
             }
-            const TileOrder order(act, act ? (int)cell_row(wk.c, p.m) : -1);
+            const int e0[1] = {0};
+            int top0[1] = {0};
+            const TileOrder order(act, act ? (int)cell_row(wk.c, p.m) : -1, e0, top0);
             if (act) {
                 long long w[3], Mf[8];
 #pragma unroll

@@ -3,11 +3,12 @@
 // Depositing a piece in FP64 takes 46 FP64 instructions and 24 L2 reductions per particle, on a
 // pipe with 1/64 of the issue rate and with one L2 request per lane and reduction (equal addresses
 // of a warp are not merged): both bound the scatters.  Every factor of a deposit is bounded (the
-// moments of orbit_cell.cuh lie in [0, 1], the weights below the warp's largest), so the products
-// and sums run in 64-bit fixed point instead: moments to 2^-62, weights to 2^-57 of the warp's
-// largest, at least as fine as the FP64 products they replace (2^-53 of each, and one more rounding
-// per addition to J), and exact sums.  The warp's particles hold few distinct cells (the store is
-// cell-sorted), so each cell's 24 sums (8 moments, 3 components) are taken by 24 lanes from a
+// moments of orbit_cell.cuh lie in [0, 1], the weights below the largest of the cell's particles), so the
+// products and sums run in 64-bit fixed point instead: moments to 2^-62, each component's weights to
+// 2^-57 of the largest that the warp adds to the same cell, and exact sums.  A cell's sum so has an error of
+// a few 2^-57 of its largest deposit, where FP64 rounds each product at 2^-53 and J at every addition; a
+// slow particle in a cell of its own keeps all its bits beside fast ones in others.  The warp's particles
+// hold few distinct cells (the store is cell-sorted), so each cell's 24 sums (8 moments, 3 components) are taken by 24 lanes from a
 // transposed shared tile, turned into node weights by three exchanges, and added to J once.
 #pragma once
 
@@ -25,23 +26,31 @@ struct TileOrder {
     unsigned group;   // lanes of this lane's cell
     int col;          // this lane's column
 
-    __device__ __forceinline__ TileOrder(bool has, int row) : group(0), col(0) {
+    // top_k: the largest e_k of the lanes of this lane's cell.
+    template <int E>
+    __device__ __forceinline__ TileOrder(bool has, int row, const int (&e)[E], int (&top)[E]) : group(0), col(0) {
         const unsigned full = 0xffffffffu, below = (1u << (threadIdx.x & 31)) - 1u;
         int base = 0;
         for (unsigned rest = __ballot_sync(full, has); rest;) {
             const int r = __shfl_sync(full, row, __ffs(rest) - 1);
-            const unsigned g = __ballot_sync(full, row == r);
-            if (row == r) {
+            const bool mine = row == r;
+            const unsigned g = __ballot_sync(full, mine);
+            int t[E];
+#pragma unroll
+            for (int k = 0; k < E; ++k) t[k] = (int)__reduce_max_sync(full, mine ? (unsigned)e[k] : 0u);
+            if (mine) {
                 group = g;
                 col = base + __popc(g & below);
+#pragma unroll
+                for (int k = 0; k < E; ++k) top[k] = t[k];
             }
             base += __popc(g);
             rest &= ~g;
         }
     }
 
-    // The tile's sums over the columns of each cell (coordinates pc of its lanes): add(sum, cell) on every
-    // lane, lane r < DEPOSIT_ROWS with the sum of row r.
+    // The tile's sums over the columns of each cell (coordinates pc of its lanes): add(sum, cell, one of
+    // its lanes) on every lane, lane r < DEPOSIT_ROWS with the sum of row r.
     template <typename F>
     __device__ __forceinline__ void sums(bool has, const int pc[3], const long long* tile, F&& add) const {
         const unsigned full = 0xffffffffu;
@@ -66,7 +75,7 @@ struct TileOrder {
                 }
             }
             base = end;
-            add(s, c);
+            add(s, c, lead);
         }
     }
 };
@@ -92,16 +101,10 @@ __device__ __forceinline__ int scatter_warp(const MeshDims& m, bool act, const C
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int64_t N = m.ncell;
-    int top[3];
     bool finite = true;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const int e = act ? exponent_of(w[a]) : 0;
-        finite = finite && exponent_of(st.f[a]) < 0x7ff;
-        // 64: the unit 2^(top - 1079) stays a normal number
-        top[a] = max((int)__reduce_max_sync(full, (unsigned)e), 64);
-    }
-    if (det || max(max(top[0], top[1]), top[2]) == 0x7ff || __any_sync(full, act && !finite)) {
+    for (int a = 0; a < 3; ++a) finite = finite && exponent_of(w[a]) < 0x7ff && exponent_of(st.f[a]) < 0x7ff;
+    if (det || __any_sync(full, act && !finite)) {
         // Deterministic mode: each deposit goes to the exact accumulators by itself (the warp's unit
         // would depend on which particles share it, and with that on the order a state was restored
         // in).  A weight or a coordinate that is not finite: the plain deposit hands it on to J.
@@ -122,9 +125,7 @@ __device__ __forceinline__ int scatter_warp(const MeshDims& m, bool act, const C
         });
     }
     if (lane < DEPOSIT_ROWS) tile[lane * DEPOSIT_STRIDE + 32] = 0;
-    // this lane's unit: component lane / 8 (lanes 24..31 sum nothing)
-    const int comp = min(lane >> 3, 2);
-    const double unit = __hiloint2double(((comp == 0 ? top[0] : (comp == 1 ? top[1] : top[2])) - 56) << 20, 0);
+    const int comp = min(lane >> 3, 2);   // this lane's component (lanes 24..31 sum nothing)
     const Fx c12 = fx_split(FX_ONE / 12);
     PieceWalk<double> wk(st, beta, m);
     bool last = !act;
@@ -136,7 +137,15 @@ __device__ __forceinline__ int scatter_warp(const MeshDims& m, bool act, const C
             has = wk.next(beta, m, h, sm, mid, pc, last);
             if (has) row = (int)cell_row(pc, m);
         }
-        const TileOrder order(has, row);
+        double hw[3];
+        int e[3], top[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            hw[a] = h * w[a];
+            e[a] = max(exponent_of(hw[a]), 64);   // (the unit 2^(top - 1079) stays a normal number)
+            top[a] = 64;
+        }
+        const TileOrder order(has, row, e, top);
         if (has) {
             long long M[8];
             Fx q[3], d[3];
@@ -154,7 +163,7 @@ __device__ __forceinline__ int scatter_warp(const MeshDims& m, bool act, const C
             M[7] = fx_mul(q[0], fx_split(M[6])) + fx_mul(q[1], fx_split(kxz)) + fx_mul(q[2], fx_split(kxy));
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
-                const long long wf = fixed_of(h * w[a], top[a], 4);
+                const long long wf = fixed_of(hw[a], top[a], 4);
                 const Fx ws = fx_split(wf);
                 tile[(8 * a) * DEPOSIT_STRIDE + order.col] = wf;
 #pragma unroll
@@ -162,7 +171,9 @@ __device__ __forceinline__ int scatter_warp(const MeshDims& m, bool act, const C
             }
         }
         __syncwarp();
-        order.sums(has, pc, tile, [&](long long sum, const int c0[3]) {
+        order.sums(has, pc, tile, [&](long long sum, const int c0[3], int lead) {
+            const int t01 = __shfl_sync(full, top[0] | top[1] << 16, lead), t2 = __shfl_sync(full, top[2], lead);
+            const double unit = __hiloint2double(((comp == 0 ? t01 & 0xffff : (comp == 1 ? t01 >> 16 : t2)) - 56) << 20, 0);
             // moments of the subsets -> weights of the nodes (inclusion--exclusion, axis by axis)
 #pragma unroll
             for (int bit = 1; bit < 8; bit <<= 1) {

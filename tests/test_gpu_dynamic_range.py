@@ -49,3 +49,29 @@ def test_push_ahead_of_a_localised_pulse(sim, ppc):
     size = np.sqrt(np.mean(want[far] ** 2))
     assert size <= 1e-3 * np.abs(want).max()
     assert np.abs(got["P"] - want)[far].max() <= 1e-12 * size
+
+
+@pytest.mark.parametrize("ppc", [1, 4, 64])
+def test_current_of_slow_particles_beside_a_fast_one(sim, ppc):
+    """One particle with velocity one among particles of 1e-9: the current at the nodes that it does
+    not touch, to 1e-12 of its size there (sums of some dozens of products)."""
+    rng = np.random.default_rng(4)
+    n = (8, 4, 5)
+    L = tuple(map(float, n))
+    npart = ppc * int(np.prod(n))
+    x = rng.uniform(0, 1, size=(npart, 3)) * L
+    v = 1e-9 * rng.normal(size=x.shape)
+    x[0], v[0] = (2.3, 1.4, 2.2), (0.6, -0.5, 0.7)
+    kw = dict(n=n, L=L, dt=0.5)
+    s = sim.PicSim(sim.pic_config_default(**kw), x, v, -1e-3, 1e-3)
+    got = s.iterate(v)
+    s.close()
+    ocfg = opic.Config(**kw)
+    grid = ocfg.grid()
+    o = opic.init(x, v, -1e-3, 1e-3, ocfg)
+    it = opic.orbit_current(o, v, ocfg, grid)
+    alone = opic.orbit_current(opic.init(x[:1], v[:1], -1e-3, 1e-3, ocfg), v[:1], ocfg, grid)
+    slow = alone == 0.0
+    size = np.sqrt(np.mean(it[slow] ** 2))
+    assert 0.0 < size <= 1e-6 * np.abs(it).max()
+    assert np.abs(got["J"] - it)[slow].max() <= 1e-12 * size
