@@ -203,8 +203,9 @@ __device__ __forceinline__ void out_adjoints(const StepParams& p, bool sl, doubl
 // A^n and grad phi, 8 subsets of the axes and 3 components each, and of the interpolant of A^{n+1} at the
 // end point.  Every particle's 72 terms a piece went to the mesh by atomics, 96 L2 reductions a particle
 // and more, which bounded the kernel (0.80 ms at 32^3 with 524,288 particles).  As in scatter_warp the
-// warp's particles are summed per cell first, in 64-bit fixed point (values to 2^-57 of the warp's
-// largest), three tiles a piece, and turned into node values once per cell: 0.43 ms.
+// warp's particles are summed per cell first, in 64-bit fixed point (each component's values to 2^-57 of the
+// largest product that the warp adds to the cell), three tiles a piece, and turned into node values once
+// per cell: 0.43 ms.
 __device__ __forceinline__ void plain_rows(double* __restrict__ col, const int c[3], const MeshDims& m, const double M[8],
                                            const double w[3]) {
     double W[8];
@@ -233,19 +234,21 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_scatter(
     const int lane = threadIdx.x & 31, comp = min(lane >> 3, 2);
     const int64_t np = p.np, nchunks = (np + ChunkLarge::SIZE - 1) / ChunkLarge::SIZE;
     if (lane < DEPOSIT_ROWS) tile[lane * DEPOSIT_STRIDE + 32] = 0;
-    auto top_of = [&](double x) { return (int)__reduce_max_sync(full, (unsigned)exponent_of(x)); };
-    // the tile's sums per cell into column `col` of lam_tab, their unit 2^(e0 + e1 - 2046) as two factors
-    auto flush = [&](const TileOrder& order, bool has, const int c[3], int col, int e0, int e1) {
-        const double u0 = pow2_biased(e0), u1 = pow2_biased(e1);
+    // the tile's sums per cell into column `col` of lam_tab, component a's unit 2^(unit_a - 2046)
+    auto flush = [&](const TileOrder& order, bool has, const int c[3], int col, const int unit[3]) {
         __syncwarp();
-        order.sums(has, c, tile, [&](long long sum, const int c0[3], int) {
+        order.sums(has, c, tile, [&](long long sum, const int c0[3], int lead) {
+            const int u01 = __shfl_sync(full, unit[0] | unit[1] << 16, lead), u2 = __shfl_sync(full, unit[2], lead);
+            const int u = comp == 0 ? u01 & 0xffff : (comp == 1 ? u01 >> 16 : u2);
             double x = (double)sum;
 #pragma unroll
             for (int bit = 1; bit < 8; bit <<= 1) {
                 const double o = __shfl_xor_sync(full, x, bit);
                 if (!(lane & bit)) x -= o;
             }
-            if (lane < DEPOSIT_ROWS) atomicAdd(lam_tab + 9 * subset_node(c0, lane, p.m) + col + comp, x * u0 * u1);
+            if (lane < DEPOSIT_ROWS)
+                atomicAdd(lam_tab + 9 * subset_node(c0, lane, p.m) + col + comp,
+                          x * pow2_biased(u >> 1) * pow2_biased(u - (u >> 1)));
         });
         __syncwarp();
     };
@@ -288,15 +291,12 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_scatter(
                 beta[a] = p.cb[a] * vs[a];
                 fs += fabs(f[a]);
             }
-            // |a piece's sums| < 1.2 fs: an exponent above that of fs
-            const int tf = max(top_of(fs), 64) + 1;
-            const int tv = max(max(top_of(vs[0]), max(top_of(vs[1]), top_of(vs[2]))), 64);
-            const int tg = max(max(top_of(lg[0]), max(top_of(lg[1]), top_of(lg[2]))), 64);
-            const int tA = max(max(top_of(lA[0]), max(top_of(lA[1]), top_of(lA[2]))), 64);
-            const bool plain = max(max(tf, tv), max(tg, tA)) >= 0x7ff;   // a value that is not finite goes on as it is
-            Fx vf[3];
+            // a value that is not finite goes on as it is
+            bool finite = exponent_of(fs) < 0x7fe;
 #pragma unroll
-            for (int a = 0; a < 3; ++a) vf[a] = fx_split(fixed_of(vs[a], tv, 9));
+            for (int a = 0; a < 3; ++a)
+                finite = finite && max(exponent_of(vs[a]), max(exponent_of(lg[a]), exponent_of(lA[a]))) < 0x7ff;
+            const bool plain = __any_sync(full, !finite);
             PieceWalk<double> wk(st, beta, p.m);
             bool last = !act;
             while (__any_sync(full, !last)) {
@@ -346,31 +346,50 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_scatter(
                     }
                     continue;
                 }
-                const int e0[1] = {0};
-                int top0[1] = {0};
-                const TileOrder order(has, has ? (int)cell_row(c, p.m) : -1, e0, top0);
+                // exponents of the factors: |a piece's sums| < 1.2 h fs, so one above that of h fs
+                const int tf = max(exponent_of(h * fs), 64) + 1;
+                double hl[3];
+                int e[6], top[6];   // of the products v (a piece's sum), and of h lg
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    hl[a] = h * lg[a];
+                    e[a] = max(exponent_of(vs[a]), 64) + tf;
+                    e[3 + a] = max(exponent_of(hl[a]), 64);
+                    top[a] = top[3 + a] = 129;
+                }
+                const TileOrder order(has, has ? (int)cell_row(c, p.m) : -1, e, top);
+                // the velocities' shift brings every lane's products to the cell's unit
+                Fx vf[3];
+                int unit[3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    vf[a] = fx_split(fixed_of(vs[a], top[a] - tf, 9));
+                    unit[a] = top[a] - 55;
+                }
 #pragma unroll
                 for (int half = 0; half < 2; ++half) {
                     if (has) {
 #pragma unroll
                         for (int k = 0; k < 8; ++k) {
-                            const Fx e = fx_split(fixed_of(half == 0 ? ab[k] - x1[k] : x1[k], tf, 4));
+                            const Fx x = fx_split(fixed_of(half == 0 ? ab[k] - x1[k] : x1[k], tf, 4));
 #pragma unroll
                             for (int a = 0; a < 3; ++a)
-                                tile[(8 * a + k) * DEPOSIT_STRIDE + order.col] = k == 0 ? 0 : fx_mul(vf[a], e);
+                                tile[(8 * a + k) * DEPOSIT_STRIDE + order.col] = k == 0 ? 0 : fx_mul(vf[a], x);
                         }
                     }
-                    flush(order, has, c, 3 * half, tv - 28, tf - 27);
+                    flush(order, has, c, 3 * half, unit);
                 }
                 if (has) {
                     long long w[3], Mf[8];
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) w[a] = fixed_of(h * lg[a], tg, 4);
+                    for (int a = 0; a < 3; ++a) w[a] = fixed_of(hl[a], top[3 + a], 4);
 #pragma unroll
                     for (int k = 1; k < 8; ++k) Mf[k] = fixed_of(M[k], 1023, 10);
                     rows(order.col, w, Mf);
                 }
-                flush(order, has, c, 6, tg - 56, 1023);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) unit[a] = top[3 + a] + 967;
+                flush(order, has, c, 6, unit);
             }
             // the end point's interpolant of A^{n+1}, transposed
             const double M[8] = {1.0, wk.te[0], wk.te[1], wk.te[0] * wk.te[1], wk.te[2], wk.te[0] * wk.te[2],
@@ -379,18 +398,24 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_scatter(
                 if (act) plain_rows(lam_tab + 3, wk.c, p.m, M, lA);
                 continue;
             }
-            const int e0[1] = {0};
-            int top0[1] = {0};
-            const TileOrder order(act, act ? (int)cell_row(wk.c, p.m) : -1, e0, top0);
+            int e[3], top[3], unit[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                e[a] = max(exponent_of(lA[a]), 64);
+                top[a] = 64;
+            }
+            const TileOrder order(act, act ? (int)cell_row(wk.c, p.m) : -1, e, top);
             if (act) {
                 long long w[3], Mf[8];
 #pragma unroll
-                for (int a = 0; a < 3; ++a) w[a] = fixed_of(lA[a], tA, 4);
+                for (int a = 0; a < 3; ++a) w[a] = fixed_of(lA[a], top[a], 4);
 #pragma unroll
                 for (int k = 1; k < 8; ++k) Mf[k] = fixed_of(M[k], 1023, 10);
                 rows(order.col, w, Mf);
             }
-            flush(order, act, wk.c, 3, tA - 56, 1023);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) unit[a] = top[a] + 967;
+            flush(order, act, wk.c, 3, unit);
         }
         __syncthreads();   // the hand-over buffers are rewritten by the next chunk
     }

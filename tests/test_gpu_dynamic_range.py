@@ -75,3 +75,38 @@ def test_current_of_slow_particles_beside_a_fast_one(sim, ppc):
     size = np.sqrt(np.mean(it[slow] ** 2))
     assert 0.0 < size <= 1e-6 * np.abs(it).max()
     assert np.abs(got["J"] - it)[slow].max() <= 1e-12 * size
+
+
+@pytest.mark.parametrize("key", ["v", "P", "A"])
+def test_adjoints_of_very_different_size(sim, key):
+    """The vjp is linear in its cotangent: a unit one on a particle and 1e-6 on others of its warp, some 16
+    cells away.  Around those the mesh adjoint is that of the small ones alone, to 1e-12: the unit one's own
+    reaches them through the solve's tail (below 1e-25) and its rounding ((4e-7)^3 = 6e-20)."""
+    import torch
+    n, dt, q = (32, 4, 4), 0.05, 1e-10
+    L = tuple(map(float, n))
+    rng = np.random.default_rng(6)
+    cells = np.stack(np.meshgrid(*[np.arange(k) for k in n], indexing="ij"), axis=-1).transpose(2, 1, 0, 3).reshape(-1, 3)
+    x = cells + rng.uniform(0.1, 0.9, size=cells.shape)        # one particle a cell, in the order of the cells
+    v = rng.normal(scale=0.5, size=x.shape)
+    npart, N = len(x), len(x)
+    s = sim.PicSim(sim.pic_config_default(n=n, L=L, dt=dt, picard_accel=0), x, v, q, 1.0)
+    assert s.step(1).converged
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    big, small = s.state_zeros(), s.state_zeros()
+    if key == "A":
+        big["A"].view(3, n[2], n[1], n[0])[:, 0, 0, 4] = 1.0
+        small["A"].view(3, n[2], n[1], n[0])[:, 0, 0, 18:23] = 1e-6 * torch.randn(3, 5, generator=gen, device="cuda", dtype=torch.float64)
+    else:
+        big[key].view(3, npart)[:, 4] = 1.0
+        small[key].view(3, npart)[:, 18:23] = 1e-6 * torch.randn(3, 5, generator=gen, device="cuda", dtype=torch.float64)
+    out = []
+    for lam in (small, {k: big[k] + small[k] for k in big}):
+        o, info = s.step_vjp(lam)
+        out.append(o)
+        assert info.residual <= 1e-11
+    s.close()
+    for name in ("A", "U"):
+        a, b = (o[name].view(3, n[2], n[1], n[0])[:, :, :, 17:25].cpu().numpy() for o in out)
+        assert np.abs(a).max() > 0.0
+        assert np.abs(b - a).max() <= 1e-12 * np.abs(a).max(), name
