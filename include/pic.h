@@ -158,7 +158,11 @@ typedef struct {
 } pic_particles;
 
 /* Optional device allocator (for example the caller's caching allocator).  When it is
- * absent the library uses cudaMalloc / cudaFree.  `stream` is the context's stream. */
+ * absent the library uses cudaMalloc / cudaFree.  `stream` is the context's stream.
+ * Optional tables (up to 1,728 bytes a cell, at most an eighth of the memory that is free at pic_init) are
+ * asked for last and may be refused.  They are given back when this or another context of the device
+ * cannot have memory that it needs: `free` may then be called from the other context's call, while this one
+ * is not in a call. */
 typedef struct {
     void* (*alloc)(size_t bytes, void* stream, void* user);
     void (*free)(void* ptr, size_t bytes, void* stream, void* user);

@@ -253,8 +253,8 @@ bool setup_pair_kernels() {
 }
 
 void launch_table_df(Ctx& c) {
-    float4* t = reinterpret_cast<float4*>(c.table_pair);
-    if (c.pair_cells) {
+    float4* t = reinterpret_cast<float4*>(c.pair_ctab ? c.pair_ctab : c.table_pair);
+    if (c.pair_ctab) {
         const int64_t n = CELL_VALUES / 2 * c.m.ncell;
         const int nb = (int)std::max<int64_t>(1, std::min<int64_t>((n + THREADS - 1) / THREADS, (int64_t)c.sms * 16));
         k_cells_df<<<nb, THREADS, 0, c.stream>>>(n, reinterpret_cast<const double2*>(c.ctab), t);
@@ -267,14 +267,14 @@ void launch_table_df(Ctx& c) {
 void launch_push_df(Ctx& c, const double* vit, double* vnew, double* Jnext) {
     cudaMemsetAsync(c.creep_count, 0, 2 * sizeof(int), c.stream);   // count, k_local queue head
     const int nb = chunk_blocks(c);
-    const float4* t = reinterpret_cast<const float4*>(c.table_pair);
+    const float4* t = reinterpret_cast<const float4*>(c.pair_ctab ? c.pair_ctab : c.table_pair);
 #define PIC_PUSH_DF(T, K)                                                                                           \
     k_push_df<T, K><<<nb, K::THREADS_, K::smem(), c.stream>>>(make_params_df(c), c.xi, c.v, c.P, vit, t, vnew, Jnext, \
                                                               c.creep_list, c.creep_count, c.slide, c.partials,    \
                                                               c.dev_status)
     const bool wide = wide_chunks(c);
-    if (c.pair_cells && wide) PIC_PUSH_DF(true, ChunkPush);
-    else if (c.pair_cells) PIC_PUSH_DF(true, ChunkLarge);
+    if (c.pair_ctab && wide) PIC_PUSH_DF(true, ChunkPush);
+    else if (c.pair_ctab) PIC_PUSH_DF(true, ChunkLarge);
     else if (wide) PIC_PUSH_DF(false, ChunkPush);
     else PIC_PUSH_DF(false, ChunkLarge);
 #undef PIC_PUSH_DF

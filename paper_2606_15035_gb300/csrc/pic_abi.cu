@@ -4,9 +4,11 @@
 // stream, converts CUDA failures and device status bits into a pic_status, and records a
 // one-line reason in ctx->err.  No entry point aborts.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <deque>
 #include <tuple>
 #include <new>
 #include <map>
@@ -24,6 +26,9 @@ using namespace pic;
 struct pic_ctx {
     Ctx c;
     std::vector<std::pair<void*, size_t>> allocs;
+    int device = 0;
+    std::vector<std::pair<void*, size_t>> evicted;   // optional tables on their way back to the allocator
+    std::atomic<bool> busy{false};                   // a call, or another context's request for the tables
 };
 
 namespace {
@@ -45,22 +50,78 @@ void* dev_alloc_once(pic_ctx* ctx, size_t bytes) {
     return p;
 }
 
-// Give the optional cell tables back (between calls: the kernels then read the gather table).
+void dev_free(pic_ctx* ctx, const std::pair<void*, size_t>& a) {
+    if (ctx->c.has_alloc) ctx->c.alloc.free(a.first, a.second, (void*)ctx->c.stream, ctx->c.alloc.user);
+    else cudaFree(a.first);
+}
+
+// ---- the optional tables of all contexts ---------------------------------------------------
+//
+// The cell tables are optional memory: a context that cannot have the memory it needs takes them back, its
+// own first, then those of other contexts on its device that are not in a call.  A context's calls hold
+// its `busy` mark, so that its tables never leave under a call that uses them.
+std::mutex g_holders_mutex;
+std::vector<pic_ctx*> g_holders;            // contexts with optional tables
+thread_local pic_ctx* tl_evicting = nullptr;   // the context whose tables this thread is giving back
+thread_local bool tl_gone = false;             // ... was destroyed on the way
+
+struct Use {
+    pic_ctx* ctx;
+    explicit Use(pic_ctx* c) : ctx(c) {
+        while (ctx->busy.exchange(true, std::memory_order_acquire)) std::this_thread::yield();
+    }
+    ~Use() { ctx->busy.store(false, std::memory_order_release); }
+    Use(const Use&) = delete;
+};
+
+void forget_holder(pic_ctx* ctx) {
+    std::lock_guard<std::mutex> lock(g_holders_mutex);
+    g_holders.erase(std::remove(g_holders.begin(), g_holders.end(), ctx), g_holders.end());
+}
+
+// Give a context's cell tables back (between its uses of them: the kernels then read the gather table).  An
+// allocator's free may end in pic_destroy of the same context (a garbage collector in a callback), which
+// then frees the rest and clears tl_evicting.
 bool drop_cell_table(pic_ctx* ctx) {
     Ctx& c = ctx->c;
     if (!c.ctab) return false;
+    forget_holder(ctx);
     cudaStreamSynchronize(c.stream);
-    for (void* t : {(void*)c.ctab, (void*)c.fxtab})
+    for (void* t : {(void*)c.ctab, (void*)c.fxtab, (void*)c.pair_ctab})
         for (size_t k = 0; t && k < ctx->allocs.size(); ++k) {
             if (ctx->allocs[k].first != t) continue;
-            if (c.has_alloc) c.alloc.free(t, ctx->allocs[k].second, (void*)c.stream, c.alloc.user);
-            else cudaFree(t);
+            ctx->evicted.push_back(ctx->allocs[k]);
             ctx->allocs.erase(ctx->allocs.begin() + (long)k);
             break;
         }
     c.ctab = nullptr;
     c.fxtab = nullptr;
-    c.pair_cells = false;   // its buffer is large enough for the pairs of the gather table
+    c.pair_ctab = nullptr;
+    tl_evicting = ctx;
+    while (tl_evicting == ctx && !ctx->evicted.empty()) {
+        const std::pair<void*, size_t> a = ctx->evicted.back();
+        ctx->evicted.pop_back();
+        dev_free(ctx, a);
+    }
+    tl_evicting = nullptr;
+    return true;
+}
+
+// The tables of one other context on this device that is not in a call; false when there is none.
+bool evict_another(pic_ctx* ctx) {
+    pic_ctx* other = nullptr;
+    {
+        std::lock_guard<std::mutex> lock(g_holders_mutex);
+        for (pic_ctx* t : g_holders)
+            if (t != ctx && t->device == ctx->device && !t->busy.exchange(true, std::memory_order_acquire)) {
+                other = t;
+                break;
+            }
+    }
+    if (!other) return false;
+    drop_cell_table(other);
+    if (tl_gone) tl_gone = false;
+    else other->busy.store(false, std::memory_order_release);
     return true;
 }
 
@@ -68,14 +129,14 @@ void* dev_alloc(pic_ctx* ctx, size_t bytes) {
     if (bytes == 0) bytes = 16;
     void* p = dev_alloc_once(ctx, bytes);
     if (!p && drop_cell_table(ctx)) p = dev_alloc_once(ctx, bytes);
+    while (!p && evict_another(ctx)) p = dev_alloc_once(ctx, bytes);
     return p;
 }
 
 void free_all(pic_ctx* ctx) {
-    for (auto& a : ctx->allocs) {
-        if (ctx->c.has_alloc) ctx->c.alloc.free(a.first, a.second, (void*)ctx->c.stream, ctx->c.alloc.user);
-        else cudaFree(a.first);
-    }
+    for (const auto& a : ctx->evicted) dev_free(ctx, a);
+    for (const auto& a : ctx->allocs) dev_free(ctx, a);
+    ctx->evicted.clear();
     ctx->allocs.clear();
     if (ctx->c.host_results) cudaFreeHost(ctx->c.host_results);
     if (ctx->c.host_status) cudaFreeHost(ctx->c.host_status);
@@ -300,12 +361,16 @@ void setup_geometry(Ctx& c) {
 // helmholtz_tol.  (On 2^p 3^q meshes every solve goes to roundoff.)
 constexpr double MESH_TOL32 = 1e-10;
 
-// Rule of the cell table (576 B per cell, orbit_cell.cuh): from one particle per cell on.  Three
-// FP64 steps measured with the table | without it: 64^3 at 1 per cell 11.18 | 11.19 ms a step, at 4
-// 15.0 | 17.9, at 16 32.6 | 45.7; 128^3 at 1 68.7 | 72.8, at 16 314 | 454; 32^3 at 1 4.34 | 4.53.
-// The byte limit keeps the table a small part of the device's memory (it is reached at 310^3).
+// Rule of the cell tables (orbit_cell.cuh, orbit_fixed.cuh, PIC_MIXED also pairs: 576 B a cell each):
+// from one particle per cell on.  Three FP64 steps, ms a step with the tables | without: 32^3 at 1 per
+// cell 2.25 | 3.02, at 4 2.29 | 3.36; 64^3 at 1 5.62 | 6.65, at 4 9.03 | 13.4; 128^3 at 1 39.9 | 48.7, at 4
+// 80.1 | 129.  PIC_MIXED: 32^3 at 1 2.27 | 2.68, 64^3 6.64 | 7.15, 128^3 44.8 | 49.0.
+// All of a context's tables take at most CELL_TABLE_SHARE of the device memory that is free when it is created,
+// so that runs side by side leave each other room, and what they hold goes to a context that cannot have
+// the memory it needs (dev_alloc).  CELL_TABLE_MAX_BYTES bounds the index arithmetic.
 constexpr int64_t CELL_TABLE_MIN_PPC = 1;
 constexpr size_t CELL_TABLE_MAX_BYTES = (size_t)16 << 30;
+constexpr double CELL_TABLE_SHARE = 0.125;
 
 #define ALLOC(ptr, type, count)                                                          \
     do {                                                                                 \
@@ -369,6 +434,11 @@ pic_status allocate(pic_ctx* ctx) {
             if (reinterpret_cast<uintptr_t>(q) % 16 != 0)
                 return fail(ctx, PIC_ERR_ARG, "the allocator returned a pointer that is not 16-byte aligned");
         ALLOC(c.table32, float, 12 * N);
+        if (c.cfg.mixed_pair_max > 0 && !c.cfg.deterministic) {
+            ALLOC(c.table_pair, float, 20 * N);
+            if (reinterpret_cast<uintptr_t>(c.table_pair) % 16 != 0)
+                return fail(ctx, PIC_ERR_ARG, "the allocator returned a pointer that is not 16-byte aligned");
+        }
     }
     if (c.cfg.deterministic) {
         ALLOC(c.acc_hi, long long, 3 * N);
@@ -463,21 +533,23 @@ pic_status allocate(pic_ctx* ctx) {
         cudaMemsetAsync(c.helm_top, 0, 8 * sizeof(int), c.stream);
         if (cudaStreamSynchronize(c.stream) != cudaSuccess) return check_cuda(ctx, "helmholtz tables");
     }
-    // last, because it is optional: the closed forms' cell table, where there are particles enough to
-    // repay building it and it stays a small part of the device's memory.
+    // last, because they are optional: the closed forms' cell tables
     const size_t cells = sizeof(double) * CELL_VALUES * (size_t)N;
-    if (c.closed && c.np >= CELL_TABLE_MIN_PPC * N && cells <= CELL_TABLE_MAX_BYTES) {
+    size_t room = 0, total = 0;
+    if (cudaMemGetInfo(&room, &total) != cudaSuccess) {
+        cudaGetLastError();
+        room = 0;
+    }
+    room = (size_t)(CELL_TABLE_SHARE * (double)room);
+    if (c.closed && c.np >= CELL_TABLE_MIN_PPC * N && cells <= CELL_TABLE_MAX_BYTES && 2 * cells <= room) {
         c.ctab = (double*)dev_alloc_once(ctx, cells);
         if (c.ctab) c.fxtab = (long long*)dev_alloc_once(ctx, cells);
         if (c.ctab && (!c.fxtab || (reinterpret_cast<uintptr_t>(c.ctab) | reinterpret_cast<uintptr_t>(c.fxtab)) % 16 != 0))
             drop_cell_table(ctx);
     }
-    if (c.cfg.precision == PIC_MIXED && c.cfg.mixed_pair_max > 0 && !c.cfg.deterministic) {
-        if (c.ctab) c.table_pair = (float*)dev_alloc_once(ctx, cells);
-        c.pair_cells = c.table_pair != nullptr;
-        if (!c.table_pair) ALLOC(c.table_pair, float, 20 * N);
-        if (reinterpret_cast<uintptr_t>(c.table_pair) % 16 != 0)
-            return fail(ctx, PIC_ERR_ARG, "the allocator returned a pointer that is not 16-byte aligned");
+    if (c.ctab && c.table_pair && 3 * cells <= room) {
+        c.pair_ctab = (float*)dev_alloc_once(ctx, cells);
+        if (c.pair_ctab && reinterpret_cast<uintptr_t>(c.pair_ctab) % 16 != 0) drop_cell_table(ctx);
     }
     std::memset(c.host_results, 0, sizeof(double) * NSLOT);
     *c.host_status = 0;
@@ -1049,6 +1121,7 @@ pic_status pic_init(const pic_config* cfg, const pic_particles* particles, const
     c.np = particles->np;
     c.q = particles->q;
     c.mass = particles->m;
+    ctx->device = dev;
     setup_geometry(c);
     pic_status s = allocate(ctx);
     if (s != PIC_OK) {
@@ -1091,6 +1164,10 @@ pic_status pic_init(const pic_config* cfg, const pic_particles* particles, const
         return s;
     }
     c.fresh_init = true;
+    if (c.ctab) {
+        std::lock_guard<std::mutex> lock(g_holders_mutex);
+        g_holders.push_back(ctx);
+    }
     *out = ctx;
     return PIC_OK;
 }
@@ -1098,6 +1175,7 @@ pic_status pic_init(const pic_config* cfg, const pic_particles* particles, const
 
 pic_status pic_step(pic_ctx* ctx, int32_t nsteps, pic_step_info* info) {
     if (!ctx || nsteps < 0) return PIC_ERR_ARG;
+    const Use use(ctx);
     ctx->c.err.clear();
     pic_step_info local{};
     pic_step_info last{};
@@ -1122,6 +1200,7 @@ pic_status pic_step(pic_ctx* ctx, int32_t nsteps, pic_step_info* info) {
 
 pic_status pic_energy(pic_ctx* ctx, pic_energy_t* out) {
     if (!ctx || !out) return PIC_ERR_ARG;
+    const Use use(ctx);
     Ctx& c = ctx->c;
     queue_energy(c);
     pic_status s = sync_results(ctx, "pic_energy");
@@ -1141,6 +1220,7 @@ pic_status pic_diagnostics(pic_ctx* ctx, pic_diag_t* out) {
 
 pic_status pic_get_state(pic_ctx* ctx, const pic_state_view* dst) {
     if (!ctx || !dst) return PIC_ERR_ARG;
+    const Use use(ctx);
     Ctx& c = ctx->c;
     const int64_t np = c.np, N = c.m.ncell;
     const cudaMemcpyKind kind = dst->on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
@@ -1166,6 +1246,7 @@ pic_status pic_get_state(pic_ctx* ctx, const pic_state_view* dst) {
 
 pic_status pic_set_state(pic_ctx* ctx, const pic_state_view* src) {
     if (!ctx || !src) return PIC_ERR_ARG;
+    const Use use(ctx);
     Ctx& c = ctx->c;
     const int64_t np = c.np, N = c.m.ncell;
     if (np > 0 && (!src->x || !src->v || !src->P || !src->vprev)) return PIC_ERR_ARG;
@@ -1193,6 +1274,7 @@ pic_status pic_set_state(pic_ctx* ctx, const pic_state_view* src) {
 
 pic_status pic_iterate(pic_ctx* ctx, const double* v_iter, int32_t on_device, const pic_iterate_out* out) {
     if (!ctx || !v_iter || !out) return PIC_ERR_ARG;
+    const Use use(ctx);
     Ctx& c = ctx->c;
     const int64_t np = c.np, N = c.m.ncell;
     const cudaMemcpyKind kin = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
@@ -1239,6 +1321,7 @@ pic_status pic_iterate(pic_ctx* ctx, const double* v_iter, int32_t on_device, co
 
 pic_status pic_get_positions(pic_ctx* ctx, double* xi, int32_t on_device) {
     if (!ctx || !xi) return PIC_ERR_ARG;
+    const Use use(ctx);
     Ctx& c = ctx->c;
     if (c.np == 0) return PIC_OK;
     launch_unpermute(c, c.xi, c.sort_tmp, 1.0, 1.0, 1.0);
@@ -1250,6 +1333,7 @@ pic_status pic_get_positions(pic_ctx* ctx, double* xi, int32_t on_device) {
 
 pic_status pic_set_positions(pic_ctx* ctx, const double* xi, int32_t on_device) {
     if (!ctx || !xi) return PIC_ERR_ARG;
+    const Use use(ctx);
     Ctx& c = ctx->c;
     if (c.np == 0) return PIC_OK;
     cudaMemcpyAsync(c.sort_tmp, xi, sizeof(double) * 3 * c.np,
@@ -1264,6 +1348,7 @@ pic_status pic_set_positions(pic_ctx* ctx, const double* xi, int32_t on_device) 
 
 pic_status pic_get_iterate(pic_ctx* ctx, double* v_iter, double* g_iter, int32_t on_device) {
     if (!ctx || !v_iter || !g_iter) return PIC_ERR_ARG;
+    const Use use(ctx);
     Ctx& c = ctx->c;
     if (c.np == 0) return PIC_OK;
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
@@ -1283,6 +1368,7 @@ pic_status pic_get_iterate(pic_ctx* ctx, double* v_iter, double* g_iter, int32_t
 
 pic_status pic_get_accepted(pic_ctx* ctx, double* v_iter, uint8_t* slide, int32_t on_device) {
     if (!ctx || (!v_iter && !slide)) return PIC_ERR_ARG;
+    const Use use(ctx);
     Ctx& c = ctx->c;
     if (!c.have_accepted)
         return fail(ctx, PIC_ERR_ARG, "pic_get_accepted: only available right after a committed pic_step");
@@ -1530,6 +1616,7 @@ extern "C" {
 pic_status pic_step_vjp(pic_ctx* ctx, const pic_state_view* lam_next, const pic_state_view* lam_prev,
                         pic_vjp_info* info) {
     if (!ctx || !lam_next || !lam_prev) return PIC_ERR_ARG;
+    const Use use(ctx);
     Ctx& c = ctx->c;
     c.err.clear();
     if (!c.have_accepted)
@@ -1595,6 +1682,7 @@ pic_status pic_step_vjp(pic_ctx* ctx, const pic_state_view* lam_next, const pic_
 
 pic_status pic_energy_vjp(pic_ctx* ctx, const pic_state_view* lam) {
     if (!ctx || !lam) return PIC_ERR_ARG;
+    const Use use(ctx);
     Ctx& c = ctx->c;
     if (c.cfg.ops != PIC_OPS_CENTRAL2) return fail(ctx, PIC_ERR_ARG, "pic_energy_vjp: needs central differences");
     pic_status s = adj_alloc(ctx);
@@ -1618,6 +1706,7 @@ pic_status pic_energy_vjp(pic_ctx* ctx, const pic_state_view* lam) {
 
 pic_status pic_init_vjp(pic_ctx* ctx, const pic_state_view* lam0, double* lam_x0, double* lam_v0, int32_t on_device) {
     if (!ctx || !lam0) return PIC_ERR_ARG;
+    const Use use(ctx);
     Ctx& c = ctx->c;
     c.err.clear();
     if (!c.fresh_init)
@@ -1667,6 +1756,7 @@ pic_status pic_set_wait_limit(pic_ctx* ctx, int64_t cycles) {
 
 pic_status pic_profile(pic_ctx* ctx, int32_t enable, pic_profile_t* out) {
     if (!ctx) return PIC_ERR_ARG;
+    const Use use(ctx);
     Ctx& c = ctx->c;
     if (cudaStreamSynchronize(c.stream) != cudaSuccess) return check_cuda(ctx, "pic_profile");
     prof_resolve(c);
@@ -1733,6 +1823,7 @@ extern "C" {
 
 pic_status pic_autotune(pic_ctx* ctx, int32_t* push_blocks_per_sm, int32_t* push32_blocks_per_sm) {
     if (!ctx) return PIC_ERR_ARG;
+    const Use use(ctx);
     Ctx& c = ctx->c;
     c.err.clear();
     const TuneKey key{{c.m.n[0], c.m.n[1], c.m.n[2]}, c.np >> 14, c.cfg.precision};
@@ -1851,6 +1942,8 @@ pic_ctx* pic_ensemble_run(pic_ensemble* e, int32_t i) {
 pic_status pic_ensemble_step(pic_ensemble* e, int32_t nsteps, pic_step_info* infos, pic_status* statuses) {
     if (!e || nsteps < 0) return PIC_ERR_ARG;
     const int R = (int)e->runs.size();
+    std::deque<Use> use;
+    for (pic_ctx* r : e->runs) use.emplace_back(r);
     std::vector<pic_step_info> acc(R), last(R);
     std::vector<pic_status> st(R, PIC_OK);
     std::vector<int> pending, finals;
@@ -1948,6 +2041,13 @@ const char* pic_last_error(const pic_ctx* ctx) {
 
 void pic_destroy(pic_ctx* ctx) {
     if (!ctx) return;
+    if (tl_evicting == ctx) {
+        tl_evicting = nullptr;
+        tl_gone = true;
+    } else {
+        while (ctx->busy.exchange(true, std::memory_order_acquire)) std::this_thread::yield();
+    }
+    forget_holder(ctx);
     cudaStreamSynchronize(ctx->c.stream);
     prof_resolve(ctx->c);
     for (cudaEvent_t e : ctx->c.ev_pool) cudaEventDestroy(e);

@@ -199,9 +199,9 @@ struct Ctx {
     int32_t* cell32 = nullptr;
     float *off32 = nullptr, *v32 = nullptr, *vit32 = nullptr, *vnew32 = nullptr;   // iterates: increments
     float* table32 = nullptr;            // 12 * ncell
-    float* table_pair = nullptr;         // FP32 pairs: the cell table (2 CELL_VALUES * ncell), or of the
-                                         // gather table (20 * ncell: A^n, A^{n+1}, grad phi, pad)
-    bool pair_cells = false;             // which of the two
+    float* table_pair = nullptr;         // FP32 pairs of the gather table (20 * ncell: A^n, A^{n+1}, grad phi,
+                                         // pad), read where there is no
+    float* pair_ctab = nullptr;          // cell table of pairs (2 CELL_VALUES * ncell, optional, with ctab)
 
     // reductions and status
     double *partials = nullptr, *results = nullptr;

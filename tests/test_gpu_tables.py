@@ -70,3 +70,54 @@ def test_the_transforms_need_no_memory_of_their_own(sim, monkeypatch, n):
     s = sim.PicSim(sim.pic_config_default(n=n, L=L, dt=0.1, deterministic=1), x, v, q, m)
     assert s.step(1).converged and limit.refused == 0
     s.close()
+
+
+TABLES = 576   # bytes a cell of one cell table
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("ensemble", [False, True])
+def test_tables_go_to_a_context_that_needs_the_memory(sim, monkeypatch, precision, ensemble):
+    """A second run whose memory fits only without the first one's tables is created, and both go on:
+    as runs alone, to rounding (the kernels without tables take the same sums in another arithmetic)."""
+    n, L = (12, 10, 8), (1.2, 1.0, 0.8)
+    N = int(np.prod(n))
+    cfg = sim.pic_config_default(n=n, L=L, dt=0.05, picard_tol=1e-13, precision=precision)
+    runs = [(cfg, *particles(n, L, 16, seed)) for seed in (31, 32)]
+    alone = []
+    for r in runs:
+        s = sim.PicSim(*r)
+        s.step(2)
+        alone.append(s.get_state())
+        s.close()
+    with monkeypatch.context() as mp:
+        bare = Limit(sim, mp, lambda b: b == TABLES * N)
+        s = sim.PicSim(*runs[0])
+        need = bare.used()
+        s.close()
+        assert bare.refused and need > 0 and not bare.live
+    limit = Limit(sim, monkeypatch)
+    first = sim.PicSim(*runs[0])
+    full = limit.used()
+    assert full >= need + (2 + precision) * TABLES * N   # the first holds its tables
+    if ensemble:
+        first.close()
+        limit.capacity = full + need - TABLES * N
+        e = sim.PicEnsemble(runs)
+        e.step(2)
+        got = [r.get_state() for r in e.runs]
+        e.close()
+    else:
+        first.step(1)
+        limit.capacity = full + need - TABLES * N
+        second = sim.PicSim(*runs[1])
+        first.step(1)                                 # from here on without tables
+        second.step(2)
+        got = [first.get_state(), second.get_state()]
+        first.close()
+        second.close()
+    assert limit.refused and not limit.live
+    for a, b in zip(got, alone):
+        for name in ("v", "P", "phi", "A"):
+            d = np.linalg.norm(getattr(a, name) - getattr(b, name)) / np.linalg.norm(getattr(b, name))
+            assert d <= (1e-11 if precision == 0 else 1e-8), (name, d)
