@@ -490,11 +490,12 @@ __global__ void k_adj_mesh_out(AdjParams ap, const double* __restrict__ y, const
 // derivatives by six dual-number evaluations of the push took 13.6 ms a sweep at 32^3 with 524,288
 // particles.
 
-template <bool CELLS>
+template <int FROM>
 __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_derivs(AdjParams ap, const double* __restrict__ xi,
                                                            const double* __restrict__ v,
                                                            const double* __restrict__ vstar,
                                                            const double* __restrict__ table,
+                                                           const double* __restrict__ ctab,
                                                            const double* __restrict__ lJ,
                                                            const double* __restrict__ lam_P,
                                                            const double* __restrict__ lam_v,
@@ -589,7 +590,7 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_derivs(AdjParam
                             for (int k = 0; k < 8; ++k)
                                 if (k & bit) K[k] -= K[k ^ bit];
                     }
-                    const FieldLoad<CELLS> ld(table, wk.c, p.m);
+                    const FieldLoad<FROM> ld({table, ctab}, wk.c, p.m);
                     double a3 = 0.0, a5 = 0.0, a6 = 0.0, a7 = 0.0, c3 = 0.0, c5 = 0.0, c6 = 0.0, c7 = 0.0;
 #pragma unroll
                     for (int pr = 0; pr < 4; ++pr) {
@@ -676,7 +677,7 @@ __global__ void __launch_bounds__(ChunkLarge::THREADS_, 4) k_adj_derivs(AdjParam
                     out_adjoints(p, (sb >> a) & 1u, lam_v[a * np + i], lam_P[a * np + i], mu[a * np + i], lP1[a],
                                  lAe[a], lg, lF);
                 }
-                const FieldLoad<CELLS> ld(table, wk.c, p.m);
+                const FieldLoad<FROM> ld({table, ctab}, wk.c, p.m);
 #pragma unroll
                 for (int pr = 0; pr < 4; ++pr)
 #pragma unroll
@@ -979,11 +980,12 @@ void launch_adj_derivs(Ctx& c, const double* xi, const double* v, const double* 
                        const double* lam_P, const double* lam_v, const double* lam_xe, const double* mu,
                        double* lam_xi, double* g, double* lvn, double* lPn) {
     const int nb = adj_blocks(c, c.np);
-#define PIC_DERIVS(T, TAB)                                                                                        \
-    k_adj_derivs<T><<<nb, ChunkLarge::THREADS_, 0, c.stream>>>(adj_params(c), xi, v, vstar, TAB, lJ, lam_P, lam_v, lam_xe, mu,    \
-                                                  c.slide, lam_xi, g, lvn, lPn, c.dev_status)
-    if (c.ctab) PIC_DERIVS(true, c.ctab);
-    else PIC_DERIVS(false, c.table);
+#define PIC_DERIVS(T)                                                                                            \
+    k_adj_derivs<T><<<nb, ChunkLarge::THREADS_, 0, c.stream>>>(adj_params(c), xi, v, vstar, c.table, c.ctab, lJ, lam_P, \
+                                                               lam_v, lam_xe, mu, c.slide, lam_xi, g, lvn, lPn,    \
+                                                               c.dev_status)
+    if (c.ctab) PIC_DERIVS(FROM_CELLS);
+    else PIC_DERIVS(FROM_NODES);
 #undef PIC_DERIVS
     ++c.launches;
 }

@@ -331,14 +331,26 @@ __device__ __forceinline__ void cell_nodes8(const int c[3], const MeshDims& m, i
     g[7] = g[6] + dx;
 }
 
-// Loader of a cell's entries for piece_impulse and cell_A1: from the FP64 cell table, or (CELLS
-// = false, contexts without that table) from the gather table, taking the differences of the
-// cell's nodes each time.
-template <bool CELLS>
-struct FieldLoad {
+// Where the particle kernels take a cell's entries from: the FP64 cell table; the gather table, taking the
+// differences of the cell's nodes each time (contexts without cell tables); or, in deterministic mode, the cell
+// table where there is one and the gather table where not, by the same instructions but for the loads.  The
+// differences are the same numbers (subtractions in the same order), so that the bits do not depend on
+// whether the table's memory was there.
+enum Fields { FROM_NODES, FROM_CELLS, FROM_EITHER };
+
+struct FieldTables {
+    const double* nodes;   // gather table
+    const double* cells;   // cell table
+};
+
+template <int FROM>
+struct FieldLoad;
+
+template <>
+struct FieldLoad<FROM_CELLS> {
     const double2* t;
-    __device__ __forceinline__ FieldLoad(const double* table, const int c[3], const MeshDims& m)
-        : t(reinterpret_cast<const double2*>(table + CELL_VALUES * cell_row(c, m))) {}
+    __device__ __forceinline__ FieldLoad(FieldTables ft, const int c[3], const MeshDims& m)
+        : t(reinterpret_cast<const double2*>(ft.cells + CELL_VALUES * cell_row(c, m))) {}
     __device__ __forceinline__ void operator()(int p, int col, double& a, double& b) const {
         const double2 q = __ldg(t + p * CELL_COLS + col);
         a = q.x;
@@ -347,10 +359,10 @@ struct FieldLoad {
 };
 
 template <>
-struct FieldLoad<false> {
+struct FieldLoad<FROM_NODES> {
     const double* t;
     int64_t g[8];
-    __device__ __forceinline__ FieldLoad(const double* table, const int c[3], const MeshDims& m) : t(table) {
+    __device__ __forceinline__ FieldLoad(FieldTables ft, const int c[3], const MeshDims& m) : t(ft.nodes) {
         cell_nodes8(c, m, g);
     }
     __device__ __forceinline__ double node(int k, int col) const {
@@ -375,6 +387,38 @@ struct FieldLoad<false> {
             a = lo - a;
             b = (node(2 * p + 1, col) - lo) - b;
         }
+    }
+};
+
+// One pair of entries from the gather table (a function of its own: FROM_EITHER's rare side).
+static __device__ __noinline__ double2 entries_of_nodes(const double* nodes, int c0, int c1, int c2, int n0, int n1, int n2,
+                                                        int p, int col) {
+    MeshDims m;
+    m.n[0] = n0;
+    m.n[1] = n1;
+    m.n[2] = n2;
+    const int c[3] = {c0, c1, c2};
+    double2 q;
+    FieldLoad<FROM_NODES>({nodes, nullptr}, c, m)(p, col, q.x, q.y);
+    return q;
+}
+
+template <>
+struct FieldLoad<FROM_EITHER> {
+    FieldTables ft;
+    const MeshDims& m;
+    const double2* t;   // the cell's entries, or null
+    int c[3];
+    __device__ __forceinline__ FieldLoad(FieldTables tables, const int cell[3], const MeshDims& dims)
+        : ft(tables), m(dims), c{cell[0], cell[1], cell[2]} {
+        t = ft.cells ? reinterpret_cast<const double2*>(ft.cells + CELL_VALUES * cell_row(c, m)) : nullptr;
+    }
+    __device__ __forceinline__ void operator()(int p, int col, double& a, double& b) const {
+        double2 q;
+        if (__builtin_expect(t != nullptr, 1)) q = __ldg(t + p * CELL_COLS + col);
+        else q = entries_of_nodes(ft.nodes, c[0], c[1], c[2], m.n[0], m.n[1], m.n[2], p, col);
+        a = q.x;
+        b = q.y;
     }
 };
 

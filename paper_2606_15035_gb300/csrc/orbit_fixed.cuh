@@ -23,12 +23,22 @@ namespace pic {
 constexpr int FX_FIELD_UP = 5;   // fixed_of's shift for the table: 58 bits
 constexpr int FX_V_UP = 9;       // ... for velocities: 62 bits
 
-// Loader of a cell's entries.  The entries k = 0 of the A columns are not used; two of them hold the
-// exponents of the cell's groups.
-struct FixedLoad {
+// Loader of a cell's entries (FROM_CELLS, or in deterministic mode FROM_EITHER: from the gather table where
+// there is no fixed-point table, the same integers).  The entries k = 0 of the A columns are not used; two of
+// them hold the exponents of the cell's groups.
+template <int FROM>
+struct FixedLoad;
+
+struct FixedTables {
+    const double* nodes;      // gather table
+    const longlong2* cells;   // fixed-point cell table
+};
+
+template <>
+struct FixedLoad<FROM_CELLS> {
     const longlong2* t;
-    __device__ __forceinline__ FixedLoad(const longlong2* table, const int c[3], const MeshDims& m)
-        : t(table + (CELL_VALUES / 2) * cell_row(c, m)) {}
+    __device__ __forceinline__ FixedLoad(FixedTables ft, const int c[3], const MeshDims& m)
+        : t(ft.cells + (CELL_VALUES / 2) * cell_row(c, m)) {}
     __device__ __forceinline__ void operator()(int p, int col, long long& a, long long& b) const {
         const longlong2 q = __ldg(t + p * CELL_COLS + col);
         a = q.x;
@@ -36,6 +46,52 @@ struct FixedLoad {
     }
     __device__ __forceinline__ int top_A() const { return (int)__ldg(&t[0].x); }
     __device__ __forceinline__ int top_g() const { return (int)__ldg(&t[1].x); }
+};
+
+// The largest exponents (at least 64) of a cell's groups, the differences of the A columns and -grad phi,
+// from the gather table.
+static __device__ __noinline__ int2 tops_of_nodes(const double* nodes, int c0, int c1, int c2, int n0, int n1, int n2) {
+    int2 top = make_int2(64, 64);
+    for (int p = 0; p < 4; ++p)
+        for (int col = 0; col < CELL_COLS; ++col) {
+            const double2 q = entries_of_nodes(nodes, c0, c1, c2, n0, n1, n2, p, col);
+            const int e = max(p == 0 && col < 6 ? 0 : exponent_of(q.x), exponent_of(q.y));
+            if (col < 6) top.x = max(top.x, e);
+            else top.y = max(top.y, e);
+        }
+    return top;
+}
+
+template <>
+struct FixedLoad<FROM_EITHER> {
+    FixedTables ft;
+    const MeshDims& m;
+    const longlong2* t;   // the cell's entries, or null
+    int c[3];
+    int2 top;
+    __device__ __forceinline__ FixedLoad(FixedTables tables, const int cell[3], const MeshDims& dims)
+        : ft(tables), m(dims), t(nullptr), c{cell[0], cell[1], cell[2]} {
+        if (__builtin_expect(ft.cells != nullptr, 1)) {
+            t = ft.cells + (CELL_VALUES / 2) * cell_row(c, m);
+            top = make_int2((int)__ldg(&t[0].x), (int)__ldg(&t[1].x));
+        } else {
+            top = tops_of_nodes(ft.nodes, c[0], c[1], c[2], m.n[0], m.n[1], m.n[2]);
+        }
+    }
+    __device__ __forceinline__ void operator()(int p, int col, long long& a, long long& b) const {
+        if (__builtin_expect(t != nullptr, 1)) {
+            const longlong2 q = __ldg(t + p * CELL_COLS + col);
+            a = q.x;
+            b = q.y;
+        } else {
+            const double2 q = entries_of_nodes(ft.nodes, c[0], c[1], c[2], m.n[0], m.n[1], m.n[2], p, col);
+            const int e = col < 6 ? top.x : top.y;
+            a = fixed_of(q.x, e, FX_FIELD_UP);
+            b = fixed_of(q.y, e, FX_FIELD_UP);
+        }
+    }
+    __device__ __forceinline__ int top_A() const { return top.x; }
+    __device__ __forceinline__ int top_g() const { return top.y; }
 };
 
 // The unit 2^e' of a sum, e' = e - 1023, of quantities whose largest biased exponent is `top`: NaN where that

@@ -675,24 +675,19 @@ __device__ __forceinline__ void push_eval(const StepParams& p, const double x0[3
 }
 
 // G(u) of the closed forms, from the start (cell, coordinate) and vs = u + v^n =
-// 2 vbar: in fixed point from the cell tables (FIXED), or from the gather table in FP64.
+// 2 vbar: in fixed point from the cell tables, or (FROM_NODES) in FP64 from the gather table.
 struct CellOut {
     double Pw[3], Ae[3], vw[3];
     int nseg;
 };
 
-struct CellFields {
-    const double* table;      // gather table
-    const longlong2* tfx;     // fixed-point cell table (FIXED)
-};
-
-template <bool FIXED>
+template <int FROM>
 __device__ __forceinline__ void push_eval_cell(const StepParams& p, CellStart<double> st, const double vs[3],
-                                               const double Pn[3], const CellFields& cf, CellOut& o) {
+                                               const double Pn[3], FixedTables ft, CellOut& o) {
     double beta[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) beta[a] = p.cb[a] * vs[a];
-    if constexpr (FIXED) {
+    if constexpr (FROM != FROM_NODES) {
         const int ev = max(max(exponent_of(vs[0]), exponent_of(vs[1])), max(exponent_of(vs[2]), 64));
         Fs v[3];
         double accF[3] = {0.0, 0.0, 0.0}, accG[3] = {0.0, 0.0, 0.0};
@@ -700,16 +695,16 @@ __device__ __forceinline__ void push_eval_cell(const StepParams& p, CellStart<do
         for (int a = 0; a < 3; ++a) v[a] = fs_of(fixed_of(vs[a], ev, FX_V_UP));
         o.nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
             const double d[3] = {h * beta[0], h * beta[1], h * beta[2]};
-            piece_impulse_fixed(h, sm, mid, d, v, ev, FixedLoad(cf.tfx, c, p.m), accF, accG);
+            piece_impulse_fixed(h, sm, mid, d, v, ev, FixedLoad<FROM>(ft, c, p.m), accF, accG);
         });
-        const FixedLoad ld(cf.tfx, st.c, p.m);
+        const FixedLoad<FROM> ld(ft, st.c, p.m);
         long long A1[3];
         cell_A1_fixed(st.f, ld, A1);
         // values that are not finite stay so (the start's coordinate: the end's is its sum with beta)
         const int ef = max(max(exponent_of(st.f[0]), exponent_of(st.f[1])), exponent_of(st.f[2]));
         const double dtq = max(ev, ef) < 0x7ff ? p.dtq : NAN;
         const double uA = pow2_biased(ld.top_A() - 57);
-        const double* low = cf.table + 12 * cell_row(st.c, p.m) + 3;   // A^{n+1} at the cell's lowest node
+        const double* low = ft.nodes + 12 * cell_row(st.c, p.m) + 3;   // A^{n+1} at the cell's lowest node
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             o.Ae[a] = __ldg(low + a) + uA * (double)A1[a];
@@ -718,9 +713,9 @@ __device__ __forceinline__ void push_eval_cell(const StepParams& p, CellStart<do
     } else {
         double acc[3] = {0.0, 0.0, 0.0};
         o.nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
-            piece_impulse(h, sm, mid, beta, vs, p.ihs, FieldLoad<false>(cf.table, c, p.m), acc);
+            piece_impulse(h, sm, mid, beta, vs, p.ihs, FieldLoad<FROM_NODES>({ft.nodes, nullptr}, c, p.m), acc);
         });
-        cell_A1(st.f, FieldLoad<false>(cf.table, st.c, p.m), o.Ae);
+        cell_A1(st.f, FieldLoad<FROM_NODES>({ft.nodes, nullptr}, st.c, p.m), o.Ae);
 #pragma unroll
         for (int a = 0; a < 3; ++a) o.Pw[a] = Pn[a] + p.dtq * acc[a];
     }
@@ -779,7 +774,7 @@ __global__ void __launch_bounds__(32 * WARPS, SCATTER_WARPS / WARPS) k_first_sca
 }
 
 // The Algorithm 1 push for the closed forms without diagnostics: as k_push (below), in fixed point
-// from the cell tables (FIXED) or in FP64 from the gather table.
+// from the cell tables or (FROM_NODES) in FP64 from the gather table.
 //
 // It was bound by the FP64 pipe (one warp instruction in 16 clocks per SM), so the steps that made it
 // faster take instructions off that pipe.  Measured at 32^3 with 2,097,152 particles (1.31 pieces
@@ -790,11 +785,11 @@ __global__ void __launch_bounds__(32 * WARPS, SCATTER_WARPS / WARPS) k_first_sca
 // sums of products shifted once; 1.03 and 0.68 with the one-crossing walk (10.3M and 7.5M); 0.96 and 0.65 with
 // eight warps a block (chunk.cuh).  At 128^3 with 134M particles the final sweep took 225, 102, 64, now 54 ms.
 // What is left is latency (36% issue-active): fixed-latency waits, shared memory, the instruction cache.
-template <bool COMMIT, bool FIXED, int WARPS, int ITEMS>
+template <bool COMMIT, int FROM, int WARPS, int ITEMS>
 __global__ void __launch_bounds__(32 * WARPS, PUSH_WARPS / WARPS) k_push_cell(StepParams p, const double* __restrict__ xi,
                                                           const double* __restrict__ v, const double* __restrict__ P,
                                                           const double* __restrict__ vit,
-                                                          CellFields cf, double* __restrict__ vnew,
+                                                          FixedTables ft, double* __restrict__ vnew,
                                                           double* __restrict__ Jnext, double* __restrict__ xi_out,
                                                           double* __restrict__ P_out,
                                                           int32_t* __restrict__ creep_list,
@@ -831,7 +826,7 @@ __global__ void __launch_bounds__(32 * WARPS, PUSH_WARPS / WARPS) k_push_cell(St
 #pragma unroll
                 for (int a = 0; a < 3; ++a) Pn[a] = P[a * np + i];
                 CellOut o;
-                push_eval_cell<FIXED>(p, st, vs, Pn, cf, o);
+                push_eval_cell<FROM>(p, st, vs, Pn, ft, o);
                 if (o.nseg < 0) atomicOr(status, DEV_ERR_SEGMENTS);
                 pieces_push += o.nseg;
                 if (!(isfinite(o.vw[0]) && isfinite(o.vw[1]) && isfinite(o.vw[2]))) atomicOr(status, DEV_ERR_NONFINITE);
@@ -992,11 +987,11 @@ __device__ __forceinline__ void piece_diag(double h, double sm, const double mid
 }
 
 // The closed forms' final sweep with the particle diagnostics, in the centred form of k_push_cell
-// (FP64; CELLS: from the cell table).  Bound by the FP64 pipe like that: some 240 operations a piece where
+// (FP64).  Bound by the FP64 pipe like that: some 240 operations a piece where
 // the integrals from the piece's start took some 700: 1.62 ms at 50 x 35 x 22 with 539,000 particles, now
 // 0.68.
 constexpr int DIAG_WARPS = 16;   // 12 (168 registers): two steps at 16^3 2.77 ms, 16 2.69
-template <bool CELLS, int WARPS, int ITEMS>
+template <int FROM, int WARPS, int ITEMS>
 __global__ void __launch_bounds__(32 * WARPS, DIAG_WARPS / WARPS) k_commit_diag(
     StepParams p, const double* __restrict__ xi, const double* __restrict__ v, const double* __restrict__ P,
     const double* __restrict__ vit, const double* __restrict__ table, const double* __restrict__ ctab,
@@ -1033,11 +1028,11 @@ __global__ void __launch_bounds__(32 * WARPS, DIAG_WARPS / WARPS) k_commit_diag(
             const int nseg = for_each_piece(st, beta, p.m, [&](double h, double s, const double mid[3], const int c[3]) {
                 int64_t g[8];
                 cell_nodes8(c, p.m, g);
-                piece_diag(h, s, mid, beta, vs, p.ihs, vh, FieldLoad<CELLS>(CELLS ? ctab : table, c, p.m), table, g, acc);
+                piece_diag(h, s, mid, beta, vs, p.ihs, vh, FieldLoad<FROM>({table, ctab}, c, p.m), table, g, acc);
             });
             if (nseg < 0) atomicOr(status, DEV_ERR_SEGMENTS);
             double Ae[3], As[3], x0[3], ra2 = 0.0;
-            cell_A1(st.f, FieldLoad<CELLS>(CELLS ? ctab : table, st.c, p.m), Ae);
+            cell_A1(st.f, FieldLoad<FROM>({table, ctab}, st.c, p.m), Ae);
 #pragma unroll
             for (int a = 0; a < 3; ++a) x0[a] = xi[a * np + i];
             {   // A_h^n(x^n)
@@ -1306,15 +1301,15 @@ __device__ __forceinline__ double pick8(const double v[8], int k) {
 
 // Lane r's share of piece_impulse: acc_j += its terms, those of the subsets r, r + LANES, ... (summed
 // over the lanes they are the piece's).
-template <bool CELLS, int LANES>
+template <int FROM, int LANES>
 __device__ __forceinline__ void piece_impulse_share(const StepParams& p, int r, double h, double sm, const double mid[3],
                                                     const double beta[3], const double vs[3], const int c[3],
-                                                    const double* __restrict__ table, double acc[3]) {
+                                                    FieldTables ft, double acc[3]) {
     const PieceMoments<double> q = piece_moments(h, mid, beta);
     const double M[8] = {1.0, mid[0], mid[1], q.Pxy, mid[2], q.Pxz, q.Pyz, q.S};
     const double E[8] = {0.0, q.e[0], q.e[1], mid[0] * q.e[1] + mid[1] * q.e[0],
                          q.e[2], mid[0] * q.e[2] + mid[2] * q.e[0], mid[1] * q.e[2] + mid[2] * q.e[1], 0.0};
-    const FieldLoad<CELLS> ld(table, c, p.m);
+    const FieldLoad<FROM> ld(ft, c, p.m);
     const double hi[3] = {h * p.ihs[0], h * p.ihs[1], h * p.ihs[2]};
 #pragma unroll
     for (int s = 0; s < 8 / LANES; ++s) {
@@ -1372,10 +1367,11 @@ __device__ __forceinline__ void basis1<1>(double x, double invH, Basis1<1>& b) {
 
 // G(u) of the particle that a group of lanes shares, u = vs - v^n: every lane gets the component `comp` of
 // v^{n+1}.  Every lane of the warp calls it (inactive groups with any valid start).
-template <int QUAD, bool CELLS>
+template <int QUAD, int FROM>
 __device__ __forceinline__ double push_eval_shared(const StepParams& p, int k, int comp, const double x0[3],
                                                    const CellStart<double>& start, const double vs[3], double Pn,
-                                                   const double* __restrict__ table, int& nseg) {
+                                                   const double* __restrict__ table,
+                                                   const double* __restrict__ ctab, int& nseg) {
     constexpr int LANES = local_lanes<QUAD>();
     double beta[3], acc[3] = {0.0, 0.0, 0.0}, Ae[3] = {0.0, 0.0, 0.0};
     CellStart<double> st = start;
@@ -1383,9 +1379,9 @@ __device__ __forceinline__ double push_eval_shared(const StepParams& p, int k, i
     for (int a = 0; a < 3; ++a) beta[a] = p.cb[a] * vs[a];
     if constexpr (QUAD == 0) {
         nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
-            piece_impulse_share<CELLS, LANES>(p, k, h, sm, mid, beta, vs, c, table, acc);
+            piece_impulse_share<FROM, LANES>(p, k, h, sm, mid, beta, vs, c, {table, ctab}, acc);
         });
-        const FieldLoad<CELLS> ld(table, st.c, p.m);
+        const FieldLoad<FROM> ld({table, ctab}, st.c, p.m);
 #pragma unroll
         for (int s = 0; s < 8 / LANES; ++s) {
             const int kk = k + s * LANES;
@@ -1438,10 +1434,11 @@ __device__ __forceinline__ double push_eval_shared(const StepParams& p, int k, i
     return (Pn + kick) * p.inv_mass;
 }
 
-template <int QUAD, bool CELLS>
+template <int QUAD, int FROM>
 __global__ void __launch_bounds__(THREADS, LOCAL_MINB) k_local(StepParams p, const double* __restrict__ xi,
                                                    const double* __restrict__ v, const double* __restrict__ P,
                                                    const double* __restrict__ vit, const double* __restrict__ table,
+                                                   const double* __restrict__ ctab,
                                                    double* __restrict__ vnew, double* __restrict__ gsave,
                                                    double* __restrict__ Jnext, const int32_t* __restrict__ creep_list,
                                                    const int* __restrict__ creep_count,
@@ -1619,7 +1616,7 @@ __global__ void __launch_bounds__(THREADS, LOCAL_MINB) k_local(StepParams p, con
         const double vsa = active ? ue + vn : 0.0;
         const double vs[3] = {of(vsa, 0), of(vsa, 1), of(vsa, 2)};
         int nseg = 0;
-        const double vw = push_eval_shared<QUAD, CELLS>(p, k, comp, x0, st, vs, Pn, table, nseg);
+        const double vw = push_eval_shared<QUAD, FROM>(p, k, comp, x0, st, vs, Pn, table, ctab, nseg);
         const double res = vw - ue;                          // g of this lane's component
         const double gp = of(res, paxis < 3 ? paxis : 0);
         const double a0 = max3(sl ? 0.0 : fabs(r0)), a1 = max3(sl ? 0.0 : fabs(res));
@@ -2029,16 +2026,24 @@ StepParams make_params(const Ctx& c) {
     return p;
 }
 
+// Where the closed-form FP64 kernels take the fields from (see Fields).
+static Fields fields_of(const Ctx& c) {
+    if (c.cfg.deterministic) return c.cell_form ? FROM_EITHER : FROM_NODES;
+    return c.ctab ? FROM_CELLS : FROM_NODES;
+}
+
 // Opt the depositing kernels in to their dynamic shared memory (above the 48 KB default where the chunk
 // is large; once per context, on its device).
 bool setup_particle_kernels() {
     const int bytes = (int)ChunkLarge::smem(), push = (int)ChunkPush::smem();
     const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
     return cudaFuncSetAttribute(k_first_scatter_cell<4, 2>, at, bytes) == cudaSuccess &&
-           cudaFuncSetAttribute(k_push_cell<false, true, 4, 2>, at, bytes) == cudaSuccess &&
-           cudaFuncSetAttribute(k_push_cell<false, false, 4, 2>, at, bytes) == cudaSuccess &&
-           cudaFuncSetAttribute(k_push_cell<false, true, 8, 2>, at, push) == cudaSuccess &&
-           cudaFuncSetAttribute(k_push_cell<false, false, 8, 2>, at, push) == cudaSuccess;
+           cudaFuncSetAttribute(k_push_cell<false, FROM_CELLS, 4, 2>, at, bytes) == cudaSuccess &&
+           cudaFuncSetAttribute(k_push_cell<false, FROM_NODES, 4, 2>, at, bytes) == cudaSuccess &&
+           cudaFuncSetAttribute(k_push_cell<false, FROM_EITHER, 4, 2>, at, bytes) == cudaSuccess &&
+           cudaFuncSetAttribute(k_push_cell<false, FROM_CELLS, 8, 2>, at, push) == cudaSuccess &&
+           cudaFuncSetAttribute(k_push_cell<false, FROM_NODES, 8, 2>, at, push) == cudaSuccess &&
+           cudaFuncSetAttribute(k_push_cell<false, FROM_EITHER, 8, 2>, at, push) == cudaSuccess;
 }
 
 // Chunks of one warp while they leave every scheduler at most two of them.
@@ -2116,11 +2121,12 @@ void launch_push(Ctx& c, const double* vit, double* vnew, double* Jnext, bool co
                                                   c.creep_list, c.creep_count, det ? c.creep_flag : nullptr,  \
                                                   c.slide,                                                    \
                                                   c.partials, c.dev_status)
-    const CellFields cf{c.table, reinterpret_cast<const longlong2*>(c.fxtab)};
+    const FixedTables ft{c.table, reinterpret_cast<const longlong2*>(c.fxtab)};
+    const Fields from = fields_of(c);
     const bool small = small_chunks(c), wide = wide_chunks(c);
 #define PIC_PUSH_CELL_AS(C, T, W, I)                                                                              \
     k_push_cell<C, T, W, I><<<chunk_blocks(c), 32 * W, C ? sizeof(ChunkOrder<W, I>) : ChunkOrder<W, I>::smem(),     \
-                              c.stream>>>(p, c.xi, c.v, c.P, vit, cf, vnew, Jnext, c.xi_new, c.P_new, c.creep_list, \
+                              c.stream>>>(p, c.xi, c.v, c.P, vit, ft, vnew, Jnext, c.xi_new, c.P_new, c.creep_list, \
                                           c.creep_count, det ? c.creep_flag : nullptr, c.slide, c.partials,        \
                                           c.dev_status)
 #define PIC_PUSH_CELL(C, T)                \
@@ -2132,19 +2138,23 @@ void launch_push(Ctx& c, const double* vit, double* vnew, double* Jnext, bool co
 #define PIC_COMMIT_DIAG(T, W, I)                                                                                  \
     k_commit_diag<T, W, I><<<chunk_blocks(c), 32 * W, sizeof(ChunkOrder<W, I>), c.stream>>>(                        \
         p, c.xi, c.v, c.P, vit, c.table, c.ctab, vnew, c.xi_new, c.P_new, c.slide, c.partials, c.dev_status)
+#define PIC_COMMIT_DIAG_AS(T)                  \
+    do {                                       \
+        if (small) PIC_COMMIT_DIAG(T, 1, 1);   \
+        else PIC_COMMIT_DIAG(T, 4, 2);         \
+    } while (0)
     if (closed && diag) {   // (commit)
-        if (c.ctab && small) PIC_COMMIT_DIAG(true, 1, 1);
-        else if (c.ctab) PIC_COMMIT_DIAG(true, 4, 2);
-        else if (small) PIC_COMMIT_DIAG(false, 1, 1);
-        else PIC_COMMIT_DIAG(false, 4, 2);
+        if (from == FROM_CELLS) PIC_COMMIT_DIAG_AS(FROM_CELLS);
+        else if (from == FROM_EITHER) PIC_COMMIT_DIAG_AS(FROM_EITHER);
+        else PIC_COMMIT_DIAG_AS(FROM_NODES);
+    } else if (closed && commit) {
+        if (from == FROM_CELLS) PIC_PUSH_CELL(true, FROM_CELLS);
+        else if (from == FROM_EITHER) PIC_PUSH_CELL(true, FROM_EITHER);
+        else PIC_PUSH_CELL(true, FROM_NODES);
     } else if (closed) {
-        if (commit) {
-            if (c.fxtab) PIC_PUSH_CELL(true, true);
-            else PIC_PUSH_CELL(true, false);
-        } else {
-            if (c.fxtab) PIC_PUSH_CELL(false, true);
-            else PIC_PUSH_CELL(false, false);
-        }
+        if (from == FROM_CELLS) PIC_PUSH_CELL(false, FROM_CELLS);
+        else if (from == FROM_EITHER) PIC_PUSH_CELL(false, FROM_EITHER);
+        else PIC_PUSH_CELL(false, FROM_NODES);
     } else if (!commit) {
         PIC_PUSH(false, false);
     } else if (!diag) {
@@ -2153,6 +2163,7 @@ void launch_push(Ctx& c, const double* vit, double* vnew, double* Jnext, bool co
         PIC_PUSH(true, true);
     }
 #undef PIC_COMMIT_DIAG
+#undef PIC_COMMIT_DIAG_AS
 #undef PIC_PUSH
 #undef PIC_PUSH_CELL
 #undef PIC_PUSH_CELL_AS
@@ -2165,13 +2176,15 @@ void launch_local(Ctx& c, const double* vit, double* vnew, double* Jnext) {
     StepParams p = make_params(c);
     const bool det = c.cfg.deterministic != 0;
     const int lb = local_blocks(c);
-#define PIC_LOCAL(Q, T, TAB)                                                                                      \
-    k_local<Q, T><<<lb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.P, vit, TAB, vnew, c.gsave, Jnext, c.creep_list,   \
-                                                c.creep_count, det ? c.creep_flag : nullptr, c.slide,              \
+#define PIC_LOCAL(Q, T)                                                                                             \
+    k_local<Q, T><<<lb, THREADS, 0, c.stream>>>(p, c.xi, c.v, c.P, vit, c.table, c.ctab, vnew, c.gsave, Jnext,        \
+                                                c.creep_list, c.creep_count, det ? c.creep_flag : nullptr, c.slide, \
                                                 c.creep_count + 1, c.partials, c.dev_status)
-    if (!c.closed) PIC_LOCAL(1, false, c.table);
-    else if (c.ctab) PIC_LOCAL(0, true, c.ctab);
-    else PIC_LOCAL(0, false, c.table);
+    const Fields from = fields_of(c);
+    if (!c.closed) PIC_LOCAL(1, FROM_NODES);
+    else if (from == FROM_CELLS) PIC_LOCAL(0, FROM_CELLS);
+    else if (from == FROM_EITHER) PIC_LOCAL(0, FROM_EITHER);
+    else PIC_LOCAL(0, FROM_NODES);
 #undef PIC_LOCAL
     ++c.launches;
     if (det && Jnext) launch_exact_finish(c, Jnext, 3 * c.m.ncell, c.inv_u_J);

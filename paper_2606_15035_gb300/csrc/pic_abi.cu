@@ -541,7 +541,8 @@ pic_status allocate(pic_ctx* ctx) {
         room = 0;
     }
     room = (size_t)(CELL_TABLE_SHARE * (double)room);
-    if (c.closed && c.np >= CELL_TABLE_MIN_PPC * N && cells <= CELL_TABLE_MAX_BYTES && 2 * cells <= room) {
+    c.cell_form = c.closed && c.np >= CELL_TABLE_MIN_PPC * N && cells <= CELL_TABLE_MAX_BYTES;
+    if (c.cell_form && 2 * cells <= room) {
         c.ctab = (double*)dev_alloc_once(ctx, cells);
         if (c.ctab) c.fxtab = (long long*)dev_alloc_once(ctx, cells);
         if (c.ctab && (!c.fxtab || (reinterpret_cast<uintptr_t>(c.ctab) | reinterpret_cast<uintptr_t>(c.fxtab)) % 16 != 0))

@@ -160,6 +160,7 @@ struct Ctx {
     double *cheb_d = nullptr, *rhs0 = nullptr, *rhs = nullptr;
     double *J[3] = {nullptr, nullptr, nullptr};
     double* table = nullptr;             // 12 * ncell gather table
+    bool cell_form = false;              // the rule of the cell tables holds (whether or not they are there)
     double* ctab = nullptr;              // closed forms: CELL_VALUES * ncell cell table (orbit_cell.cuh)
     long long* fxtab = nullptr;          // ... in fixed point (orbit_fixed.cuh; both or neither)
 

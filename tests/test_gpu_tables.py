@@ -121,3 +121,22 @@ def test_tables_go_to_a_context_that_needs_the_memory(sim, monkeypatch, precisio
         for name in ("v", "P", "phi", "A"):
             d = np.linalg.norm(getattr(a, name) - getattr(b, name)) / np.linalg.norm(getattr(b, name))
             assert d <= (1e-11 if precision == 0 else 1e-8), (name, d)
+
+
+@pytest.mark.parametrize("n", [(6, 5, 4), (11, 7, 5)])
+@pytest.mark.parametrize("precision,diagnostics", [(0, 0), (0, 1), (1, 0)])
+def test_deterministic_bits_do_not_depend_on_memory(sim, monkeypatch, n, precision, diagnostics):
+    """The cell tables refused or granted: the same bits."""
+    L, N = (1.2, 1.0, 0.8), int(np.prod(n))
+    x, v, q, m = particles(n, L, 17, 21)
+    out = []
+    for refuse in (False, True):
+        with monkeypatch.context() as mp:
+            Limit(sim, mp, lambda b: refuse and b == TABLES * N)
+            s = sim.PicSim(sim.pic_config_default(n=n, L=L, dt=0.1, deterministic=1, precision=precision,
+                                                  diagnostics=diagnostics), x, v, q, m)
+            s.step(3)
+            out.append(s.get_state())
+            s.close()
+    for name in ("x", "v", "P", "phi", "psi", "rho", "A", "U"):
+        assert np.array_equal(getattr(out[0], name), getattr(out[1], name)), name
