@@ -91,9 +91,9 @@ typedef struct {
                                      helmholtz_tol times the solution's norm, from the warm start's
                                      residual (at most the schedule that reduces any start by it).
                                      On a mesh whose sizes are all <= 1024 with no prime factor
-                                     above 127 the central2 solve is by FFT instead, to this
-                                     accuracy or better (to roundoff where all are 2^p 3^q, where
-                                     this does not apply) */
+                                     above 127 the central2 solve is by FFT instead, where that is
+                                     cheaper, to this accuracy or better (to roundoff, and always,
+                                     where all are 2^p 3^q, where this does not apply) */
     double mixed_tol32;           /* PIC_MIXED: leave the FP32 iterations once e_v <= this */
     int32_t mixed_max32;          /* PIC_MIXED: at most this many FP32 iterations per step */
     int32_t deterministic;        /* 1: bitwise reproducible steps.  The particle sort is a stable

@@ -173,13 +173,17 @@ extern "C" pic_status pic_cn_update_static(const int32_t n[3], const double L[3]
     Fields4 src = {{rho_half, J, J + N, J + 2 * N}};
     const double c_rho = 0.5 * dt * dt * kappa * kappa * sigma1;
     const double c_J = 0.5 * dt * dt * kappa * kappa * sigma2;
-    // By transforms where they take the mesh and are cheaper than the Chebyshev steps: a correction
-    // (five launches) costs about five steps, 23 against 4.6 us at 32^3.  The whole call at 32^3 with
-    // helmholtz_tol = 1e-17: 326 us by 30 steps (8.2 us each with 64-bit index divisions), 122 by transforms.
+    // By transforms where they take the mesh and are cheaper than the Chebyshev steps, which take 4 us each up to
+    // 5,000 nodes and 10.5 at 32,768: the whole call at 32^3 with helmholtz_tol = 1e-17, lmax 3, steps | transforms
+    // 346 | 107 us, 31^3 344 | 170; at lmax 1.05 131 | 107 and 129 | 170; (8, 61, 61) 343 | 396, 8^3 at lmax 1.05 53 | 62.
     bool fft = true;
     for (int ax = 0; ax < 3; ++ax) fft = fft && pic::helm32_factor(n[ax]);
     const int corrections = fft ? pic::helm32_corrections(lmax, std::fmax(helmholtz_tol, 1e-16)) : 0;
-    fft = corrections > 0 && iters > 5 * corrections && pic::setup_helm_kernels();
+    pic::MeshDims dims;
+    for (int ax = 0; ax < 3; ++ax) dims.n[ax] = n[ax];
+    dims.ncell = N;
+    const double step = std::fmax(4.0, 2.7 + (double)N / 4150.0);
+    fft = corrections > 0 && 10.0 + corrections * pic::helm32_micros(dims, sms) < iters * step && pic::setup_helm_kernels();
     // the transforms' buffers: z in place of the second iterate, the tables and exponents in the
     // directions' place
     float2* tw = fft ? reinterpret_cast<float2*>(dir) : nullptr;
@@ -191,11 +195,8 @@ extern "C" pic_status pic_cn_update_static(const int32_t n[3], const double L[3]
     double* x = xa;
     if (fft) {
         pic::HelmPlan plan;
-        plan.m.ncell = N;
-        for (int ax = 0; ax < 3; ++ax) {
-            plan.m.n[ax] = n[ax];
-            plan.invH[ax] = d.invH[ax];
-        }
+        plan.m = dims;
+        for (int ax = 0; ax < 3; ++ax) plan.invH[ax] = d.invH[ax];
         plan.a = a;
         plan.sms = sms;
         plan.z = reinterpret_cast<float2*>(xb);

@@ -361,6 +361,40 @@ int helm32_corrections(double lmax, double to) {
     return k > HELM_MAX_CORRECTIONS ? 0 : std::max(1, (int)k);
 }
 
+namespace {
+
+// Adjacent x of a block of k_helm_plane, fewer while the blocks do not fill the SMs, and its threads.
+int plane_lines(const MeshDims& m, int sms) {
+    const int64_t plane = (int64_t)m.n[1] * m.n[2];
+    int lb = 4;
+    while (lb > 1 && (lb * plane > PLANE || 2 * ((m.n[0] + lb - 1) / lb) < sms / 2)) lb /= 2;
+    return lb;
+}
+int plane_threads(int64_t elements) { return (int)std::max<int64_t>(64, std::min<int64_t>(512, (elements / 4 + 31) / 32 * 32)); }
+
+}  // namespace
+
+// Measured on 18 meshes up to 430,784 nodes (8^3 to 127 x 64 x 53, primes to 127 on each axis, sizes to 1024): 17
+// us and a share of the nodes, two launches more where y and z go apart, and 0.05 us for each product that
+// a thread sums in the stages of larger primes.  Between -10% and +30% of the times.
+double helm32_micros(const MeshDims& m, int sms) {
+    HelmPlan c{};
+    c.m = m;
+    c.sms = sms;
+    const Axis32 ax[3] = {make_axis32(c, 0), make_axis32(c, 1), make_axis32(c, 2)};
+    const int64_t plane = (int64_t)m.n[1] * m.n[2];
+    const bool fused = plane <= PLANE;
+    double products = 0.0;
+    for (int a = 0; a < 3; ++a) {
+        const bool in_plane = fused && a > 0;
+        const int64_t elements = in_plane ? plane_lines(m, sms) * plane : (int64_t)ax[a].lb * ax[a].n;
+        const int threads = in_plane ? plane_threads(elements) : 256;
+        for (int s = 0; s < ax[a].nst; ++s)
+            if (ax[a].st[s].R > 4) products += 2.0 * (double)((elements + threads - 1) / threads) * ax[a].st[s].R;
+    }
+    return 17.5 + (double)m.ncell / 2400.0 + 0.05 * products + (fused ? 0.0 : 8.0);
+}
+
 int helm32_solve(const HelmPlan& c, const double* b, double* x, const int* top, int corrections, cudaStream_t stream) {
     Helm32 h;
     h.m = c.m;
@@ -379,18 +413,15 @@ int helm32_solve(const HelmPlan& c, const double* b, double* x, const int* top, 
     const dim3 gx = grid((c.m.ncell / ax.n + ax.lb - 1) / ax.lb);
     const dim3 gy = grid((int64_t)((c.m.n[0] + ay.lb - 1) / ay.lb) * c.m.n[2]);
     const dim3 gz = grid(((int64_t)c.m.n[0] * c.m.n[1] + az.lb - 1) / az.lb);
-    // one launch for y and z where a plane fits (PLANE elements): lb adjacent x a block, fewer while the
-    // blocks do not fill the SMs
+    // one launch for y and z where a plane fits (PLANE elements): lb adjacent x a block
     const int64_t plane = (int64_t)ay.n * az.n;
     const bool fused = plane <= PLANE;
-    int lb = 4;
-    while (lb > 1 && (lb * plane > PLANE || 2 * ((c.m.n[0] + lb - 1) / lb) < c.sms / 2)) lb /= 2;
+    const int lb = plane_lines(c.m, c.sms);
     for (int k = 0; k < corrections; ++k) {
         h.up = 20 * k;   // each correction leaves a residual some 2^20 smaller
         k_helm_x<false><<<gx, 256, smem(ax), stream>>>(h, ax);
         if (fused) {
-            const int threads = (int)std::max<int64_t>(64, std::min<int64_t>(512, (lb * plane / 4 + 31) / 32 * 32));
-            k_helm_plane<<<dim3((c.m.n[0] + lb - 1) / lb, 2), threads, 2 * sizeof(float2) * lb * plane, stream>>>(h, ay, az, lb);
+            k_helm_plane<<<dim3((c.m.n[0] + lb - 1) / lb, 2), plane_threads(lb * plane), 2 * sizeof(float2) * lb * plane, stream>>>(h, ay, az, lb);
             k_helm_x<true><<<gx, 256, smem(ax), stream>>>(h, ax);
             continue;
         }

@@ -467,8 +467,10 @@ pic_status allocate(pic_ctx* ctx) {
         c.inv_u_rho = inv_u(wq);
     }
     // central differences: the CN Helmholtz solves by FP32 transforms where they take the mesh, to roundoff
-    // on 2^p 3^q meshes (else by FP64 transforms) and to helmholtz_tol on others (else by Chebyshev steps:
-    // a mesh phase's solves took 520 us at (37, 41, 43), now 208; 1966 and 429 at 62^3, 28.6 and 8.6 ms at 127^3)
+    // on 2^p 3^q meshes (else by FP64 transforms) and to helmholtz_tol on others, where they are cheaper than the
+    // Chebyshev steps (a mesh phase at dt = 0.1, steps | transforms: (37, 41, 43) 520 | 208 us, 62^3 1176 | 515,
+    // 61^3 1064 | 689; where a plane of large primes keeps few blocks busy it is the other way round: (8, 61, 61)
+    // 330 | 392 us, (1, 61, 61) 119 | 366, and more so at small steps: (61, 61, 61) at dt = 0.02 461 | 689).
     if (c.cfg.ops == PIC_OPS_CENTRAL2) {
         bool ok = true, ok32 = true;
         for (int a = 0; a < 3; ++a) {
@@ -480,6 +482,10 @@ pic_status allocate(pic_ctx* ctx) {
         if (ok32) {
             c.helm_corrections = helm32_corrections(c.cheb_lmax, ok ? 1e-16 : std::max(c.cfg.helmholtz_tol, 1e-16));
             c.helm_corrections32 = ok ? c.helm_corrections : helm32_corrections(c.cheb_lmax, MESH_TOL32);
+            // a phase takes 15 us beside its corrections, 47 beside its Chebyshev steps of 2.4 us and the nodes' share
+            const double nodes = (double)N, step = 2.4 + std::min(nodes / 5000.0, 3.0 + nodes / 8000.0);
+            if (!ok && 15.0 + c.helm_corrections * helm32_micros(c.m, c.sms) > 47.0 + c.cheb_iters * step)
+                c.helm_corrections = c.helm_corrections32 = 0;
         }
     }
     if (c.helm_fft && c.helm_corrections == 0) {

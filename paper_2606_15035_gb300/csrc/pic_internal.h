@@ -332,7 +332,8 @@ constexpr int HELM_MAX_CORRECTIONS = 8;
 // longest: no less than 5e-7 is counted on.
 int helm32_corrections(double lmax, double to);
 // Largest prime factor of an axis (its stage costs that many products a point): at 127^3 the transforms
-// still take a third of the Chebyshev steps' time.
+// still take a third of the Chebyshev steps' time.  Estimate of a correction's time in us, for the choice between the two.
+double helm32_micros(const MeshDims& m, int sms);
 constexpr int HELM_MAX_RADIX = 127;
 bool helm32_factor(int n);   // whether the FP32 transforms take n: at most FFT_MAX, primes to HELM_MAX_RADIX
 bool setup_helm_kernels();   // their shared memory, on the current device

@@ -41,3 +41,29 @@ def test_loose_tolerances_are_met(sim, n, L, tol):
                            opic.Config(n=n, L=L, dt=dt).grid())
     for g, w in ((got["phi"], want[0]), *zip(got["A"], want[2])):
         assert np.linalg.norm(g - w) <= (tol + 1e-15) * np.linalg.norm(w)
+
+
+@pytest.mark.parametrize("n,dt,transforms", [((1, 61, 61), 0.02, False), ((8, 61, 61), 0.1, False), ((1, 61, 61), 1.0, True),
+                                             ((50, 35, 22), 0.1, True), ((62, 62, 62), 0.1, True)])
+def test_solver_by_its_cost(sim, n, dt, transforms):
+    """Transforms where they are the cheaper solve, Chebyshev steps (one launch) where not, by the launches of
+    one body; the fields are the exact update's either way."""
+    rng = np.random.default_rng(9)
+    L = tuple(0.0654 * k for k in n)
+    x = rng.uniform(0, 1, size=(8, 3)) * L
+    v = 1e-3 * rng.normal(size=x.shape)
+    launches = []
+    for size in (n, (131, 2, 2)):                             # 131: never by transforms
+        s = sim.PicSim(sim.pic_config_default(n=size, L=tuple(0.0654 * k for k in size), dt=dt), np.mod(x, 0.13), v, -1e-5, 1e-5)
+        st = s.get_state()
+        st.psi = rng.normal(size=st.psi.shape)
+        s.set_state(st)
+        s.profile(True)
+        got = s.iterate(v)
+        launches.append(s.profile(False).launches)
+        s.close()
+        if size == n:
+            want = omesh.cn_fields(st.phi, st.psi, st.A, st.U, 0.5 * (got["rho"] + st.rho), got["J"], dt, 1.0, 1.0, 1.0,
+                                   opic.Config(n=n, L=L, dt=dt).grid())[0]
+            assert np.linalg.norm(got["phi"] - want) <= 1e-12 * np.linalg.norm(want)
+    assert (launches[0] > launches[1]) == transforms, launches
