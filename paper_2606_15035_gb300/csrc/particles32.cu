@@ -431,8 +431,11 @@ __global__ void k_to32(Params32 p, const double* __restrict__ xi, const double* 
         cell_start(x0, p.m, st);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            off[a * p.stride + i] = to_float(st.f[a]);
-            packed |= (st.c[a] & CELL_MASK) << (a * CELL_BITS);
+            // (an offset that rounds to one is the start of the next cell, which a resting orbit's box holds)
+            const float f = to_float(st.f[a]);
+            const int c = f == 1.f ? next_cell(st.c[a], p.m.n[a]) : st.c[a];
+            off[a * p.stride + i] = f == 1.f ? 0.f : f;
+            packed |= (c & CELL_MASK) << (a * CELL_BITS);
             v32[a * p.stride + i] = to_float(vn[a]);
             vit32[a * p.stride + i] = to_float(vn[a] - vprev[a * np + i]);   // (2 v^n - v^{n-1}) - v^n
         }
