@@ -248,6 +248,7 @@ class PicSim:
         self.ncell = self.n[0] * self.n[1] * self.n[2]
         self.np = int(np.shape(x)[0])
         self._owned = True
+        self._stream = (stream if stream is not None else _torch().cuda.current_stream()).cuda_stream
         self.ctx, self._alloc, self._keep = pic_init(cfg, x, v, q, m, stream)
 
     @classmethod
@@ -260,6 +261,7 @@ class PicSim:
         self.np = int(npart)
         self._owned = False
         self._owner = owner
+        self._stream = None   # (the ensemble's own)
         self.ctx = C.c_void_p(ctx)
         return self
 
@@ -330,7 +332,16 @@ class PicSim:
         sizes = {"x": 3 * self.np, "v": 3 * self.np, "P": 3 * self.np, "vprev": 3 * self.np, "phi": self.ncell,
                  "psi": self.ncell, "rho": self.ncell, "A": 3 * self.ncell, "U": 3 * self.ncell}
         torch = _torch()
-        return {k: (make if n else torch.zeros)(max(n, 1), dtype=torch.float64, device="cuda") for k, n in sizes.items()}
+        d = {k: (make if n else torch.zeros)(max(n, 1), dtype=torch.float64, device="cuda") for k, n in sizes.items()}
+        self._settle()
+        return d
+
+    def _settle(self):
+        """Before the library writes tensors just made: their memory may be a former tensor's that torch's
+        stream still uses, and it may still be clearing them, while the library writes on its own stream."""
+        now = _torch().cuda.current_stream()
+        if now.cuda_stream != self._stream:
+            now.synchronize()
 
     def state_zeros(self):
         """A dict of zero float64 CUDA tensors in the state layout: particles SoA (3 np),
@@ -353,6 +364,7 @@ class PicSim:
         that restore() brings the run back bit for bit (pic_set_positions)."""
         d = self.get_state_device()
         xi = _torch().zeros(max(3 * self.np, 1), dtype=_torch().float64, device="cuda")
+        self._settle()
         _check(_lib.lib().pic_get_positions(self.ctx, C.c_void_p(xi.data_ptr()), 1), self.ctx)
         d["xi"] = xi
         return d
@@ -381,6 +393,7 @@ class PicSim:
         torch = _torch()
         lx = torch.zeros(max(3 * self.np, 1), dtype=torch.float64, device="cuda")
         lv = torch.zeros_like(lx)
+        self._settle()
         _check(_lib.lib().pic_init_vjp(self.ctx, C.byref(self._dview(lam0)), lx.data_ptr(), lv.data_ptr(), 1),
                self.ctx)
         return lx, lv
