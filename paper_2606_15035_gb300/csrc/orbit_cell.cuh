@@ -335,7 +335,8 @@ __device__ __forceinline__ void cell_nodes8(const int c[3], const MeshDims& m, i
 // differences of the cell's nodes each time (contexts without cell tables); or, in deterministic mode, the cell
 // table where there is one and the gather table where not, by the same instructions but for the loads.  The
 // differences are the same numbers (subtractions in the same order), so that the bits do not depend on
-// whether the table's memory was there.
+// whether the table's memory was there.  24^3, 442,368 particles: 4.4 ms a step with the table, 9.6 without
+// (15.0 when each entry was made at its use); the loads through a generic pointer cost 7% beside FROM_CELLS.
 enum Fields { FROM_NODES, FROM_CELLS, FROM_EITHER };
 
 struct FieldTables {
@@ -390,33 +391,35 @@ struct FieldLoad<FROM_NODES> {
     }
 };
 
-// One pair of entries from the gather table (a function of its own: FROM_EITHER's rare side).
-static __device__ __noinline__ double2 entries_of_nodes(const double* nodes, int c0, int c1, int c2, int n0, int n1, int n2,
-                                                        int p, int col) {
+// A cell's entries from the gather table (a function of its own: FROM_EITHER's rare side).
+static __device__ __noinline__ void entries_of_nodes(const double* nodes, int c0, int c1, int c2, int n0, int n1, int n2,
+                                                     double2* out) {
     MeshDims m;
     m.n[0] = n0;
     m.n[1] = n1;
     m.n[2] = n2;
     const int c[3] = {c0, c1, c2};
-    double2 q;
-    FieldLoad<FROM_NODES>({nodes, nullptr}, c, m)(p, col, q.x, q.y);
-    return q;
+    const FieldLoad<FROM_NODES> ld({nodes, nullptr}, c, m);
+    for (int col = 0; col < CELL_COLS; ++col)
+#pragma unroll
+        for (int p = 0; p < 4; ++p) ld(p, col, out[p * CELL_COLS + col].x, out[p * CELL_COLS + col].y);
 }
 
 template <>
 struct FieldLoad<FROM_EITHER> {
-    FieldTables ft;
-    const MeshDims& m;
-    const double2* t;   // the cell's entries, or null
-    int c[3];
-    __device__ __forceinline__ FieldLoad(FieldTables tables, const int cell[3], const MeshDims& dims)
-        : ft(tables), m(dims), c{cell[0], cell[1], cell[2]} {
-        t = ft.cells ? reinterpret_cast<const double2*>(ft.cells + CELL_VALUES * cell_row(c, m)) : nullptr;
+    const double2* t;                     // the table's entries, or own
+    double2 own[CELL_VALUES / 2];         // (local memory, untouched where there is a table)
+    __device__ __forceinline__ FieldLoad(FieldTables ft, const int c[3], const MeshDims& m) {
+        if (__builtin_expect(ft.cells != nullptr, 1)) {
+            t = reinterpret_cast<const double2*>(ft.cells + CELL_VALUES * cell_row(c, m));
+        } else {
+            entries_of_nodes(ft.nodes, c[0], c[1], c[2], m.n[0], m.n[1], m.n[2], own);
+            t = own;
+        }
     }
+    FieldLoad(const FieldLoad&) = delete;
     __device__ __forceinline__ void operator()(int p, int col, double& a, double& b) const {
-        double2 q;
-        if (__builtin_expect(t != nullptr, 1)) q = __ldg(t + p * CELL_COLS + col);
-        else q = entries_of_nodes(ft.nodes, c[0], c[1], c[2], m.n[0], m.n[1], m.n[2], p, col);
+        const double2 q = t[p * CELL_COLS + col];
         a = q.x;
         b = q.y;
     }

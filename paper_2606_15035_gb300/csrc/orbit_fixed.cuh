@@ -48,50 +48,45 @@ struct FixedLoad<FROM_CELLS> {
     __device__ __forceinline__ int top_g() const { return (int)__ldg(&t[1].x); }
 };
 
-// The largest exponents (at least 64) of a cell's groups, the differences of the A columns and -grad phi,
-// from the gather table.
-static __device__ __noinline__ int2 tops_of_nodes(const double* nodes, int c0, int c1, int c2, int n0, int n1, int n2) {
-    int2 top = make_int2(64, 64);
-    for (int p = 0; p < 4; ++p)
-        for (int col = 0; col < CELL_COLS; ++col) {
-            const double2 q = entries_of_nodes(nodes, c0, c1, c2, n0, n1, n2, p, col);
-            const int e = max(p == 0 && col < 6 ? 0 : exponent_of(q.x), exponent_of(q.y));
-            if (col < 6) top.x = max(top.x, e);
-            else top.y = max(top.y, e);
-        }
-    return top;
+// A cell's entries as its fixed-point table has them, from the gather table.
+static __device__ __noinline__ void fixed_of_nodes(const double* nodes, int c0, int c1, int c2, int n0, int n1, int n2,
+                                                   longlong2* out) {
+    double2 q[CELL_VALUES / 2];
+    entries_of_nodes(nodes, c0, c1, c2, n0, n1, n2, q);
+    int top[2] = {64, 64};
+    for (int k = 0; k < CELL_VALUES / 2; ++k) {
+        const int col = k % CELL_COLS;
+        const int e = max(k < 6 ? 0 : exponent_of(q[k].x), exponent_of(q[k].y));
+        if (col < 6) top[0] = max(top[0], e);
+        else top[1] = max(top[1], e);
+    }
+    for (int k = 0; k < CELL_VALUES / 2; ++k) {
+        const int e = k % CELL_COLS < 6 ? top[0] : top[1];
+        out[k].x = k < 2 ? top[k] : (k < 6 ? 0 : fixed_of(q[k].x, e, FX_FIELD_UP));
+        out[k].y = fixed_of(q[k].y, e, FX_FIELD_UP);
+    }
 }
 
 template <>
 struct FixedLoad<FROM_EITHER> {
-    FixedTables ft;
-    const MeshDims& m;
-    const longlong2* t;   // the cell's entries, or null
-    int c[3];
-    int2 top;
-    __device__ __forceinline__ FixedLoad(FixedTables tables, const int cell[3], const MeshDims& dims)
-        : ft(tables), m(dims), t(nullptr), c{cell[0], cell[1], cell[2]} {
+    const longlong2* t;                   // the table's entries, or own
+    longlong2 own[CELL_VALUES / 2];
+    __device__ __forceinline__ FixedLoad(FixedTables ft, const int c[3], const MeshDims& m) {
         if (__builtin_expect(ft.cells != nullptr, 1)) {
             t = ft.cells + (CELL_VALUES / 2) * cell_row(c, m);
-            top = make_int2((int)__ldg(&t[0].x), (int)__ldg(&t[1].x));
         } else {
-            top = tops_of_nodes(ft.nodes, c[0], c[1], c[2], m.n[0], m.n[1], m.n[2]);
+            fixed_of_nodes(ft.nodes, c[0], c[1], c[2], m.n[0], m.n[1], m.n[2], own);
+            t = own;
         }
     }
+    FixedLoad(const FixedLoad&) = delete;
     __device__ __forceinline__ void operator()(int p, int col, long long& a, long long& b) const {
-        if (__builtin_expect(t != nullptr, 1)) {
-            const longlong2 q = __ldg(t + p * CELL_COLS + col);
-            a = q.x;
-            b = q.y;
-        } else {
-            const double2 q = entries_of_nodes(ft.nodes, c[0], c[1], c[2], m.n[0], m.n[1], m.n[2], p, col);
-            const int e = col < 6 ? top.x : top.y;
-            a = fixed_of(q.x, e, FX_FIELD_UP);
-            b = fixed_of(q.y, e, FX_FIELD_UP);
-        }
+        const longlong2 q = t[p * CELL_COLS + col];
+        a = q.x;
+        b = q.y;
     }
-    __device__ __forceinline__ int top_A() const { return top.x; }
-    __device__ __forceinline__ int top_g() const { return top.y; }
+    __device__ __forceinline__ int top_A() const { return (int)t[0].x; }
+    __device__ __forceinline__ int top_g() const { return (int)t[1].x; }
 };
 
 // The unit 2^e' of a sum, e' = e - 1023, of quantities whose largest biased exponent is `top`: NaN where that
