@@ -51,18 +51,18 @@ CPU_STEPS = 10            # timed oracle steps of the cpu_baseline leg
 
 # FP64 operations (add, mul, division = 1, FMA = 2) left on the FP64 pipe in the fused push +
 # next-orbit scatter kernel, counted from its source: per particle hand-over, displacement, end
-# point, momentum and velocity update and residual; per push piece the walk (12, and 5 a crossing);
-# per scatter piece the walk and weights (26) and the next orbit's setup (34).  The pieces'
-# moments, contractions and deposits, some 290 a piece, run in 64-bit fixed point on the integer pipe
-# and are not counted.
-FLOPS_PER_PARTICLE = 73
-FLOPS_PER_PUSH_PIECE = 17
+# point, momentum and velocity update and residual; per push piece the walk (12, and 5 a crossing)
+# and the sums of its integrals (12); per scatter piece the walk and weights (26) and the next orbit's
+# setup (34).  The pieces' moments, contractions and deposits, some 290 a piece, run in 64-bit fixed
+# point on the integer pipe and are not counted.
+FLOPS_PER_PARTICLE = 70
+FLOPS_PER_PUSH_PIECE = 29
 FLOPS_PER_SCATTER_PIECE = 60
 # The survey's lower estimate of the same work (its per-orbit count split into a per-particle part
 # and a per-piece part: weights 110, grad phi 24, A^(m) and C 72, contraction 48, transverse 72,
 # D sum 48 and scatter 24 per piece; point gather 36, push and orbit 30, next-orbit weights 20 per
-# particle), reported beside the source count.  Its fraction of the FP64 peak passes 1: most of that
-# work is off the FP64 pipe.
+# particle), reported beside the source count as a rate of work (not a fraction of the FP64 peak: most of
+# that work is off the FP64 pipe).
 MIN_FLOPS_PER_PARTICLE = 86
 MIN_FLOPS_PER_PIECE = 398
 # Bytes per particle-iteration of the FP32 push (read cell 4, offset 12, v^n 12, increment 12;
@@ -70,14 +70,14 @@ MIN_FLOPS_PER_PIECE = 398
 BYTES32_PER_PARTICLE = 52
 # DRAM bytes (read + write) per launch from one ncu capture of the kernel version in the tree,
 # keyed by kernel and workload, with how the figure was obtained (absent: not captured for this
-# version).  The 128^3 run is too large for a multi-pass capture, so its k_push figure is the
+# version).  The 128^3 run is too large for a multi-pass capture, so its k_push_cell figure is the
 # 32^3 capture (2,097,152 particles, third Picard iteration) scaled by the particle count: the
-# kernel's traffic is its particle streams, 163 B per particle-iteration there.
+# kernel's traffic is its particle streams, 176 B per particle-iteration there.
 NCU_TRAFFIC = {
-    ("k_push", "twostream-32c-2M"): (342.53e6, "ncu capture, one launch (dram read 278.20 MB + write 64.33 MB)"),
-    ("k_push", "twostream-128c-134M"): (342.53e6 * 64, "the 32^3 capture scaled by particles (x 64)"),
-    ("k_push32", "twostream-32c-2M"): (96.59e6, "ncu capture, one launch (dram read 86.46 MB + write 10.13 MB)"),
-    ("k_push32", "twostream-128c-134M"): (96.59e6 * 64, "the 32^3 capture scaled by particles (x 64)"),
+    ("k_push_cell", "twostream-32c-2M"): (369.95e6, "ncu capture, one launch (dram read 277.52 MB + write 92.43 MB)"),
+    ("k_push_cell", "twostream-128c-134M"): (369.95e6 * 64, "the 32^3 capture scaled by particles (x 64)"),
+    ("k_push32", "twostream-32c-2M"): (96.48e6, "ncu capture, one launch (dram read 86.53 MB + write 9.95 MB)"),
+    ("k_push32", "twostream-128c-134M"): (96.48e6 * 64, "the 32^3 capture scaled by particles (x 64)"),
 }
 
 
@@ -394,7 +394,7 @@ def run_ensemble(args, world, rank, local):
                    "l2": "inputs larger than L2"},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                      "frac": achieved / FP64_PEAK_TFLOPS if achieved else None, "traffic": None,
-                     "kernel": "k_push (all runs; algorithmic flops over the summed k_push event durations)",
+                     "kernel": "k_push_cell (all runs; algorithmic flops over the summed event durations of the pushes)",
                      "peak_note": "derived: 152 SMs x 4 flop/clk x 2070 MHz"},
         "sequential": {"value": total / t_seq, "unit": UNIT,
                        "what": "the same runs, one pic_step each, one after another"},
@@ -433,7 +433,7 @@ def mean_pieces(prof, npart):
 
 
 def fp64_push_roofline(prof, workload):
-    """k_push (FP64 push + next-orbit scatter) against the FP64 ALU peak."""
+    """k_push_cell (FP64 push + next-orbit scatter) against the FP64 ALU peak."""
     pushes = prof.particle_pushes
     if not prof.push_launches or prof.push_ms <= 0:
         return None
@@ -447,15 +447,15 @@ def fp64_push_roofline(prof, workload):
     achieved_min = min_flops / (prof.push_ms / 1e3) / 1e12
     return {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
             "frac": achieved / FP64_PEAK_TFLOPS,
-            "flops_basis": "FP64 pipe only, from the kernel source (add, mul = 1, FMA = 2): 73 per particle + 17 per push "
+            "flops_basis": "FP64 pipe only, from the kernel source (add, mul = 1, FMA = 2): 70 per particle + 29 per push "
                            "piece + 60 per scatter piece; the pieces' contractions and deposits run on the integer pipe",
-            "frac_survey_minimum": achieved_min / FP64_PEAK_TFLOPS,
-            "survey_minimum_basis": "86 per particle + 398 per orbit piece (the survey's per-orbit estimate), over the FP64 "
-                                    "peak; above 1 where that work runs on the integer pipe",
-            "traffic": NCU_TRAFFIC.get(("k_push", workload), (None, None))[0],
+            "survey_work_tflops": achieved_min,
+            "survey_work_basis": "rate of the survey's per-orbit estimate of the work, 86 per particle + 398 per orbit "
+                                 "piece, most of which runs on the integer pipe: no fraction of the FP64 peak",
+            "traffic": NCU_TRAFFIC.get(("k_push_cell", workload), (None, None))[0],
             "traffic_unit": "DRAM bytes per launch (ncu dram read + write)",
-            "traffic_source": NCU_TRAFFIC.get(("k_push", workload), (None, "not captured"))[1],
-            "kernel": "k_push (fused FP64 orbit push + next-orbit current scatter, Picard iterations)",
+            "traffic_source": NCU_TRAFFIC.get(("k_push_cell", workload), (None, "not captured"))[1],
+            "kernel": "k_push_cell (k_push with Gauss rules): fused FP64 orbit push + next-orbit current scatter, Picard iterations",
             "peak_note": "FP64 ALU, of derived: 152 SMs x 4 flop/clk x 2070 MHz (the live probe is in fma_probe)",
             "launches": int(prof.push_launches), "ms_per_launch": prof.push_ms / prof.push_launches,
             "flops_per_launch": flops / prof.push_launches,
@@ -463,7 +463,7 @@ def fp64_push_roofline(prof, workload):
 
 
 def final_sweep_roofline(prof, workload, npart):
-    """The FP64 final sweep (k_push, commit: the push of the accepted orbit, no scatter) against
+    """The FP64 final sweep (k_push_cell, commit: the push of the accepted orbit, no scatter) against
     the FP64 ALU peak.  Its orbit is the one the last iteration scattered, so its pieces per
     particle are taken as the iterations' scatter pieces per particle."""
     if not prof.commit_launches or prof.commit_ms <= 0:
@@ -474,14 +474,14 @@ def final_sweep_roofline(prof, workload, npart):
     min_flops = prof.commit_launches * npart * (MIN_FLOPS_PER_PARTICLE + MIN_FLOPS_PER_PIECE * msc)
     return {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
             "frac": achieved / FP64_PEAK_TFLOPS,
-            "flops_basis": "FP64 pipe only, from the kernel source (add, mul = 1, FMA = 2): 73 per particle + 17 per push "
+            "flops_basis": "FP64 pipe only, from the kernel source (add, mul = 1, FMA = 2): 70 per particle + 29 per push "
                            "piece (no scatter in the final sweep); the contractions run on the integer pipe",
-            "frac_survey_minimum": min_flops / (prof.commit_ms / 1e3) / 1e12 / FP64_PEAK_TFLOPS,
-            "survey_minimum_basis": "86 per particle + 398 per orbit piece (the survey's per-orbit estimate), over the FP64 "
-                                    "peak; above 1 where that work runs on the integer pipe",
+            "survey_work_tflops": min_flops / (prof.commit_ms / 1e3) / 1e12,
+            "survey_work_basis": "rate of the survey's per-orbit estimate of the work, 86 per particle + 398 per orbit "
+                                 "piece, most of which runs on the integer pipe: no fraction of the FP64 peak",
             "traffic": None, "traffic_unit": "DRAM bytes per launch (ncu dram read + write)",
             "traffic_source": "not captured for the commit variant",
-            "kernel": "k_push (FP64 final sweep: push of the accepted orbit, commit, residual sums)",
+            "kernel": "k_push_cell (k_push with Gauss rules), FP64 final sweep: push of the accepted orbit, commit, residual sums",
             "peak_note": "FP64 ALU, of derived: 152 SMs x 4 flop/clk x 2070 MHz (the live probe is in fma_probe)",
             "launches": int(prof.commit_launches), "ms_per_launch": prof.commit_ms / prof.commit_launches,
             "flops_per_launch": flops / prof.commit_launches, "mean_orbit_pieces": msc}

@@ -205,7 +205,7 @@ __device__ __forceinline__ void out_adjoints(const StepParams& p, bool sl, doubl
 // and more, which bounded the kernel (0.80 ms at 32^3 with 524,288 particles).  As in scatter_warp the
 // warp's particles are summed per cell first, in 64-bit fixed point (each component's values to 2^-57 of the
 // largest product that the warp adds to the cell), three tiles a piece, and turned into node values once
-// per cell: 0.43 ms.
+// per cell: 0.43 ms, 0.46 with the units by cell (one a warp lost the bits of small cotangents beside large ones).
 __device__ __forceinline__ void plain_rows(double* __restrict__ col, const int c[3], const MeshDims& m, const double M[8],
                                            const double w[3]) {
     double W[8];

@@ -783,7 +783,9 @@ __global__ void __launch_bounds__(32 * WARPS, SCATTER_WARPS / WARPS) k_first_sca
 // differences (25.6M); 1.43 with the fixed-point deposit; 1.22 and 0.77 with the fixed-point pieces
 // (11.4M and 9.0M, the pipe 52% and 62% busy); 1.13 and 0.73 with chunks whose warps have equal work and
 // sums of products shifted once; 1.03 and 0.68 with the one-crossing walk (10.3M and 7.5M); 0.96 and 0.65 with
-// eight warps a block (chunk.cuh).  At 128^3 with 134M particles the final sweep took 225, 102, 64, now 54 ms.
+// eight warps a block (chunk.cuh); 1.00 and 0.66 (10.7M and 7.7M) with each cell's own exponents and units, which
+// keep the bits of fields and particles far smaller than others elsewhere.  At 128^3 with 134M particles the final
+// sweep took 225, 102, 64, 54, now 56 ms.
 // What is left is latency (36% issue-active): fixed-latency waits, shared memory, the instruction cache.
 template <bool COMMIT, int FROM, int WARPS, int ITEMS>
 __global__ void __launch_bounds__(32 * WARPS, PUSH_WARPS / WARPS) k_push_cell(StepParams p, const double* __restrict__ xi,

@@ -90,7 +90,8 @@ __device__ __forceinline__ int64_t subset_node(const int c0[3], int k, const Mes
 
 // Measured at 32^3 with 2,097,152 particles (1.31 pieces each): the first scatter 0.82 -> 0.49 ms with
 // 4.5M L2 reduction requests where there were 67M; at 128^3 with 134M (2.2 pieces) 96 -> 44 ms;
-// 0.35 and 29.8 ms now, with balanced chunks, the one-crossing walk and columns by cell.
+// 0.34 and 29.8 ms with balanced chunks, the one-crossing walk and columns by cell, 0.35 and 31.5 with each
+// cell's own unit (one a warp lost what separates slow particles from fast ones in other cells).
 // In the push it takes 46 FP64 instructions a piece off the pipe that bounds it (1.59 -> 1.43 ms).
 //
 // Add the orbit currents q v_bar S_bar / dV (weights w, orbits st.f + s beta) of the lanes with `act`

@@ -187,7 +187,8 @@ __global__ void k_spec_cn(SpecParams p, const double2* __restrict__ Jh, const do
         mode_k(p, g, k);
         const double lam = -(k[0] * k[0] + k[1] * k[1] + k[2] * k[2]);
         const double b = hdt * p.kappa2 * lam, det = 1.0 - hdt * b, inv = 1.0 / det;
-        // x / det by the reciprocal and one correction from the exact remainder (16 divisions bound the kernel)
+        // x / det by Markstein's method: the quotient by the reciprocal, and one correction from the exact
+        // remainder (16 divisions bound the kernel)
         auto over = [&](double x) {
             const double q = x * inv;
             return fma(fma(-q, det, x), inv, q);
