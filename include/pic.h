@@ -75,7 +75,11 @@ typedef struct {
     int32_t precision;            /* PIC_FP64, or PIC_MIXED: the first Picard iterations of each step
                                      in FP32 (orbit integrals, push, scatter; mesh solve and sums in
                                      FP64), then FP64 iterations to picard_tol and the FP64 final
-                                     sweep; needs n_a <= 1024 */
+                                     sweep; needs n_a <= 1024.  The FP64 closed forms sum parts of
+                                     their products in 64-bit fixed point: an orbit piece's impulse
+                                     to a few 2^-55 of its cell's largest field difference times the
+                                     particle's largest velocity component, a cell's current to a
+                                     few 2^-57 of the largest deposit in it */
     int32_t sort_every;           /* re-sort particles by cell every k steps (0: never) */
     int32_t diagnostics;          /* 1: accumulate the §5.1-§5.3 diagnostics during each step */
     int32_t accept_unconverged;   /* 1: commit a step that hit p_max (Algorithm 1 as printed) */
