@@ -333,10 +333,10 @@ __device__ __forceinline__ void cell_nodes8(const int c[3], const MeshDims& m, i
 
 // Where the particle kernels take a cell's entries from: the FP64 cell table; the gather table, taking the
 // differences of the cell's nodes each time (contexts without cell tables); or, in deterministic mode, the cell
-// table where there is one and the gather table where not, by the same instructions but for the loads.  The
-// differences are the same numbers (subtractions in the same order), so that the bits do not depend on
-// whether the table's memory was there.  24^3, 442,368 particles: 4.4 ms a step with the table, 9.6 without
-// (15.0 when each entry was made at its use); the loads through a generic pointer cost 7% beside FROM_CELLS.
+// table where there is one and the gather table where not, with the same bits: the differences are the same
+// numbers (subtractions in the same order), and what is made of them is integers (orbit_fixed.cuh) or runs
+// through the same instructions.  24^3, 442,368 particles: 4.1 ms a step with the table, 7.9 without (9.95
+// before there were tables).
 enum Fields { FROM_NODES, FROM_CELLS, FROM_EITHER };
 
 struct FieldTables {

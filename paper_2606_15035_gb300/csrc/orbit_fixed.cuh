@@ -23,19 +23,14 @@ namespace pic {
 constexpr int FX_FIELD_UP = 5;   // fixed_of's shift for the table: 58 bits
 constexpr int FX_V_UP = 9;       // ... for velocities: 62 bits
 
-// Loader of a cell's entries (FROM_CELLS, or in deterministic mode FROM_EITHER: from the gather table where
-// there is no fixed-point table, the same integers).  The entries k = 0 of the A columns are not used; two of
-// them hold the exponents of the cell's groups.
-template <int FROM>
-struct FixedLoad;
-
 struct FixedTables {
     const double* nodes;      // gather table
     const longlong2* cells;   // fixed-point cell table
 };
 
-template <>
-struct FixedLoad<FROM_CELLS> {
+// Loader of a cell's entries from the fixed-point table, or from a copy of the cell's part of it.  The
+// entries k = 0 of the A columns are not used; two of them hold the exponents of the cell's groups.
+struct FixedLoad {
     const longlong2* t;
     __device__ __forceinline__ FixedLoad(FixedTables ft, const int c[3], const MeshDims& m)
         : t(ft.cells + (CELL_VALUES / 2) * cell_row(c, m)) {}
@@ -48,42 +43,28 @@ struct FixedLoad<FROM_CELLS> {
     __device__ __forceinline__ int top_g() const { return (int)__ldg(&t[1].x); }
 };
 
-// A cell's entries as its fixed-point table has them, from the gather table.
-static __device__ __noinline__ void fixed_of_nodes(const double* nodes, int c0, int c1, int c2, int n0, int n1, int n2,
-                                                   longlong2* out) {
-    double2 q[CELL_VALUES / 2];
-    entries_of_nodes(nodes, c0, c1, c2, n0, n1, n2, q);
-    int top[2] = {64, 64};
-    for (int k = 0; k < CELL_VALUES / 2; ++k) {
-        const int col = k % CELL_COLS;
-        const int e = max(k < 6 ? 0 : exponent_of(q[k].x), exponent_of(q[k].y));
-        if (col < 6) top[0] = max(top[0], e);
-        else top[1] = max(top[1], e);
-    }
-    for (int k = 0; k < CELL_VALUES / 2; ++k) {
-        const int e = k % CELL_COLS < 6 ? top[0] : top[1];
-        out[k].x = k < 2 ? top[k] : (k < 6 ? 0 : fixed_of(q[k].x, e, FX_FIELD_UP));
-        out[k].y = fixed_of(q[k].y, e, FX_FIELD_UP);
-    }
-}
-
-template <>
-struct FixedLoad<FROM_EITHER> {
-    const longlong2* t;                   // the table's entries, or own
-    longlong2 own[CELL_VALUES / 2];
-    __device__ __forceinline__ FixedLoad(FixedTables ft, const int c[3], const MeshDims& m) {
-        if (__builtin_expect(ft.cells != nullptr, 1)) {
-            t = ft.cells + (CELL_VALUES / 2) * cell_row(c, m);
-        } else {
-            fixed_of_nodes(ft.nodes, c[0], c[1], c[2], m.n[0], m.n[1], m.n[2], own);
-            t = own;
+// A cell's entries as the fixed-point table has them, made from the gather table.
+struct FixedOfNodes {
+    longlong2 t[CELL_VALUES / 2];
+    __device__ __forceinline__ FixedOfNodes(const double* nodes, const int c[3], const int n[3]) {
+        double2 q[CELL_VALUES / 2];
+        entries_of_nodes(nodes, c[0], c[1], c[2], n[0], n[1], n[2], q);
+        int top[2] = {64, 64};
+        for (int k = 0; k < CELL_VALUES / 2; ++k) {
+            const int col = k % CELL_COLS;
+            const int e = max(k < 6 ? 0 : exponent_of(q[k].x), exponent_of(q[k].y));
+            if (col < 6) top[0] = max(top[0], e);
+            else top[1] = max(top[1], e);
+        }
+        for (int k = 0; k < CELL_VALUES / 2; ++k) {
+            const int e = k % CELL_COLS < 6 ? top[0] : top[1];
+            t[k].x = k < 2 ? top[k] : (k < 6 ? 0 : fixed_of(q[k].x, e, FX_FIELD_UP));
+            t[k].y = fixed_of(q[k].y, e, FX_FIELD_UP);
         }
     }
-    FixedLoad(const FixedLoad&) = delete;
     __device__ __forceinline__ void operator()(int p, int col, long long& a, long long& b) const {
-        const longlong2 q = t[p * CELL_COLS + col];
-        a = q.x;
-        b = q.y;
+        a = t[p * CELL_COLS + col].x;
+        b = t[p * CELL_COLS + col].y;
     }
     __device__ __forceinline__ int top_A() const { return (int)t[0].x; }
     __device__ __forceinline__ int top_g() const { return (int)t[1].x; }
@@ -209,6 +190,38 @@ __device__ __forceinline__ void cell_A1_fixed(const double r[3], const L& ld, lo
         s.add(fs_of(k7), xyz);
         out[c] = s.value();
     }
+}
+
+// The same two from the gather table, for deterministic runs whose cell tables were refused: integers and
+// single FP64 multiply-adds throughout, so that the bits are those of the table's (values in and out, which keeps
+// the callers' in registers).
+struct PieceSums {
+    double F[3], G[3];
+};
+struct PieceOrbit {
+    double h, sm, mid[3], d[3];
+    Fs v[3];
+    int ev, c[3], n[3];
+};
+static __device__ __noinline__ PieceSums piece_impulse_of_nodes(const double* nodes, PieceOrbit o, PieceSums s) {
+    const FixedOfNodes ld(nodes, o.c, o.n);
+    piece_impulse_fixed(o.h, o.sm, o.mid, o.d, o.v, o.ev, ld, s.F, s.G);
+    return s;
+}
+
+struct CellA1 {
+    long long a[3];
+    int top;
+};
+static __device__ __noinline__ CellA1 cell_A1_of_nodes(const double* nodes, int c0, int c1, int c2, int n0, int n1, int n2,
+                                                       double r0, double r1, double r2) {
+    const int c[3] = {c0, c1, c2}, n[3] = {n0, n1, n2};
+    const double r[3] = {r0, r1, r2};
+    const FixedOfNodes ld(nodes, c, n);
+    CellA1 A;
+    cell_A1_fixed(r, ld, A.a);
+    A.top = ld.top_A();
+    return A;
 }
 
 }  // namespace pic

@@ -695,19 +695,37 @@ __device__ __forceinline__ void push_eval_cell(const StepParams& p, CellStart<do
         for (int a = 0; a < 3; ++a) v[a] = fs_of(fixed_of(vs[a], ev, FX_V_UP));
         o.nseg = for_each_piece(st, beta, p.m, [&](double h, double sm, const double mid[3], const int c[3]) {
             const double d[3] = {h * beta[0], h * beta[1], h * beta[2]};
-            piece_impulse_fixed(h, sm, mid, d, v, ev, FixedLoad<FROM>(ft, c, p.m), accF, accG);
+            if (FROM == FROM_CELLS || ft.cells) {
+                piece_impulse_fixed(h, sm, mid, d, v, ev, FixedLoad(ft, c, p.m), accF, accG);
+            } else {
+                const PieceOrbit o = {h, sm, {mid[0], mid[1], mid[2]}, {d[0], d[1], d[2]}, {v[0], v[1], v[2]},
+                                      ev, {c[0], c[1], c[2]}, {p.m.n[0], p.m.n[1], p.m.n[2]}};
+                const PieceSums s = piece_impulse_of_nodes(
+                    ft.nodes, o, PieceSums{{accF[0], accF[1], accF[2]}, {accG[0], accG[1], accG[2]}});
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    accF[a] = s.F[a];
+                    accG[a] = s.G[a];
+                }
+            }
         });
-        const FixedLoad<FROM> ld(ft, st.c, p.m);
-        long long A1[3];
-        cell_A1_fixed(st.f, ld, A1);
+        CellA1 A1;
+        if (FROM == FROM_CELLS || ft.cells) {
+            const FixedLoad ld(ft, st.c, p.m);
+            cell_A1_fixed(st.f, ld, A1.a);
+            A1.top = ld.top_A();
+        } else {
+            A1 = cell_A1_of_nodes(ft.nodes, st.c[0], st.c[1], st.c[2], p.m.n[0], p.m.n[1], p.m.n[2], st.f[0], st.f[1],
+                                  st.f[2]);
+        }
         // values that are not finite stay so (the start's coordinate: the end's is its sum with beta)
         const int ef = max(max(exponent_of(st.f[0]), exponent_of(st.f[1])), exponent_of(st.f[2]));
         const double dtq = max(ev, ef) < 0x7ff ? p.dtq : NAN;
-        const double uA = pow2_biased(ld.top_A() - 57);
+        const double uA = pow2_biased(A1.top - 57);
         const double* low = ft.nodes + 12 * cell_row(st.c, p.m) + 3;   // A^{n+1} at the cell's lowest node
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            o.Ae[a] = __ldg(low + a) + uA * (double)A1[a];
+            o.Ae[a] = __ldg(low + a) + uA * (double)A1.a[a];
             o.Pw[a] = Pn[a] + dtq * (accG[a] + p.ihs[a] * accF[a]);
         }
     } else {
