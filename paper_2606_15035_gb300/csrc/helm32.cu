@@ -370,7 +370,9 @@ int plane_lines(const MeshDims& m, int sms) {
     while (lb > 1 && (lb * plane > PLANE || 2 * ((m.n[0] + lb - 1) / lb) < sms / 2)) lb /= 2;
     return lb;
 }
-int plane_threads(int64_t elements) { return (int)std::max<int64_t>(64, std::min<int64_t>(512, (elements / 4 + 31) / 32 * 32)); }
+int plane_threads(int64_t elements) {
+    return (int)std::max<int64_t>(64, std::min<int64_t>(512, (elements / 4 + 31) / 32 * 32));
+}
 
 }  // namespace
 
@@ -421,7 +423,8 @@ int helm32_solve(const HelmPlan& c, const double* b, double* x, const int* top, 
         h.up = 20 * k;   // each correction leaves a residual some 2^20 smaller
         k_helm_x<false><<<gx, 256, smem(ax), stream>>>(h, ax);
         if (fused) {
-            k_helm_plane<<<dim3((c.m.n[0] + lb - 1) / lb, 2), plane_threads(lb * plane), 2 * sizeof(float2) * lb * plane, stream>>>(h, ay, az, lb);
+            k_helm_plane<<<dim3((c.m.n[0] + lb - 1) / lb, 2), plane_threads(lb * plane),
+                           2 * sizeof(float2) * lb * plane, stream>>>(h, ay, az, lb);
             k_helm_x<true><<<gx, 256, smem(ax), stream>>>(h, ax);
             continue;
         }

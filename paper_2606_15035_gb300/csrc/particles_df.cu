@@ -95,8 +95,8 @@ struct PairLoad<false> {
 
 // The FP32-pair iteration (239 -> 88.5 ms at 128^3 with 134M particles, from start-based integrals, a
 // node table and shared 64-bit atomics before; 70.9 with the one-crossing walk, deposit columns by cell and
-// blocks of eight warps, 73.0 with the deposits' units by cell): G(v^p) for every particle, creeping ones listed for k_local (as in
-// k_push_cell), the e_v partial sums, and the orbit current of v^{p+1} = G(v^p) into Jnext.
+// blocks of eight warps, 73.0 with the deposits' units by cell): G(v^p) for every particle, creeping ones
+// listed for k_local (as in k_push_cell), the e_v partial sums, and the orbit current of v^{p+1} = G(v^p) into Jnext.
 template <bool CELLS, typename Chunk>
 __global__ void __launch_bounds__(Chunk::THREADS_, 32 * DF_WARPS / Chunk::THREADS_) k_push_df(ParamsDF pd, const double* __restrict__ xi,
                                                                const double* __restrict__ v,

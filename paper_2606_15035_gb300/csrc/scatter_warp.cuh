@@ -8,8 +8,8 @@
 // 2^-57 of the largest that the warp adds to the same cell, and exact sums.  A cell's sum so has an error of
 // a few 2^-57 of its largest deposit, where FP64 rounds each product at 2^-53 and J at every addition; a
 // slow particle in a cell of its own keeps all its bits beside fast ones in others.  The warp's particles
-// hold few distinct cells (the store is cell-sorted), so each cell's 24 sums (8 moments, 3 components) are taken by 24 lanes from a
-// transposed shared tile, turned into node weights by three exchanges, and added to J once.
+// hold few distinct cells (the store is cell-sorted), so each cell's 24 sums (8 moments, 3 components) are
+// taken by 24 lanes from a transposed shared tile, turned into node weights by three exchanges, and added to J once.
 #pragma once
 
 #include "fixed.cuh"
